@@ -67,14 +67,13 @@ __device__ __forceinline__ DF operator*(DF a, DF b) {
   e = __fmaf_rn(a.lo, b.hi, e);
   return df_fast_two_sum(p, e);
 }
-// a * b + c with one normalisation.  Generic code calls fma, sqrt, fabs and
-// sincos unqualified; the using-declarations keep the float and double
+// a * b + c with one normalisation.  Generic code calls fma, sqrt and
+// fabs unqualified; the using-declarations keep the float and double
 // overloads visible next to the double-float ones declared here (otherwise
 // those would hide them, and a float argument would convert to DF).
 using ::fma;
 using ::sqrt;
 using ::fabs;
-using ::sincos;
 __device__ __forceinline__ DF fma(DF a, DF b, DF c) {
   const float p = __fmul_rn(a.hi, b.hi);
   float e = __fmaf_rn(a.hi, b.hi, -p);
@@ -132,60 +131,6 @@ __device__ __forceinline__ DF sqrt(DF a) {
   const DF y = df_fast_two_sum(s, __fdiv_rn(d, __fadd_rn(s, s)));
   const DF r = a - y * y;
   return y + DF(__fdiv_rn(r.hi, __fadd_rn(y.hi, y.hi)));
-}
-
-// sin and cos of a double-float argument.  Arguments beyond pi/4 are first
-// reduced by n pi/2 (Cody and Waite's additive reduction, with pi/2 split
-// into three floats; the first two products are formed exactly), then the
-// Taylor series run on y / 2^k, |y / 2^k| <= 1/8, followed by k double-angle
-// steps (sin 2y = 2 sin y cos y, cos 2y = 1 - 2 sin^2 y), and the quadrant
-// n mod 4 permutes the result.  The series stop at y^11 and y^10: the first
-// omitted terms are below 3e-20 of the result.  A truncation error has one
-// sign, so it must stay far below the rounding: stopping one term earlier
-// (cos short by up to 2.6e-16) made every exp(iA) shrink the links by
-// ~1e-15, and over 16 drifts of 4.2 M links that moved S by ~1e-6 on 32^4.
-// Each doubling at most doubles the absolute rounding error and k <= 3
-// after the reduction, so the error stays near 3e-14 plus the 2^-48 |x| that
-// the argument itself carries.  Arguments here are rotation angles of link
-// updates, usually below 1.
-__device__ __forceinline__ void sincos(DF x, DF* s, DF* c) {
-  int quadrant = 0;
-  if (fabsf(x.hi) > 0.785398163f) {
-    const float n = rintf(__fmul_rn(x.hi, 0.636619772f));  // round(2 x / pi)
-    constexpr float p1 = 1.57079637050628662109375f, p2 = -4.37113882867379300296306610107421875e-8f,
-                    p3 = -1.71512451000588190e-15f;         // p1 + p2 + p3 = pi/2 to ~1e-23
-    const float q1 = __fmul_rn(n, p1), q2 = __fmul_rn(n, p2);
-    x = x - DF(q1, __fmaf_rn(n, p1, -q1));
-    x = x - DF(q2, __fmaf_rn(n, p2, -q2));
-    x = x - DF(__fmul_rn(n, p3));
-    quadrant = (int)n & 3;
-  }
-  // k = max(0, e + 3) with |x.hi| = m 2^e, m in [0.5, 1)
-  const int e = (int)((__float_as_uint(x.hi) >> 23) & 0xffu) - 126;
-  const int k = e + 3 > 0 ? (e + 3 < 60 ? e + 3 : 60) : 0;
-  const float sc = __uint_as_float((uint32_t)(127 - k) << 23);  // 2^-k, exact scaling
-  const DF y(__fmul_rn(x.hi, sc), __fmul_rn(x.lo, sc));
-  const DF z = y * y;
-  constexpr DF s3(-1.0 / 6.0), s5(1.0 / 120.0), s7(-1.0 / 5040.0), s9(1.0 / 362880.0), s11(-1.0 / 39916800.0);
-  constexpr DF c4(1.0 / 24.0), c6(-1.0 / 720.0), c8(1.0 / 40320.0), c10(-1.0 / 3628800.0);
-  DF ps = fma(z, s11, s9);
-  ps = fma(z, ps, s7);
-  ps = fma(z, ps, s5);
-  ps = fma(z, ps, s3);
-  DF sn = fma(y * z, ps, y);
-  DF pc = fma(z, c10, c8);
-  pc = fma(z, pc, c6);
-  pc = fma(z, pc, c4);
-  DF cs = fma(z * z, pc, DF(1.0f) - z * 0.5f);
-  for (int i = 0; i < k; ++i) {
-    const DF s2 = sn * sn;
-    sn = (sn * cs) * 2.0f;
-    cs = DF(1.0f) - s2 * 2.0f;
-  }
-  // sin(y + n pi/2), cos(y + n pi/2)
-  const DF ms = -sn, mc = -cs;
-  *s = quadrant == 0 ? sn : (quadrant == 1 ? cs : (quadrant == 2 ? ms : mc));
-  *c = quadrant == 0 ? cs : (quadrant == 1 ? ms : (quadrant == 2 ? mc : sn));
 }
 
 // Storage: one complex double-float is a float4 (re.hi, re.lo, im.hi, im.lo),
@@ -246,112 +191,18 @@ __device__ __forceinline__ void block_reduce_store_df(DF v[NV], double* __restri
   }
 }
 
-// exp(i A) for Hermitian traceless A in double-float: the closed form of
-// Morningstar and Peardon (Phys. Rev. D 69 (2004) 054501, section III),
-// exp(iA) = f0 + f1 A + f2 A^2, as in the generic expi_herm, with the
-// scalars computed to double-float accuracy on the FP32 pipes:
-//   * 2u, the largest eigenvalue of A for c0 = det A >= 0 (negative c0 is
-//     mapped through f_j(-c0) = (-1)^j conj(f_j(c0))), is a simple root of the
-//     characteristic polynomial lambda^3 - c1 lambda - c0 separated from the
-//     others by at least sqrt(c1); it starts from the FP32 angle formula and
-//     takes two Newton steps in double-float (1e-7 -> 1e-14 -> rounding);
-//   * w^2 = c1 - 3 u^2 (the eigenvalues are 2u and -u +- w, and
-//     c1 = Tr A^2 / 2 = 3 u^2 + w^2), so cos w and sin(w)/w, the only
-//     functions of w that enter, are even in w and need no angle;
-//   * sin and cos by the double-float series above.
-// Below c1 = 1e-12 (|A| < 1.5e-6) the exponential series to A^4 is used, with
-// A^3 = c1 A + c0 and A^4 = c1 A^2 + c0 A (Cayley-Hamilton); the omitted
-// terms are below |A|^5 / 120 < 1e-31.
-template <>
-__device__ __forceinline__ M3<DF> expi_herm<DF>(const M3<DF>& a) {
-  const M3<DF> a2 = herm_sq(a);
-  const DF c1 = (a2.e[0][0].re + a2.e[1][1].re + a2.e[2][2].re) * 0.5f;
-  constexpr DF third(1.0 / 3.0), sixth(1.0 / 6.0), c24(1.0 / 24.0);
-  const DF c0 = re_tr_mul(a, a2) * third;
-  Cx<DF> f0, f1, f2;
-  if (c1.hi < 1e-12f) {
-    f0 = cx<DF>(DF(1.0f), -(c0 * sixth));
-    f1 = cx<DF>(c0 * c24, DF(1.0f) - c1 * sixth);
-    f2 = cx<DF>(DF(-0.5f) + c1 * c24, DF(0.0f));
-  } else {
-    const bool neg = c0.hi < 0.0f;
-    const DF c0a = neg ? -c0 : c0;
-    // FP32 seed: u = r cos(theta / 3), r = sqrt(c1 / 3), cos theta = c0 / (2 r^3)
-    const float r32 = sqrtf(c1.hi * (1.0f / 3.0f));
-    const float ratio = fminf(c0a.hi / (2.0f * r32 * r32 * r32), 1.0f);
-    DF lam(2.0f * r32 * cosf(acosf(ratio) * (1.0f / 3.0f)));
+// Horner's rule of exp_coeffs in double-float, to order 16 (the first
+// omitted term is below 1e-17, far below the rounding, as it must be: a
+// truncation error has one sign).  Orders 16 to 10 contribute less than 2e-9
+// and run in FP32 (1e-16); a conversion to double-float follows.
+template <> __device__ __forceinline__ void exp_coeffs<DF>(DF c0, DF c1, Cx<DF> f[3]) {
+  Cx<float> q[3] = {cx<float>(0.0f, 0.0f), cx<float>(0.0f, 0.0f), cx<float>(0.0f, 0.0f)};
+  exp_horner<float, 16, 10>(c0.hi, c1.hi, q);
 #pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      const DF l2 = lam * lam;
-      const DF pv = (l2 - c1) * lam - c0a;
-      const DF dp = l2 * 3.0f - c1;
-      // the correction is ~1e-7 of lam or less: FP32 accuracy suffices
-      lam = lam - DF(__fdiv_rn(pv.hi, dp.hi));
-    }
-    const DF u = lam * 0.5f;
-    const DF u2 = u * u;
-    DF w2 = c1 - u2 * 3.0f;
-    if (w2.hi < 0.0f) w2 = DF(0.0f);
-    const DF w = sqrt(w2);
-    // sin and cos of u and of w through one copy of the series code (two
-    // inlined copies cost instruction-cache misses in the force kernel)
-    DF su, cu, sw, cw;
-#pragma unroll 1
-    for (int i = 0; i < 2; ++i) {
-      DF sv, cv;
-      sincos(i ? w : u, &sv, &cv);
-      if (i) {
-        sw = sv;
-        cw = cv;
-      } else {
-        su = sv;
-        cu = cv;
-      }
-    }
-    DF xi0;
-    if (w2.hi < 0.0025f) {
-      // |w| < 0.05: sin(w)/w from its series in w^2 (first omitted term
-      // below 3e-21), not from a quotient of small numbers
-      constexpr DF x2(-1.0 / 6.0), x4(1.0 / 120.0), x6(-1.0 / 5040.0), x8(1.0 / 362880.0);
-      DF q = fma(w2, x8, x6);
-      q = fma(w2, q, x4);
-      q = fma(w2, q, x2);
-      xi0 = fma(w2, q, DF(1.0f));
-    } else {
-      xi0 = sw / w;
-    }
-    const DF s2u = (su * cu) * 2.0f;
-    const DF c2u = (cu - su) * (cu + su);
-    const Cx<DF> e2 = cx<DF>(c2u, s2u);
-    const Cx<DF> em = cx<DF>(cu, -su);
-    const DF u2x3 = u2 * 3.0f;
-    const Cx<DF> h0 = cx<DF>(u2 - w2, DF(0.0f)) * e2 +
-                      em * cx<DF>(u2 * cw * 8.0f, (u * (u2x3 + w2) * xi0) * 2.0f);
-    const Cx<DF> h1 = cx<DF>(u * 2.0f, DF(0.0f)) * e2 - em * cx<DF>((u * cw) * 2.0f, -((u2x3 - w2) * xi0));
-    const Cx<DF> h2 = e2 - em * cx<DF>(cw, (u * xi0) * 3.0f);
-    const DF inv = DF(1.0f) / (u2 * 9.0f - w2);
-    f0 = inv * h0;
-    f1 = inv * h1;
-    f2 = inv * h2;
-    if (neg) {
-      f0 = conj(f0);
-      f1 = cx<DF>(-f1.re, f1.im);
-      f2 = conj(f2);
-    }
-  }
-  M3<DF> e;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      Cx<DF> s = f1 * a.e[i][j];
-      cmac(s, f2, a2.e[i][j]);
-      if (i == j) s = s + f0;
-      e.e[i][j] = s;
-    }
-  return e;
+  for (int j = 0; j < 3; ++j) f[j] = cx<DF>(DF(q[j].re), DF(q[j].im));
+  exp_horner<DF, 9, 0>(c0, c1, f);
 }
-
+template <> __device__ __forceinline__ int exp_halvings<DF>(DF c1) { return exp_halvings(c1.hi); }
 
 // ---------------------------------------------------------------------------
 // Products of SU(3) matrices in double-float with an anchored accumulator.

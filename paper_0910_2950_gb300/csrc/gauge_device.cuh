@@ -114,6 +114,21 @@ __device__ __forceinline__ M3<R> staple_sum(const Gauge<R, NC>& U, const Geom& g
   return a;
 }
 
+// Stores exp(i P) u, re-projected onto SU(3) if reunit is set (then rows 0
+// and 1 of the product suffice).
+template <typename R, int NC>
+__device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const Gauge<R, NC>& Uout, int mu, int s,
+                                            int reunit) {
+  const M3<R> e = expi_herm(alg_to_mat(p));
+  if (reunit) {
+    M3<R> un = mul_rows01(e, u);
+    reunitarize(un);
+    Uout.store(mu, s, un);
+  } else {
+    Uout.store(mu, s, link_mul(e, u));
+  }
+}
+
 // Everything after the staple sum a of U_mu(x): the force, then what MODE
 // does with it on this link.
 template <typename R, int NC, int MODE>
@@ -160,11 +175,7 @@ __device__ __forceinline__ void force_finish(const Gauge<R, NC>& U, const Mom<R>
     if (MODE == FM_KICK_DRIFT) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) p[k] *= cdrift;
-      const M3<R> e = expi_herm(alg_to_mat(p));
-      const M3<R> ub = (Ubase.p == U.p) ? ul : Ubase.load(mu, s);
-      M3<R> un = link_mul(e, ub);
-      if (reunit) reunitarize(un);
-      Uout.store(mu, s, un);
+      drift_store(p, (Ubase.p == U.p) ? ul : Ubase.load(mu, s), Uout, mu, s, reunit);
     }
   } else {  // FM_DISPLACE
     // The displaced links only serve one force evaluation and are then
@@ -322,10 +333,7 @@ __device__ __forceinline__ void drift_link(const Gauge<R, NC>& Uin, const Mom<R>
   P.load(mu, s, p);
 #pragma unroll
   for (int k = 0; k < 8; ++k) p[k] *= c;
-  const M3<R> e = expi_herm(alg_to_mat(p));
-  M3<R> un = link_mul(e, Uin.load(mu, s));
-  if (reunit) reunitarize(un);
-  Uout.store(mu, s, un);
+  drift_store(p, Uin.load(mu, s), Uout, mu, s, reunit);
 }
 
 // Per-site energy h(x) = T(x) + S_G(x) (T = 0 if P is null), with
