@@ -756,6 +756,7 @@ def precision_measurement(fg, stream, rank, L=16, n_time=5):
         lat.timing_reset()
         lat.trajectory("fg", 0.25, TAU, refresh=True, u_accept=0.0)
         f_ms, f_n = lat.kernel_time("gauge_force")
+        f_ms += lat.kernel_time("plaquette")[0]   # the other launch of a force in FP64 and double-float
         lat.timing(False)
         lat.close()
         esize = 4 if prec == "fp32" else 8

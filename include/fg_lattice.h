@@ -193,7 +193,9 @@ void fg_lattice_destroy(fg_lattice *h);
 const char *fg_last_error(const fg_lattice *h);
 
 /* Gauge field in and out (host layout above).  fg_set_gauge does not check
- * unitarity; links are stored in the handle's precision. */
+ * unitarity; links are stored in the handle's precision.  They are taken to
+ * be special unitary to rounding: 12-real storage rebuilds a row from the
+ * other two, and the FP64 and double-float forces use U^dagger U = 1. */
 fg_status fg_set_gauge(fg_lattice *h, const double *host_links);
 fg_status fg_get_gauge(fg_lattice *h, double *host_links);
 
@@ -325,7 +327,9 @@ fg_status fg_reunitarize(fg_lattice *h);
  * precision), "cg_blas", "fermion_force", "convert", "dslash_fp64" (the
  * FP64-arithmetic Dslash of the heat bath, of fg_apply_mhat and of the
  * reliable update that certifies convergence), "dslash_df" (the
- * double-float Dslash of the FP32 solver's other reliable updates). */
+ * double-float Dslash of the FP32 solver's other reliable updates),
+ * "plaquette" (the plaquette products of an FP64 or FG_DF64 force
+ * evaluation, launched before its "gauge_force"). */
 fg_status fg_timing_enable(fg_lattice *h, int on);
 fg_status fg_timing_reset(fg_lattice *h);
 fg_status fg_kernel_time(fg_lattice *h, const char *kernel_class, double *total_ms,

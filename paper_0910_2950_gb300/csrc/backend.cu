@@ -70,6 +70,10 @@ class Backend final : public IBackend {
     U_ = buf_[0];
     if ((s = alloc(&P_, mom_bytes)) != FG_OK) return s;
     if ((s = alloc(&F_, mom_bytes)) != FG_OK) return s;
+    if (kPlaquetteForce<R>) {
+      if ((s = alloc(&W_, (size_t)6 * 4 * V * sizeof(C2))) != FG_OK) return s;
+      if ((s = init_force_rows()) != FG_OK) return s;
+    }
     if ((s = alloc((void**)&h0_, V * sizeof(double))) != FG_OK) return s;
     for (int k = 0; k < 2; ++k)
       if ((s = alloc((void**)&sgc_[k], V * sizeof(double))) != FG_OK) return s;
@@ -425,6 +429,8 @@ class Backend final : public IBackend {
   void* U_ = nullptr;
   void* P_ = nullptr;
   void* F_ = nullptr;
+  ForceRows rows_{};
+  void* W_ = nullptr;   // plaquette field of the force evaluation in progress
   double* h0_ = nullptr;
   // per-site gauge action of the current links (sgc_[sgc_cur_]) and of the
   // end of the running trajectory (the other one); valid while only
@@ -539,6 +545,19 @@ class Backend final : public IBackend {
   int solves_ = 0;
   long long cg_iters_ = 0;
 
+  // Lattice description of the plaquette-form force launches.
+  fg_status init_force_rows() {
+    std::vector<char> cd(chain_bytes());
+    fill_chain(cd.data(), g_, h_->prm.beta, 0, 0, 0, 0, 0);
+    void* chain;
+    fg_status s;
+    if ((s = alloc(&chain, cd.size())) != FG_OK) return s;
+    if (cudaMemcpyAsync(chain, cd.data(), cd.size(), cudaMemcpyHostToDevice, st_) != cudaSuccess)
+      return cuda_fail("lattice description upload");
+    rows_ = ForceRows{chain, nullptr, (g_.Vh + 31) / 32};
+    return sync();  // the host copy goes out of scope
+  }
+
   size_t gauge_bytes() const { return (size_t)4 * NC * g_.V * sizeof(C2); }
   int nvec() const { return 12 * g_.Vh; }
 
@@ -624,6 +643,7 @@ class Backend final : public IBackend {
     ForceArgs a;
     std::memset(&a, 0, sizeof(a));
     a.U = Uf;
+    a.W = W_;
     a.P = P_;
     a.Ubase = Uf;
     a.beta = h_->prm.beta;
@@ -655,22 +675,26 @@ class Backend final : public IBackend {
     return e ? e[0] == '1' : std::is_same<R, DF>::value;
   }();
   fg_status gauge_launch(int mode, const ForceArgs& a) {
+    if constexpr (kPlaquetteForce<R>) {
+      const fg_status w = run(KC_PLAQUETTE, [&] { return launch_plaquettes<R, NC>(rows_, a.U, W_, st_); });
+      if (w != FG_OK) return w;
+    }
     if (split_exp_ && (mode == FM_KICK_DRIFT || mode == FM_DISPLACE)) {
       ForceArgs f = a;
       fg_status s;
       if (mode == FM_KICK_DRIFT) {
-        if ((s = run(KC_GAUGE_FORCE, [&] { return launch_gauge_force<R, NC>(g_, FM_KICK, f, st_); })) != FG_OK)
+        if ((s = run(KC_GAUGE_FORCE, [&] { return launch_gauge_force<R, NC>(g_, rows_, FM_KICK, f, st_); })) != FG_OK)
           return s;
         return run(KC_DRIFT, [&] {
           return launch_drift<R, NC>(g_, a.Ubase, P_, a.Uout, a.cdrift, a.reunit, st_);
         });
       }
       f.F = F_;
-      if ((s = run(KC_GAUGE_FORCE, [&] { return launch_gauge_force<R, NC>(g_, FM_STORE, f, st_); })) != FG_OK)
+      if ((s = run(KC_GAUGE_FORCE, [&] { return launch_gauge_force<R, NC>(g_, rows_, FM_STORE, f, st_); })) != FG_OK)
         return s;
       return run(KC_DRIFT, [&] { return launch_drift<R, NC>(g_, a.U, F_, a.Uout, -a.cdisp, 0, st_); });
     }
-    return run(KC_GAUGE_FORCE, [&] { return launch_gauge_force<R, NC>(g_, mode, a, st_); });
+    return run(KC_GAUGE_FORCE, [&] { return launch_gauge_force<R, NC>(g_, rows_, mode, a, st_); });
   }
 
   fg_status ensure_fg_buffers() {

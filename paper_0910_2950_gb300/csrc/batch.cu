@@ -34,15 +34,6 @@
 
 namespace fg {
 
-struct ChainDesc {
-  Geom g;
-  long long goff;  // byte offset of the chain's links in a link buffer
-  long long moff;  // byte offset of its momenta
-  long long soff;  // offset of its sites in per-site arrays
-  double beta;
-  int tile0, ntiles;
-};
-
 struct Tile {
   int chain;
   int i0;  // first half-site index of the tile
@@ -60,72 +51,52 @@ __device__ __forceinline__ bool tile_site(const Tile& t, const Geom& g, int& s) 
   return true;
 }
 
+// FP32 force: one block a tile, its warps 8 H / 32 of the tile's links, with
+// the registers of the single-lattice kernel.
 template <int H> struct TileBounds;
 template <> struct TileBounds<16> { static constexpr int min_blocks = 4; };
 template <> struct TileBounds<32> { static constexpr int min_blocks = 2; };
 template <> struct TileBounds<64> { static constexpr int min_blocks = 1; };
-// Register cap of the force kernel: 128 per thread for FP32 and FP64 links;
-// double-float links get up to 255 (as in the single-lattice kernel).
-template <typename R, int H>
-constexpr int kBatchMinBlocks =
-    std::is_same<R, DF>::value ? (H == 16 ? 2 * FG_FORCE_DF_MIN_BLOCKS : FG_FORCE_DF_MIN_BLOCKS) : TileBounds<H>::min_blocks;
 
-// Double-float links: a block barrier after each tile keeps the warps of an
-// SM on the same tile.  Left to drift apart, some warps run the staple
-// products while others run the exponential, and the two long code paths
-// together overflow the instruction cache: a 64-chain FG trajectory took
-// 80 ms without the barrier and 45 ms with it.  FG_BATCH_TILE_SYNC (tuning
-// macro): 0 no barrier, 1 double-float only, 2 also FP32.
-#ifndef FG_BATCH_TILE_SYNC
-#define FG_BATCH_TILE_SYNC 1
-#endif
-template <typename R>
-constexpr bool kTileSync =
-    (std::is_same<R, DF>::value && FG_BATCH_TILE_SYNC >= 1) || (std::is_same<R, float>::value && FG_BATCH_TILE_SYNC >= 2);
-
-template <typename R, int NC, int MODE, int H>
-__global__ void __launch_bounds__(8 * H, (kBatchMinBlocks<R, H>))
-    batch_force_kernel(const Tile* __restrict__ tiles, int ntiles, const ChainDesc* __restrict__ chains,
-                       char* U, char* P, char* F, char* Ubase, char* Uout, double ckick, double cdrift, double cdisp,
-                       int reunit) {
+template <int NC, int MODE, int H>
+__global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
+    batch_force_kernel(const Tile* __restrict__ tiles, int ntiles, const ChainDesc* __restrict__ chains, char* U,
+                       char* P, char* F, char* Ubase, char* Uout, float ckick, float cdrift, float cdisp, int reunit) {
   for (int b = blockIdx.x; b < ntiles; b += gridDim.x) {
     const Tile t = tiles[b];
     const ChainDesc& cd = chains[t.chain];
     const Geom g = cd.g;
     int s;
     const bool ok = tile_site<H>(t, g, s);
-    if (!kForceSharedT<R, NC> && !kTileSync<R> && !ok) continue;
-    Gauge<R, NC> u, ub, uo;
+    if (!kForceSharedT<float, NC> && !ok) continue;
+    Gauge<float, NC> u, ub, uo;
     u.p = U + cd.goff; u.V = g.V;
     ub.p = Ubase ? Ubase + cd.goff : nullptr; ub.V = g.V;
     uo.p = Uout ? Uout + cd.goff : nullptr; uo.V = g.V;
-    Mom<R> p, f, ff;
+    Mom<float> p, f, ff;
     p.p = P ? P + cd.moff : nullptr; p.V = g.V;
     f.p = F ? F + cd.moff : nullptr; f.V = g.V;
     ff.p = nullptr; ff.V = g.V;
-    if constexpr (kForceSharedT<R, NC>) {
+    if constexpr (kForceSharedT<float, NC>) {
       // the same staple arithmetic as the single-lattice kernel; the whole
       // block takes the barriers (uniform tile loop)
       extern __shared__ float2 batch_tsh[];
       force_link_shared<NC, MODE, 2 * H>(reinterpret_cast<float2(*)[9][2 * H]>(batch_tsh), ok, s, u, p, f, ff, ub,
-                                         uo, g, R(cd.beta / 6.0), R(ckick), R(cdrift), R(cdisp), reunit, R(1));
+                                         uo, g, cd.beta6_hi, ckick, cdrift, cdisp, reunit, 1.0f);
       __syncthreads();   // the next tile rewrites the slots
     } else {
-      if (ok) {
-        int c[4], par;
-        cb_coords(g, s, c, par);
-        force_link<R, NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, R(cd.beta / 6.0), R(ckick),
-                                R(cdrift), R(cdisp), reunit);
-      }
-      if constexpr (kTileSync<R>) __syncthreads();  // every thread of the block runs the same tiles
+      int c[4], par;
+      cb_coords(g, s, c, par);
+      force_link_staples<NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, cd.beta6_hi, ckick, cdrift, cdisp,
+                                   reunit, 1.0f);
     }
   }
 }
 
 // Dynamic shared memory of batch_force_kernel with H half-sites per tile.
-template <typename R, int NC, int H>
+template <int NC, int H>
 constexpr size_t batch_force_smem() {
-  return kForceSharedT<R, NC> ? (size_t)6 * 9 * 2 * H * sizeof(float2) : 0;
+  return kForceSharedT<float, NC> ? (size_t)6 * 9 * 2 * H * sizeof(float2) : 0;
 }
 
 template <typename R, int NC, int H>
@@ -311,15 +282,12 @@ struct fg_batch {
 
 namespace fg {
 
-static Geom geom_of(const int* d) {
-  Geom g;
+static GeomH geom_of(const int* d) {
+  GeomH g;
   for (int i = 0; i < 4; ++i) g.L[i] = d[i];
   g.V = d[0] * d[1] * d[2] * d[3];
   g.Vh = g.V / 2;
   g.Lxh = d[0] / 2;
-  g.dLxh = make_fastdiv((uint32_t)g.Lxh);
-  g.dLy = make_fastdiv((uint32_t)d[1]);
-  g.dLz = make_fastdiv((uint32_t)d[2]);
   return g;
 }
 
@@ -341,30 +309,27 @@ class Batch final : public IBatch {
   fg_status init() {
     // 64-half-site tiles of the FP32 force kernel use more than the default
     // 48 KB of dynamic shared memory
-    if constexpr (batch_force_smem<R, NC, 64>() > 48 * 1024) {
-      const int bytes = (int)batch_force_smem<R, NC, 64>();
-      if (cudaFuncSetAttribute(batch_force_kernel<R, NC, FM_STORE, 64>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-          cudaFuncSetAttribute(batch_force_kernel<R, NC, FM_KICK, 64>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-          cudaFuncSetAttribute(batch_force_kernel<R, NC, FM_KICK_DRIFT, 64>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-          cudaFuncSetAttribute(batch_force_kernel<R, NC, FM_DISPLACE, 64>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
+    if constexpr (!kPlaquetteForce<R> && batch_force_smem<NC, 64>() > 48 * 1024) {
+      const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+      const int bytes = (int)batch_force_smem<NC, 64>();
+      if (cudaFuncSetAttribute(batch_force_kernel<NC, FM_STORE, 64>, a, bytes) != cudaSuccess ||
+          cudaFuncSetAttribute(batch_force_kernel<NC, FM_KICK, 64>, a, bytes) != cudaSuccess ||
+          cudaFuncSetAttribute(batch_force_kernel<NC, FM_KICK_DRIFT, 64>, a, bytes) != cudaSuccess ||
+          cudaFuncSetAttribute(batch_force_kernel<NC, FM_DISPLACE, 64>, a, bytes) != cudaSuccess)
         return cuda_fail("force kernel shared-memory attribute");
     }
     const int n = b_->prm.nchains;
     std::vector<ChainDesc> cds(n);
-    long long goff = 0, moff = 0, soff = 0;
+    std::vector<int> row_chain;
+    long long goff = 0, moff = 0, woff = 0, soff = 0;
     for (int c = 0; c < n; ++c) {
       ChainDesc& cd = cds[c];
-      cd.g = geom_of(&b_->dims[4 * c]);
-      cd.beta = b_->beta[c];
-      cd.goff = goff;
-      cd.moff = moff;
-      cd.soff = soff;
+      const GeomH gh = geom_of(&b_->dims[4 * c]);
+      fill_chain(&cd, gh, b_->beta[c], goff, moff, woff, soff, (int)row_chain.size());
+      row_chain.insert(row_chain.end(), (gh.Vh + 31) / 32, c);
       goff += align256((long long)4 * NC * cd.g.V * sizeof(C2));
       moff += align256((long long)4 * 4 * cd.g.V * sizeof(C2));
+      woff += align256((long long)6 * 4 * cd.g.V * sizeof(C2));
       soff += cd.g.V;
     }
     gauge_bytes_ = goff;
@@ -377,6 +342,7 @@ class Batch final : public IBatch {
     cur_ = 0;
     if ((s = alloc(&P_, mom_bytes_)) != FG_OK) return s;
     if ((s = alloc(&F_, mom_bytes_)) != FG_OK) return s;
+    if (kPlaquetteForce<R> && (s = alloc(&W_, woff)) != FG_OK) return s;
     if ((s = alloc((void**)&h0_, sites_ * sizeof(double))) != FG_OK) return s;
     if ((s = alloc((void**)&d_out_, (size_t)n * kChainOut * sizeof(double))) != FG_OK) return s;
     if ((s = alloc((void**)&d_acc_, (size_t)n * sizeof(int))) != FG_OK) return s;
@@ -409,6 +375,7 @@ class Batch final : public IBatch {
         return cuda_fail("descriptor upload");
       if ((s = alloc((void**)&d_partial_[hi], (size_t)3 * tl.size() * sizeof(double))) != FG_OK) return s;
     }
+    if (kPlaquetteForce<R> && (s = init_force_rows(row_chain)) != FG_OK) return s;
     if (b_->prm.tile == 16) hsel_ = 0;
     else if (b_->prm.tile == 32) hsel_ = 1;
     else if (b_->prm.tile == 64) hsel_ = 2;
@@ -560,6 +527,8 @@ class Batch final : public IBatch {
   int cur_ = 0;
   void* P_ = nullptr;
   void* F_ = nullptr;
+  void* W_ = nullptr;     // plaquette field of the force evaluation in progress
+  ForceRows rows_{};
   double* h0_ = nullptr;
   ChainDesc* d_chains_h_[3] = {nullptr, nullptr, nullptr};
   Tile* d_tiles_[3] = {nullptr, nullptr, nullptr};
@@ -574,6 +543,18 @@ class Batch final : public IBatch {
   int hsel_ = 1;
   int sms_ = 152;
   std::vector<GraphEntry> graphs_;
+
+  // The rows of all chains for the plaquette-form force launches.
+  fg_status init_force_rows(const std::vector<int>& row_chain) {
+    int* rc;
+    fg_status s;
+    const size_t bytes = row_chain.size() * sizeof(int);
+    if ((s = alloc((void**)&rc, bytes)) != FG_OK) return s;
+    if (cudaMemcpyAsync(rc, row_chain.data(), bytes, cudaMemcpyHostToDevice, st_) != cudaSuccess)
+      return cuda_fail("row list upload");
+    rows_ = ForceRows{d_chains_h_[0], rc, (int)row_chain.size()};
+    return sync();  // the host copy goes out of scope
+  }
 
   static long long align256(long long x) { return (x + 255) & ~255LL; }
   GeomH geomh(int c) const {
@@ -622,42 +603,48 @@ class Batch final : public IBatch {
   // grid of a persistent launch: enough blocks to fill every SM once
   int grid(int ntiles, int blocks_per_sm) const { return std::max(1, std::min(ntiles, sms_ * blocks_per_sm)); }
 
+  // The FP32 force launch over the tiles of H half-sites.
   template <int H>
-  fg_status force_h(int hi, int mode, void* U, void* Ubase, void* Uout, void* F, double ckick, double cdrift,
-                    double cdisp) {
+  fg_status staples_h(int hi, int mode, const ForceArgs& a) {
     const int nt = ntiles_[hi];
     const dim3 blk(2 * H, 4);
-    const int gr = grid(nt, kBatchMinBlocks<R, H>);
-    const int reunit = b_->prm.reunitarize;
-    char* Pp = (char*)P_;
+    const int gr = grid(nt, TileBounds<H>::min_blocks);
     return lrun([&] {
-      const size_t sm = batch_force_smem<R, NC, H>();
+      const size_t sm = batch_force_smem<NC, H>();
       const Tile* tl = d_tiles_[hi];
       const ChainDesc* cds = d_chains_h_[hi];
+#define FG_FORCE(M)                                                                                                \
+  batch_force_kernel<NC, M, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)a.U, (char*)a.P, (char*)a.F, (char*)a.Ubase, \
+                                                     (char*)a.Uout, (float)a.ckick, (float)a.cdrift,              \
+                                                     (float)a.cdisp, a.reunit)
       switch (mode) {
-        case FM_STORE:
-          batch_force_kernel<R, NC, FM_STORE, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)U, Pp, (char*)F,
-                                                                      (char*)Ubase, (char*)Uout, ckick, cdrift,
-                                                                      cdisp, reunit);
-          break;
-        case FM_KICK:
-          batch_force_kernel<R, NC, FM_KICK, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)U, Pp, (char*)F,
-                                                                     (char*)Ubase, (char*)Uout, ckick, cdrift,
-                                                                     cdisp, reunit);
-          break;
-        case FM_KICK_DRIFT:
-          batch_force_kernel<R, NC, FM_KICK_DRIFT, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)U, Pp, (char*)F,
-                                                                           (char*)Ubase, (char*)Uout, ckick,
-                                                                           cdrift, cdisp, reunit);
-          break;
-        default:
-          batch_force_kernel<R, NC, FM_DISPLACE, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)U, Pp, (char*)F,
-                                                                         (char*)Ubase, (char*)Uout, ckick, cdrift,
-                                                                         cdisp, reunit);
-          break;
+        case FM_STORE: FG_FORCE(FM_STORE); break;
+        case FM_KICK: FG_FORCE(FM_KICK); break;
+        case FM_KICK_DRIFT: FG_FORCE(FM_KICK_DRIFT); break;
+        default: FG_FORCE(FM_DISPLACE); break;
       }
+#undef FG_FORCE
       return cudaGetLastError();
     });
+  }
+  fg_status force_launch(int mode, void* U, void* Ubase, void* Uout, double ckick, double cdrift, double cdisp) {
+    ForceArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.U = U; a.W = W_; a.P = P_; a.F = F_;
+    a.Ubase = Ubase; a.Uout = Uout;
+    a.ckick = ckick; a.cdrift = cdrift; a.cdisp = cdisp;
+    a.reunit = b_->prm.reunitarize;
+    if constexpr (kPlaquetteForce<R>) {
+      const fg_status s = lrun([&] { return launch_plaquettes<R, NC>(rows_, U, W_, st_); });
+      if (s != FG_OK) return s;
+      return lrun([&] { return launch_gauge_force<R, NC>(geomh(0), rows_, mode, a, st_); });
+    } else {
+      switch (hsel_) {
+        case 0: return staples_h<16>(0, mode, a);
+        case 2: return staples_h<64>(2, mode, a);
+        default: return staples_h<32>(1, mode, a);
+      }
+    }
   }
   // Double-float: the exponential of a kick-and-drift or a displacement runs
   // in a launch of its own after the force (the same arithmetic, the same
@@ -670,25 +657,16 @@ class Batch final : public IBatch {
   }();
   fg_status force(int mode, void* U, void* Ubase, void* Uout, double ckick, double cdrift, double cdisp) {
     if (split_exp_ && mode == FM_KICK_DRIFT) {
-      fg_status s = force_tiles(FM_KICK, U, nullptr, nullptr, ckick, 0, 0);
+      fg_status s = force_launch(FM_KICK, U, nullptr, nullptr, ckick, 0, 0);
       if (s != FG_OK) return s;
       return drift(Ubase, Uout, cdrift);
     }
     if (split_exp_ && mode == FM_DISPLACE) {
-      fg_status s = force_tiles(FM_STORE, U, nullptr, nullptr, 0, 0, 0);
+      fg_status s = force_launch(FM_STORE, U, nullptr, nullptr, 0, 0, 0);
       if (s != FG_OK) return s;
       return drift(U, Uout, -cdisp, F_, 0);
     }
-    return force_tiles(mode, U, Ubase, Uout, ckick, cdrift, cdisp);
-  }
-  fg_status force_tiles(int mode, void* U, void* Ubase, void* Uout, double ckick, double cdrift, double cdisp) {
-    switch (hsel_) {
-      case 0: return force_h<16>(0, mode, U, Ubase, Uout, F_, ckick, cdrift, cdisp);
-      case 2:
-        if constexpr (kTileSizes > 2) return force_h<64>(2, mode, U, Ubase, Uout, F_, ckick, cdrift, cdisp);
-        [[fallthrough]];
-      default: return force_h<32>(1, mode, U, Ubase, Uout, F_, ckick, cdrift, cdisp);
-    }
+    return force_launch(mode, U, Ubase, Uout, ckick, cdrift, cdisp);
   }
   // Uout = exp(i c G) Uin for the generator G (the momenta, or the force
   // buffer for a displacement); reunit < 0: the handle's setting.
@@ -823,8 +801,9 @@ class Batch final : public IBatch {
     return FG_OK;
   }
 
-  // Times the force kernel (store mode, all chains) for every tile size and
-  // keeps the fastest.
+  // Times the launches that walk the tiles for every tile size and keeps the
+  // fastest: in FP32 a displacement (the force and the exponential, as in most
+  // launches of a trajectory), otherwise a drift and an energy launch.
   fg_status autotune() {
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return cuda_fail("event");
@@ -835,10 +814,14 @@ class Batch final : public IBatch {
       float tmin = 1e30f;
       for (int rep = 0; rep < 4; ++rep) {
         cudaEventRecord(a, st_);
-        // a displacement into a scratch buffer: the force and the exponential,
-        // as in the kick-and-drift and displace launches that dominate a
-        // trajectory (the exponential's code decides the tile for double-float)
-        fg_status s = force(FM_DISPLACE, buf_[cur_], nullptr, buf_[(cur_ + 1) % 3], 0, 0, 0.01);
+        void* const scratch = buf_[(cur_ + 1) % 3];
+        fg_status s;
+        if (kPlaquetteForce<R>) {
+          s = drift(buf_[cur_], scratch, 0.01);
+          if (s == FG_OK) s = misc(1, buf_[cur_], 2);
+        } else {
+          s = force(FM_DISPLACE, buf_[cur_], nullptr, scratch, 0, 0, 0.01);
+        }
         if (s != FG_OK) {
           cudaEventDestroy(a);
           cudaEventDestroy(b);

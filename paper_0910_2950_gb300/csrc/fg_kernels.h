@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace fg {
 
 struct GeomH {
@@ -23,6 +25,7 @@ enum ForceMode {
 
 struct ForceArgs {
   const void* U;       // links at which the force is evaluated
+  const void* W;       // their plaquette field (launch_plaquettes; unused in FP32)
   void* P;             // momenta
   void* F;             // force out (FM_STORE)
   const void* FF;      // extra force added to the gauge force (fermions) or nullptr
@@ -34,8 +37,28 @@ struct ForceArgs {
   int reunit;
 };
 
+// Whether the force of links in precision R is formed by plaquettes (two
+// launches) or by staples (one).
+template <typename R>
+constexpr bool kPlaquetteForce = !std::is_same<R, float>::value;
+
+// The lattices of a plaquette-form launch, cut into rows of 32 half-sites.
+struct ForceRows {
+  const void* chains;     // device array of lattice descriptions (fill_chain)
+  const int* row_chain;   // lattice of each row, or null for one lattice
+  int nrows;
+};
+void fill_chain(void* dst, const GeomH& g, double beta, long long goff, long long moff, long long woff,
+                long long soff, int row0);
+size_t chain_bytes();
+
+// The plaquette field of links U into W (6 x 8 reals a site), which the force
+// launch that follows reads.
 template <typename R, int NC>
-cudaError_t launch_gauge_force(const GeomH& g, int mode, const ForceArgs& a, cudaStream_t st);
+cudaError_t launch_plaquettes(const ForceRows& rows, const void* U, void* W, cudaStream_t st);
+// `rows` is used in the plaquette form, `g` otherwise.
+template <typename R, int NC>
+cudaError_t launch_gauge_force(const GeomH& g, const ForceRows& rows, int mode, const ForceArgs& a, cudaStream_t st);
 
 // P -= c FF on every link (a kick with an externally computed force).
 template <typename R>

@@ -33,7 +33,7 @@ namespace fg {
 
 const char* kKernelClasses[] = {"gauge_force", "drift", "energy", "reduce", "momenta",
                                 "dslash", "cg_blas", "fermion_force", "convert", "dslash_fp64",
-                                "dslash_df"};
+                                "dslash_df", "plaquette"};
 
 // ---------------------------------------------------------------------------
 // Integrator sequences (Table 1 and section 3).

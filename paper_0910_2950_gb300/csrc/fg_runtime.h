@@ -42,9 +42,10 @@ int count_forces(const std::vector<Op>& ops);
 
 enum KernelClass {
   KC_GAUGE_FORCE = 0, KC_DRIFT, KC_ENERGY, KC_REDUCE, KC_MOMENTA,
-  KC_DSLASH, KC_CG_BLAS, KC_FERMION_FORCE, KC_CONVERT, KC_DSLASH64, KC_DSLASH_DF
+  KC_DSLASH, KC_CG_BLAS, KC_FERMION_FORCE, KC_CONVERT, KC_DSLASH64, KC_DSLASH_DF,
+  KC_PLAQUETTE
 };
-constexpr int kNumKernelClasses = 11;
+constexpr int kNumKernelClasses = 12;
 extern const char* kKernelClasses[];
 
 // Per-launch CUDA-event timing.  Events come from a pool that grows on

@@ -1,10 +1,11 @@
 // Pure-gauge kernels of the force-gradient HMC step (sm_103a).
 //
-//  * gauge_force_kernel: Wilson staple force F^a = (beta/6) Im Tr(lambda^a U A)
-//    (the S-hat vector field of section 3), fused with what the integrator does
-//    next on the same link: store it, kick the momentum, kick then drift the
-//    link, or displace the link along the force for the force-gradient step
-//    of Table 1 (U' = exp(-i dt^2/24 F) U).
+//  * staple_force_kernel (FP32), plaquette_kernel and link_force_kernel
+//    (double-float and FP64): Wilson force F^a = (beta/6) Im Tr(lambda^a U A), A the sum of the
+//    link's staples (the S-hat vector field of section 3), fused with what
+//    the integrator does next on the same link: store it, kick the momentum,
+//    kick then drift the link, or displace the link along the force for the
+//    force-gradient step of Table 1 (U' = exp(-i dt^2/24 F) U).
 //  * drift_kernel: the exact T-hat flow U <- exp(i c P) U (section 2).
 //  * energy_kernel: per-site T(x) + S_G(x), in double-float for FP32 fields
 //    and FP64 for FP64 fields, block partial sums for the dH of section 5
@@ -32,14 +33,15 @@ static Geom to_dev(const GeomH& h) {
 }
 
 constexpr int kSitesPerBlock = 64;
+constexpr int kSms = 152;  // SMs of a GB300
 
 
-template <typename R, int NC, int MODE>
-__global__ void __launch_bounds__(256, (kForceMinBlocks<R, NC>)) gauge_force_kernel(Gauge<R, NC> U, Mom<R> P, Mom<R> F,
-                                                          Mom<R> FF, Gauge<R, NC> Ubase,
-                                                          Gauge<R, NC> Uout, Geom g, R beta6,
-                                                          R ckick, R cdrift, R cdisp, int reunit, R ffw) {
-  if constexpr (kForceSharedT<R, NC>) {
+template <int NC, int MODE>
+__global__ void __launch_bounds__(256, kStapleMinBlocks<NC>) staple_force_kernel(Gauge<float, NC> U, Mom<float> P, Mom<float> F,
+                                                          Mom<float> FF, Gauge<float, NC> Ubase,
+                                                          Gauge<float, NC> Uout, Geom g, float beta6,
+                                                          float ckick, float cdrift, float cdisp, int reunit, float ffw) {
+  if constexpr (kForceSharedT<float, NC>) {
     __shared__ float2 tsh[6][9][64];   // 64 sites: both parities x 32 half-sites (link_site)
     int s;
     const bool ok = link_site(g, s);
@@ -50,9 +52,73 @@ __global__ void __launch_bounds__(256, (kForceMinBlocks<R, NC>)) gauge_force_ker
     if (!link_site(g, s)) return;
     int c[4], par;
     cb_coords(g, s, c, par);
-    force_link<R, NC, MODE>(U, P, F, FF, Ubase, Uout, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
+    force_link_staples<NC, MODE>(U, P, F, FF, Ubase, Uout, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
                             reunit, ffw);
   }
+}
+
+// The plaquette form walks the lattices of a launch by warps (rows of 32
+// consecutive half-sites of one parity): warp w takes part w % parts (a plane
+// or a direction) of row w / parts; all parts and both parities of the same
+// half-sites are in consecutive warps and share the links in L1.
+struct RowSite {
+  const ChainDesc* cd;
+  int s, part;
+};
+__device__ __forceinline__ bool row_site(const ForceRows& r, int parts, RowSite& o) {
+  const unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const unsigned q = w / (unsigned)parts;
+  o.part = (int)(w - q * (unsigned)parts);
+  int row = (int)(q >> 1);
+  if (row >= r.nrows) return false;
+  const ChainDesc* cd = (const ChainDesc*)r.chains;
+  if (r.row_chain != nullptr) {
+    cd += r.row_chain[row];
+    row -= cd->row0;
+  }
+  const int i = row * 32 + (int)(threadIdx.x & 31);
+  if (i >= cd->g.Vh) return false;
+  o.cd = cd;
+  o.s = (int)(q & 1) * cd->g.Vh + i;
+  return true;
+}
+
+// Q of every site and plane (gauge_device.cuh).
+template <typename R, int NC>
+__global__ void __launch_bounds__(kForceThreads, FG_PLAQ_MIN_BLOCKS)
+    plaquette_kernel(const __grid_constant__ ForceRows r, char* U, char* W) {
+  RowSite o;
+  if (!row_site(r, 6, o)) return;
+  const Geom g = o.cd->g;
+  Gauge<R, NC> u;
+  u.p = U + o.cd->goff; u.V = g.V;
+  Mom<R> w;
+  w.p = W + o.cd->woff; w.V = g.V;
+  R q[8];
+  plaquette_herm(u, g, o.s, o.part, q);
+  w.store(o.part, o.s, q);
+}
+
+// The force of every link from Q, and what MODE does with it.
+template <typename R, int NC, int MODE>
+__global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
+    link_force_kernel(const __grid_constant__ ForceRows r, char* U, char* W, char* P, char* F, char* FF, char* Ubase,
+                      char* Uout, R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+  RowSite o;
+  if (!row_site(r, 4, o)) return;
+  const ChainDesc& cd = *o.cd;
+  const Geom g = cd.g;
+  Gauge<R, NC> u, ub, uo;
+  u.p = U + cd.goff; u.V = g.V;
+  ub.p = Ubase + cd.goff; ub.V = g.V;
+  uo.p = Uout + cd.goff; uo.V = g.V;
+  Mom<R> w, p, f, ff;
+  w.p = W + cd.woff; w.V = g.V;
+  p.p = P + cd.moff; p.V = g.V;
+  f.p = F + cd.moff; f.V = g.V;
+  ff.p = FF == nullptr ? nullptr : FF + cd.moff; ff.V = g.V;
+  force_link_plaquettes<R, NC, MODE>(u, w, p, f, ff, ub, uo, g, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, cdisp,
+                                     reunit, ffw);
 }
 
 template <typename R, int NC>
@@ -260,19 +326,19 @@ static inline dim3 link_grid(int V) { return dim3((V + kSitesPerBlock - 1) / kSi
 static inline dim3 pair_grid(int V) { return dim3((V / 2 + 31) / 32); }
 static inline dim3 link_block() { return dim3(kSitesPerBlock, 4); }
 
-template <typename R, int NC>
-cudaError_t launch_gauge_force(const GeomH& gh, int mode, const ForceArgs& a, cudaStream_t st) {
-  if constexpr (kForceSharedT<R, NC> && FG_FORCE_CARVEOUT > 0) {
+template <int NC>
+static cudaError_t launch_staple_force(const GeomH& gh, int mode, const ForceArgs& a, cudaStream_t st) {
+  if constexpr (kForceSharedT<float, NC> && FG_FORCE_CARVEOUT > 0) {
     // keep the L1 share of the unified L1/shared storage as large as the
     // staple-product slots allow: the kernel's neighbour loads live in L1.
     // A preference only (once per process, thread-safe static initialisation);
     // a refusal leaves the driver's choice and is not an error.
     static const bool carved = [] {
       const cudaFuncAttribute a = cudaFuncAttributePreferredSharedMemoryCarveout;
-      cudaFuncSetAttribute(gauge_force_kernel<R, NC, FM_STORE>, a, FG_FORCE_CARVEOUT);
-      cudaFuncSetAttribute(gauge_force_kernel<R, NC, FM_KICK>, a, FG_FORCE_CARVEOUT);
-      cudaFuncSetAttribute(gauge_force_kernel<R, NC, FM_KICK_DRIFT>, a, FG_FORCE_CARVEOUT);
-      cudaFuncSetAttribute(gauge_force_kernel<R, NC, FM_DISPLACE>, a, FG_FORCE_CARVEOUT);
+      cudaFuncSetAttribute(staple_force_kernel<NC, FM_STORE>, a, FG_FORCE_CARVEOUT);
+      cudaFuncSetAttribute(staple_force_kernel<NC, FM_KICK>, a, FG_FORCE_CARVEOUT);
+      cudaFuncSetAttribute(staple_force_kernel<NC, FM_KICK_DRIFT>, a, FG_FORCE_CARVEOUT);
+      cudaFuncSetAttribute(staple_force_kernel<NC, FM_DISPLACE>, a, FG_FORCE_CARVEOUT);
       cudaGetLastError();
       return true;
     }();
@@ -280,35 +346,94 @@ cudaError_t launch_gauge_force(const GeomH& gh, int mode, const ForceArgs& a, cu
   }
   const Geom g = to_dev(gh);
   const int V = g.V;
-  auto U = gauge_of<R, NC>(a.U, V);
-  auto P = mom_of<R>(a.P, V);
-  auto F = mom_of<R>(a.F, V);
-  auto FF = mom_of<R>(a.FF, V);
-  auto Ub = gauge_of<R, NC>(a.Ubase, V);
-  auto Uo = gauge_of<R, NC>(a.Uout, V);
-  const R b6 = R(a.beta / 6.0);
-  const R ffw = R(a.ffw == 0.0 ? 1.0 : a.ffw);
+  auto U = gauge_of<float, NC>(a.U, V);
+  auto P = mom_of<float>(a.P, V);
+  auto F = mom_of<float>(a.F, V);
+  auto FF = mom_of<float>(a.FF, V);
+  auto Ub = gauge_of<float, NC>(a.Ubase, V);
+  auto Uo = gauge_of<float, NC>(a.Uout, V);
+  const float b6 = float(a.beta / 6.0);
+  const float ffw = float(a.ffw == 0.0 ? 1.0 : a.ffw);
   switch (mode) {
     case FM_STORE:
-      gauge_force_kernel<R, NC, FM_STORE><<<pair_grid(V), link_block(), 0, st>>>(
-          U, P, F, FF, Ub, Uo, g, b6, R(a.ckick), R(a.cdrift), R(a.cdisp), a.reunit, ffw);
+      staple_force_kernel<NC, FM_STORE><<<pair_grid(V), link_block(), 0, st>>>(
+          U, P, F, FF, Ub, Uo, g, b6, float(a.ckick), float(a.cdrift), float(a.cdisp), a.reunit, ffw);
       break;
     case FM_KICK:
-      gauge_force_kernel<R, NC, FM_KICK><<<pair_grid(V), link_block(), 0, st>>>(
-          U, P, F, FF, Ub, Uo, g, b6, R(a.ckick), R(a.cdrift), R(a.cdisp), a.reunit, ffw);
+      staple_force_kernel<NC, FM_KICK><<<pair_grid(V), link_block(), 0, st>>>(
+          U, P, F, FF, Ub, Uo, g, b6, float(a.ckick), float(a.cdrift), float(a.cdisp), a.reunit, ffw);
       break;
     case FM_KICK_DRIFT:
-      gauge_force_kernel<R, NC, FM_KICK_DRIFT><<<pair_grid(V), link_block(), 0, st>>>(
-          U, P, F, FF, Ub, Uo, g, b6, R(a.ckick), R(a.cdrift), R(a.cdisp), a.reunit, ffw);
+      staple_force_kernel<NC, FM_KICK_DRIFT><<<pair_grid(V), link_block(), 0, st>>>(
+          U, P, F, FF, Ub, Uo, g, b6, float(a.ckick), float(a.cdrift), float(a.cdisp), a.reunit, ffw);
       break;
     case FM_DISPLACE:
-      gauge_force_kernel<R, NC, FM_DISPLACE><<<pair_grid(V), link_block(), 0, st>>>(
-          U, P, F, FF, Ub, Uo, g, b6, R(a.ckick), R(a.cdrift), R(a.cdisp), a.reunit, ffw);
+      staple_force_kernel<NC, FM_DISPLACE><<<pair_grid(V), link_block(), 0, st>>>(
+          U, P, F, FF, Ub, Uo, g, b6, float(a.ckick), float(a.cdrift), float(a.cdisp), a.reunit, ffw);
       break;
     default:
       return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+void fill_chain(void* dst, const GeomH& gh, double beta, long long goff, long long moff, long long woff,
+                long long soff, int row0) {
+  ChainDesc* cd = (ChainDesc*)dst;
+  cd->g = to_dev(gh);
+  cd->goff = goff; cd->moff = moff; cd->woff = woff; cd->soff = soff;
+  cd->beta = beta;
+  cd->beta6 = beta / 6.0;
+  cd->beta6_hi = (float)cd->beta6;
+  cd->beta6_lo = (float)(cd->beta6 - (double)cd->beta6_hi);
+  cd->row0 = row0;
+  cd->tile0 = cd->ntiles = 0;
+}
+size_t chain_bytes() { return sizeof(ChainDesc); }
+
+// Warps of a block: `most` while that leaves two blocks for every SM, fewer on
+// small lattices, so that their few warps spread over the SMs instead of
+// queueing on some of them.
+static inline int warps_per_block(long long warps, int most) {
+  int w = most;
+  while (w > 1 && warps < (long long)w * 2 * kSms) w /= 2;
+  return w;
+}
+
+template <typename R, int NC>
+cudaError_t launch_plaquettes(const ForceRows& r, const void* U, void* W, cudaStream_t st) {
+  const long long warps = 12LL * r.nrows;
+  const int w = warps_per_block(warps, kForceThreads / 32);
+  plaquette_kernel<R, NC><<<(unsigned)((warps + w - 1) / w), 32 * w, 0, st>>>(r, (char*)U, (char*)W);
+  return cudaGetLastError();
+}
+
+template <typename R, int NC>
+static cudaError_t launch_link_force(const ForceRows& r, int mode, const ForceArgs& a, cudaStream_t st) {
+  const R ffw = R(a.ffw == 0.0 ? 1.0 : a.ffw);
+  const long long warps = 8LL * r.nrows;
+  const int w = warps_per_block(warps, kForceThreads / 32);
+  const unsigned nb = (unsigned)((warps + w - 1) / w);
+#define FG_FORCE(M)                                                                                                 \
+  link_force_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.W, (char*)a.P, (char*)a.F, (char*)a.FF, \
+                                                     (char*)a.Ubase, (char*)a.Uout, R(a.ckick), R(a.cdrift),         \
+                                                     R(a.cdisp), a.reunit, ffw)
+  switch (mode) {
+    case FM_STORE: FG_FORCE(FM_STORE); break;
+    case FM_KICK: FG_FORCE(FM_KICK); break;
+    case FM_KICK_DRIFT: FG_FORCE(FM_KICK_DRIFT); break;
+    case FM_DISPLACE: FG_FORCE(FM_DISPLACE); break;
+    default: return cudaErrorInvalidValue;
+  }
+#undef FG_FORCE
+  return cudaGetLastError();
+}
+
+template <typename R, int NC>
+cudaError_t launch_gauge_force(const GeomH& gh, const ForceRows& rows, int mode, const ForceArgs& a,
+                               cudaStream_t st) {
+  if constexpr (kPlaquetteForce<R>) return launch_link_force<R, NC>(rows, mode, a, st);
+  else return launch_staple_force<NC>(gh, mode, a, st);
 }
 
 template <typename R, int NC>
@@ -414,8 +539,14 @@ template cudaError_t launch_kick_ff<double>(const GeomH&, void*, const void*, do
 template cudaError_t launch_kick_ff<float>(const GeomH&, void*, const void*, double, cudaStream_t);
 template cudaError_t launch_kick_ff<DF>(const GeomH&, void*, const void*, double, cudaStream_t);
 
+template cudaError_t launch_plaquettes<double, 9>(const ForceRows&, const void*, void*, cudaStream_t);
+template cudaError_t launch_plaquettes<double, 6>(const ForceRows&, const void*, void*, cudaStream_t);
+template cudaError_t launch_plaquettes<DF, 9>(const ForceRows&, const void*, void*, cudaStream_t);
+template cudaError_t launch_plaquettes<DF, 6>(const ForceRows&, const void*, void*, cudaStream_t);
+
 #define FG_INST_RNC(R, NC)                                                                          \
-  template cudaError_t launch_gauge_force<R, NC>(const GeomH&, int, const ForceArgs&, cudaStream_t); \
+  template cudaError_t launch_gauge_force<R, NC>(const GeomH&, const ForceRows&, int, const ForceArgs&,   \
+                                                 cudaStream_t);                                   \
   template cudaError_t launch_drift<R, NC>(const GeomH&, const void*, const void*, void*, double,   \
                                            int, cudaStream_t);                                      \
   template cudaError_t launch_reunitarize<R, NC>(const GeomH&, void*, cudaStream_t);                \

@@ -11,20 +11,16 @@
 
 namespace fg {
 
-// Tuning knobs of the gauge-force kernel: minimum resident blocks of 256
-// threads per SM (register cap) and whether the loop over the three staple
+// Tuning knobs of the staple kernel: minimum resident blocks of 256 threads
+// per SM (register cap) and whether the loop over the three staple
 // directions is unrolled.
-#ifndef FG_FORCE_MIN_BLOCKS
-#define FG_FORCE_MIN_BLOCKS 2
+#ifndef FG_STAPLE_MIN_BLOCKS
+#define FG_STAPLE_MIN_BLOCKS 2
 #endif
 #ifndef FG_FORCE_UNROLL_NU
 #define FG_FORCE_UNROLL_NU 0
 #endif
 
-// Sum of the six staples that close a plaquette with U_mu(x).  Neighbour
-// indices are formed with selects, so mu and nu may be run-time values
-// without the coordinate array going to local memory; one copy of the body
-// keeps the kernel small enough for the instruction cache.
 // Changes dp, dm of the half index lex/2 when coordinate nu of c moves by
 // +1 and -1 (periodic); the parity flips.  Only that coordinate moves, so the change
 // is (v>>1) - (c>>1) in x and (v - c) times the half stride of nu otherwise,
@@ -52,6 +48,70 @@ __device__ __forceinline__ M3<R> link_mul(const M3<R>& a, const M3<R>& b) {
   else return mul(a, b);
 }
 
+// Stores exp(i P) u, re-projected onto SU(3) if reunit is set (then rows 0
+// and 1 of the product suffice).
+template <typename R, int NC>
+__device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const Gauge<R, NC>& Uout, int mu, int s,
+                                            int reunit) {
+  const M3<R> e = expi_herm(alg_to_mat(p));
+  if (reunit) {
+    M3<R> un = mul_rows01(e, u);
+    reunitarize(un);
+    Uout.store(mu, s, un);
+  } else {
+    Uout.store(mu, s, link_mul(e, u));
+  }
+}
+
+// What MODE does with link (s, mu), f^a = Im Tr(lambda^a U A) given.
+template <typename R, int NC, int MODE>
+__device__ __forceinline__ void force_apply(const Gauge<R, NC>& U, const Mom<R>& P, const Mom<R>& F, const Mom<R>& FF,
+                                            const Gauge<R, NC>& Ubase, const Gauge<R, NC>& Uout, int s, int mu,
+                                            R f[8], R beta6, R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) f[k] = f[k] * beta6;
+  if (FF.p != nullptr) {
+    R ff[8];
+    FF.load(mu, s, ff);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] = fma(ffw, ff[k], f[k]);
+  }
+  if (MODE == FM_STORE) {
+    F.store(mu, s, f);
+  } else if (MODE == FM_KICK || MODE == FM_KICK_DRIFT) {
+    R p[8];
+    P.load(mu, s, p);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) p[k] = fma(-ckick, f[k], p[k]);
+    P.store(mu, s, p);
+    if (MODE == FM_KICK_DRIFT) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) p[k] *= cdrift;
+      drift_store(p, Ubase.load(mu, s), Uout, mu, s, reunit);
+    }
+  } else {  // FM_DISPLACE
+    // The displaced links only serve one force evaluation and are then
+    // dropped, so they are not re-projected.  (FP32 exp(i A) U comes out
+    // short of unitary by ~7e-9 of |U|^2 on average, but re-projecting the
+    // displaced FP32 links as the drifted ones are raised the FP32 dH error
+    // of a 24^4 trajectory from 2.5e-2 to 3.4e-2: the projection's own
+    // rounding is not of random sign either.)
+    (void)reunit;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] *= -cdisp;
+    const M3<R> e = expi_herm(alg_to_mat(f));
+    Uout.store(mu, s, link_mul(e, U.load(mu, s)));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The Wilson force by staples (FP32 links): one thread sums the six staples
+// of its link.
+
+// Sum of the six staples that close a plaquette with U_mu(x).  Neighbour
+// indices are formed with selects, so mu and nu may be run-time values
+// without the coordinate array going to local memory; one copy of the body
+// keeps the kernel small enough for the instruction cache.
 template <typename R, int NC>
 __device__ __forceinline__ M3<R> staple_sum(const Gauge<R, NC>& U, const Geom& g, const int c[4], int s, int mu) {
   M3<R> a;
@@ -73,133 +133,31 @@ __device__ __forceinline__ M3<R> staple_sum(const Gauge<R, NC>& U, const Geom& g
     const int nu = (mu + k) & 3;
     int dp, dm;
     cb_half_steps(g, c, nu, dp, dm);
-    if constexpr (std::is_same<R, DF>::value) {
-      // Double-float: every staple is a product of links, hence unitary, so
-      // the anchored products (df64.cuh) apply.  Both staples of the plane
-      // are written as X Y^dag Z with run-time daggers,
-      //   upper  U_nu(x+mu)          U_mu(x+nu)^dag U_nu(x)^dag,
-      //   lower  U_nu(x+mu-nu)^dag   U_mu(x-nu)^dag U_nu(x-nu),
-      // and the two products of each run through one loop body: unrolled,
-      // the double-float code of four products per plane overflowed the
-      // instruction cache (most issue stalls were instruction fetch).
+    {
+      // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
+      const M3<R> t = mul_nd(U.load(nu, s_pmu), U.load(mu, other + dp));
+      mac_nd(a, t, U.load(nu, s));
+    }
+    {
+      // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) = (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)
       const int s_mnu = other + dm;
-#pragma unroll 1
-      for (int up = 1; up >= 0; --up) {
-        M3<DF> l = dagger_if(U.load(nu, up ? s_pmu : s + dm + dmu), !up);
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-          // Y^dag = U_mu(x+nu)^dag or U_mu(x-nu)^dag, then Z
-          const int sr = q ? (up ? s : s_mnu) : (up ? other + dp : s_mnu);
-          l = su3_mul(l, dagger_if(U.load(q ? nu : mu, sr), q ? up != 0 : true));
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) a.e[i][j] = a.e[i][j] + l.e[i][j];
-      }
-    } else {
-      {
-        // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-        const M3<R> t = mul_nd(U.load(nu, s_pmu), U.load(mu, other + dp));
-        mac_nd(a, t, U.load(nu, s));
-      }
-      {
-        // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) = (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)
-        const int s_mnu = other + dm;
-        const M3<R> t = mul(U.load(mu, s_mnu), U.load(nu, s + dm + dmu));
-        mac_dn(a, t, U.load(nu, s_mnu));
-      }
+      const M3<R> t = mul(U.load(mu, s_mnu), U.load(nu, s + dm + dmu));
+      mac_dn(a, t, U.load(nu, s_mnu));
     }
   }
   return a;
 }
 
-// Stores exp(i P) u, re-projected onto SU(3) if reunit is set (then rows 0
-// and 1 of the product suffice).
-template <typename R, int NC>
-__device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const Gauge<R, NC>& Uout, int mu, int s,
-                                            int reunit) {
-  const M3<R> e = expi_herm(alg_to_mat(p));
-  if (reunit) {
-    M3<R> un = mul_rows01(e, u);
-    reunitarize(un);
-    Uout.store(mu, s, un);
-  } else {
-    Uout.store(mu, s, link_mul(e, u));
-  }
-}
-
-// Everything after the staple sum a of U_mu(x): the force, then what MODE
-// does with it on this link.
-template <typename R, int NC, int MODE>
-__device__ __forceinline__ void force_finish(const Gauge<R, NC>& U, const Mom<R>& P, const Mom<R>& F,
-                                             const Mom<R>& FF, const Gauge<R, NC>& Ubase,
-                                             const Gauge<R, NC>& Uout, int s, int mu, const M3<R>& a, R beta6,
-                                             R ckick, R cdrift, R cdisp, int reunit, R ffw) {
-  const M3<R> ul = U.load(mu, s);
-  R f[8];
-  if constexpr (std::is_same<R, DF>::value) {
-    // a is a sum of six unitary staples, so a / 8 has columns of norm <= 3/4
-    // and U (a / 8) is within the anchored products' bounds; scaling by a
-    // power of two is exact
-    M3<DF> a8;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        a8.e[i][j] = cx<DF>(DF(a.e[i][j].re.hi * 0.125f, a.e[i][j].re.lo * 0.125f),
-                            DF(a.e[i][j].im.hi * 0.125f, a.e[i][j].im.lo * 0.125f));
-    im_tr_gellmann(su3_mul(ul, a8), f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] = (f[k] * 8.0f) * beta6;
-  } else {
-    const M3<R> omega = mul(ul, a);
-    im_tr_gellmann(omega, f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] *= beta6;
-  }
-  if (FF.p != nullptr) {
-    R ff[8];
-    FF.load(mu, s, ff);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] = fma(ffw, ff[k], f[k]);
-  }
-  if (MODE == FM_STORE) {
-    F.store(mu, s, f);
-  } else if (MODE == FM_KICK || MODE == FM_KICK_DRIFT) {
-    R p[8];
-    P.load(mu, s, p);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) p[k] = fma(-ckick, f[k], p[k]);
-    P.store(mu, s, p);
-    if (MODE == FM_KICK_DRIFT) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) p[k] *= cdrift;
-      drift_store(p, (Ubase.p == U.p) ? ul : Ubase.load(mu, s), Uout, mu, s, reunit);
-    }
-  } else {  // FM_DISPLACE
-    // The displaced links only serve one force evaluation and are then
-    // dropped, so they are not re-projected.  (FP32 exp(i A) U comes out
-    // short of unitary by ~7e-9 of |U|^2 on average, but re-projecting the
-    // displaced FP32 links as the drifted ones are raised the FP32 dH error
-    // of a 24^4 trajectory from 2.5e-2 to 3.4e-2: the projection's own
-    // rounding is not of random sign either.)
-    (void)reunit;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] *= -cdisp;
-    const M3<R> e = expi_herm(alg_to_mat(f));
-    Uout.store(mu, s, link_mul(e, ul));
-  }
-}
-
-template <typename R, int NC, int MODE>
-__device__ __forceinline__ void force_link(const Gauge<R, NC>& U, const Mom<R>& P, const Mom<R>& F,
-                                           const Mom<R>& FF, const Gauge<R, NC>& Ubase,
-                                           const Gauge<R, NC>& Uout, const Geom& g, const int c[4], int s,
-                                           int mu, R beta6, R ckick, R cdrift, R cdisp, int reunit,
-                                           R ffw = R(1)) {
-  const M3<R> a = staple_sum(U, g, c, s, mu);
-  force_finish<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, a, beta6, ckick, cdrift, cdisp, reunit, ffw);
+template <int NC, int MODE>
+__device__ __forceinline__ void force_link_staples(const Gauge<float, NC>& U, const Mom<float>& P, const Mom<float>& F,
+                                                   const Mom<float>& FF, const Gauge<float, NC>& Ubase,
+                                                   const Gauge<float, NC>& Uout, const Geom& g, const int c[4], int s,
+                                                   int mu, float beta6, float ckick, float cdrift, float cdisp,
+                                                   int reunit, float ffw) {
+  const M3<float> a = staple_sum(U, g, c, s, mu);
+  float f[8];
+  im_tr_gellmann(mul(U.load(mu, s), a), f);
+  force_apply<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
 }
 
 // Whether the FP32 12-real force kernels share the upper-staple products of
@@ -239,18 +197,8 @@ __device__ __forceinline__ void force_link(const Gauge<R, NC>& U, const Mom<R>& 
 // barrier.  The caller separates two calls on the same tsh by a barrier.
 template <typename R, int NC>
 constexpr bool kForceSharedT = FG_FORCE_SHARED_T && std::is_same<R, float>::value && NC == 6;
-#ifndef FG_FORCE_DF_MIN_BLOCKS
-#define FG_FORCE_DF_MIN_BLOCKS 2
-#endif
-// Double-float links need about twice the registers of FP32 ones.  With the
-// exponential in a launch of its own the force launch fits two blocks of
-// 256 threads per SM (128 registers a thread): 2-3% faster than one block
-// with up to 255 registers (32^4 trajectory 34.7 against 35.5 ms, 64-chain
-// batch 39.7 against 40.5 ms).
-template <typename R, int NC>
-constexpr int kForceMinBlocks = std::is_same<R, DF>::value
-                                    ? FG_FORCE_DF_MIN_BLOCKS
-                                    : (kForceSharedT<R, NC> ? FG_FORCE_SHARED_MIN_BLOCKS : FG_FORCE_MIN_BLOCKS);
+template <int NC>
+constexpr int kStapleMinBlocks = kForceSharedT<float, NC> ? FG_FORCE_SHARED_MIN_BLOCKS : FG_STAPLE_MIN_BLOCKS;
 
 template <int NC, int MODE, int NS>
 __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok, int s, const Gauge<float, NC>& U,
@@ -322,7 +270,327 @@ __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok,
         a.e[i][j] = conj(acc);
       }
   }
-  force_finish<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, a, beta6, ckick, cdrift, cdisp, reunit, ffw);
+  float f[8];
+  im_tr_gellmann(mul(U.load(mu, s), a), f);
+  force_apply<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
+}
+
+// ---------------------------------------------------------------------------
+// The Wilson force by plaquettes (double-float and FP64 links).
+//
+// The four links of a plaquette share its force.  With
+//   W_{mu nu}(x) = U_mu(x) U_nu(x+mu) (U_nu(x) U_mu(x+nu))^dag,   mu < nu,
+// and Q the Hermitian traceless part of W (W = ... + i Q),
+//   * U_mu(x) takes +Q and U_nu(x) takes -Q (their products with the staple
+//     are W and W^dag);
+//   * U_mu(x+nu) takes -U_nu(x)^dag Q U_nu(x) and U_nu(x+mu) takes
+//     +U_mu(x)^dag Q U_mu(x) (the same closed path read from another corner;
+//     this step uses U^dag U = 1).
+// plaquette_kernel forms Q once for every site and plane (two products and
+// half of a third), link_force_kernel sums six of them for every link, three
+// of them rotated by one neighbour link (90 + 48 multiply-adds, H being
+// Hermitian).  A site then takes 6 x 306 + 12 x 138 = 3492 multiply-adds
+// instead of the 4 x 13 x 108 = 5616 of a staple sum for every link.
+// Double-float and FP64 forces are bound by that arithmetic (FP32 and FP64
+// issue), so they take this form: a trajectory against the staple sums takes
+// 1.94 instead of 2.51 ms (double-float 16^4), 12.1 instead of 16.0 ms
+// (64-chain double-float batch), 3.03 instead of 4.6 ms (FP64 12^4), and on
+// small lattices, where a thread's serial chain counts, 0.45 instead of
+// 0.55 ms (double-float 8^4) and 1.32 instead of 3.00 ms (FP64 4^4, with its
+// warps spread over the SMs).  The FP32 force executes 18% fewer instructions
+// this way but waits for the memory traffic of Q (193 + 233 us a launch pair
+// against 405 us at 32^4; 12% slower at 8^4): it stays with the staples.  One
+// launch of both kinds of work, link blocks waiting for the plaquettes they
+// read, was 5 to 25% slower than two launches (idle SMs, spilled registers).
+// Q is kept in the momenta's layout, [plane][2][site], as Q / 2 (for the
+// double-float products below) by its entries
+// (q00, q11, Re q01, Im q01, Re q02, Im q02, Re q12, Im q12).
+
+// Most threads of a block of the two kernels, and resident blocks of that
+// size asked of the register allocator: 168 and 128 registers a thread, where
+// neither spills (plaquettes at 128 registers: 5-7% slower in double-float).
+#ifndef FG_PLAQ_THREADS
+#define FG_PLAQ_THREADS 128
+#endif
+#ifndef FG_PLAQ_MIN_BLOCKS
+#define FG_PLAQ_MIN_BLOCKS 3
+#endif
+#ifndef FG_LINK_MIN_BLOCKS
+#define FG_LINK_MIN_BLOCKS 4
+#endif
+constexpr int kForceThreads = FG_PLAQ_THREADS;
+
+// One lattice of a launch: its geometry, coupling and the byte offsets of its
+// links, momenta and plaquette field in the launch's buffers.
+struct ChainDesc {
+  Geom g;
+  long long goff, moff, woff;
+  long long soff;  // offset of its sites in per-site arrays
+  double beta, beta6;          // beta, beta / 6
+  float beta6_hi, beta6_lo;    // beta / 6 as a double-float: no FP64 arithmetic (1/64 of the FP32 rate) there
+  int row0;                    // first of its rows of 32 half-sites
+  int tile0, ntiles;           // its tiles (batch.cu)
+};
+template <typename R> __device__ __forceinline__ R beta6_of(const ChainDesc& cd);
+template <> __device__ __forceinline__ double beta6_of<double>(const ChainDesc& cd) { return cd.beta6; }
+template <> __device__ __forceinline__ float beta6_of<float>(const ChainDesc& cd) { return cd.beta6_hi; }
+template <> __device__ __forceinline__ DF beta6_of<DF>(const ChainDesc& cd) { return DF(cd.beta6_hi, cd.beta6_lo); }
+
+// Plane pl = 0..5 as directions mu < nu, and back.
+__device__ __forceinline__ void plane_dirs(int pl, int& mu, int& nu) {
+  mu = pl < 3 ? 0 : (pl < 5 ? 1 : 2);
+  nu = pl < 3 ? pl + 1 : (pl < 5 ? pl - 1 : 3);
+}
+__device__ __forceinline__ int plane_of(int a, int b) {
+  const int mu = a < b ? a : b, nu = a < b ? b : a;
+  return mu == 0 ? nu - 1 : (mu == 1 ? nu + 1 : 5);
+}
+
+// q = (Hermitian traceless part of W_pl(s)) / 2.
+template <typename R, int NC>
+__device__ __forceinline__ void plaquette_herm(const Gauge<R, NC>& U, const Geom& g, int s, int pl, R q[8]) {
+  int c[4], par, mu, nu;
+  cb_coords(g, s, c, par);
+  plane_dirs(pl, mu, nu);
+  const int other = s + (par ? -g.Vh : g.Vh);
+  int dmu, dnu, dm;
+  cb_half_steps(g, c, mu, dmu, dm);
+  cb_half_steps(g, c, nu, dnu, dm);
+  (void)dm;
+  if constexpr (std::is_same<R, DF>::value) {
+    // both corner products through one loop body (instruction cache)
+    M3<DF> a, b;
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+      const M3<DF> m = su3_mul(U.load(k ? nu : mu, s), U.load(k ? mu : nu, other + (k ? dnu : dmu)));
+      if (k) b = m;
+      else a = m;
+    }
+    // half of a (exact) keeps the sums of two entries of W within the
+    // anchored accumulator's [-1, 1]
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        a.e[i][j] = cx<DF>(DF(0.5f * a.e[i][j].re.hi, 0.5f * a.e[i][j].re.lo),
+                           DF(0.5f * a.e[i][j].im.hi, 0.5f * a.e[i][j].im.lo));
+    DF d[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      Anchored t;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        t.add(a.e[i][k].im, b.e[i][k].re);
+        t.sub(a.e[i][k].re, b.e[i][k].im);
+      }
+      d[i] = t.value();
+    }
+    constexpr DF third(1.0 / 3.0);
+    const DF tr = (d[0] + d[1] + d[2]) * third;
+    q[0] = d[0] - tr;
+    q[1] = d[1] - tr;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const int i = p < 2 ? 0 : 1, j = p == 0 ? 1 : 2;
+      Anchored re, im;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        re.add(a.e[i][k].im, b.e[j][k].re);
+        re.sub(a.e[i][k].re, b.e[j][k].im);
+        re.add(a.e[j][k].im, b.e[i][k].re);
+        re.sub(a.e[j][k].re, b.e[i][k].im);
+        im.sub(a.e[i][k].re, b.e[j][k].re);
+        im.sub(a.e[i][k].im, b.e[j][k].im);
+        im.add(a.e[j][k].re, b.e[i][k].re);
+        im.add(a.e[j][k].im, b.e[i][k].im);
+      }
+      const DF vr = re.value(), vi = im.value();
+      q[2 + 2 * p] = DF(0.5f * vr.hi, 0.5f * vr.lo);
+      q[3 + 2 * p] = DF(0.5f * vi.hi, 0.5f * vi.lo);
+    }
+  } else {
+    const M3<R> a = mul(U.load(mu, s), U.load(nu, other + dmu));
+    const M3<R> b = mul(U.load(nu, s), U.load(mu, other + dnu));
+    R d[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      R t = R(0);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        t = fma(a.e[i][k].im, b.e[i][k].re, t);
+        t = fma(-a.e[i][k].re, b.e[i][k].im, t);
+      }
+      d[i] = t;
+    }
+    const R tr = (d[0] + d[1] + d[2]) * R(1.0 / 3.0);
+    q[0] = R(0.5) * (d[0] - tr);
+    q[1] = R(0.5) * (d[1] - tr);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const int i = p < 2 ? 0 : 1, j = p == 0 ? 1 : 2;
+      R re = R(0), im = R(0);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        re = fma(a.e[i][k].im, b.e[j][k].re, re);
+        re = fma(-a.e[i][k].re, b.e[j][k].im, re);
+        re = fma(a.e[j][k].im, b.e[i][k].re, re);
+        re = fma(-a.e[j][k].re, b.e[i][k].im, re);
+        im = fma(-a.e[i][k].re, b.e[j][k].re, im);
+        im = fma(-a.e[i][k].im, b.e[j][k].im, im);
+        im = fma(a.e[j][k].re, b.e[i][k].re, im);
+        im = fma(a.e[j][k].im, b.e[i][k].im, im);
+      }
+      q[2 + 2 * p] = R(0.25) * re;
+      q[3 + 2 * p] = R(0.25) * im;
+    }
+  }
+}
+
+// acc += u^dag H u for the Hermitian traceless H given by h (entries as
+// above), a column of H u at a time.
+template <typename R>
+__device__ __forceinline__ void rotate_add(R acc[8], const R h[8], const M3<R>& u) {
+  const R h22 = -(h[0] + h[1]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const Cx<R> u0 = u.e[0][j], u1 = u.e[1][j], u2 = u.e[2][j];
+    Cx<R> v[3];
+    v[0] = cx<R>(h[0] * u0.re, h[0] * u0.im);
+    cmac(v[0], cx<R>(h[2], h[3]), u1);
+    cmac(v[0], cx<R>(h[4], h[5]), u2);
+    v[1] = cx<R>(h[1] * u1.re, h[1] * u1.im);
+    cmac_cj(v[1], cx<R>(h[2], h[3]), u0);
+    cmac(v[1], cx<R>(h[6], h[7]), u2);
+    v[2] = cx<R>(h22 * u2.re, h22 * u2.im);
+    cmac_cj(v[2], cx<R>(h[4], h[5]), u0);
+    cmac_cj(v[2], cx<R>(h[6], h[7]), u1);
+    if (j < 2) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        acc[j] = fma(u.e[k][j].re, v[k].re, acc[j]);
+        acc[j] = fma(u.e[k][j].im, v[k].im, acc[j]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < j; ++i) {
+      const int p = i + j;  // (0,1) -> 1, (0,2) -> 2, (1,2) -> 3
+      Cx<R> t = cx<R>(acc[2 * p], acc[2 * p + 1]);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) cmac_cj(t, u.e[k][i], v[k]);
+      acc[2 * p] = t.re;
+      acc[2 * p + 1] = t.im;
+    }
+  }
+}
+
+// Double-float: H / 2 has norm at most 2/3 (Q's eigenvalues are sines less
+// their mean), so the entries of H u / 2 and u^dag H u / 2 and all their
+// partial sums lie within the anchored products' [-1, 1].
+template <>
+__device__ __forceinline__ void rotate_add<DF>(DF acc[8], const DF h[8], const M3<DF>& u) {
+  const DF h22 = -(h[0] + h[1]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    Cx<DF> v[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      Anchored re, im;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const Cx<DF> x = u.e[k][j];
+        if (k == r) {
+          const DF d = r == 0 ? h[0] : (r == 1 ? h[1] : h22);
+          re.add(d, x.re);
+          im.add(d, x.im);
+        } else {
+          const int p = k + r;  // the entry above the diagonal; its conjugate below
+          const DF hr = h[2 * p], hi = h[2 * p + 1];
+          re.add(hr, x.re);
+          im.add(hr, x.im);
+          if (k > r) {
+            re.sub(hi, x.im);
+            im.add(hi, x.re);
+          } else {
+            re.add(hi, x.im);
+            im.sub(hi, x.re);
+          }
+        }
+      }
+      v[r] = cx<DF>(re.value(), im.value());
+    }
+#pragma unroll
+    for (int i = 0; i <= j; ++i) {
+      if (i == 2) continue;  // the trace is zero
+      Anchored re, im;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        re.add(u.e[k][i].re, v[k].re);
+        re.add(u.e[k][i].im, v[k].im);
+        if (i < j) {
+          im.add(u.e[k][i].re, v[k].im);
+          im.sub(u.e[k][i].im, v[k].re);
+        }
+      }
+      if (i == j) {
+        acc[i] = acc[i] + re.value();
+      } else {
+        acc[2 * (i + j)] = acc[2 * (i + j)] + re.value();
+        acc[2 * (i + j) + 1] = acc[2 * (i + j) + 1] + im.value();
+      }
+    }
+  }
+}
+
+template <typename R> __device__ __forceinline__ R flip_if(R x, bool n) { return n ? -x : x; }
+
+// f^a = Im Tr(lambda^a U_mu(s) A_mu(s)), A the staple sum, from the
+// plaquette field W of these links.
+template <typename R, int NC>
+__device__ __forceinline__ void link_force(const Gauge<R, NC>& U, const Mom<R>& W, const Geom& g, int s, int mu,
+                                           R f[8]) {
+  int c[4], par;
+  cb_coords(g, s, c, par);
+  const int other = s + (par ? -g.Vh : g.Vh);
+  R acc[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k] = R(0);
+  // one copy of the body (instruction cache)
+#pragma unroll 1
+  for (int d = 1; d < 4; ++d) {
+    const int nu = (mu + d) & 3;
+    const int pl = plane_of(mu, nu);
+    int dp, dm;
+    cb_half_steps(g, c, nu, dp, dm);
+    (void)dp;
+    const int sm = other + dm;  // x - nu
+    R h[8];
+    W.load(pl, s, h);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = acc[k] + flip_if(h[k], mu > nu);
+    W.load(pl, sm, h);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) h[k] = flip_if(h[k], mu < nu);
+    rotate_add(acc, h, U.load(nu, sm));
+  }
+  const R four = R(4.0f), two = R(2.0f), s12 = R(3.46410161513775458705);  // 2 sqrt(3)
+  f[0] = four * acc[2];
+  f[1] = -(four * acc[3]);
+  f[2] = two * (acc[0] - acc[1]);
+  f[3] = four * acc[4];
+  f[4] = -(four * acc[5]);
+  f[5] = four * acc[6];
+  f[6] = -(four * acc[7]);
+  f[7] = s12 * (acc[0] + acc[1]);
+}
+
+template <typename R, int NC, int MODE>
+__device__ __forceinline__ void force_link_plaquettes(const Gauge<R, NC>& U, const Mom<R>& W, const Mom<R>& P,
+                                                      const Mom<R>& F, const Mom<R>& FF, const Gauge<R, NC>& Ubase,
+                                                      const Gauge<R, NC>& Uout, const Geom& g, int s, int mu, R beta6,
+                                                      R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+  R f[8];
+  link_force(U, W, g, s, mu, f);
+  force_apply<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
 }
 
 // U_out(s, mu) = exp(i c P) U_in(s, mu), the exact T-hat flow of section 2.
@@ -387,7 +655,7 @@ __device__ __forceinline__ void site_energy(const Gauge<R, NC>& U, const Mom<R>&
   } else {
     int c[4], par;
     cb_coords(g, s, c, par);
-    // x + mu as a half-index step from s (see staple_sum)
+    // x + mu as a half-index step from s (cb_half_steps)
     const int other = s + (par ? -g.Vh : g.Vh);
     int dp[4];
 #pragma unroll

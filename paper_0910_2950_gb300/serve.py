@@ -91,7 +91,8 @@ class Result:
 def footprint_bytes(spec: ChainSpec, precision: str = "fp32", link_reals: int = 18,
                     l2_bytes: int = 126 << 20) -> int:
     """Device bytes a chain holds, from the library's allocation plan: three
-    link buffers, momenta and force, per-site energies and the stored per-site
+    link buffers, momenta and force, the plaquette field of the double-float and
+    FP64 force, per-site energies and the stored per-site
     gauge actions, block partials and
     result scalars, the FP64 host-layout staging buffer, and for fermions 8
     FP64 and 10 working half-lattice spinors (plus 2 double-float ones for the
@@ -108,7 +109,8 @@ def footprint_bytes(spec: ChainSpec, precision: str = "fp32", link_reals: int = 
     r = 8 if precision in ("fp64", "df64") else 4     # bytes per real (double-float: two floats)
     gauge = 4 * v * link_reals * r
     mom = 4 * v * 8 * r
-    total = 3 * gauge + 2 * mom + 3 * 8 * v + 4 * 8 * ((v + 255) // 256 + 1) + 32 * 8 + 4 * v * 18 * 8
+    plaq = 6 * 8 * r * v if r == 8 else 0     # plaquette field of the double-float and FP64 force
+    total = 3 * gauge + 2 * mom + plaq + 3 * 8 * v + 4 * 8 * ((v + 255) // 256 + 1) + 32 * 8 + 4 * v * 18 * 8
     if spec.kappa > 0:
         vh = v // 2
         nvec = 12 * vh
