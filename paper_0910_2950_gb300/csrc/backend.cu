@@ -1146,7 +1146,7 @@ class Backend final : public IBackend {
   }
   cudaError_t fold_update(const void* U) {
     if constexpr (kMixed || std::is_same<R, double>::value) {
-      const cudaError_t e = launch_cg_fold<R, NC>(g_, to_, xs_, rs_, ap_, p_, rs2_, p2_, U, part_rr_, cgd_,
+      const cudaError_t e = launch_cg_fold<R, NC>(g_, to_, xs_, rs_, ap_, p_, rs2_, p2_, U, part_pap_, cgd_,
                                                   mapped_->hist, &mapped_->dev_iter, h_->prm.cg_maxiter, st_);
       std::swap(rs_, rs2_);
       std::swap(p_, p2_);

@@ -40,6 +40,87 @@ template <> struct DslashMinBlocks<float> { static constexpr int value = FG_DSLA
 #define FG_DSLASH_DF_MIN_BLOCKS 4
 #endif
 template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_DF_MIN_BLOCKS; };
+// The one-direction-a-warp kernels: five blocks a SM (102 registers); four
+// (128) are 10% slower at 12^3 x 24, six 2-3% slower at 8^3 x 16.
+#ifndef FG_SPLIT_MIN_BLOCKS
+#define FG_SPLIT_MIN_BLOCKS 5
+#endif
+// Most sites of a parity that get one direction a warp.  Eight hops to a
+// thread need the fewest instructions and fill the GPU at 16^3 x 32 (65536
+// sites); below some 30 thousand sites they leave it waiting for a few warps'
+// serial loads.  Whole solves, split against whole: FP32 8^3 x 16 (4096
+// sites) 3.43 against 4.95 ms, 12^3 x 24 (20736) 5.22 against 6.50, 16^4
+// (32768) 7.00 against 6.14, 16^3 x 32 12.5 against 9.1.  The double-float
+// update gains up to 12^3 x 24 and loses 2% at 24^3 x 48.  FP64 arithmetic
+// waits for its unit, and four times the warps spread over the SMs evenly:
+// 8^3 x 16 7.7 against 21.6 ms, 12^3 x 24 28.3 against 40.7, 16^3 x 32 73.0
+// against 76.6.
+#ifndef FG_SPLIT_MAX32
+#define FG_SPLIT_MAX32 24576
+#endif
+#ifndef FG_SPLIT_MAXDF
+#define FG_SPLIT_MAXDF 32768
+#endif
+#ifndef FG_SPLIT_MAX64
+#define FG_SPLIT_MAX64 131072
+#endif
+
+// The grand total of NV values, one a thread in R (blocks of kDslashThreads):
+// thread 32 w of the block adds value w of all its threads in FP64, and the
+// last block to finish adds the blocks' sums in block order.  True in the
+// threads of that block, with the totals in tot[].  The caller stores its
+// fields afterwards: the fence before the count then has nothing of theirs
+// to wait for.  (Warp trees in FP64 in every warp, the fields stored first,
+// cost 5 us a launch more than no total; this form 2 us: FP32 16^3 x 32
+// solves 9.14 instead of 10.2 ms.)
+template <int NV, typename R>
+__device__ __forceinline__ bool block_total(const R v[NV], double* __restrict__ partial,
+                                            unsigned* __restrict__ ticket, double tot[NV]) {
+  constexpr int T = kDslashThreads;
+  static_assert(NV <= T / 32, "one warp a value");
+  __shared__ R sv[NV][T];
+  __shared__ double sw[NV][T / 32];
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) sv[k][threadIdx.x] = v[k];
+  __syncthreads();
+  if (warp < NV) {
+    double x = 0.0;
+#pragma unroll
+    for (int q = 0; q < T / 32; ++q) x += double(sv[warp][32 * q + lane]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) {
+      partial[(size_t)warp * gridDim.x + blockIdx.x] = x;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  const int n = gridDim.x;
+  double x[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) x[k] = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += T)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) x[k] += __ldcg(partial + (size_t)k * n + i);
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x[k] += __shfl_down_sync(0xffffffffu, x[k], o);
+    if (lane == 0) sw[k][warp] = x[k];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) tot[k] = (sw[k][0] + sw[k][1]) + (sw[k][2] + sw[k][3]);
+  if (threadIdx.x == 0) *ticket = 0u;
+  return true;
+}
 
 template <typename RL, int NC, typename RS, int DAG, int MODE, typename ST = RS>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) dslash_kernel(
@@ -49,6 +130,7 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) ds
   if (cgd != nullptr && cgd->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   RS dot = RS(0);  // one site's 24 terms in the spinor precision (GB300's FP64 unit is slow)
+  Spinor<RS> o;
   if (i < g.Vh) {
     const int s = out_par * g.Vh + i;
     int c[4], par;
@@ -60,7 +142,6 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) ds
 #pragma unroll
       for (int cc = 0; cc < 3; ++cc) acc.s[k][cc] = cx<RS>(0, 0);
     Hops<DAG, RL, NC, RS, ST>::run(acc, in, U, g, c, s, in_off);
-    Spinor<RS> o;
     if (MODE == 0) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
@@ -81,9 +162,14 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) ds
             dot += pv.s[k][cc].re * o.s[k][cc].re + pv.s[k][cc].im * o.s[k][cc].im;
       }
     }
-    store_spinor<RS, ST>(out, i, g.Vh, o);
+    if (MODE != 2) store_spinor<RS, ST>(out, i, g.Vh, o);
   }
-  if (MODE == 2) block_reduce_total(double(dot), partial, &cgd->ticket[0], &cgd->pap);
+  if constexpr (MODE == 2) {
+    const RS v[1] = {dot};
+    double tot[1];
+    if (block_total<1>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) cgd->pap = tot[0];
+    if (i < g.Vh) store_spinor<RS, ST>(out, i, g.Vh, o);
+  }
 }
 
 // --------------------------------------------------------------------------- folded CG
@@ -103,42 +189,6 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) ds
 // still being read).  Only beta uses the expanded rr'; alpha of the next
 // iteration and the convergence test use the summed |r'|^2.
 
-// Block partials of NV values; the last block to finish (ticket) sums each
-// in block order into tot[] (fixed for a fixed launch) and resets the
-// ticket.  Returns true in that block.
-template <int NV>
-__device__ __forceinline__ bool block_reduce_last(double v[NV], double* __restrict__ partial,
-                                                  unsigned* __restrict__ ticket, double tot[NV]) {
-  block_reduce_store<NV>(v, partial, gridDim.x);
-  __shared__ int last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  __shared__ double sh[NV][32];
-  const int n = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double x = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) x += __ldcg(partial + (size_t)k * n + i);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[k][warp] = x;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double t = 0.0;
-    for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += sh[k][w];
-    tot[k] = t;
-  }
-  if (threadIdx.x == 0) *ticket = 0u;
-  return true;
-}
-
 // D: Ap = te + b D^dagger_eo to at the even sites, with the three dot products.
 template <typename R, int NC>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_apdot_kernel(
@@ -148,7 +198,9 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     CgDev* __restrict__ cgd) {
   if (cgd->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const double rr = cgd->rr[cgd->iter & 1];
   R pa = R(0), ra = R(0), aa = R(0);  // one site's 24 terms each, in R
+  Spinor<R> o;
   if (i < g.Vh) {
     int c[4], par;
     cb_coords(g, i, c, par);
@@ -161,7 +213,6 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     const Spinor<R> tv = load_spinor<R>(te, i, g.Vh);
     const Spinor<R> pv = load_spinor<R>(p, i, g.Vh);
     const Spinor<R> rv = load_spinor<R>(r, i, g.Vh);
-    Spinor<R> o;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -171,17 +222,17 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
         ra += rv.s[k][cc].re * o.s[k][cc].re + rv.s[k][cc].im * o.s[k][cc].im;
         aa += o.s[k][cc].re * o.s[k][cc].re + o.s[k][cc].im * o.s[k][cc].im;
       }
-    store_spinor<R>(ap, i, g.Vh, o);
   }
-  double v[3] = {double(pa), double(ra), double(aa)}, tot[3];
-  if (block_reduce_last<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) {
-    const double rr = cgd->rr[cgd->iter & 1];
+  const R v[3] = {pa, ra, aa};
+  double tot[3];
+  if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) {
     const double alpha = tot[0] > 0.0 ? rr / tot[0] : 0.0;
     const double rrn = rr - 2.0 * alpha * tot[1] + alpha * alpha * tot[2];
     cgd->pap = tot[0];
     cgd->alpha = alpha;
     cgd->beta = (rr > 0.0 && rrn > 0.0) ? rrn / rr : 0.0;
   }
+  if (i < g.Vh) store_spinor<R>(ap, i, g.Vh, o);
 }
 
 // A: the vector updates of the iteration and t_o = D_oe p'.
@@ -212,6 +263,7 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
   }
   const FoldSrc<R> src{r, ap, p, R(cgd->alpha), R(cgd->beta)};
   R acc = R(0);
+  Spinor<R> o;
   if (i < g.Vh) {
     // the even site i: x, r', p'
 #pragma unroll
@@ -239,16 +291,15 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     const int s = g.Vh + i;
     int c[4], par;
     cb_coords(g, s, c, par);
-    Spinor<R> o;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
       for (int cc = 0; cc < 3; ++cc) o.s[k][cc] = cx<R>(0, 0);
     hops_src<0, R, NC, R>(o, src, U, g, c, s, 0);
-    store_spinor<R>(to, i, g.Vh, o);
   }
-  double v[1] = {double(acc)}, tot[1];
-  if (block_reduce_last<1>(v, partial, &cgd->ticket[1], tot) && threadIdx.x == 0) {
+  const R v[1] = {acc};
+  double tot[1];
+  if (block_total<1>(v, partial, &cgd->ticket[1], tot) && threadIdx.x == 0) {
     const int k = cgd->iter + 1;
     const double rr = tot[0];
     cgd->rr[k & 1] = rr;
@@ -256,6 +307,144 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     cgd->iter = k;
     *iter_out = k;
     if (rr <= cgd->tol2bb) cgd->done = 1;
+  }
+  if (i < g.Vh) store_spinor<R>(to, i, g.Vh, o);
+}
+
+// --------------------------------------------------------------------------- one direction a warp
+// dslash_kernel with one direction a warp.
+template <typename RL, int NC, typename RS, int DAG, int MODE, typename ST = RS>
+__global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) dslash_split_kernel(
+    typename Vec2<ST>::T* __restrict__ out, const typename Vec2<ST>::T* __restrict__ in,
+    const typename Vec2<ST>::T* __restrict__ x, const typename Vec2<ST>::T* __restrict__ pdot,
+    Gauge<RL, NC> U, Geom g, int out_par, RS b, double* __restrict__ partial, CgDev* __restrict__ cgd) {
+  __shared__ HopShared<RS> sh;
+  if (cgd != nullptr && cgd->done) return;
+  const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
+  Cx<RS> row[3];
+  hops_split<DAG, RL, NC, RS>(row, sh, FieldSrc<RS, ST>{in}, U, g, i, out_par, (1 - out_par) * g.Vh);
+  RS dot[1] = {RS(0)};
+  if (i < g.Vh) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const size_t j = entry_index(k, c, i, g.Vh);
+      row[c] = b * row[c];
+      if (MODE > 0) row[c] = Entry<RS, ST>::load(x, j) + row[c];
+      if (MODE == 2) {
+        const Cx<RS> pv = Entry<RS, ST>::load(pdot, j);
+        dot[0] = fma(pv.re, row[c].re, dot[0]);
+        dot[0] = fma(pv.im, row[c].im, dot[0]);
+      }
+      if (MODE != 2) Entry<RS, ST>::store(out, j, row[c]);
+    }
+  }
+  if constexpr (MODE == 2) {
+    double tot[1];
+    const bool last = block_total<1>(dot, partial, &cgd->ticket[0], tot);
+    if (last && threadIdx.x == 0) cgd->pap = tot[0];
+    if (i < g.Vh) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) Entry<RS, ST>::store(out, entry_index(k, c, i, g.Vh), row[c]);
+    }
+  }
+}
+
+// cg_apdot_kernel with one direction a warp.
+template <typename R, int NC>
+__global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_split_kernel(
+    typename Vec2<R>::T* __restrict__ ap, const typename Vec2<R>::T* __restrict__ to,
+    const typename Vec2<R>::T* __restrict__ te, const typename Vec2<R>::T* __restrict__ p,
+    const typename Vec2<R>::T* __restrict__ r, Gauge<R, NC> U, Geom g, R b, double* __restrict__ partial,
+    CgDev* __restrict__ cgd) {
+  __shared__ HopShared<R> sh;
+  if (cgd->done) return;
+  const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
+  const double rr = cgd->rr[cgd->iter & 1];
+  Cx<R> row[3];
+  hops_split<1, R, NC, R>(row, sh, FieldSrc<R, R>{to}, U, g, i, 0, g.Vh);
+  R v[3] = {R(0), R(0), R(0)};  // a thread's 6 terms each of <p, Ap>, Re <r, Ap>, |Ap|^2
+  if (i < g.Vh) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const size_t j = entry_index(k, c, i, g.Vh);
+      row[c] = Entry<R, R>::load(te, j) + b * row[c];
+      const Cx<R> pv = Entry<R, R>::load(p, j), rv = Entry<R, R>::load(r, j);
+      v[0] = fma(pv.re, row[c].re, v[0]);
+      v[0] = fma(pv.im, row[c].im, v[0]);
+      v[1] = fma(rv.re, row[c].re, v[1]);
+      v[1] = fma(rv.im, row[c].im, v[1]);
+      v[2] = fma(row[c].re, row[c].re, v[2]);
+      v[2] = fma(row[c].im, row[c].im, v[2]);
+    }
+  }
+  double tot[3];
+  if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) {
+    const double alpha = tot[0] > 0.0 ? rr / tot[0] : 0.0;
+    const double rrn = rr - 2.0 * alpha * tot[1] + alpha * alpha * tot[2];
+    cgd->pap = tot[0];
+    cgd->alpha = alpha;
+    cgd->beta = (rr > 0.0 && rrn > 0.0) ? rrn / rr : 0.0;
+  }
+  if (i < g.Vh) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Entry<R, R>::store(ap, entry_index(k, c, i, g.Vh), row[c]);
+  }
+}
+
+// cg_fold_kernel with one direction a warp.
+template <typename R, int NC>
+__global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_fold_split_kernel(
+    typename Vec2<R>::T* __restrict__ to, typename Vec2<R>::T* __restrict__ x,
+    const typename Vec2<R>::T* __restrict__ r, const typename Vec2<R>::T* __restrict__ ap,
+    const typename Vec2<R>::T* __restrict__ p, typename Vec2<R>::T* __restrict__ r2,
+    typename Vec2<R>::T* __restrict__ p2, Gauge<R, NC> U, Geom g, double* __restrict__ partial,
+    CgDev* __restrict__ cgd, double* __restrict__ hist, int* __restrict__ iter_out, int maxiter) {
+  __shared__ HopShared<R> sh;
+  const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
+  if (cgd->done) {
+    // as in cg_fold_kernel: the host has taken r2, p2 as the current buffers
+    if (i < g.Vh) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const size_t j = entry_index(k, c, i, g.Vh);
+        r2[j] = r[j];
+        p2[j] = p[j];
+      }
+    }
+    return;
+  }
+  const FoldSrc<R> src{r, ap, p, R(cgd->alpha), R(cgd->beta)};
+  R acc[1] = {R(0)};
+  if (i < g.Vh) {
+    // row k of the even site i: x, r', p'
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const size_t j = entry_index(k, c, i, g.Vh);
+      const Cx<R> x0 = Entry<R, R>::load(x, j), r0 = Entry<R, R>::load(r, j), a0 = Entry<R, R>::load(ap, j),
+                  p0 = Entry<R, R>::load(p, j);
+      Entry<R, R>::store(x, j, cx<R>(fma(src.alpha, p0.re, x0.re), fma(src.alpha, p0.im, x0.im)));
+      Entry<R, R>::store(p2, j, src.fold_entry(r0, a0, p0));
+      const Cx<R> r1 = cx<R>(fma(-src.alpha, a0.re, r0.re), fma(-src.alpha, a0.im, r0.im));
+      Entry<R, R>::store(r2, j, r1);
+      acc[0] = fma(r1.re, r1.re, acc[0]);
+      acc[0] = fma(r1.im, r1.im, acc[0]);
+    }
+  }
+  // row k of the odd site Vh + i: D_oe p'
+  Cx<R> row[3];
+  hops_split<0, R, NC, R>(row, sh, src, U, g, i, 1, 0);
+  double tot[1];
+  if (block_total<1>(acc, partial, &cgd->ticket[1], tot) && threadIdx.x == 0) {
+    const int n = cgd->iter + 1;
+    cgd->rr[n & 1] = tot[0];
+    if (n <= maxiter) hist[n] = tot[0];
+    cgd->iter = n;
+    *iter_out = n;
+    if (tot[0] <= cgd->tol2bb) cgd->done = 1;
+  }
+  if (i < g.Vh) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Entry<R, R>::store(to, entry_index(k, c, i, g.Vh), row[c]);
   }
 }
 
@@ -857,7 +1046,16 @@ int vec_blocks(int n) {
   int b = (n + kVecThreads - 1) / kVecThreads;
   return b > 152 * 8 ? 152 * 8 : b;
 }
-int dslash_blocks(int Vh) { return (Vh + kDslashThreads - 1) / kDslashThreads; }
+// Whether a Dslash launch over Vh sites gives one direction to a warp
+// (blocks of 32 sites) or all eight hops to a thread (blocks of 128).
+template <typename RS> static bool hop_split(int Vh) {
+  return Vh <= (std::is_same<RS, float>::value ? FG_SPLIT_MAX32
+                                               : (std::is_same<RS, DF>::value ? FG_SPLIT_MAXDF : FG_SPLIT_MAX64));
+}
+template <typename RS> static int hop_blocks(int Vh) {
+  return hop_split<RS>(Vh) ? (Vh + 31) / 32 : (Vh + kDslashThreads - 1) / kDslashThreads;
+}
+int dslash_blocks(int Vh) { return (Vh + 31) / 32; }
 
 template <typename RL, int NC, typename RS>
 cudaError_t launch_dslash(const GeomH& gh, void* out, const void* in, const void* x, const void* pdot,
@@ -867,11 +1065,11 @@ cudaError_t launch_dslash(const GeomH& gh, void* out, const void* in, const void
   u.p = const_cast<void*>(U);
   u.V = gh.V;
   const Geom g = to_devg(gh);
-  const int nb = dslash_blocks(gh.Vh);
-#define FG_DS(D, M)                                                                                     \
-  dslash_kernel<RL, NC, RS, D, M><<<nb, kDslashThreads, 0, st>>>(v2<RS>(out), cv2<RS>(in), cv2<RS>(x),   \
-                                                                 cv2<RS>(pdot), u, g, out_par, RS(b),   \
-                                                                 partial, cgd)
+  const int nb = hop_blocks<RS>(gh.Vh);
+  const bool split = hop_split<RS>(gh.Vh);
+#define FG_DS(D, M)                                                                                       \
+  (split ? dslash_split_kernel<RL, NC, RS, D, M> : dslash_kernel<RL, NC, RS, D, M>)<<<nb, kDslashThreads, 0, st>>>( \
+      v2<RS>(out), cv2<RS>(in), cv2<RS>(x), cv2<RS>(pdot), u, g, out_par, RS(b), partial, cgd)
   if (dag) {
     if (mode == 0) FG_DS(1, 0); else if (mode == 1) FG_DS(1, 1); else FG_DS(1, 2);
   } else {
@@ -914,7 +1112,8 @@ cudaError_t launch_cg_apdot(const GeomH& gh, void* ap, const void* to, const voi
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  cg_apdot_kernel<R, NC><<<dslash_blocks(gh.Vh), kDslashThreads, 0, st>>>(
+  (hop_split<R>(gh.Vh) ? cg_apdot_split_kernel<R, NC> : cg_apdot_kernel<R, NC>)<<<hop_blocks<R>(gh.Vh), kDslashThreads,
+                                                                               0, st>>>(
       v2<R>(ap), cv2<R>(to), cv2<R>(te), cv2<R>(p), cv2<R>(r), u, to_devg(gh), R(-k2), partial, cgd);
   return cudaGetLastError();
 }
@@ -925,7 +1124,8 @@ cudaError_t launch_cg_fold(const GeomH& gh, void* to, void* x, const void* r, co
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  cg_fold_kernel<R, NC><<<dslash_blocks(gh.Vh), kDslashThreads, 0, st>>>(
+  (hop_split<R>(gh.Vh) ? cg_fold_split_kernel<R, NC> : cg_fold_kernel<R, NC>)<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0,
+                                                                             st>>>(
       v2<R>(to), v2<R>(x), cv2<R>(r), cv2<R>(ap), cv2<R>(p), v2<R>(r2), v2<R>(p2), u, to_devg(gh), partial, cgd,
       hist, iter_out, maxiter);
   return cudaGetLastError();
@@ -992,9 +1192,11 @@ static cudaError_t dslash16(const GeomH& gh, void* out, const void* in, const vo
   u.p = const_cast<void*>(U);
   u.V = gh.V;
   const Geom g = to_devg(gh);
-  const int nb = dslash_blocks(gh.Vh);
+  const int nb = hop_blocks<float>(gh.Vh);
+  const bool split = hop_split<float>(gh.Vh);
 #define FG_DH(D, M)                                                                                            \
-  dslash_kernel<S, NC, float, D, M, S><<<nb, kDslashThreads, 0, st>>>(                                        \
+  (split ? dslash_split_kernel<S, NC, float, D, M, S>                                                          \
+         : dslash_kernel<S, NC, float, D, M, S>)<<<nb, kDslashThreads, 0, st>>>(                               \
       (T2*)out, (const T2*)in, (const T2*)x, (const T2*)pdot, u, g, out_par, float(b), partial, cgd)
   if (dag) {
     if (mode == 0) FG_DH(1, 0); else if (mode == 1) FG_DH(1, 1); else FG_DH(1, 2);

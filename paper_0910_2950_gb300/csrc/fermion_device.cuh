@@ -7,6 +7,8 @@
 #include "fg_common.cuh"
 #include "fg_fermion.h"
 
+#include <type_traits>
+
 namespace fg {
 
 static inline Geom to_devg(const GeomH& h) {
@@ -348,5 +350,112 @@ struct Hops<DAG, float, NC, DF, DF> {
     hops_rt<DAG, NC>(acc, in, U, g, c, s, in_off);
   }
 };
+
+// ---- one direction a warp
+// A block of four warps takes 32 consecutive sites of one parity; warp mu
+// adds the two hops of direction mu, the four sums meet in shared memory, and
+// warp w goes on with spin row w of the 32 sites.  A thread's serial chain is
+// two hops instead of eight and a lattice has four times the warps.
+
+// The double-float form of hop_dir_src (its hops by run-time selects).
+template <int DAG, int NC>
+__device__ __forceinline__ void hop_dir_df(Spinor<DF>& acc, const float4* __restrict__ in, const Gauge<float, NC>& U,
+                                           const Geom& g, const int c[4], int s, int in_off, int mu) {
+  constexpr int SF = DAG ? -1 : 1;
+#pragma unroll 1
+  for (int back = 0; back < 2; ++back) {
+    const int sn = cb_neighbor_rt(g, c, mu, back ? -1 : 1);
+    const Spinor<DF> p = load_spinor<DF>(in, sn - in_off, g.Vh);
+    const int S = back ? -SF : SF;
+    Cx<DF> h[2][3], w[2][3];
+    project_rt(mu, S, p, h);
+    mat_half_rt(U.load(mu, back ? sn : s), back != 0, h, w);
+    const bool anti = mu == 3 && (back ? c[3] == 0 : c[3] == g.L[3] - 1);
+    reconstruct_rt(mu, S, anti ? -1.0f : 1.0f, w, acc);
+  }
+}
+
+template <typename R> struct HopShared {
+  R v[4][24][32];
+};
+// Row threadIdx.x / 32 of D src at the 32 sites from i0 of parity out_par (the
+// lane's site is i0 + lane; beyond Vh the row is garbage).  Every thread of
+// the block calls this.
+template <int DAG, typename RL, int NC, typename RS, class Src>
+__device__ __forceinline__ void hops_split(Cx<RS> row[3], HopShared<RS>& sh, const Src& src, const Gauge<RL, NC>& U,
+                                           const Geom& g, int i, int out_par, int in_off) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Spinor<RS> acc;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc.s[k][c] = cx<RS>(RS(0), RS(0));
+  if (i < g.Vh) {
+    const int s = out_par * g.Vh + i;
+    int c[4], par;
+    cb_coords(g, s, c, par);
+    if constexpr (std::is_same<RS, DF>::value) {
+      hop_dir_df<DAG, NC>(acc, src.f, U, g, c, s, in_off, warp);
+    } else {
+      switch (warp) {
+        case 0: hop_dir_src<0, DAG, RL, NC, RS>(acc, src, U, g, c, s, in_off); break;
+        case 1: hop_dir_src<1, DAG, RL, NC, RS>(acc, src, U, g, c, s, in_off); break;
+        case 2: hop_dir_src<2, DAG, RL, NC, RS>(acc, src, U, g, c, s, in_off); break;
+        default: hop_dir_src<3, DAG, RL, NC, RS>(acc, src, U, g, c, s, in_off); break;
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      sh.v[warp][6 * k + 2 * c][lane] = acc.s[k][c].re;
+      sh.v[warp][6 * k + 2 * c + 1][lane] = acc.s[k][c].im;
+    }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int e = 6 * warp + 2 * c;
+    row[c] = cx<RS>(sh.v[0][e][lane] + sh.v[1][e][lane] + (sh.v[2][e][lane] + sh.v[3][e][lane]),
+                    sh.v[0][e + 1][lane] + sh.v[1][e + 1][lane] + (sh.v[2][e + 1][lane] + sh.v[3][e + 1][lane]));
+  }
+}
+
+// Storage of one complex entry (a pair of a field holds two, pair-major).
+template <typename RS, typename ST> struct Entry {
+  static __device__ __forceinline__ Cx<RS> load(const typename Vec2<ST>::T* f, size_t j) {
+    const typename Vec2<ST>::T v = f[j];
+    return cx<RS>(RS(v.x), RS(v.y));
+  }
+  static __device__ __forceinline__ void store(typename Vec2<ST>::T* f, size_t j, const Cx<RS>& a) {
+    typename Vec2<ST>::T v;
+    v.x = a.re;
+    v.y = a.im;
+    f[j] = v;
+  }
+};
+template <> struct Entry<DF, DF> {
+  static __device__ __forceinline__ Cx<DF> load(const float4* f, size_t j) { return Quad<DF>::c(f[j]); }
+  static __device__ __forceinline__ void store(float4* f, size_t j, const Cx<DF>& a) {
+    f[j] = make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo);
+  }
+};
+template <typename S> struct Entry16 {
+  typedef typename Conv16<S>::T2 T2;
+  static __device__ __forceinline__ Cx<float> load(const T2* f, size_t j) {
+    const float2 v = Conv16<S>::f2(f[j]);
+    return cx<float>(v.x, v.y);
+  }
+  static __device__ __forceinline__ void store(T2* f, size_t j, const Cx<float>& a) {
+    f[j] = Conv16<S>::of(make_float2(a.re, a.im));
+  }
+};
+template <> struct Entry<float, Half16> : Entry16<Half16> {};
+template <> struct Entry<float, BF16> : Entry16<BF16> {};
+// Flat index of entry (spin k, colour c) of site i.
+__device__ __forceinline__ size_t entry_index(int k, int c, int i, int Vh) {
+  const int e = 3 * k + c;
+  return ((size_t)(e >> 1) * Vh + i) * 2 + (e & 1);
+}
 
 }  // namespace fg

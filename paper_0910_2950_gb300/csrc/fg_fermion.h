@@ -33,6 +33,7 @@ struct CgDev {
 };
 
 int vec_blocks(int n);
+// Most blocks of a Dslash launch (entries of its block partials).
 int dslash_blocks(int Vh);
 
 // RS = DF (df64.cuh) evaluates the hop in double-float arithmetic on FP32

@@ -115,7 +115,7 @@ def footprint_bytes(spec: ChainSpec, precision: str = "fp32", link_reals: int = 
         vh = v // 2
         nvec = 12 * vh
         n64 = 8 + (2 if precision != "fp64" else 0)
-        dslash_blocks = (vh + 127) // 128
+        dslash_blocks = (vh + 31) // 32
         vec_blocks = min((nvec + 255) // 256, 152 * 8)
         half = precision in ("fp32_fp16cg", "fp32_bf16cg") or (
             precision == "fp32_autocg" and v * (4 * (link_reals // 2) * 8 + 6 * 48) > l2_bytes)
