@@ -983,7 +983,7 @@ class Backend final : public IBackend {
       if ((s = alloc(&FF_, (size_t)4 * 4 * g_.V * sizeof(C2))) != FG_OK) return s;
       if ((s = alloc((void**)&cgd_, sizeof(CgDev))) != FG_OK) return s;
       if (cudaMemsetAsync(cgd_, 0, sizeof(CgDev), st_) != cudaSuccess) return cuda_fail("cg state init");
-      if ((s = alloc((void**)&part_pap_, (3 * dslash_blocks(g_.Vh) + 1) * sizeof(double))) != FG_OK) return s;
+      if ((s = alloc((void**)&part_pap_, 4 * dslash_blocks(g_.Vh) * sizeof(double))) != FG_OK) return s;
       if ((s = alloc((void**)&part_rr_, (vec_blocks(nvec()) + 1) * sizeof(double))) != FG_OK) return s;
       if ((s = alloc((void**)&part_b_, (vec_blocks(nvec()) + 1) * sizeof(double))) != FG_OK) return s;
       const size_t mbytes = sizeof(Mapped) + (size_t)(h_->prm.cg_maxiter + 8) * sizeof(double);
@@ -1155,6 +1155,21 @@ class Backend final : public IBackend {
       return cudaErrorNotSupported;
     }
   }
+  cudaError_t fold_hop(const void* U) {
+    if constexpr (kMixed || std::is_same<R, double>::value) {
+      const double k2 = h_->prm.kappa * h_->prm.kappa;
+      return launch_cg_hop<R, NC>(g_, te_, to_, p_, U, k2, part_pap_, cgd_, mapped_->hist, &mapped_->dev_iter,
+                                  h_->prm.cg_maxiter, st_);
+    } else {
+      return cudaErrorNotSupported;
+    }
+  }
+  // Whether a batch of folded iterations ends with a launch that publishes
+  // the last one, and that launch.
+  bool fold_deferred() const { return fold_ && cg_deferred(g_.Vh, !kMixed); }
+  cudaError_t fold_publish() {
+    return launch_cg_publish(g_, part_pap_, cgd_, mapped_->hist, &mapped_->dev_iter, h_->prm.cg_maxiter, st_);
+  }
   // t_o = D_oe p, which the folded iteration expects on entry (after the
   // setup and after every reliable update, which may replace p).
   fg_status fold_prime(const void* U) {
@@ -1169,7 +1184,7 @@ class Backend final : public IBackend {
     const int n = nvec();
     cudaError_t e;
     if (fold_) {
-      if ((e = inner_dslash(te_, to_, p_, nullptr, U, 0, 0, 1, -k2, nullptr)) != cudaSuccess) return e;
+      if ((e = fold_hop(U)) != cudaSuccess) return e;
       if ((e = inner_dslash(to_, te_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr)) != cudaSuccess) return e;
       if ((e = fold_apdot(U)) != cudaSuccess) return e;
       return fold_update(U);
@@ -1196,9 +1211,7 @@ class Backend final : public IBackend {
     const int n = nvec();
     fg_status s;
     if (fold_) {
-      if ((s = run(KC_DSLASH, [&] { return inner_dslash(te_, to_, p_, nullptr, U, 0, 0, 1, -k2, nullptr); })) !=
-          FG_OK)
-        return s;
+      if ((s = run(KC_DSLASH, [&] { return fold_hop(U); })) != FG_OK) return s;
       if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, te_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr); })) !=
           FG_OK)
         return s;
@@ -1263,6 +1276,7 @@ class Backend final : public IBackend {
     }
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < n && e == cudaSuccess; ++i) e = cg_iteration_raw(U);
+    if (e == cudaSuccess && fold_deferred()) e = fold_publish();
     cudaError_t e2 = cudaStreamEndCapture(st_, &graph);
     if (rs_ != r_at_capture) {  // a capture that stopped after an odd number of folded iterations
       std::swap(rs_, rs2_);
@@ -1289,7 +1303,7 @@ class Backend final : public IBackend {
       if (g != nullptr) {
         if (cudaGraphLaunch(g, st_) != cudaSuccess) return cuda_fail("cg graph launch");
         // an even number of folded iterations leaves rs_ and p_ where they were
-        h_->launches += (fold_ ? 4 : 6) * n;
+        h_->launches += (fold_ ? 4 : 6) * n + (fold_deferred() ? 1 : 0);
         return FG_OK;
       }
     }
@@ -1297,6 +1311,7 @@ class Backend final : public IBackend {
       fg_status s = cg_iteration(U);
       if (s != FG_OK) return s;
     }
+    if (fold_deferred()) return run(KC_REDUCE, [&] { return fold_publish(); });
     return FG_OK;
   }
 

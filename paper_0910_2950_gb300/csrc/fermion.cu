@@ -58,6 +58,10 @@ template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_
 #ifndef FG_SPLIT_MAX32
 #define FG_SPLIT_MAX32 24576
 #endif
+// Most sites with deferred totals (cg_fold_split_kernel).
+#ifndef FG_DEFER_MAX
+#define FG_DEFER_MAX 24576
+#endif
 #ifndef FG_SPLIT_MAXDF
 #define FG_SPLIT_MAXDF 32768
 #endif
@@ -189,6 +193,31 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) ds
 // still being read).  Only beta uses the expanded rr'; alpha of the next
 // iteration and the convergence test use the summed |r'|^2.
 
+// alpha = rr / <p, Ap> and beta = |r - alpha Ap|^2 / rr from rr and the three sums.
+__device__ __forceinline__ void alpha_beta(double rr, const double tot[3], double& alpha, double& beta) {
+  alpha = tot[0] > 0.0 ? rr / tot[0] : 0.0;
+  const double rrn = rr - 2.0 * alpha * tot[1] + alpha * alpha * tot[2];
+  beta = (rr > 0.0 && rrn > 0.0) ? rrn / rr : 0.0;
+}
+__device__ __forceinline__ void set_alpha_beta(CgDev* cgd, const double tot[3]) {
+  double alpha, beta;
+  alpha_beta(cgd->rr[cgd->iter & 1], tot, alpha, beta);
+  cgd->pap = tot[0];
+  cgd->alpha = alpha;
+  cgd->beta = beta;
+}
+// |r|^2 of the iteration just done: rr, the history, the count (also to the
+// host), done.
+__device__ __forceinline__ void publish(CgDev* cgd, double rr, double* __restrict__ hist, int* __restrict__ iter_out,
+                                        int maxiter) {
+  const int k = cgd->iter + 1;
+  cgd->rr[k & 1] = rr;
+  if (k <= maxiter) hist[k] = rr;
+  cgd->iter = k;
+  *iter_out = k;
+  if (rr <= cgd->tol2bb) cgd->done = 1;
+}
+
 // D: Ap = te + b D^dagger_eo to at the even sites, with the three dot products.
 template <typename R, int NC>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_apdot_kernel(
@@ -198,7 +227,6 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     CgDev* __restrict__ cgd) {
   if (cgd->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const double rr = cgd->rr[cgd->iter & 1];
   R pa = R(0), ra = R(0), aa = R(0);  // one site's 24 terms each, in R
   Spinor<R> o;
   if (i < g.Vh) {
@@ -225,13 +253,7 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
   }
   const R v[3] = {pa, ra, aa};
   double tot[3];
-  if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) {
-    const double alpha = tot[0] > 0.0 ? rr / tot[0] : 0.0;
-    const double rrn = rr - 2.0 * alpha * tot[1] + alpha * alpha * tot[2];
-    cgd->pap = tot[0];
-    cgd->alpha = alpha;
-    cgd->beta = (rr > 0.0 && rrn > 0.0) ? rrn / rr : 0.0;
-  }
+  if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_alpha_beta(cgd, tot);
   if (i < g.Vh) store_spinor<R>(ap, i, g.Vh, o);
 }
 
@@ -299,15 +321,8 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
   }
   const R v[1] = {acc};
   double tot[1];
-  if (block_total<1>(v, partial, &cgd->ticket[1], tot) && threadIdx.x == 0) {
-    const int k = cgd->iter + 1;
-    const double rr = tot[0];
-    cgd->rr[k & 1] = rr;
-    if (k <= maxiter) hist[k] = rr;
-    cgd->iter = k;
-    *iter_out = k;
-    if (rr <= cgd->tol2bb) cgd->done = 1;
-  }
+  if (block_total<1>(v, partial, &cgd->ticket[1], tot) && threadIdx.x == 0)
+    publish(cgd, tot[0], hist, iter_out, maxiter);
   if (i < g.Vh) store_spinor<R>(to, i, g.Vh, o);
 }
 
@@ -349,8 +364,86 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) dslash_sp
   }
 }
 
-// cg_apdot_kernel with one direction a warp.
+// The folded iteration with one direction a warp.  DEFER: D and A leave block
+// sums and no totals: A adds D's when it starts and A's are added by one more
+// block of the next B, beside its Dslash, or by cg_publish_kernel at the end
+// of a batch.  Otherwise the last block to finish adds them, as above: 4 us
+// more in each of D and A on a small lattice (8^3 x 16: an FP32 solve 3.48
+// against 2.82 ms; 12^3 x 24: 5.22 against 4.93), no difference where A's
+// blocks add a thousand sums each (FP64 16^4: 37.5 against 37.4 ms).
+
+// Block sums of NV values, one a thread in R: warp w adds value w in FP64.
+template <int NV, typename R>
+__device__ __forceinline__ void block_sums(const R v[NV], double* __restrict__ partial, int nblocks) {
+  constexpr int T = kDslashThreads;
+  static_assert(NV <= T / 32, "one warp a value");
+  __shared__ R sv[NV][T];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) sv[k][threadIdx.x] = v[k];
+  __syncthreads();
+  if (warp < NV) {
+    double x = 0.0;
+#pragma unroll
+    for (int q = 0; q < T / 32; ++q) x += double(sv[warp][32 * q + lane]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) partial[(size_t)warp * nblocks + blockIdx.x] = x;
+  }
+}
+// Sum of n block sums by one warp, in a fixed order (lane 0 has it).
+__device__ __forceinline__ double warp_sum(const double* __restrict__ part, int n) {
+  double x = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 31; i < n; i += 32) x += part[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  return x;
+}
+// Publishes |r|^2 of the iteration whose A left its block sums: rr, the
+// history, the iteration count (also to the host), done.
+__device__ __forceinline__ void publish_iteration(const double* __restrict__ part, int n, CgDev* __restrict__ cgd,
+                                                  double* __restrict__ hist, int* __restrict__ iter_out,
+                                                  int maxiter) {
+  if (threadIdx.x >= 32 || !cgd->pending) return;
+  const double rr = warp_sum(part, n);
+  if (threadIdx.x == 0) {
+    cgd->pending = 0;
+    publish(cgd, rr, hist, iter_out, maxiter);
+  }
+}
+__global__ void cg_publish_kernel(const double* __restrict__ part, int n, CgDev* __restrict__ cgd,
+                                  double* __restrict__ hist, int* __restrict__ iter_out, int maxiter) {
+  publish_iteration(part, n, cgd, hist, iter_out, maxiter);
+}
+
+// B: te = p + b D_eo to, and in the last block the iteration before is published.
 template <typename R, int NC>
+__global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_hop_split_kernel(
+    typename Vec2<R>::T* __restrict__ te, const typename Vec2<R>::T* __restrict__ to,
+    const typename Vec2<R>::T* __restrict__ p, Gauge<R, NC> U, Geom g, R b, const double* __restrict__ partial,
+    CgDev* __restrict__ cgd, double* __restrict__ hist, int* __restrict__ iter_out, int maxiter) {
+  __shared__ HopShared<R> sh;
+  const int n = (int)gridDim.x - 1;
+  if ((int)blockIdx.x == n) {
+    publish_iteration(partial + (size_t)3 * n, n, cgd, hist, iter_out, maxiter);
+    return;
+  }
+  if (cgd->done) return;
+  const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
+  Cx<R> row[3];
+  hops_split<0, R, NC, R>(row, sh, FieldSrc<R, R>{to}, U, g, i, 0, g.Vh);
+  if (i < g.Vh) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const size_t j = entry_index(k, c, i, g.Vh);
+      Entry<R, R>::store(te, j, Entry<R, R>::load(p, j) + b * row[c]);
+    }
+  }
+}
+
+// D: Ap = te + b D^dagger_eo to, block sums of <p, Ap>, Re <r, Ap>, |Ap|^2.
+template <typename R, int NC, bool DEFER>
 __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_split_kernel(
     typename Vec2<R>::T* __restrict__ ap, const typename Vec2<R>::T* __restrict__ to,
     const typename Vec2<R>::T* __restrict__ te, const typename Vec2<R>::T* __restrict__ p,
@@ -359,15 +452,15 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_
   __shared__ HopShared<R> sh;
   if (cgd->done) return;
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
-  const double rr = cgd->rr[cgd->iter & 1];
   Cx<R> row[3];
   hops_split<1, R, NC, R>(row, sh, FieldSrc<R, R>{to}, U, g, i, 0, g.Vh);
-  R v[3] = {R(0), R(0), R(0)};  // a thread's 6 terms each of <p, Ap>, Re <r, Ap>, |Ap|^2
+  R v[3] = {R(0), R(0), R(0)};  // a thread's 6 terms each
   if (i < g.Vh) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const size_t j = entry_index(k, c, i, g.Vh);
       row[c] = Entry<R, R>::load(te, j) + b * row[c];
+      if (DEFER) Entry<R, R>::store(ap, j, row[c]);
       const Cx<R> pv = Entry<R, R>::load(p, j), rv = Entry<R, R>::load(r, j);
       v[0] = fma(pv.re, row[c].re, v[0]);
       v[0] = fma(pv.im, row[c].im, v[0]);
@@ -377,22 +470,21 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_
       v[2] = fma(row[c].im, row[c].im, v[2]);
     }
   }
-  double tot[3];
-  if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) {
-    const double alpha = tot[0] > 0.0 ? rr / tot[0] : 0.0;
-    const double rrn = rr - 2.0 * alpha * tot[1] + alpha * alpha * tot[2];
-    cgd->pap = tot[0];
-    cgd->alpha = alpha;
-    cgd->beta = (rr > 0.0 && rrn > 0.0) ? rrn / rr : 0.0;
-  }
-  if (i < g.Vh) {
+  if constexpr (DEFER) {
+    block_sums<3>(v, partial, gridDim.x);
+  } else {
+    double tot[3];
+    if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_alpha_beta(cgd, tot);
+    if (i < g.Vh) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) Entry<R, R>::store(ap, entry_index(k, c, i, g.Vh), row[c]);
+      for (int c = 0; c < 3; ++c) Entry<R, R>::store(ap, entry_index(k, c, i, g.Vh), row[c]);
+    }
   }
 }
 
-// cg_fold_kernel with one direction a warp.
-template <typename R, int NC>
+// A: alpha and beta from D's block sums (every block, the same bits), the
+// vector updates and to = D_oe p', block sums of |r'|^2.
+template <typename R, int NC, bool DEFER>
 __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_fold_split_kernel(
     typename Vec2<R>::T* __restrict__ to, typename Vec2<R>::T* __restrict__ x,
     const typename Vec2<R>::T* __restrict__ r, const typename Vec2<R>::T* __restrict__ ap,
@@ -400,6 +492,7 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_fold_s
     typename Vec2<R>::T* __restrict__ p2, Gauge<R, NC> U, Geom g, double* __restrict__ partial,
     CgDev* __restrict__ cgd, double* __restrict__ hist, int* __restrict__ iter_out, int maxiter) {
   __shared__ HopShared<R> sh;
+  __shared__ double dot[3], ab[2];
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
   if (cgd->done) {
     // as in cg_fold_kernel: the host has taken r2, p2 as the current buffers
@@ -413,7 +506,25 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_fold_s
     }
     return;
   }
-  const FoldSrc<R> src{r, ap, p, R(cgd->alpha), R(cgd->beta)};
+  if constexpr (DEFER) {
+    if (k < 3) {
+      const double t = warp_sum(partial + (size_t)k * gridDim.x, gridDim.x);
+      if ((threadIdx.x & 31) == 0) dot[k] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      alpha_beta(cgd->rr[cgd->iter & 1], dot, ab[0], ab[1]);
+      if (blockIdx.x == 0) cgd->pending = 1;
+    }
+    __syncthreads();
+  } else {
+    if (threadIdx.x == 0) {
+      ab[0] = cgd->alpha;
+      ab[1] = cgd->beta;
+    }
+    __syncthreads();
+  }
+  const FoldSrc<R> src{r, ap, p, R(ab[0]), R(ab[1])};
   R acc[1] = {R(0)};
   if (i < g.Vh) {
     // row k of the even site i: x, r', p'
@@ -433,19 +544,16 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_fold_s
   // row k of the odd site Vh + i: D_oe p'
   Cx<R> row[3];
   hops_split<0, R, NC, R>(row, sh, src, U, g, i, 1, 0);
-  double tot[1];
-  if (block_total<1>(acc, partial, &cgd->ticket[1], tot) && threadIdx.x == 0) {
-    const int n = cgd->iter + 1;
-    cgd->rr[n & 1] = tot[0];
-    if (n <= maxiter) hist[n] = tot[0];
-    cgd->iter = n;
-    *iter_out = n;
-    if (tot[0] <= cgd->tol2bb) cgd->done = 1;
+  if constexpr (!DEFER) {
+    double tot[1];
+    if (block_total<1>(acc, partial, &cgd->ticket[1], tot) && threadIdx.x == 0)
+      publish(cgd, tot[0], hist, iter_out, maxiter);
   }
   if (i < g.Vh) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) Entry<R, R>::store(to, entry_index(k, c, i, g.Vh), row[c]);
   }
+  if constexpr (DEFER) block_sums<1>(acc, partial + (size_t)3 * gridDim.x, gridDim.x);
 }
 
 // --------------------------------------------------------------------------- force
@@ -776,6 +884,7 @@ __global__ void cg_init_h16_kernel(const double* __restrict__ part, int nparts, 
     cgd->done = bb == 0.0 ? 1 : 0;
     cgd->iter = 0;
     cgd->k_axpy = 0;
+    cgd->pending = 0;
     cgd->restart = 0;
     *bb_out = bb;
   }
@@ -932,6 +1041,7 @@ __global__ void cg_init_kernel(const double* __restrict__ part, int n, CgDev* __
     cgd->done = bb == 0.0 ? 1 : 0;
     cgd->iter = 0;
     cgd->k_axpy = 0;
+    cgd->pending = 0;
     cgd->restart = 0;
     *bb_out = bb;
   }
@@ -951,6 +1061,7 @@ __global__ void cg_init_guess_kernel(const double* __restrict__ part_b, const do
     cgd->done = (bb == 0.0 || rr <= tol2 * bb) ? 1 : 0;
     cgd->iter = 0;
     cgd->k_axpy = 0;
+    cgd->pending = 0;
     cgd->restart = 0;
     *bb_out = bb;
     *rr0_out = rr;
@@ -1106,14 +1217,35 @@ cudaError_t launch_cg_xpay(void* p, const void* r, CgDev* cgd, double* hist, int
   cg_xpay_kernel<R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(p), cv2<R>(r), cgd, hist, iter_out, maxiter, n);
   return cudaGetLastError();
 }
+template <typename R> static bool cg_defer(int Vh) { return hop_split<R>(Vh) && Vh <= FG_DEFER_MAX; }
+bool cg_deferred(int Vh, bool fp64) { return fp64 ? cg_defer<double>(Vh) : cg_defer<float>(Vh); }
+template <typename R, int NC>
+cudaError_t launch_cg_hop(const GeomH& gh, void* te, const void* to, const void* p, const void* U, double k2,
+                          double* partial, CgDev* cgd, double* hist, int* iter_out, int maxiter, cudaStream_t st) {
+  if (!cg_defer<R>(gh.Vh))
+    return launch_dslash<R, NC, R>(gh, te, to, p, nullptr, U, 0, 0, 1, -k2, nullptr, cgd, st);
+  Gauge<R, NC> u;
+  u.p = const_cast<void*>(U);
+  u.V = gh.V;
+  cg_hop_split_kernel<R, NC><<<hop_blocks<R>(gh.Vh) + 1, kDslashThreads, 0, st>>>(
+      v2<R>(te), cv2<R>(to), cv2<R>(p), u, to_devg(gh), R(-k2), partial, cgd, hist, iter_out, maxiter);
+  return cudaGetLastError();
+}
+cudaError_t launch_cg_publish(const GeomH& gh, const double* partial, CgDev* cgd, double* hist, int* iter_out,
+                              int maxiter, cudaStream_t st) {
+  const int n = (gh.Vh + 31) / 32;
+  cg_publish_kernel<<<1, 32, 0, st>>>(partial + (size_t)3 * n, n, cgd, hist, iter_out, maxiter);
+  return cudaGetLastError();
+}
 template <typename R, int NC>
 cudaError_t launch_cg_apdot(const GeomH& gh, void* ap, const void* to, const void* te, const void* p, const void* r,
                             const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st) {
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  (hop_split<R>(gh.Vh) ? cg_apdot_split_kernel<R, NC> : cg_apdot_kernel<R, NC>)<<<hop_blocks<R>(gh.Vh), kDslashThreads,
-                                                                               0, st>>>(
+  auto* const k = cg_defer<R>(gh.Vh) ? cg_apdot_split_kernel<R, NC, true>
+                                     : (hop_split<R>(gh.Vh) ? cg_apdot_split_kernel<R, NC, false> : cg_apdot_kernel<R, NC>);
+  k<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0, st>>>(
       v2<R>(ap), cv2<R>(to), cv2<R>(te), cv2<R>(p), cv2<R>(r), u, to_devg(gh), R(-k2), partial, cgd);
   return cudaGetLastError();
 }
@@ -1124,10 +1256,10 @@ cudaError_t launch_cg_fold(const GeomH& gh, void* to, void* x, const void* r, co
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  (hop_split<R>(gh.Vh) ? cg_fold_split_kernel<R, NC> : cg_fold_kernel<R, NC>)<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0,
-                                                                             st>>>(
-      v2<R>(to), v2<R>(x), cv2<R>(r), cv2<R>(ap), cv2<R>(p), v2<R>(r2), v2<R>(p2), u, to_devg(gh), partial, cgd,
-      hist, iter_out, maxiter);
+  auto* const k = cg_defer<R>(gh.Vh) ? cg_fold_split_kernel<R, NC, true>
+                                     : (hop_split<R>(gh.Vh) ? cg_fold_split_kernel<R, NC, false> : cg_fold_kernel<R, NC>);
+  k<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0, st>>>(v2<R>(to), v2<R>(x), cv2<R>(r), cv2<R>(ap), cv2<R>(p), v2<R>(r2),
+                                                     v2<R>(p2), u, to_devg(gh), partial, cgd, hist, iter_out, maxiter);
   return cudaGetLastError();
 }
 template <typename RI>
@@ -1374,6 +1506,8 @@ template cudaError_t launch_cg_axpy<float>(void*, void*, const void*, const void
 template cudaError_t launch_cg_xpay<double>(void*, const void*, CgDev*, double*, int*, int, int, cudaStream_t);
 template cudaError_t launch_cg_xpay<float>(void*, const void*, CgDev*, double*, int*, int, int, cudaStream_t);
 #define FG_INST_FOLD(R, NC)                                                                                    \
+  template cudaError_t launch_cg_hop<R, NC>(const GeomH&, void*, const void*, const void*, const void*, double, \
+                                            double*, CgDev*, double*, int*, int, cudaStream_t);                \
   template cudaError_t launch_cg_apdot<R, NC>(const GeomH&, void*, const void*, const void*, const void*,      \
                                               const void*, const void*, double, double*, CgDev*, cudaStream_t); \
   template cudaError_t launch_cg_fold<R, NC>(const GeomH&, void*, void*, const void*, const void*, const void*, \

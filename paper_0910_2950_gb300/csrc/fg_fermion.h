@@ -30,6 +30,9 @@ struct CgDev {
   // reset at every reliable update to |r|^2 / n, and rho rescales p then
   double sigma2;
   double rho;
+  // folded iteration with one direction a warp: block sums of |r'|^2 are left
+  // and not yet published
+  int pending;
 };
 
 int vec_blocks(int n);
@@ -135,17 +138,27 @@ cudaError_t launch_cg_init(const double* part, int n, CgDev* cgd, double tol2, d
 cudaError_t launch_cg_init_guess(const double* part_b, const double* part_r, int n, CgDev* cgd, double tol2,
                                  double* bb_out, double* rr0_out, cudaStream_t st);
 
-// ---- folded CG iteration (FP32 / FP64 inner vectors, links R with NC entries)
-// Ap = te - k2 D_eo^dagger to on the even sites; grand totals of <p, Ap>,
-// Re <r, Ap>, |Ap|^2 through `partial` (3 x dslash_blocks(Vh) entries); the
-// last block sets cgd->alpha = rr / <p, Ap> and
-// cgd->beta = (rr - 2 alpha Re <r, Ap> + alpha^2 |Ap|^2) / rr, rr = cgd->rr[iter & 1].
+// ---- folded CG iteration (FP32 / FP64 inner vectors, links R with NC
+// entries): B, C (launch_dslash), D and A (see fermion.cu); `partial` has
+// 4 x dslash_blocks(Vh) entries.
+// Whether the launches of such an iteration on Vh sites publish it in the
+// next one's B (launch_cg_publish then ends a batch of them) or in A.
+bool cg_deferred(int Vh, bool fp64);
+// B: te = p - k2 D_eo to (and publishes the iteration before).
+template <typename R, int NC>
+cudaError_t launch_cg_hop(const GeomH& g, void* te, const void* to, const void* p, const void* U, double k2,
+                          double* partial, CgDev* cgd, double* hist, int* iter_out, int maxiter, cudaStream_t st);
+cudaError_t launch_cg_publish(const GeomH& g, const double* partial, CgDev* cgd, double* hist, int* iter_out,
+                              int maxiter, cudaStream_t st);
+// D: Ap = te - k2 D_eo^dagger to on the even sites, and the sums of <p, Ap>,
+// Re <r, Ap>, |Ap|^2 from which alpha = rr / <p, Ap> and
+// beta = (rr - 2 alpha Re <r, Ap> + alpha^2 |Ap|^2) / rr follow, rr = cgd->rr[iter & 1].
 template <typename R, int NC>
 cudaError_t launch_cg_apdot(const GeomH& g, void* ap, const void* to, const void* te, const void* p, const void* r,
                             const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st);
-// x += alpha p; r2 = r - alpha Ap; p2 = r2 + beta p (even sites) and
-// to = D_oe p2 (odd sites); |r2|^2 published as iteration iter + 1 (rr[],
-// hist, *iter_out, done).  r, p and r2, p2 are different buffers.
+// A: x += alpha p; r2 = r - alpha Ap; p2 = r2 + beta p (even sites) and
+// to = D_oe p2 (odd sites); |r2|^2 is the residual of iteration iter + 1
+// (rr[], hist, *iter_out, done).  r, p and r2, p2 are different buffers.
 template <typename R, int NC>
 cudaError_t launch_cg_fold(const GeomH& g, void* to, void* x, const void* r, const void* ap, const void* p,
                            void* r2, void* p2, const void* U, double* partial, CgDev* cgd, double* hist,

@@ -99,7 +99,7 @@ def footprint_bytes(spec: ChainSpec, precision: str = "fp32", link_reals: int = 
     FP32 solver's reliable updates, and the second r and p buffers of the
     folded CG iteration, which the library runs while the solver's links
     and six vectors fit in L2 and never with 16-bit inner vectors), the
-    pseudofermion force, the CG scalars and the Dslash (three values) and
+    pseudofermion force, the CG scalars and the Dslash (four values) and
     vector block partials (two arrays of the latter).  4 KiB are added for allocator
     rounding of the small buffers.  (The closed-form force gradient's
     buffers are not included: the server does not offer that integrator.)
@@ -123,7 +123,7 @@ def footprint_bytes(spec: ChainSpec, precision: str = "fp32", link_reals: int = 
         # estimate stays an upper bound whatever L2 size the library sees
         folded = not half and v * (4 * (link_reals // 2) * 2 + 6 * 12) * r <= 1.25 * l2_bytes
         n_inner = 12 if folded else 10
-        total += n64 * nvec * 16 + n_inner * nvec * 2 * r + mom + 128 + 8 * (3 * dslash_blocks + 2 * vec_blocks + 3)
+        total += n64 * nvec * 16 + n_inner * nvec * 2 * r + mom + 136 + 8 * (4 * dslash_blocks + 2 * vec_blocks + 2)
         if half:
             total += 4 * v * link_reals * 2      # 16-bit links of the inner solver
     return total + 4096
