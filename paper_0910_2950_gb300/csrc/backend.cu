@@ -77,9 +77,9 @@ class Backend final : public IBackend {
     if ((s = alloc((void**)&h0_, V * sizeof(double))) != FG_OK) return s;
     for (int k = 0; k < 2; ++k)
       if ((s = alloc((void**)&sgc_[k], V * sizeof(double))) != FG_OK) return s;
-    const size_t nb = (V + 255) / 256 + 1;
-    if ((s = alloc((void**)&partial_, 4 * nb * sizeof(double))) != FG_OK) return s;
-    if ((s = alloc((void**)&dout_, 32 * sizeof(double))) != FG_OK) return s;
+    if ((s = alloc((void**)&partial_, (size_t)3 * energy_blocks(g_) * sizeof(double))) != FG_OK) return s;
+    if ((s = alloc((void**)&dout_, 32 * sizeof(double))) != FG_OK) return s;  // the last one: energy()'s counter
+    if (cudaMemsetAsync(dout_, 0, 32 * sizeof(double), st_) != cudaSuccess) return cuda_fail("memset");
     if (cudaMallocHost((void**)&host_out_, 32 * sizeof(double)) != cudaSuccess) {
       host_out_ = nullptr;
       return h_->fail(FG_ENOMEM, "pinned host allocation failed");
@@ -624,14 +624,12 @@ class Backend final : public IBackend {
     return sync();
   }
 
-  // energy kernel + fixed-order reduction into dout_[off .. off+2]
+  // energy sums into dout_[off .. off+2]
   fg_status energy(int mode, const void* P, int off, const double* sg_in = nullptr, double* sg_out = nullptr) {
-    int nb = 0;
-    fg_status s = run(KC_ENERGY, [&] {
-      return launch_energy<R, NC>(g_, U_, P, h_->prm.beta, mode, h0_, partial_, &nb, st_, sg_in, sg_out);
+    return run(KC_ENERGY, [&] {
+      return launch_energy<R, NC>(g_, U_, P, h_->prm.beta, mode, h0_, partial_, (unsigned*)(dout_ + 31), dout_ + off,
+                                  st_, sg_in, sg_out);
     });
-    if (s != FG_OK) return s;
-    return run(KC_REDUCE, [&] { return launch_reduce(partial_, nb, 3, dout_ + off, 0, st_); });
   }
   fg_status fetch(int n) {
     if (cudaMemcpyAsync(host_out_, dout_, n * sizeof(double), cudaMemcpyDeviceToHost, st_) != cudaSuccess)

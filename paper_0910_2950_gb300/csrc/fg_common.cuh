@@ -439,16 +439,6 @@ __device__ __forceinline__ bool link_site(const Geom& g, int& s) {
   s = (threadIdx.x >> 5) * g.Vh + i;
   return true;
 }
-// The same for one thread per site and blocks of 2 * H threads: half-site
-// indices [H b, H b + H) of both parities.  Launch with (V/2 + H - 1) / H blocks.
-template <int H>
-__device__ __forceinline__ bool pair_site(const Geom& g, int& s) {
-  const int i = blockIdx.x * H + (threadIdx.x % H);
-  if (i >= g.Vh) return false;
-  s = (threadIdx.x / H) * g.Vh + i;
-  return true;
-}
-
 // ---------------------------------------------------------------------------
 // Field access.  Fields are stored "pair-major": complex entries are grouped
 // in pairs, and pair q of every site is contiguous, so that one thread moves

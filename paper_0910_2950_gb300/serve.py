@@ -110,7 +110,7 @@ def footprint_bytes(spec: ChainSpec, precision: str = "fp32", link_reals: int = 
     gauge = 4 * v * link_reals * r
     mom = 4 * v * 8 * r
     plaq = 6 * 8 * r * v if r == 8 else 0     # plaquette field of the double-float and FP64 force
-    total = 3 * gauge + 2 * mom + plaq + 3 * 8 * v + 4 * 8 * ((v + 255) // 256 + 1) + 32 * 8 + 4 * v * 18 * 8
+    total = 3 * gauge + 2 * mom + plaq + 3 * 8 * v + 3 * 8 * ((v + 31) // 32 + 2) + 32 * 8 + 4 * v * 18 * 8
     if spec.kappa > 0:
         vh = v // 2
         nvec = 12 * vh
