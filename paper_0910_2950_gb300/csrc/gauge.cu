@@ -371,7 +371,6 @@ static Mom<R> mom_of(const void* p, int V) {
 }
 
 static inline dim3 link_grid(int V) { return dim3((V + kSitesPerBlock - 1) / kSitesPerBlock); }
-static inline dim3 pair_grid(int V) { return dim3((V / 2 + 31) / 32); }
 static inline dim3 link_block() { return dim3(kSitesPerBlock, 4); }
 
 template <int NC>

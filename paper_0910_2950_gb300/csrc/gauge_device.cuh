@@ -302,8 +302,7 @@ __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok,
 // against 405 us at 32^4; 12% slower at 8^4): it stays with the staples.  One
 // launch of both kinds of work, link blocks waiting for the plaquettes they
 // read, was 5 to 25% slower than two launches (idle SMs, spilled registers).
-// Q is kept in the momenta's layout, [plane][2][site], as Q / 2 (for the
-// double-float products below) by its entries
+// Q is kept in the momenta's layout, [plane][2][site], by its entries
 // (q00, q11, Re q01, Im q01, Re q02, Im q02, Re q12, Im q12).
 
 // Most threads of a block of the two kernels, and resident blocks of that
@@ -346,7 +345,7 @@ __device__ __forceinline__ int plane_of(int a, int b) {
   return mu == 0 ? nu - 1 : (mu == 1 ? nu + 1 : 5);
 }
 
-// q = (Hermitian traceless part of W_pl(s)) / 2.
+// q = Hermitian traceless part of W_pl(s).
 template <typename R, int NC>
 __device__ __forceinline__ void plaquette_herm(const Gauge<R, NC>& U, const Geom& g, int s, int pl, R q[8]) {
   int c[4], par, mu, nu;
@@ -387,8 +386,8 @@ __device__ __forceinline__ void plaquette_herm(const Gauge<R, NC>& U, const Geom
     }
     constexpr DF third(1.0 / 3.0);
     const DF tr = (d[0] + d[1] + d[2]) * third;
-    q[0] = d[0] - tr;
-    q[1] = d[1] - tr;
+    q[0] = (d[0] - tr) * 2.0f;
+    q[1] = (d[1] - tr) * 2.0f;
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
       const int i = p < 2 ? 0 : 1, j = p == 0 ? 1 : 2;
@@ -404,9 +403,8 @@ __device__ __forceinline__ void plaquette_herm(const Gauge<R, NC>& U, const Geom
         im.add(a.e[j][k].re, b.e[i][k].re);
         im.add(a.e[j][k].im, b.e[i][k].im);
       }
-      const DF vr = re.value(), vi = im.value();
-      q[2 + 2 * p] = DF(0.5f * vr.hi, 0.5f * vr.lo);
-      q[3 + 2 * p] = DF(0.5f * vi.hi, 0.5f * vi.lo);
+      q[2 + 2 * p] = re.value();
+      q[3 + 2 * p] = im.value();
     }
   } else {
     const M3<R> a = mul(U.load(mu, s), U.load(nu, other + dmu));
@@ -423,8 +421,8 @@ __device__ __forceinline__ void plaquette_herm(const Gauge<R, NC>& U, const Geom
       d[i] = t;
     }
     const R tr = (d[0] + d[1] + d[2]) * R(1.0 / 3.0);
-    q[0] = R(0.5) * (d[0] - tr);
-    q[1] = R(0.5) * (d[1] - tr);
+    q[0] = d[0] - tr;
+    q[1] = d[1] - tr;
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
       const int i = p < 2 ? 0 : 1, j = p == 0 ? 1 : 2;
@@ -440,8 +438,8 @@ __device__ __forceinline__ void plaquette_herm(const Gauge<R, NC>& U, const Geom
         im = fma(a.e[j][k].re, b.e[i][k].re, im);
         im = fma(a.e[j][k].im, b.e[i][k].im, im);
       }
-      q[2 + 2 * p] = R(0.25) * re;
-      q[3 + 2 * p] = R(0.25) * im;
+      q[2 + 2 * p] = R(0.5) * re;
+      q[3 + 2 * p] = R(0.5) * im;
     }
   }
 }
@@ -483,9 +481,11 @@ __device__ __forceinline__ void rotate_add(R acc[8], const R h[8], const M3<R>& 
   }
 }
 
-// Double-float: H / 2 has norm at most 2/3 (Q's eigenvalues are sines less
-// their mean), so the entries of H u / 2 and u^dag H u / 2 and all their
-// partial sums lie within the anchored products' [-1, 1].
+// Double-float: the entries of H u and u^dag H u and their partial sums are
+// bounded by the norm of H, which stays below the anchored products' 1 unless
+// the plaquette is far from the unit matrix (Q's eigenvalues are sines less
+// their mean, 4/3 at most); beyond, the accumulator's grid is twice as coarse.
+// (H / 2 is always within the bound but doubles the rounding of every force.)
 template <>
 __device__ __forceinline__ void rotate_add<DF>(DF acc[8], const DF h[8], const M3<DF>& u) {
   const DF h22 = -(h[0] + h[1]);
@@ -572,15 +572,15 @@ __device__ __forceinline__ void link_force(const Gauge<R, NC>& U, const Mom<R>& 
     for (int k = 0; k < 8; ++k) h[k] = flip_if(h[k], mu < nu);
     rotate_add(acc, h, U.load(nu, sm));
   }
-  const R four = R(4.0f), two = R(2.0f), s12 = R(3.46410161513775458705);  // 2 sqrt(3)
-  f[0] = four * acc[2];
-  f[1] = -(four * acc[3]);
-  f[2] = two * (acc[0] - acc[1]);
-  f[3] = four * acc[4];
-  f[4] = -(four * acc[5]);
-  f[5] = four * acc[6];
-  f[6] = -(four * acc[7]);
-  f[7] = s12 * (acc[0] + acc[1]);
+  const R two = R(2.0f), s3 = R(1.73205080756887729353);
+  f[0] = two * acc[2];
+  f[1] = -(two * acc[3]);
+  f[2] = acc[0] - acc[1];
+  f[3] = two * acc[4];
+  f[4] = -(two * acc[5]);
+  f[5] = two * acc[6];
+  f[6] = -(two * acc[7]);
+  f[7] = s3 * (acc[0] + acc[1]);
 }
 
 template <typename R, int NC, int MODE>
