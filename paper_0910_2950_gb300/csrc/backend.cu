@@ -240,10 +240,10 @@ class Backend final : public IBackend {
           return s;
       }
       if ((s = run(KC_DSLASH, [&] {
-             return inner_dslash(to_, rs_, nullptr, nullptr, Uin, 1, dagger, 0, 1.0, nullptr, false);
+             return inner_dslash(to_, rs_, nullptr, Uin, 1, dagger, 0, 1.0, false);
            })) != FG_OK)
         return s;
-      if ((s = run(KC_DSLASH, [&] { return inner_dslash(te_, to_, rs_, nullptr, Uin, 0, dagger, 1, -k2, nullptr, false); })) !=
+      if ((s = run(KC_DSLASH, [&] { return inner_dslash(te_, to_, rs_, Uin, 0, dagger, 1, -k2, false); })) !=
           FG_OK)
         return s;
       if (half_links_) s = run(KC_CONVERT, [&] { return launch_h16_to_double_scaled(s16_, ax64_, te_, cgd_, n, st_); });
@@ -729,10 +729,8 @@ class Backend final : public IBackend {
       auto ds = [&](void* out, const void* in, const void* x, const void* links, bool tangent, int out_par, int dag,
                     int mode, double b) {
         return run(KC_DSLASH, [&] {
-          return tangent ? launch_dslash<R, 9, R>(g_, out, in, x, nullptr, links, out_par, dag, mode, b, nullptr,
-                                                  nullptr, st_)
-                         : launch_dslash<R, NC, R>(g_, out, in, x, nullptr, links, out_par, dag, mode, b, nullptr,
-                                                   nullptr, st_);
+          return tangent ? launch_dslash<R, 9, R>(g_, out, in, x, links, out_par, dag, mode, b, nullptr, st_)
+                         : launch_dslash<R, NC, R>(g_, out, in, x, links, out_par, dag, mode, b, nullptr, st_);
         });
       };
       auto lc = [&](auto launch) { return run(KC_CG_BLAS, launch); };
@@ -1021,11 +1019,11 @@ class Backend final : public IBackend {
   fg_status apply_mhat64(void* out, const void* in, const void* U, int dag) {
     const double k2 = h_->prm.kappa * h_->prm.kappa;
     fg_status s = run(KC_DSLASH64, [&] {
-      return launch_dslash<R, NC, double>(g_, to64_, in, nullptr, nullptr, U, 1, dag, 0, 1.0, nullptr, nullptr, st_);
+      return launch_dslash<R, NC, double>(g_, to64_, in, nullptr, U, 1, dag, 0, 1.0, nullptr, st_);
     });
     if (s != FG_OK) return s;
     return run(KC_DSLASH64, [&] {
-      return launch_dslash<R, NC, double>(g_, out, to64_, in, nullptr, U, 0, dag, 1, -k2, nullptr, nullptr, st_);
+      return launch_dslash<R, NC, double>(g_, out, to64_, in, U, 0, dag, 1, -k2, nullptr, st_);
     });
   }
   fg_status apply_mdagm64(void* out, const void* in, const void* U) {
@@ -1039,11 +1037,11 @@ class Backend final : public IBackend {
     if constexpr (kMixed) {
       const double k2 = h_->prm.kappa * h_->prm.kappa;
       fg_status s = run(KC_DSLASH_DF, [&] {
-        return launch_dslash<R, NC, DF>(g_, to64_, in, nullptr, nullptr, U, 1, dag, 0, 1.0, nullptr, nullptr, st_);
+        return launch_dslash<R, NC, DF>(g_, to64_, in, nullptr, U, 1, dag, 0, 1.0, nullptr, st_);
       });
       if (s != FG_OK) return s;
       return run(KC_DSLASH_DF, [&] {
-        return launch_dslash<R, NC, DF>(g_, out, to64_, in, nullptr, U, 0, dag, 1, -k2, nullptr, nullptr, st_);
+        return launch_dslash<R, NC, DF>(g_, out, to64_, in, U, 0, dag, 1, -k2, nullptr, st_);
       });
     } else {
       return h_->fail(FG_ESTATE, "double-float Dslash needs FP32 links");
@@ -1103,13 +1101,13 @@ class Backend final : public IBackend {
       if ((s = run(KC_CG_BLAS, [&] { return launch_convert<R, double>(Xe_, x64_, nullptr, n, st_); })) != FG_OK) return s;
       // X_o = D_oe X_e; Y_e = X_e - kappa^2 D_eo X_o; Y_o = g5 D_oe g5 Y_e
       if ((s = run(KC_DSLASH, [&] {
-             return launch_dslash<R, NC, R>(g_, Xo_, Xe_, nullptr, nullptr, U, 1, 0, 0, 1.0, nullptr, nullptr, st_);
+             return launch_dslash<R, NC, R>(g_, Xo_, Xe_, nullptr, U, 1, 0, 0, 1.0, nullptr, st_);
            })) != FG_OK) return s;
       if ((s = run(KC_DSLASH, [&] {
-             return launch_dslash<R, NC, R>(g_, Ye_, Xo_, Xe_, nullptr, U, 0, 0, 1, -k2, nullptr, nullptr, st_);
+             return launch_dslash<R, NC, R>(g_, Ye_, Xo_, Xe_, U, 0, 0, 1, -k2, nullptr, st_);
            })) != FG_OK) return s;
       if ((s = run(KC_DSLASH, [&] {
-             return launch_dslash<R, NC, R>(g_, Yo_, Ye_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr, nullptr, st_);
+             return launch_dslash<R, NC, R>(g_, Yo_, Ye_, nullptr, U, 1, 1, 0, 1.0, nullptr, st_);
            })) != FG_OK) return s;
       return run(KC_FERMION_FORCE, [&] {
         return launch_fermion_force<R, NC, R>(g_, U, Xe_, Xo_, Ye_, Yo_, FF_, k2, 0, st_);
@@ -1122,25 +1120,36 @@ class Backend final : public IBackend {
   // spinors.
   // `solver` = false: outside a solve (no early return on the solver's
   // converged flag).
-  cudaError_t inner_dslash(void* out, const void* in, const void* x, const void* pdot, const void* U, int out_par,
-                           int dag, int mode, double b, double* partial, bool solver = true) {
-    CgDev* const cgd = solver ? cgd_ : nullptr;
+  cudaError_t inner_dslash(void* out, const void* in, const void* x, const void* U, int out_par, int dag, int mode,
+                           double b, bool solver = true) {
+    const CgDev* const cgd = solver ? cgd_ : nullptr;
     if constexpr (kMixed) {
-      if (half_links_)
-        return launch_dslash_h16<NC>(s16_, g_, out, in, x, pdot, U, out_par, dag, mode, b, partial, cgd, st_);
+      if (half_links_) return launch_dslash_h16<NC>(s16_, g_, out, in, x, U, out_par, dag, mode, b, cgd, st_);
     }
-    return launch_dslash<R, NC, R>(g_, out, in, x, pdot, U, out_par, dag, mode, b, partial, cgd, st_);
+    return launch_dslash<R, NC, R>(g_, out, in, x, U, out_par, dag, mode, b, cgd, st_);
   }
 
-  // Folded iteration, launches D and A (B and C are plain Dslash launches).
-  // A swaps the current and other buffers of r and p.
-  cudaError_t fold_apdot(const void* U) {
+  // Launch D of an iteration, and the last one: the vector update of the
+  // five-launch form or A of the folded one, which swaps the current and
+  // other buffers of r and p.
+  cudaError_t cg_apdot(const void* U) {
     if constexpr (kMixed || std::is_same<R, double>::value) {
       const double k2 = h_->prm.kappa * h_->prm.kappa;
-      return launch_cg_apdot<R, NC>(g_, ap_, to_, te_, p_, rs_, U, k2, part_pap_, cgd_, st_);
+      if constexpr (kMixed) {
+        if (half_links_)
+          return launch_cg_apdot_h16<NC>(s16_, g_, ap_, to_, te_, p_, rs_, U, k2, part_pap_, cgd_, st_);
+      }
+      return launch_cg_apdot<R, NC>(g_, ap_, to_, te_, p_, rs_, U, k2, part_pap_, cgd_, st_, fold_);
     } else {
       return cudaErrorNotSupported;
     }
+  }
+  cudaError_t cg_update() {
+    double* const hist = mapped_->hist;
+    int* const it = &mapped_->dev_iter;
+    const int n = nvec(), most = h_->prm.cg_maxiter;
+    if (half_links_) return launch_cg_update_h16(s16_, xs_, rs_, p_, ap_, cgd_, part_rr_, hist, it, most, n, st_);
+    return launch_cg_update<R>(xs_, rs_, p_, ap_, cgd_, part_rr_, hist, it, most, n, st_);
   }
   cudaError_t fold_update(const void* U) {
     if constexpr (kMixed || std::is_same<R, double>::value) {
@@ -1171,11 +1180,11 @@ class Backend final : public IBackend {
   // t_o = D_oe p, which the folded iteration expects on entry (after the
   // setup and after every reliable update, which may replace p).
   fg_status fold_prime(const void* U) {
-    return run(KC_DSLASH, [&] { return inner_dslash(to_, p_, nullptr, nullptr, U, 1, 0, 0, 1.0, nullptr); });
+    return run(KC_DSLASH, [&] { return inner_dslash(to_, p_, nullptr, U, 1, 0, 0, 1.0); });
   }
 
-  // One CG iteration in the inner precision R: 4 Dslash + 2 vector kernels,
-  // which all return at once after convergence (cgd_->done).  Raw launches,
+  // One CG iteration in the inner precision R: 4 Dslash launches and a vector
+  // one, which all return at once after convergence (cgd_->done).  Raw launches,
   // usable inside stream capture.
   cudaError_t cg_iteration_raw(const void* U) {
     const double k2 = h_->prm.kappa * h_->prm.kappa;
@@ -1183,23 +1192,15 @@ class Backend final : public IBackend {
     cudaError_t e;
     if (fold_) {
       if ((e = fold_hop(U)) != cudaSuccess) return e;
-      if ((e = inner_dslash(to_, te_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr)) != cudaSuccess) return e;
-      if ((e = fold_apdot(U)) != cudaSuccess) return e;
+      if ((e = inner_dslash(to_, te_, nullptr, U, 1, 1, 0, 1.0)) != cudaSuccess) return e;
+      if ((e = cg_apdot(U)) != cudaSuccess) return e;
       return fold_update(U);
     }
-    if ((e = inner_dslash(to_, p_, nullptr, nullptr, U, 1, 0, 0, 1.0, nullptr)) != cudaSuccess) return e;
-    if ((e = inner_dslash(te_, to_, p_, nullptr, U, 0, 0, 1, -k2, nullptr)) != cudaSuccess) return e;
-    if ((e = inner_dslash(to_, te_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr)) != cudaSuccess) return e;
-    if ((e = inner_dslash(ap_, to_, te_, p_, U, 0, 1, 2, -k2, part_pap_)) != cudaSuccess) return e;
-    if (half_links_) {
-      if ((e = launch_cg_axpy_h16(s16_, xs_, rs_, p_, ap_, cgd_, part_rr_, n, st_)) != cudaSuccess) return e;
-      return launch_cg_xpay_h16(s16_, p_, rs_, cgd_, mapped_->hist, &mapped_->dev_iter, h_->prm.cg_maxiter, n, st_);
-    }
-    if ((e = launch_cg_axpy<R>(xs_, rs_, p_, ap_, cgd_, part_rr_, n, st_)) !=
-        cudaSuccess)
-      return e;
-    return launch_cg_xpay<R>(p_, rs_, cgd_, mapped_->hist, &mapped_->dev_iter,
-                             h_->prm.cg_maxiter, n, st_);
+    if ((e = inner_dslash(to_, p_, nullptr, U, 1, 0, 0, 1.0)) != cudaSuccess) return e;
+    if ((e = inner_dslash(te_, to_, p_, U, 0, 0, 1, -k2)) != cudaSuccess) return e;
+    if ((e = inner_dslash(to_, te_, nullptr, U, 1, 1, 0, 1.0)) != cudaSuccess) return e;
+    if ((e = cg_apdot(U)) != cudaSuccess) return e;
+    return cg_update();
   }
 
   // The same through run(), so that per-kernel timing and launch counting see
@@ -1210,37 +1211,22 @@ class Backend final : public IBackend {
     fg_status s;
     if (fold_) {
       if ((s = run(KC_DSLASH, [&] { return fold_hop(U); })) != FG_OK) return s;
-      if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, te_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr); })) !=
+      if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, te_, nullptr, U, 1, 1, 0, 1.0); })) !=
           FG_OK)
         return s;
-      if ((s = run(KC_DSLASH, [&] { return fold_apdot(U); })) != FG_OK) return s;
+      if ((s = run(KC_DSLASH, [&] { return cg_apdot(U); })) != FG_OK) return s;
       return run(KC_DSLASH, [&] { return fold_update(U); });
     }
-    if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, p_, nullptr, nullptr, U, 1, 0, 0, 1.0, nullptr); })) !=
+    if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, p_, nullptr, U, 1, 0, 0, 1.0); })) !=
         FG_OK)
       return s;
-    if ((s = run(KC_DSLASH, [&] { return inner_dslash(te_, to_, p_, nullptr, U, 0, 0, 1, -k2, nullptr); })) != FG_OK)
+    if ((s = run(KC_DSLASH, [&] { return inner_dslash(te_, to_, p_, U, 0, 0, 1, -k2); })) != FG_OK)
       return s;
-    if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, te_, nullptr, nullptr, U, 1, 1, 0, 1.0, nullptr); })) !=
+    if ((s = run(KC_DSLASH, [&] { return inner_dslash(to_, te_, nullptr, U, 1, 1, 0, 1.0); })) !=
         FG_OK)
       return s;
-    if ((s = run(KC_DSLASH, [&] { return inner_dslash(ap_, to_, te_, p_, U, 0, 1, 2, -k2, part_pap_); })) != FG_OK)
-      return s;
-    if (half_links_) {
-      if ((s = run(KC_CG_BLAS, [&] { return launch_cg_axpy_h16(s16_, xs_, rs_, p_, ap_, cgd_, part_rr_, n, st_); })) !=
-          FG_OK)
-        return s;
-      return run(KC_CG_BLAS, [&] {
-        return launch_cg_xpay_h16(s16_, p_, rs_, cgd_, mapped_->hist, &mapped_->dev_iter, h_->prm.cg_maxiter, n, st_);
-      });
-    }
-    if ((s = run(KC_CG_BLAS, [&] {
-           return launch_cg_axpy<R>(xs_, rs_, p_, ap_, cgd_, part_rr_, n, st_);
-         })) != FG_OK) return s;
-    return run(KC_CG_BLAS, [&] {
-      return launch_cg_xpay<R>(p_, rs_, cgd_, mapped_->hist, &mapped_->dev_iter,
-                               h_->prm.cg_maxiter, n, st_);
-    });
+    if ((s = run(KC_DSLASH, [&] { return cg_apdot(U); })) != FG_OK) return s;
+    return run(KC_CG_BLAS, [&] { return cg_update(); });
   }
 
   // A CUDA graph of n iterations (n = 2, 4 or 8) on links U, captured on first
@@ -1301,7 +1287,7 @@ class Backend final : public IBackend {
       if (g != nullptr) {
         if (cudaGraphLaunch(g, st_) != cudaSuccess) return cuda_fail("cg graph launch");
         // an even number of folded iterations leaves rs_ and p_ where they were
-        h_->launches += (fold_ ? 4 : 6) * n + (fold_deferred() ? 1 : 0);
+        h_->launches += (fold_ ? 4 : 5) * n + (fold_deferred() ? 1 : 0);
         return FG_OK;
       }
     }

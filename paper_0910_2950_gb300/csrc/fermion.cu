@@ -24,8 +24,8 @@ namespace fg {
 
 constexpr int kDslashThreads = 128;
 
-// out = b D in (MODE 0), out = x + b D in (MODE 1), and MODE 2 also writes the
-// block partial sum of Re <pdot, out>.  `in` has parity 1 - out_par.
+// out = b D in (MODE 0), out = x + b D in (MODE 1).  `in` has parity
+// 1 - out_par.
 // Resident blocks asked of the register allocator.  The FP32 hop is bound by
 // memory latency: six blocks of 128 (80 registers, 24 warps per SM) beat the
 // unconstrained five (90 registers) by 8% at 16^3 x 32 and 24^3 x 48.  The
@@ -69,7 +69,7 @@ template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_
 #define FG_SPLIT_MAX64 131072
 #endif
 
-// The grand total of NV values, one a thread in R (blocks of kDslashThreads):
+// The grand total of NV values, one a thread in R (blocks of T threads):
 // thread 32 w of the block adds value w of all its threads in FP64, and the
 // last block to finish adds the blocks' sums in block order.  True in the
 // threads of that block, with the totals in tot[].  The caller stores its
@@ -77,10 +77,9 @@ template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_
 // to wait for.  (Warp trees in FP64 in every warp, the fields stored first,
 // cost 5 us a launch more than no total; this form 2 us: FP32 16^3 x 32
 // solves 9.14 instead of 10.2 ms.)
-template <int NV, typename R>
+template <int NV, int T = kDslashThreads, typename R>
 __device__ __forceinline__ bool block_total(const R v[NV], double* __restrict__ partial,
                                             unsigned* __restrict__ ticket, double tot[NV]) {
-  constexpr int T = kDslashThreads;
   static_assert(NV <= T / 32, "one warp a value");
   __shared__ R sv[NV][T];
   __shared__ double sw[NV][T / 32];
@@ -121,7 +120,11 @@ __device__ __forceinline__ bool block_total(const R v[NV], double* __restrict__ 
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < NV; ++k) tot[k] = (sw[k][0] + sw[k][1]) + (sw[k][2] + sw[k][3]);
+  for (int k = 0; k < NV; ++k) {
+    tot[k] = sw[k][0];
+#pragma unroll
+    for (int w = 1; w < T / 32; ++w) tot[k] += sw[k][w];
+  }
   if (threadIdx.x == 0) *ticket = 0u;
   return true;
 }
@@ -129,51 +132,34 @@ __device__ __forceinline__ bool block_total(const R v[NV], double* __restrict__ 
 template <typename RL, int NC, typename RS, int DAG, int MODE, typename ST = RS>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<RS>::value) dslash_kernel(
     typename Vec2<ST>::T* __restrict__ out, const typename Vec2<ST>::T* __restrict__ in,
-    const typename Vec2<ST>::T* __restrict__ x, const typename Vec2<ST>::T* __restrict__ pdot,
-    Gauge<RL, NC> U, Geom g, int out_par, RS b, double* __restrict__ partial, CgDev* __restrict__ cgd) {
+    const typename Vec2<ST>::T* __restrict__ x, Gauge<RL, NC> U, Geom g, int out_par, RS b,
+    const CgDev* __restrict__ cgd) {
   if (cgd != nullptr && cgd->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  RS dot = RS(0);  // one site's 24 terms in the spinor precision (GB300's FP64 unit is slow)
+  if (i >= g.Vh) return;
+  const int s = out_par * g.Vh + i;
+  int c[4], par;
+  cb_coords(g, s, c, par);
+  const int in_off = (1 - out_par) * g.Vh;
   Spinor<RS> o;
-  if (i < g.Vh) {
-    const int s = out_par * g.Vh + i;
-    int c[4], par;
-    cb_coords(g, s, c, par);
-    const int in_off = (1 - out_par) * g.Vh;
-    Spinor<RS> acc;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) o.s[k][cc] = cx<RS>(0, 0);
+  Hops<DAG, RL, NC, RS, ST>::run(o, in, U, g, c, s, in_off);
+  if (MODE == 0) {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-      for (int cc = 0; cc < 3; ++cc) acc.s[k][cc] = cx<RS>(0, 0);
-    Hops<DAG, RL, NC, RS, ST>::run(acc, in, U, g, c, s, in_off);
-    if (MODE == 0) {
+      for (int cc = 0; cc < 3; ++cc) o.s[k][cc] = b * o.s[k][cc];
+  } else {
+    const Spinor<RS> xv = load_spinor<RS, ST>(x, i, g.Vh);
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) o.s[k][cc] = b * acc.s[k][cc];
-    } else {
-      const Spinor<RS> xv = load_spinor<RS, ST>(x, i, g.Vh);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) o.s[k][cc] = xv.s[k][cc] + b * acc.s[k][cc];
-      if (MODE == 2) {
-        const Spinor<RS> pv = load_spinor<RS, ST>(pdot, i, g.Vh);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc)
-            dot += pv.s[k][cc].re * o.s[k][cc].re + pv.s[k][cc].im * o.s[k][cc].im;
-      }
-    }
-    if (MODE != 2) store_spinor<RS, ST>(out, i, g.Vh, o);
+      for (int cc = 0; cc < 3; ++cc) o.s[k][cc] = xv.s[k][cc] + b * o.s[k][cc];
   }
-  if constexpr (MODE == 2) {
-    const RS v[1] = {dot};
-    double tot[1];
-    if (block_total<1>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) cgd->pap = tot[0];
-    if (i < g.Vh) store_spinor<RS, ST>(out, i, g.Vh, o);
-  }
+  store_spinor<RS, ST>(out, i, g.Vh, o);
 }
 
 // --------------------------------------------------------------------------- folded CG
@@ -208,22 +194,23 @@ __device__ __forceinline__ void set_alpha_beta(CgDev* cgd, const double tot[3]) 
 }
 // |r|^2 of the iteration just done: rr, the history, the count (also to the
 // host), done.
+// `unit`: what |r|^2 is measured in (sigma^2 in the 16-bit solvers).
 __device__ __forceinline__ void publish(CgDev* cgd, double rr, double* __restrict__ hist, int* __restrict__ iter_out,
-                                        int maxiter) {
+                                        int maxiter, double unit = 1.0) {
   const int k = cgd->iter + 1;
   cgd->rr[k & 1] = rr;
-  if (k <= maxiter) hist[k] = rr;
+  if (k <= maxiter) hist[k] = rr * unit;
   cgd->iter = k;
   *iter_out = k;
-  if (rr <= cgd->tol2bb) cgd->done = 1;
+  if (rr * unit <= cgd->tol2bb) cgd->done = 1;
 }
 
 // D: Ap = te + b D^dagger_eo to at the even sites, with the three dot products.
-template <typename R, int NC>
+template <typename RL, int NC, typename R, typename ST = R>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_apdot_kernel(
-    typename Vec2<R>::T* __restrict__ ap, const typename Vec2<R>::T* __restrict__ to,
-    const typename Vec2<R>::T* __restrict__ te, const typename Vec2<R>::T* __restrict__ p,
-    const typename Vec2<R>::T* __restrict__ r, Gauge<R, NC> U, Geom g, R b, double* __restrict__ partial,
+    typename Vec2<ST>::T* __restrict__ ap, const typename Vec2<ST>::T* __restrict__ to,
+    const typename Vec2<ST>::T* __restrict__ te, const typename Vec2<ST>::T* __restrict__ p,
+    const typename Vec2<ST>::T* __restrict__ r, Gauge<RL, NC> U, Geom g, R b, double* __restrict__ partial,
     CgDev* __restrict__ cgd) {
   if (cgd->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -237,10 +224,10 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     for (int k = 0; k < 4; ++k)
 #pragma unroll
       for (int cc = 0; cc < 3; ++cc) acc.s[k][cc] = cx<R>(0, 0);
-    hops_src<1, R, NC, R>(acc, FieldSrc<R, R>{to}, U, g, c, i, g.Vh);
-    const Spinor<R> tv = load_spinor<R>(te, i, g.Vh);
-    const Spinor<R> pv = load_spinor<R>(p, i, g.Vh);
-    const Spinor<R> rv = load_spinor<R>(r, i, g.Vh);
+    hops_src<1, RL, NC, R>(acc, FieldSrc<R, ST>{to}, U, g, c, i, g.Vh);
+    const Spinor<R> tv = load_spinor<R, ST>(te, i, g.Vh);
+    const Spinor<R> pv = load_spinor<R, ST>(p, i, g.Vh);
+    const Spinor<R> rv = load_spinor<R, ST>(r, i, g.Vh);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -254,7 +241,7 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
   const R v[3] = {pa, ra, aa};
   double tot[3];
   if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_alpha_beta(cgd, tot);
-  if (i < g.Vh) store_spinor<R>(ap, i, g.Vh, o);
+  if (i < g.Vh) store_spinor<R, ST>(ap, i, g.Vh, o);
 }
 
 // A: the vector updates of the iteration and t_o = D_oe p'.
@@ -331,35 +318,20 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
 template <typename RL, int NC, typename RS, int DAG, int MODE, typename ST = RS>
 __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) dslash_split_kernel(
     typename Vec2<ST>::T* __restrict__ out, const typename Vec2<ST>::T* __restrict__ in,
-    const typename Vec2<ST>::T* __restrict__ x, const typename Vec2<ST>::T* __restrict__ pdot,
-    Gauge<RL, NC> U, Geom g, int out_par, RS b, double* __restrict__ partial, CgDev* __restrict__ cgd) {
+    const typename Vec2<ST>::T* __restrict__ x, Gauge<RL, NC> U, Geom g, int out_par, RS b,
+    const CgDev* __restrict__ cgd) {
   __shared__ HopShared<RS> sh;
   if (cgd != nullptr && cgd->done) return;
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
   Cx<RS> row[3];
   hops_split<DAG, RL, NC, RS>(row, sh, FieldSrc<RS, ST>{in}, U, g, i, out_par, (1 - out_par) * g.Vh);
-  RS dot[1] = {RS(0)};
   if (i < g.Vh) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const size_t j = entry_index(k, c, i, g.Vh);
       row[c] = b * row[c];
       if (MODE > 0) row[c] = Entry<RS, ST>::load(x, j) + row[c];
-      if (MODE == 2) {
-        const Cx<RS> pv = Entry<RS, ST>::load(pdot, j);
-        dot[0] = fma(pv.re, row[c].re, dot[0]);
-        dot[0] = fma(pv.im, row[c].im, dot[0]);
-      }
-      if (MODE != 2) Entry<RS, ST>::store(out, j, row[c]);
-    }
-  }
-  if constexpr (MODE == 2) {
-    double tot[1];
-    const bool last = block_total<1>(dot, partial, &cgd->ticket[0], tot);
-    if (last && threadIdx.x == 0) cgd->pap = tot[0];
-    if (i < g.Vh) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) Entry<RS, ST>::store(out, entry_index(k, c, i, g.Vh), row[c]);
+      Entry<RS, ST>::store(out, j, row[c]);
     }
   }
 }
@@ -443,25 +415,25 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_hop_sp
 }
 
 // D: Ap = te + b D^dagger_eo to, block sums of <p, Ap>, Re <r, Ap>, |Ap|^2.
-template <typename R, int NC, bool DEFER>
+template <bool DEFER, typename RL, int NC, typename R, typename ST = R>
 __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_split_kernel(
-    typename Vec2<R>::T* __restrict__ ap, const typename Vec2<R>::T* __restrict__ to,
-    const typename Vec2<R>::T* __restrict__ te, const typename Vec2<R>::T* __restrict__ p,
-    const typename Vec2<R>::T* __restrict__ r, Gauge<R, NC> U, Geom g, R b, double* __restrict__ partial,
+    typename Vec2<ST>::T* __restrict__ ap, const typename Vec2<ST>::T* __restrict__ to,
+    const typename Vec2<ST>::T* __restrict__ te, const typename Vec2<ST>::T* __restrict__ p,
+    const typename Vec2<ST>::T* __restrict__ r, Gauge<RL, NC> U, Geom g, R b, double* __restrict__ partial,
     CgDev* __restrict__ cgd) {
   __shared__ HopShared<R> sh;
   if (cgd->done) return;
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
   Cx<R> row[3];
-  hops_split<1, R, NC, R>(row, sh, FieldSrc<R, R>{to}, U, g, i, 0, g.Vh);
+  hops_split<1, RL, NC, R>(row, sh, FieldSrc<R, ST>{to}, U, g, i, 0, g.Vh);
   R v[3] = {R(0), R(0), R(0)};  // a thread's 6 terms each
   if (i < g.Vh) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const size_t j = entry_index(k, c, i, g.Vh);
-      row[c] = Entry<R, R>::load(te, j) + b * row[c];
-      if (DEFER) Entry<R, R>::store(ap, j, row[c]);
-      const Cx<R> pv = Entry<R, R>::load(p, j), rv = Entry<R, R>::load(r, j);
+      row[c] = Entry<R, ST>::load(te, j) + b * row[c];
+      if (DEFER) Entry<R, ST>::store(ap, j, row[c]);
+      const Cx<R> pv = Entry<R, ST>::load(p, j), rv = Entry<R, ST>::load(r, j);
       v[0] = fma(pv.re, row[c].re, v[0]);
       v[0] = fma(pv.im, row[c].im, v[0]);
       v[1] = fma(rv.re, row[c].re, v[1]);
@@ -477,7 +449,7 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_
     if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_alpha_beta(cgd, tot);
     if (i < g.Vh) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Entry<R, R>::store(ap, entry_index(k, c, i, g.Vh), row[c]);
+      for (int c = 0; c < 3; ++c) Entry<R, ST>::store(ap, entry_index(k, c, i, g.Vh), row[c]);
     }
   }
 }
@@ -650,69 +622,56 @@ __device__ __forceinline__ double block_sum_partials(const double* __restrict__ 
   return r;
 }
 
-// Iteration k = iter + 1 (iter was published by the previous iteration's
-// xpay kernel): alpha = rr[(k-1)&1] / pAp; x += alpha p; r -= alpha Ap;
-// |r|^2 into cgd->rr_next.  Block 0 passes k on to xpay through k_axpy.
-// The kernels take no iteration argument, so a batch of iterations can be
+// The vector part of a five-launch iteration (Dslash launches to, te, to, D,
+// then this one): x += alpha p, r -= alpha Ap, p = r + beta p with D's alpha
+// and beta; the last block publishes |r|^2.  One pass where an axpy, whose
+// total |r|^2 beta waited for, and an xpay took two (half precision
+// 24^3 x 48: 23.3 + 11.2 us; each thread also divided in FP64).  The search
+// direction is formed on the converging iteration too, so that a reliable
+// update that finds the true residual still too large can simply continue.
+// x has pairs X (FP32 in the 16-bit solvers, whose r, p and Ap are stored as
+// ST and in units of sigma; `scaled` then publishes |r|^2 sigma^2).  The
+// kernels take no iteration argument, so a batch of iterations can be
 // captured once in a CUDA graph and replayed.
-template <typename R>
-__global__ void __launch_bounds__(kVecThreads) cg_axpy_kernel(
-    typename Vec2<R>::T* __restrict__ x, typename Vec2<R>::T* __restrict__ r,
-    const typename Vec2<R>::T* __restrict__ p, const typename Vec2<R>::T* __restrict__ ap,
-    CgDev* __restrict__ cgd, double* __restrict__ rr_part, int n) {
-  if (cgd->done) return;
-  const int k = cgd->iter + 1;
-  const double pap = cgd->pap;
-  const double rr = cgd->rr[(k - 1) & 1];
-  const double alpha = pap > 0.0 ? rr / pap : 0.0;
-  const R a = R(alpha);
-  R acc = R(0);  // a thread's few entries in R; blocks and the total in FP64
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    typename Vec2<R>::T xv = x[i], rv = r[i];
-    const typename Vec2<R>::T pv = p[i], av = ap[i];
-    xv.x = fma(a, pv.x, xv.x); xv.y = fma(a, pv.y, xv.y);
-    rv.x = fma(-a, av.x, rv.x); rv.y = fma(-a, av.y, rv.y);
-    x[i] = xv;
-    r[i] = rv;
-    acc = fma(rv.x, rv.x, acc);
-    acc = fma(rv.y, rv.y, acc);
+// A value as its storage holds it.
+template <typename ST, typename R> __device__ __forceinline__ Cx<R> stored(const Cx<R>& v) {
+  if constexpr (std::is_same<ST, R>::value) {
+    return v;
+  } else {
+    const float2 f = Conv16<ST>::f2(Conv16<ST>::of(make_float2(v.re, v.im)));
+    return cx<float>(f.x, f.y);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    cgd->alpha = alpha;
-    cgd->k_axpy = k;
-  }
-  block_reduce_total(double(acc), rr_part, &cgd->ticket[1], &cgd->rr_next);
 }
-
-// rr_new = cgd->rr_next; done if rr_new <= tol2 bb; beta = rr_new / rr_old;
-// p = r + beta p (also on the converging iteration, so that a reliable update
-// that finds the true residual still too large can simply continue).
-// Block 0 publishes rr[k&1], the history entry, iter = k (also to the host
-// through iter_out) and `done`; no block of this kernel reads those.
-template <typename R>
-__global__ void __launch_bounds__(kVecThreads) cg_xpay_kernel(
-    typename Vec2<R>::T* __restrict__ p, const typename Vec2<R>::T* __restrict__ r,
-    CgDev* __restrict__ cgd, double* __restrict__ hist, int* __restrict__ iter_out, int maxiter, int n) {
+template <typename R, typename ST>
+__global__ void __launch_bounds__(kVecThreads) cg_update_kernel(
+    typename Vec2<R>::T* __restrict__ x, typename Vec2<ST>::T* __restrict__ r, typename Vec2<ST>::T* __restrict__ p,
+    const typename Vec2<ST>::T* __restrict__ ap, CgDev* __restrict__ cgd, double* __restrict__ rr_part,
+    double* __restrict__ hist, int* __restrict__ iter_out, int maxiter, int scaled, int n) {
   if (cgd->done) return;
-  const int k = cgd->k_axpy;
-  const double rr_new = cgd->rr_next;
-  const double rr_old = cgd->rr[(k - 1) & 1];
-  const bool conv = rr_new <= cgd->tol2bb;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    cgd->rr[k & 1] = rr_new;
-    if (k <= maxiter) hist[k] = rr_new;
-    cgd->iter = k;
-    *iter_out = k;
-    if (conv) cgd->done = 1;
+  const R a = R(cgd->alpha), b = R(cgd->beta);
+  R acc = R(0);  // a thread's few entries in R; blocks and the total in FP64
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += gridDim.x * blockDim.x) {
+    Cx<R> xv[2], rv[2], pv[2], av[2];
+    Quad<R>::load_cg(x, i, xv[0], xv[1]);
+    Quad<ST>::load_cg(r, i, rv[0], rv[1]);
+    Quad<ST>::load_cg(p, i, pv[0], pv[1]);
+    Quad<ST>::load_cg(ap, i, av[0], av[1]);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      xv[k] = cx<R>(fma(a, pv[k].re, xv[k].re), fma(a, pv[k].im, xv[k].im));
+      rv[k] = stored<ST>(cx<R>(fma(-a, av[k].re, rv[k].re), fma(-a, av[k].im, rv[k].im)));
+      pv[k] = cx<R>(fma(b, pv[k].re, rv[k].re), fma(b, pv[k].im, rv[k].im));
+      acc = fma(rv[k].re, rv[k].re, acc);
+      acc = fma(rv[k].im, rv[k].im, acc);
+    }
+    Quad<R>::store(x, i, xv[0], xv[1]);
+    Quad<ST>::store(r, i, rv[0], rv[1]);
+    Quad<ST>::store(p, i, pv[0], pv[1]);
   }
-  const R beta = R(rr_old > 0.0 ? rr_new / rr_old : 0.0);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    typename Vec2<R>::T pv = p[i];
-    const typename Vec2<R>::T rv = r[i];
-    pv.x = fma(beta, pv.x, rv.x);
-    pv.y = fma(beta, pv.y, rv.y);
-    p[i] = pv;
-  }
+  const R v[1] = {acc};
+  double tot[1];
+  if (block_total<1, kVecThreads>(v, rr_part, &cgd->ticket[1], tot) && threadIdx.x == 0)
+    publish(cgd, tot[0], hist, iter_out, maxiter, scaled ? cgd->sigma2 : 1.0);
 }
 
 // Reliable update, first half: x64 += x_s; x_s = 0.
@@ -809,68 +768,6 @@ __global__ void __launch_bounds__(kVecThreads) df_to_double_kernel(double2* __re
 // |r / sigma|^2 = n after every reliable update keeps the entries O(1), far
 // from the ends of the half range.  Scalars (rr, pAp, alpha, beta) are in the scaled units;
 // the history and the convergence test use rr sigma^2.
-template <typename S>
-__global__ void __launch_bounds__(kVecThreads) cg_axpy_h16_kernel(float2* __restrict__ x,
-                                                                  typename Conv16<S>::T2* __restrict__ r,
-                                                                  const typename Conv16<S>::T2* __restrict__ p,
-                                                                  const typename Conv16<S>::T2* __restrict__ ap,
-                                                                  CgDev* __restrict__ cgd, double* __restrict__ rr_part,
-                                                                  int n) {
-  if (cgd->done) return;
-  const int k = cgd->iter + 1;
-  const double pap = cgd->pap;
-  const double rr = cgd->rr[(k - 1) & 1];
-  const double alpha = pap > 0.0 ? rr / pap : 0.0;
-  const float a = float(alpha);
-  float acc = 0.0f;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float2 xv = x[i];
-    float2 rv = Conv16<S>::f2(r[i]);
-    const float2 pv = Conv16<S>::f2(p[i]), av = Conv16<S>::f2(ap[i]);
-    xv.x = fmaf(a, pv.x, xv.x); xv.y = fmaf(a, pv.y, xv.y);
-    rv.x = fmaf(-a, av.x, rv.x); rv.y = fmaf(-a, av.y, rv.y);
-    x[i] = xv;
-    const typename Conv16<S>::T2 rh = Conv16<S>::of(rv);
-    r[i] = rh;
-    const float2 rq = Conv16<S>::f2(rh);   // |r|^2 of the stored residual
-    acc = fmaf(rq.x, rq.x, acc);
-    acc = fmaf(rq.y, rq.y, acc);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    cgd->alpha = alpha;
-    cgd->k_axpy = k;
-  }
-  block_reduce_total(double(acc), rr_part, &cgd->ticket[1], &cgd->rr_next);
-}
-
-template <typename S>
-__global__ void __launch_bounds__(kVecThreads) cg_xpay_h16_kernel(typename Conv16<S>::T2* __restrict__ p,
-                                                                  const typename Conv16<S>::T2* __restrict__ r,
-                                                                  CgDev* __restrict__ cgd, double* __restrict__ hist,
-                                                                  int* __restrict__ iter_out, int maxiter, int n) {
-  if (cgd->done) return;
-  const int k = cgd->k_axpy;
-  const double rr_new = cgd->rr_next;
-  const double rr_old = cgd->rr[(k - 1) & 1];
-  const double rr_true = rr_new * cgd->sigma2;
-  const bool conv = rr_true <= cgd->tol2bb;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    cgd->rr[k & 1] = rr_new;
-    if (k <= maxiter) hist[k] = rr_true;
-    cgd->iter = k;
-    *iter_out = k;
-    if (conv) cgd->done = 1;
-  }
-  const float beta = float(rr_old > 0.0 ? rr_new / rr_old : 0.0);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float2 pv = Conv16<S>::f2(p[i]);
-    const float2 rv = Conv16<S>::f2(r[i]);
-    pv.x = fmaf(beta, pv.x, rv.x);
-    pv.y = fmaf(beta, pv.y, rv.y);
-    p[i] = Conv16<S>::of(pv);
-  }
-}
-
 __global__ void cg_init_h16_kernel(const double* __restrict__ part, int nparts, CgDev* __restrict__ cgd, double tol2,
                                    double* __restrict__ bb_out, int n) {
   const double bb = block_sum_partials(part, nparts);
@@ -883,7 +780,6 @@ __global__ void cg_init_h16_kernel(const double* __restrict__ part, int nparts, 
     cgd->rr[0] = cgd->rr[1] = bb / s2;
     cgd->done = bb == 0.0 ? 1 : 0;
     cgd->iter = 0;
-    cgd->k_axpy = 0;
     cgd->pending = 0;
     cgd->restart = 0;
     *bb_out = bb;
@@ -1040,7 +936,6 @@ __global__ void cg_init_kernel(const double* __restrict__ part, int n, CgDev* __
     cgd->rr[0] = cgd->rr[1] = bb;
     cgd->done = bb == 0.0 ? 1 : 0;
     cgd->iter = 0;
-    cgd->k_axpy = 0;
     cgd->pending = 0;
     cgd->restart = 0;
     *bb_out = bb;
@@ -1060,7 +955,6 @@ __global__ void cg_init_guess_kernel(const double* __restrict__ part_b, const do
     cgd->rr[0] = cgd->rr[1] = rr;
     cgd->done = (bb == 0.0 || rr <= tol2 * bb) ? 1 : 0;
     cgd->iter = 0;
-    cgd->k_axpy = 0;
     cgd->pending = 0;
     cgd->restart = 0;
     *bb_out = bb;
@@ -1169,9 +1063,8 @@ template <typename RS> static int hop_blocks(int Vh) {
 int dslash_blocks(int Vh) { return (Vh + 31) / 32; }
 
 template <typename RL, int NC, typename RS>
-cudaError_t launch_dslash(const GeomH& gh, void* out, const void* in, const void* x, const void* pdot,
-                          const void* U, int out_par, int dag, int mode, double b, double* partial,
-                          CgDev* cgd, cudaStream_t st) {
+cudaError_t launch_dslash(const GeomH& gh, void* out, const void* in, const void* x, const void* U, int out_par,
+                          int dag, int mode, double b, const CgDev* cgd, cudaStream_t st) {
   Gauge<RL, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
@@ -1180,11 +1073,11 @@ cudaError_t launch_dslash(const GeomH& gh, void* out, const void* in, const void
   const bool split = hop_split<RS>(gh.Vh);
 #define FG_DS(D, M)                                                                                       \
   (split ? dslash_split_kernel<RL, NC, RS, D, M> : dslash_kernel<RL, NC, RS, D, M>)<<<nb, kDslashThreads, 0, st>>>( \
-      v2<RS>(out), cv2<RS>(in), cv2<RS>(x), cv2<RS>(pdot), u, g, out_par, RS(b), partial, cgd)
+      v2<RS>(out), cv2<RS>(in), cv2<RS>(x), u, g, out_par, RS(b), cgd)
   if (dag) {
-    if (mode == 0) FG_DS(1, 0); else if (mode == 1) FG_DS(1, 1); else FG_DS(1, 2);
+    if (mode == 0) FG_DS(1, 0); else FG_DS(1, 1);
   } else {
-    if (mode == 0) FG_DS(0, 0); else if (mode == 1) FG_DS(0, 1); else FG_DS(0, 2);
+    if (mode == 0) FG_DS(0, 0); else FG_DS(0, 1);
   }
 #undef FG_DS
   return cudaGetLastError();
@@ -1205,16 +1098,10 @@ cudaError_t launch_fermion_force(const GeomH& gh, const void* U, const void* Xe,
 }
 
 template <typename R>
-cudaError_t launch_cg_axpy(void* x, void* r, const void* p, const void* ap, CgDev* cgd, double* rr_part, int n,
-                           cudaStream_t st) {
-  cg_axpy_kernel<R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(x), v2<R>(r), cv2<R>(p), cv2<R>(ap), cgd,
-                                                           rr_part, n);
-  return cudaGetLastError();
-}
-template <typename R>
-cudaError_t launch_cg_xpay(void* p, const void* r, CgDev* cgd, double* hist, int* iter_out, int maxiter, int n,
-                           cudaStream_t st) {
-  cg_xpay_kernel<R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(p), cv2<R>(r), cgd, hist, iter_out, maxiter, n);
+cudaError_t launch_cg_update(void* x, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part, double* hist,
+                             int* iter_out, int maxiter, int n, cudaStream_t st) {
+  cg_update_kernel<R, R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(x), v2<R>(r), v2<R>(p), cv2<R>(ap), cgd, rr_part,
+                                                               hist, iter_out, maxiter, 0, n);
   return cudaGetLastError();
 }
 template <typename R> static bool cg_defer(int Vh) { return hop_split<R>(Vh) && Vh <= FG_DEFER_MAX; }
@@ -1223,7 +1110,7 @@ template <typename R, int NC>
 cudaError_t launch_cg_hop(const GeomH& gh, void* te, const void* to, const void* p, const void* U, double k2,
                           double* partial, CgDev* cgd, double* hist, int* iter_out, int maxiter, cudaStream_t st) {
   if (!cg_defer<R>(gh.Vh))
-    return launch_dslash<R, NC, R>(gh, te, to, p, nullptr, U, 0, 0, 1, -k2, nullptr, cgd, st);
+    return launch_dslash<R, NC, R>(gh, te, to, p, U, 0, 0, 1, -k2, cgd, st);
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
@@ -1239,12 +1126,14 @@ cudaError_t launch_cg_publish(const GeomH& gh, const double* partial, CgDev* cgd
 }
 template <typename R, int NC>
 cudaError_t launch_cg_apdot(const GeomH& gh, void* ap, const void* to, const void* te, const void* p, const void* r,
-                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st) {
+                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st, bool deferred) {
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  auto* const k = cg_defer<R>(gh.Vh) ? cg_apdot_split_kernel<R, NC, true>
-                                     : (hop_split<R>(gh.Vh) ? cg_apdot_split_kernel<R, NC, false> : cg_apdot_kernel<R, NC>);
+  // totals are deferred only with a folded iteration's A behind
+  auto* const k = deferred && cg_defer<R>(gh.Vh)
+                      ? cg_apdot_split_kernel<true, R, NC, R>
+                      : (hop_split<R>(gh.Vh) ? cg_apdot_split_kernel<false, R, NC, R> : cg_apdot_kernel<R, NC, R>);
   k<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0, st>>>(
       v2<R>(ap), cv2<R>(to), cv2<R>(te), cv2<R>(p), cv2<R>(r), u, to_devg(gh), R(-k2), partial, cgd);
   return cudaGetLastError();
@@ -1316,9 +1205,8 @@ cudaError_t launch_df_to_double(void* dst, const void* src, int n, cudaStream_t 
   return cudaGetLastError();
 }
 template <typename S, int NC>
-static cudaError_t dslash16(const GeomH& gh, void* out, const void* in, const void* x, const void* pdot,
-                            const void* U, int out_par, int dag, int mode, double b, double* partial, CgDev* cgd,
-                            cudaStream_t st) {
+static cudaError_t dslash16(const GeomH& gh, void* out, const void* in, const void* x, const void* U, int out_par,
+                            int dag, int mode, double b, const CgDev* cgd, cudaStream_t st) {
   typedef typename Conv16<S>::T2 T2;
   Gauge<S, NC> u;
   u.p = const_cast<void*>(U);
@@ -1329,27 +1217,48 @@ static cudaError_t dslash16(const GeomH& gh, void* out, const void* in, const vo
 #define FG_DH(D, M)                                                                                            \
   (split ? dslash_split_kernel<S, NC, float, D, M, S>                                                          \
          : dslash_kernel<S, NC, float, D, M, S>)<<<nb, kDslashThreads, 0, st>>>(                               \
-      (T2*)out, (const T2*)in, (const T2*)x, (const T2*)pdot, u, g, out_par, float(b), partial, cgd)
+      (T2*)out, (const T2*)in, (const T2*)x, u, g, out_par, float(b), cgd)
   if (dag) {
-    if (mode == 0) FG_DH(1, 0); else if (mode == 1) FG_DH(1, 1); else FG_DH(1, 2);
+    if (mode == 0) FG_DH(1, 0); else FG_DH(1, 1);
   } else {
-    if (mode == 0) FG_DH(0, 0); else if (mode == 1) FG_DH(0, 1); else FG_DH(0, 2);
+    if (mode == 0) FG_DH(0, 0); else FG_DH(0, 1);
   }
 #undef FG_DH
   return cudaGetLastError();
 }
 template <int NC>
-cudaError_t launch_dslash_h16(int s16, const GeomH& gh, void* out, const void* in, const void* x, const void* pdot,
-                              const void* U, int out_par, int dag, int mode, double b, double* partial,
-                              CgDev* cgd, cudaStream_t st) {
-  return s16 == S16_BF16
-             ? dslash16<BF16, NC>(gh, out, in, x, pdot, U, out_par, dag, mode, b, partial, cgd, st)
-             : dslash16<Half16, NC>(gh, out, in, x, pdot, U, out_par, dag, mode, b, partial, cgd, st);
+cudaError_t launch_dslash_h16(int s16, const GeomH& gh, void* out, const void* in, const void* x, const void* U,
+                              int out_par, int dag, int mode, double b, const CgDev* cgd, cudaStream_t st) {
+  return s16 == S16_BF16 ? dslash16<BF16, NC>(gh, out, in, x, U, out_par, dag, mode, b, cgd, st)
+                         : dslash16<Half16, NC>(gh, out, in, x, U, out_par, dag, mode, b, cgd, st);
 }
-template cudaError_t launch_dslash_h16<9>(int, const GeomH&, void*, const void*, const void*, const void*,
-                                          const void*, int, int, int, double, double*, CgDev*, cudaStream_t);
-template cudaError_t launch_dslash_h16<6>(int, const GeomH&, void*, const void*, const void*, const void*,
-                                          const void*, int, int, int, double, double*, CgDev*, cudaStream_t);
+template cudaError_t launch_dslash_h16<9>(int, const GeomH&, void*, const void*, const void*, const void*, int, int,
+                                          int, double, const CgDev*, cudaStream_t);
+template cudaError_t launch_dslash_h16<6>(int, const GeomH&, void*, const void*, const void*, const void*, int, int,
+                                          int, double, const CgDev*, cudaStream_t);
+template <typename S, int NC>
+static cudaError_t apdot16(const GeomH& gh, void* ap, const void* to, const void* te, const void* p, const void* r,
+                           const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st) {
+  typedef typename Conv16<S>::T2 T2;
+  Gauge<S, NC> u;
+  u.p = const_cast<void*>(U);
+  u.V = gh.V;
+  auto* const k = hop_split<float>(gh.Vh) ? cg_apdot_split_kernel<false, S, NC, float, S> : cg_apdot_kernel<S, NC, float, S>;
+  k<<<hop_blocks<float>(gh.Vh), kDslashThreads, 0, st>>>((T2*)ap, (const T2*)to, (const T2*)te, (const T2*)p,
+                                                        (const T2*)r, u, to_devg(gh), float(-k2), partial, cgd);
+  return cudaGetLastError();
+}
+template <int NC>
+cudaError_t launch_cg_apdot_h16(int s16, const GeomH& gh, void* ap, const void* to, const void* te, const void* p,
+                                const void* r, const void* U, double k2, double* partial, CgDev* cgd,
+                                cudaStream_t st) {
+  return s16 == S16_BF16 ? apdot16<BF16, NC>(gh, ap, to, te, p, r, U, k2, partial, cgd, st)
+                         : apdot16<Half16, NC>(gh, ap, to, te, p, r, U, k2, partial, cgd, st);
+}
+template cudaError_t launch_cg_apdot_h16<9>(int, const GeomH&, void*, const void*, const void*, const void*,
+                                            const void*, const void*, double, double*, CgDev*, cudaStream_t);
+template cudaError_t launch_cg_apdot_h16<6>(int, const GeomH&, void*, const void*, const void*, const void*,
+                                            const void*, const void*, double, double*, CgDev*, cudaStream_t);
 // Runs KERNEL<S> with the arguments that follow for the 16-bit format s16.
 #define FG_S16(KERNEL, GRID, ...)                                                                              \
   do {                                                                                                         \
@@ -1361,15 +1270,16 @@ template cudaError_t launch_dslash_h16<6>(int, const GeomH&, void*, const void*,
       KERNEL<Half16><<<GRID, kVecThreads, 0, st>>>(__VA_ARGS__);                                               \
     }                                                                                                          \
   } while (0)
-cudaError_t launch_cg_axpy_h16(int s16, void* xs, void* r, const void* p, const void* ap, CgDev* cgd,
-                               double* rr_part, int n, cudaStream_t st) {
-  FG_S16(cg_axpy_h16_kernel, vec_blocks(n), (float2*)xs, (T2*)r, (const T2*)p, (const T2*)ap, cgd, rr_part, n);
-  return cudaGetLastError();
-}
-cudaError_t launch_cg_xpay_h16(int s16, void* p, const void* r, CgDev* cgd, double* hist, int* iter_out,
-                               int maxiter, int n, cudaStream_t st) {
-  FG_S16(cg_xpay_h16_kernel, vec_blocks(n), (T2*)p, (const T2*)r, cgd, hist, iter_out, maxiter, n);
-  return cudaGetLastError();
+cudaError_t launch_cg_update_h16(int s16, void* xs, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part,
+                                 double* hist, int* iter_out, int maxiter, int n, cudaStream_t st) {
+  auto run = [&](auto s) {
+    typedef decltype(s) S;
+    typedef typename Conv16<S>::T2 T2;
+    cg_update_kernel<float, S><<<vec_blocks(n), kVecThreads, 0, st>>>((float2*)xs, (T2*)r, (T2*)p, (const T2*)ap, cgd,
+                                                                     rr_part, hist, iter_out, maxiter, 1, n);
+    return cudaGetLastError();
+  };
+  return s16 == S16_BF16 ? run(BF16{}) : run(Half16{});
 }
 cudaError_t launch_cg_init_h16(const double* part, int nparts, CgDev* cgd, double tol2, double* bb_out, int n,
                                cudaStream_t st) {
@@ -1447,9 +1357,8 @@ cudaError_t launch_spinor_to_canon(const void* f, double* canon, int Vh, cudaStr
 }
 
 #define FG_INST_F(RL, NC, RS)                                                                                  \
-  template cudaError_t launch_dslash<RL, NC, RS>(const GeomH&, void*, const void*, const void*, const void*,  \
-                                                 const void*, int, int, int, double, double*, CgDev*,        \
-                                                 cudaStream_t);                                               \
+  template cudaError_t launch_dslash<RL, NC, RS>(const GeomH&, void*, const void*, const void*, const void*, int, \
+                                                 int, int, double, const CgDev*, cudaStream_t);                \
   template cudaError_t launch_fermion_force<RL, NC, RS>(const GeomH&, const void*, const void*, const void*,  \
                                                         const void*, const void*, void*, double, int,         \
                                                         cudaStream_t);
@@ -1459,12 +1368,10 @@ FG_INST_F(float, 9, float)
 FG_INST_F(float, 6, float)
 FG_INST_F(float, 9, double)
 FG_INST_F(float, 6, double)
-template cudaError_t launch_dslash<Half16, 9, float>(const GeomH&, void*, const void*, const void*,
-                                                     const void*, const void*, int, int, int, double, double*,
-                                                     CgDev*, cudaStream_t);
-template cudaError_t launch_dslash<Half16, 6, float>(const GeomH&, void*, const void*, const void*,
-                                                     const void*, const void*, int, int, int, double, double*,
-                                                     CgDev*, cudaStream_t);
+template cudaError_t launch_dslash<Half16, 9, float>(const GeomH&, void*, const void*, const void*, const void*, int, int, int,
+                                                     double, const CgDev*, cudaStream_t);
+template cudaError_t launch_dslash<Half16, 6, float>(const GeomH&, void*, const void*, const void*, const void*, int, int, int,
+                                                     double, const CgDev*, cudaStream_t);
 
 template <typename S, int NC>
 __global__ void __launch_bounds__(256) links_to_half_kernel(Gauge<float, NC> in, Gauge<S, NC> out, int V) {
@@ -1494,22 +1401,21 @@ cudaError_t launch_links_to_half(int s16, const GeomH& gh, const void* U32, void
 template cudaError_t launch_links_to_half<9>(int, const GeomH&, const void*, void*, cudaStream_t);
 template cudaError_t launch_links_to_half<6>(int, const GeomH&, const void*, void*, cudaStream_t);
 
-template cudaError_t launch_dslash<float, 9, DF>(const GeomH&, void*, const void*, const void*, const void*,
-                                                 const void*, int, int, int, double, double*, CgDev*, cudaStream_t);
-template cudaError_t launch_dslash<float, 6, DF>(const GeomH&, void*, const void*, const void*, const void*,
-                                                 const void*, int, int, int, double, double*, CgDev*, cudaStream_t);
+template cudaError_t launch_dslash<float, 9, DF>(const GeomH&, void*, const void*, const void*, const void*, int, int, int,
+                                                     double, const CgDev*, cudaStream_t);
+template cudaError_t launch_dslash<float, 6, DF>(const GeomH&, void*, const void*, const void*, const void*, int, int, int,
+                                                     double, const CgDev*, cudaStream_t);
 
-template cudaError_t launch_cg_axpy<double>(void*, void*, const void*, const void*, CgDev*, double*, int,
-                                            cudaStream_t);
-template cudaError_t launch_cg_axpy<float>(void*, void*, const void*, const void*, CgDev*, double*, int,
-                                           cudaStream_t);
-template cudaError_t launch_cg_xpay<double>(void*, const void*, CgDev*, double*, int*, int, int, cudaStream_t);
-template cudaError_t launch_cg_xpay<float>(void*, const void*, CgDev*, double*, int*, int, int, cudaStream_t);
+template cudaError_t launch_cg_update<double>(void*, void*, void*, const void*, CgDev*, double*, double*, int*, int, int,
+                                              cudaStream_t);
+template cudaError_t launch_cg_update<float>(void*, void*, void*, const void*, CgDev*, double*, double*, int*, int, int,
+                                             cudaStream_t);
 #define FG_INST_FOLD(R, NC)                                                                                    \
   template cudaError_t launch_cg_hop<R, NC>(const GeomH&, void*, const void*, const void*, const void*, double, \
                                             double*, CgDev*, double*, int*, int, cudaStream_t);                \
   template cudaError_t launch_cg_apdot<R, NC>(const GeomH&, void*, const void*, const void*, const void*,      \
-                                              const void*, const void*, double, double*, CgDev*, cudaStream_t); \
+                                              const void*, const void*, double, double*, CgDev*, cudaStream_t,  \
+                                              bool);                                                           \
   template cudaError_t launch_cg_fold<R, NC>(const GeomH&, void*, void*, const void*, const void*, const void*, \
                                              void*, void*, const void*, double*, CgDev*, double*, int*, int,    \
                                              cudaStream_t);

@@ -19,12 +19,10 @@ struct CgDev {
   double tol2bb;
   double alpha;
   int done;
-  int iter;     // last completed iteration (written by xpay's block 0)
-  int k_axpy;   // iteration in progress (written by axpy's block 0)
+  int iter;     // last completed iteration
   int restart;  // set by a reliable update whose true residual left the recursion far behind
-  double pap;       // <p, Ap> of the iteration in progress (grand total of the Dslash partials)
-  double rr_next;   // |r|^2 after the iteration in progress (grand total of the axpy partials)
-  double beta;      // folded iteration: beta of the update in progress
+  double pap;       // <p, Ap> of the iteration in progress
+  double beta;      // beta of the update in progress
   unsigned ticket[2];  // blocks finished, for the two grand totals; the last block resets it to 0
   // half-precision inner vectors hold r / sigma and p / sigma; sigma^2 is
   // reset at every reliable update to |r|^2 / n, and rho rescales p then
@@ -41,16 +39,14 @@ int dslash_blocks(int Vh);
 
 // RS = DF (df64.cuh) evaluates the hop in double-float arithmetic on FP32
 // links (instantiated for RL = float; the solver uses modes 0 and 1).
-// out = b D in (mode 0); out = x + b D in (mode 1); mode 2 (CG only) also
-// sums Re <pdot, out> into cgd->pap through the block partials `partial`.
+// out = b D in (mode 0); out = x + b D in (mode 1).
 // D hops from parity 1-out_par to out_par; dag = 1 applies g5 D g5.  Links
 // stored as RL with NC complex entries, spinors and arithmetic in RS.  If
 // `cgd` is non-null and cgd->done != 0 the kernel returns at once (converged
 // CG).
 template <typename RL, int NC, typename RS>
-cudaError_t launch_dslash(const GeomH& g, void* out, const void* in, const void* x, const void* pdot,
-                          const void* U, int out_par, int dag, int mode, double b, double* partial,
-                          CgDev* cgd, cudaStream_t st);
+cudaError_t launch_dslash(const GeomH& g, void* out, const void* in, const void* x, const void* U, int out_par,
+                          int dag, int mode, double b, const CgDev* cgd, cudaStream_t st);
 
 // 16-bit formats of the inner solver's links and vectors (argument s16).
 enum { S16_HALF = 0, S16_BF16 = 1 };
@@ -66,16 +62,12 @@ template <typename RL, int NC, typename RS>
 cudaError_t launch_fermion_force(const GeomH& g, const void* U, const void* Xe, const void* Xo, const void* Ye,
                                  const void* Yo, void* FF, double kappa2, int accumulate, cudaStream_t st);
 
-// x += alpha p, r -= alpha Ap with alpha = rr / cgd->pap; |r|^2 into
-// cgd->rr_next through the block partials rr_part.
+// x += alpha p, r -= alpha Ap, p = r + beta p with cgd's alpha and beta;
+// |r|^2 is published as the residual of iteration iter + 1 (rr[], hist,
+// *iter_out, done).
 template <typename R>
-cudaError_t launch_cg_axpy(void* x, void* r, const void* p, const void* ap, CgDev* cgd, double* rr_part, int n,
-                           cudaStream_t st);
-// p = r + beta p with beta = cgd->rr_next / rr; hist[k] receives |r_k|^2 for
-// k <= maxiter and *iter_out the iteration k.
-template <typename R>
-cudaError_t launch_cg_xpay(void* p, const void* r, CgDev* cgd, double* hist, int* iter_out, int maxiter, int n,
-                           cudaStream_t st);
+cudaError_t launch_cg_update(void* x, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part, double* hist,
+                             int* iter_out, int maxiter, int n, cudaStream_t st);
 template <typename RI>
 cudaError_t launch_ru_accumulate(void* x64, void* xs, int n, cudaStream_t st);
 template <typename RI>
@@ -94,13 +86,16 @@ cudaError_t launch_df_to_double(void* dst, const void* src, int n, cudaStream_t 
 // 1/sigma; the solution increment x_s stays FP32)
 // Dslash with 16-bit links and spinors of format s16, FP32 arithmetic.
 template <int NC>
-cudaError_t launch_dslash_h16(int s16, const GeomH& g, void* out, const void* in, const void* x, const void* pdot,
-                              const void* U, int out_par, int dag, int mode, double b, double* partial,
-                              CgDev* cgd, cudaStream_t st);
-cudaError_t launch_cg_axpy_h16(int s16, void* xs, void* r, const void* p, const void* ap, CgDev* cgd,
-                               double* rr_part, int n, cudaStream_t st);
-cudaError_t launch_cg_xpay_h16(int s16, void* p, const void* r, CgDev* cgd, double* hist, int* iter_out,
-                               int maxiter, int n, cudaStream_t st);
+cudaError_t launch_dslash_h16(int s16, const GeomH& g, void* out, const void* in, const void* x, const void* U,
+                              int out_par, int dag, int mode, double b, const CgDev* cgd, cudaStream_t st);
+// launch_cg_apdot and launch_cg_update on 16-bit vectors (hist and done in
+// units of |b|).
+template <int NC>
+cudaError_t launch_cg_apdot_h16(int s16, const GeomH& g, void* ap, const void* to, const void* te, const void* p,
+                                const void* r, const void* U, double k2, double* partial, CgDev* cgd,
+                                cudaStream_t st);
+cudaError_t launch_cg_update_h16(int s16, void* xs, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part,
+                                 double* hist, int* iter_out, int maxiter, int n, cudaStream_t st);
 // Start of a solve: bb from the partials of |b|^2, sigma^2 = bb / n, rr = n, tol2bb, done.
 cudaError_t launch_cg_init_h16(const double* part, int nparts, CgDev* cgd, double tol2, double* bb_out, int n,
                                cudaStream_t st);
@@ -152,10 +147,12 @@ cudaError_t launch_cg_publish(const GeomH& g, const double* partial, CgDev* cgd,
                               int maxiter, cudaStream_t st);
 // D: Ap = te - k2 D_eo^dagger to on the even sites, and the sums of <p, Ap>,
 // Re <r, Ap>, |Ap|^2 from which alpha = rr / <p, Ap> and
-// beta = (rr - 2 alpha Re <r, Ap> + alpha^2 |Ap|^2) / rr follow, rr = cgd->rr[iter & 1].
+// beta = (rr - 2 alpha Re <r, Ap> + alpha^2 |Ap|^2) / rr follow, rr =
+// cgd->rr[iter & 1]: set in cgd, or with `deferred` (a folded iteration) left
+// as block sums to A where cg_deferred().
 template <typename R, int NC>
 cudaError_t launch_cg_apdot(const GeomH& g, void* ap, const void* to, const void* te, const void* p, const void* r,
-                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st);
+                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st, bool deferred);
 // A: x += alpha p; r2 = r - alpha Ap; p2 = r2 + beta p (even sites) and
 // to = D_oe p2 (odd sites); |r2|^2 is the residual of iteration iter + 1
 // (rr[], hist, *iter_out, done).  r, p and r2, p2 are different buffers.
