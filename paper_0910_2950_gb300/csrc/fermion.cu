@@ -862,6 +862,9 @@ __global__ void ru_publish_h16_kernel(const double* __restrict__ part, int npart
     cgd->restart = (rr > 2.0 * rr_iter) ? 1 : 0;
     cgd->rho = sqrt(cgd->sigma2 / s2);
     cgd->sigma2 = s2;
+    const DF inv(1.0 / sqrt(s2));
+    cgd->inv_hi = inv.hi;
+    cgd->inv_lo = inv.lo;
     cgd->rr[cgd->iter & 1] = rr / s2;
     cgd->done = rr <= cgd->tol2bb ? 1 : 0;
     *true_rr = rr;
@@ -873,21 +876,22 @@ __global__ void __launch_bounds__(kVecThreads) ru_rescale_h16_kernel(const RV* _
                                                                      typename Conv16<S>::T2* __restrict__ rs,
                                                                      typename Conv16<S>::T2* __restrict__ p,
                                                                      const CgDev* __restrict__ cgd, int n) {
-  const double inv = 1.0 / sqrt(cgd->sigma2);
+  // 1 / sigma as ru_publish_h16 left it: a root and a division in FP64 in every
+  // thread, and FP64 products, made this pass 87 us at 24^3 x 48
+  const DF inv(cgd->inv_hi, cgd->inv_lo);
   const float rho = float(cgd->rho);
   const bool restart = cgd->restart != 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double re, im;
+    float2 f;
     if constexpr (std::is_same<RV, float4>::value) {   // double-float residual
       const float4 v = ((const float4*)r)[i];
-      re = double(DF(v.x, v.y));
-      im = double(DF(v.z, v.w));
+      f = make_float2((DF(v.x, v.y) * inv).hi, (DF(v.z, v.w) * inv).hi);
     } else {
       const double2 v = ((const double2*)r)[i];
-      re = v.x;
-      im = v.y;
+      const double d = double(inv);
+      f = make_float2(float(v.x * d), float(v.y * d));
     }
-    const typename Conv16<S>::T2 h = Conv16<S>::of(make_float2(float(re * inv), float(im * inv)));
+    const typename Conv16<S>::T2 h = Conv16<S>::of(f);
     rs[i] = h;
     if (restart) {
       p[i] = h;

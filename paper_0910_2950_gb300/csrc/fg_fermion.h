@@ -28,6 +28,7 @@ struct CgDev {
   // reset at every reliable update to |r|^2 / n, and rho rescales p then
   double sigma2;
   double rho;
+  float inv_hi, inv_lo;  // 1 / sigma as a double-float
   // folded iteration with one direction a warp: block sums of |r'|^2 are left
   // and not yet published
   int pending;
