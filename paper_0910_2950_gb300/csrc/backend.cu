@@ -499,17 +499,17 @@ class Backend final : public IBackend {
   // rs_ and p_ always name the current ones
   void *rs2_ = nullptr, *p2_ = nullptr;
   // Folded CG iterations (four launches, vector updates inside the Dslash
-  // launches) or six (four Dslash, axpy, xpay) for FP32 and FP64 inner
-  // vectors.  The folded form forms p' at each of a site's eight neighbours,
-  // reading r, Ap and p per hop, to save two streaming vector passes and two
-  // launches.  While the solver's links and vectors fit in L2 the extra hop
-  // reads hit L2 and the saved launches count (served 8^3 x 16 and
-  // 12^3 x 24 chains; 16^3 x 32 FP32 within run-to-run spread: 8.9 against
-  // 9.0 and 8.1 against 7.5 ms per solve on two fields); beyond L2 they
-  // cost DRAM bandwidth (FP32 25.7 against 17.9 ms at 20^3 x 40, 38.8
-  // against 34.2 at 24^3 x 48; FP64 at 16^3 x 32 61.7 against 56.6).
+  // launches) or five (four Dslash, one vector update) for FP32 and FP64
+  // inner vectors.  The folded form forms p' at each of a site's eight
+  // neighbours, reading r, Ap and p per hop, to save a streaming vector pass
+  // and a launch.  While the solver's links and vectors fit in L2 the extra
+  // hop reads hit L2 and the saved launch counts (served 8^3 x 16 and
+  // 12^3 x 24 chains); beyond L2 they cost DRAM bandwidth (against six
+  // launches, axpy and xpay apart: FP32 25.7 against 17.9 ms at 20^3 x 40,
+  // 38.8 against 34.2 at 24^3 x 48; FP64 at 16^3 x 32 61.7 against 56.6; the
+  // fifth launch takes another 2% off the FP32 ones).
   // Default: folded when the fields fit in L2; FG_CG_FOLD=1 or 0 in the
-  // environment forces either form.  The 16-bit solvers always take six
+  // environment forces either form.  The 16-bit solvers always take five
   // launches.
   const bool fold_ = [this] {
     const char* e = std::getenv("FG_CG_FOLD");
@@ -663,10 +663,9 @@ class Backend final : public IBackend {
   // The fused gauge-force kernel with whatever a.FF holds (no solve).  With
   // split_exp_ (the default for double-float) the exponential of a
   // kick-and-drift or a displacement runs in a launch of its own after the
-  // force (the same arithmetic, the same bits): the staple products and the
-  // double-float exponential together overflow the instruction cache, and
-  // the split takes 16-21% off a double-float trajectory, while FP32 runs 9%
-  // faster fused.  FG_SPLIT_EXP=0 / =1 in the environment turns the split
+  // force (the same arithmetic, the same bits): the force's products and the
+  // double-float exponential in one kernel cost registers and instruction
+  // fetches, while FP32 runs 9% faster fused.  FG_SPLIT_EXP=0 / =1 in the environment turns the split
   // off / on for any precision.
   const bool split_exp_ = [] {
     const char* e = std::getenv("FG_SPLIT_EXP");

@@ -8,13 +8,14 @@
 // single-lattice layout (fg_common.cuh) at its own offset; a tile list
 // assigns blocks of H half-sites (both parities, four directions) to chains,
 // and the kernels walk it with a grid-stride loop over a grid sized to fill
-// the GPU once (a persistent launch).  Per-link arithmetic is the same code
+// the GPU once (a persistent launch).  The double-float and FP64 force takes
+// the single-lattice launches instead, over the rows of all chains.  Per-link arithmetic is the same code
 // as for one lattice (gauge_device.cuh), so a chain gives the same links alone
 // and in a batch.  The dH of every chain is summed in FP64 per chain and the
 // Metropolis step runs on the device, so a whole trajectory of all chains is
 // one CUDA graph: refresh, start energies, the fused force launches, end
 // energies, accept/reject, restore of rejected chains.  The tile size H is
-// chosen by timing the force kernel at the first trajectory (autotuning).
+// chosen by timing the launches that walk it at the first trajectory (autotuning).
 #include <cuda_runtime.h>
 
 #include <algorithm>

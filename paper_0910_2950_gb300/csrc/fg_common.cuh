@@ -152,15 +152,6 @@ template <typename R> __device__ __forceinline__ void mac_dn(M3<R>& acc, const M
       for (int k = 0; k < 3; ++k) cmac_cj(acc.e[i][j], a.e[k][i], b.e[k][j]);
 }
 
-// Re Tr(a * b)
-template <typename R> __device__ __forceinline__ R re_tr_mul(const M3<R>& a, const M3<R>& b) {
-  R s = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) s += a.e[i][k].re * b.e[k][i].re - a.e[i][k].im * b.e[k][i].im;
-  return s;
-}
 // Re Tr(a * b^dagger) = sum Re(a_ik conj(b_ik))
 template <typename R> __device__ __forceinline__ R re_tr_mul_nd(const M3<R>& a, const M3<R>& b) {
   R s = 0;
