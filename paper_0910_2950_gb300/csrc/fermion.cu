@@ -55,15 +55,20 @@ template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_
 // waits for its unit, and four times the warps spread over the SMs evenly:
 // 8^3 x 16 7.7 against 21.6 ms, 12^3 x 24 28.3 against 40.7, 16^3 x 32 73.0
 // against 76.6.
+// The line of FP32 and double-float lies lower than those solves put it: with
+// many chains served at once the GPU is full, the extra instructions of the
+// split form count, and eight concurrent slots of the Poisson mix (8^3 x 16
+// and 12^3 x 24 chains) ran 61 trajectories/s with the line at 24576, 74 at
+// 8192, 78 before and 81 with no split.
 #ifndef FG_SPLIT_MAX32
-#define FG_SPLIT_MAX32 24576
+#define FG_SPLIT_MAX32 8192
 #endif
 // Most sites with deferred totals (cg_fold_split_kernel).
 #ifndef FG_DEFER_MAX
 #define FG_DEFER_MAX 24576
 #endif
 #ifndef FG_SPLIT_MAXDF
-#define FG_SPLIT_MAXDF 32768
+#define FG_SPLIT_MAXDF 8192
 #endif
 #ifndef FG_SPLIT_MAX64
 #define FG_SPLIT_MAX64 131072
