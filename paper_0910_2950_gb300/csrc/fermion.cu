@@ -210,6 +210,11 @@ __device__ __forceinline__ void publish(CgDev* cgd, double rr, double* __restric
   if (rr * unit <= cgd->tol2bb) cgd->done = 1;
 }
 
+// Between iterations (one thread, no other launch of the solver in flight).
+__device__ __forceinline__ void set_done(CgDev* cgd, bool d) {
+  cgd->done = cgd->stop = d ? 1 : 0;
+}
+
 // D: Ap = te + b D^dagger_eo to at the even sites, with the three dot products.
 template <typename RL, int NC, typename R, typename ST = R>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_apdot_kernel(
@@ -394,7 +399,12 @@ __global__ void cg_publish_kernel(const double* __restrict__ part, int n, CgDev*
   publish_iteration(part, n, cgd, hist, iter_out, maxiter);
 }
 
-// B: te = p + b D_eo to, and in the last block the iteration before is published.
+// B: te = p + b D_eo to, and in the last block the iteration before is
+// published.  That block sets done while the others start: they look at stop
+// instead, which A sets when it finds done, so every thread of a block takes
+// the same way past the barrier of hops_split.  On the converging iteration te
+// is therefore still formed (C, D and A return and nothing reads it); from
+// the next iteration on B returns too.
 template <typename R, int NC>
 __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_hop_split_kernel(
     typename Vec2<R>::T* __restrict__ te, const typename Vec2<R>::T* __restrict__ to,
@@ -406,7 +416,7 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_hop_sp
     publish_iteration(partial + (size_t)3 * n, n, cgd, hist, iter_out, maxiter);
     return;
   }
-  if (cgd->done) return;
+  if (cgd->stop) return;
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
   Cx<R> row[3];
   hops_split<0, R, NC, R>(row, sh, FieldSrc<R, R>{to}, U, g, i, 0, g.Vh);
@@ -473,6 +483,7 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_fold_s
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
   if (cgd->done) {
     // as in cg_fold_kernel: the host has taken r2, p2 as the current buffers
+    if (DEFER && blockIdx.x == 0 && threadIdx.x == 0) cgd->stop = 1;
     if (i < g.Vh) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -783,7 +794,7 @@ __global__ void cg_init_h16_kernel(const double* __restrict__ part, int nparts, 
     cgd->sigma2 = s2;
     cgd->rho = 1.0;
     cgd->rr[0] = cgd->rr[1] = bb / s2;
-    cgd->done = bb == 0.0 ? 1 : 0;
+    set_done(cgd, bb == 0.0);
     cgd->iter = 0;
     cgd->pending = 0;
     cgd->restart = 0;
@@ -871,7 +882,7 @@ __global__ void ru_publish_h16_kernel(const double* __restrict__ part, int npart
     cgd->inv_hi = inv.hi;
     cgd->inv_lo = inv.lo;
     cgd->rr[cgd->iter & 1] = rr / s2;
-    cgd->done = rr <= cgd->tol2bb ? 1 : 0;
+    set_done(cgd, rr <= cgd->tol2bb);
     *true_rr = rr;
   }
 }
@@ -921,7 +932,7 @@ __global__ void ru_publish_kernel(const double* __restrict__ part, int n, CgDev*
     cgd->rr[cgd->iter & 1] = rr;
     // only the certifying update ends the solve; after an intermediate one
     // the next iteration publishes the residual, which the host watches
-    cgd->done = (final && rr <= cgd->tol2bb) ? 1 : 0;
+    set_done(cgd, final && rr <= cgd->tol2bb);
     *true_rr = rr;
   }
 }
@@ -943,7 +954,7 @@ __global__ void cg_init_kernel(const double* __restrict__ part, int n, CgDev* __
     cgd->bb = bb;
     cgd->tol2bb = tol2 * bb;
     cgd->rr[0] = cgd->rr[1] = bb;
-    cgd->done = bb == 0.0 ? 1 : 0;
+    set_done(cgd, bb == 0.0);
     cgd->iter = 0;
     cgd->pending = 0;
     cgd->restart = 0;
@@ -962,7 +973,7 @@ __global__ void cg_init_guess_kernel(const double* __restrict__ part_b, const do
     cgd->bb = bb;
     cgd->tol2bb = tol2 * bb;
     cgd->rr[0] = cgd->rr[1] = rr;
-    cgd->done = (bb == 0.0 || rr <= tol2 * bb) ? 1 : 0;
+    set_done(cgd, bb == 0.0 || rr <= tol2 * bb);
     cgd->iter = 0;
     cgd->pending = 0;
     cgd->restart = 0;

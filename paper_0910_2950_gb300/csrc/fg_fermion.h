@@ -19,6 +19,10 @@ struct CgDev {
   double tol2bb;
   double alpha;
   int done;
+  // folded iteration with deferred totals: done, one launch late.  B's extra
+  // block sets done while B's other blocks run, so those look at stop, which
+  // only launches other than B write.
+  int stop;
   int iter;     // last completed iteration
   int restart;  // set by a reliable update whose true residual left the recursion far behind
   double pap;       // <p, Ap> of the iteration in progress
