@@ -102,7 +102,7 @@ class Backend final : public IBackend {
     if (s != FG_OK) return s;
     sf0_valid_ = false;
     sgc_valid_ = false;
-    return sync();
+    return check_links();
   }
   fg_status get_gauge(double* host) override {
     const size_t n = (size_t)4 * g_.V * 18;
@@ -304,7 +304,7 @@ class Backend final : public IBackend {
     if (s != FG_OK) return s;
     sf0_valid_ = false;
     sgc_valid_ = false;
-    return sync();
+    return check_links();
   }
 
   fg_status random_gauge() override {
@@ -313,7 +313,7 @@ class Backend final : public IBackend {
     if (s != FG_OK) return s;
     sf0_valid_ = false;
     sgc_valid_ = false;
-    return sync();
+    return check_links();
   }
   fg_status set_rng_position(unsigned long long pos) override {
     draw_ = (uint32_t)pos;
@@ -329,7 +329,7 @@ class Backend final : public IBackend {
     if (s != FG_OK) return s;
     sf0_valid_ = false;
     sgc_valid_ = false;
-    return sync();
+    return check_links();
   }
 
   fg_status trajectory(int integ, double dt, int nsteps, int refresh, double u_accept,
@@ -379,9 +379,11 @@ class Backend final : public IBackend {
     sf0_valid_ = false;
     if ((s = execute(ops, dt, start)) != FG_OK) return s;
     if ((s = energy(1, P_, 3, nullptr, sgc_[1 - sgc_cur_])) != FG_OK) return s;
-    if ((s = fetch(6)) != FG_OK) return s;
+    if ((s = queue_unitarity()) != FG_OK) return s;
+    if ((s = fetch(7)) != FG_OK) return s;
     double o[6];
     std::memcpy(o, host_out_, sizeof(o));
+    const bool unitary1 = read_unitarity();
     double sf1 = 0.0;
     if (ferm_ && (s = fermion_action(U_, &sf1)) != FG_OK) return s;
     r->S_gauge0 = o[0];
@@ -402,6 +404,7 @@ class Backend final : public IBackend {
     // the stored per-site gauge action follows the links kept
     if (r->accepted) sgc_cur_ = 1 - sgc_cur_;
     sgc_valid_ = true;
+    if (r->accepted) unitary_ = unitary1;
     if (!r->accepted) {
       U_ = start;
       sf0_ = sf0;             // phi unchanged and the links are back: S_F is S_F0 again
@@ -431,6 +434,12 @@ class Backend final : public IBackend {
   void* F_ = nullptr;
   ForceRows rows_{};
   void* W_ = nullptr;   // plaquette field of the force evaluation in progress
+  // Whether the current links are unitary to R, which the plaquette form of
+  // the force needs (kUnitaryWithin): measured whenever links enter and after
+  // every trajectory and step, so that the form depends on the links alone
+  // and a chain goes on from a stored configuration with the same bits.
+  bool unitary_ = true;
+  bool flag_set_ = false;   // the device's flag (dout_ + 6) is up
   double* h0_ = nullptr;
   // per-site gauge action of the current links (sgc_[sgc_cur_]) and of the
   // end of the running trajectory (the other one); valid while only
@@ -545,10 +554,38 @@ class Backend final : public IBackend {
   int solves_ = 0;
   long long cg_iters_ = 0;
 
-  // Lattice description of the plaquette-form force launches.
+  // Queues the measurement of the current links' unitarity into dout_ + 6.
+  fg_status queue_unitarity() {
+    if constexpr (kPlaquetteForce<R>) {
+      if (flag_set_ && cudaMemsetAsync(dout_ + 6, 0, sizeof(double), st_) != cudaSuccess) return cuda_fail("memset");
+      flag_set_ = false;
+      return run(KC_REDUCE, [&] { return launch_unitarity<R, NC>(rows_, U_, dout_ + 6, 1, st_); });
+    } else {
+      return FG_OK;
+    }
+  }
+  // Its result, after fetch(7).
+  bool read_unitarity() {
+    flag_set_ = host_out_[6] != 0.0;
+    return !flag_set_;
+  }
+  // New links have entered: measure them and wait.
+  fg_status check_links() {
+    if constexpr (kPlaquetteForce<R>) {
+      fg_status s = queue_unitarity();
+      if (s != FG_OK) return s;
+      if ((s = fetch(7)) != FG_OK) return s;
+      unitary_ = read_unitarity();
+      return FG_OK;
+    } else {
+      return sync();
+    }
+  }
+
+  // Lattice description of the FP64 and double-float force launches.
   fg_status init_force_rows() {
     std::vector<char> cd(chain_bytes());
-    fill_chain(cd.data(), g_, h_->prm.beta, 0, 0, 0, 0, 0);
+    fill_chain(cd.data(), g_, h_->prm.beta, 0, 0, 0, 0);
     void* chain;
     fg_status s;
     if ((s = alloc(&chain, cd.size())) != FG_OK) return s;
@@ -641,7 +678,7 @@ class Backend final : public IBackend {
     ForceArgs a;
     std::memset(&a, 0, sizeof(a));
     a.U = Uf;
-    a.W = W_;
+    a.W = unitary_ ? W_ : nullptr;
     a.P = P_;
     a.Ubase = Uf;
     a.beta = h_->prm.beta;
@@ -673,8 +710,10 @@ class Backend final : public IBackend {
   }();
   fg_status gauge_launch(int mode, const ForceArgs& a) {
     if constexpr (kPlaquetteForce<R>) {
-      const fg_status w = run(KC_PLAQUETTE, [&] { return launch_plaquettes<R, NC>(rows_, a.U, W_, st_); });
-      if (w != FG_OK) return w;
+      if (a.W != nullptr) {
+        const fg_status w = run(KC_PLAQUETTE, [&] { return launch_plaquettes<R, NC>(rows_, a.U, W_, st_); });
+        if (w != FG_OK) return w;
+      }
     }
     if (split_exp_ && (mode == FM_KICK_DRIFT || mode == FM_DISPLACE)) {
       ForceArgs f = a;

@@ -42,6 +42,7 @@ struct Tile {
 
 // Per-chain results, FP64: S_G and T at start and end, dH, accepted.
 constexpr int kChainOut = 8;
+constexpr int kOutOffUnitary = 7;   // result slot: links off unitarity at the end
 
 // Site of thread threadIdx.x in tile t (H half-sites, both parities).
 template <int H>
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
     } else {
       int c[4], par;
       cb_coords(g, s, c, par);
-      force_link_staples<NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, cd.beta6_hi, ckick, cdrift, cdisp,
+      force_link_staples<float, NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, cd.beta6_hi, ckick, cdrift, cdisp,
                                    reunit, 1.0f);
     }
   }
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(256) batch_chain_reduce_kernel(const ChainDesc
                                                                  double* __restrict__ out, int off) {
   const ChainDesc& cd = chains[blockIdx.x];
   __shared__ double sh[8];
+  if (threadIdx.x == 0 && off == 0) out[(size_t)blockIdx.x * kChainOut + kOutOffUnitary] = 0.0;
   for (int k = 0; k < 3; ++k) {
     double x = 0.0;
     for (int i = threadIdx.x; i < cd.ntiles; i += blockDim.x) x += partial[(size_t)k * ntiles + cd.tile0 + i];
@@ -321,13 +323,11 @@ class Batch final : public IBatch {
     }
     const int n = b_->prm.nchains;
     std::vector<ChainDesc> cds(n);
-    std::vector<int> row_chain;
     long long goff = 0, moff = 0, woff = 0, soff = 0;
     for (int c = 0; c < n; ++c) {
       ChainDesc& cd = cds[c];
       const GeomH gh = geom_of(&b_->dims[4 * c]);
-      fill_chain(&cd, gh, b_->beta[c], goff, moff, woff, soff, (int)row_chain.size());
-      row_chain.insert(row_chain.end(), (gh.Vh + 31) / 32, c);
+      fill_chain(&cd, gh, b_->beta[c], goff, moff, woff, soff);
       goff += align256((long long)4 * NC * cd.g.V * sizeof(C2));
       moff += align256((long long)4 * 4 * cd.g.V * sizeof(C2));
       woff += align256((long long)6 * 4 * cd.g.V * sizeof(C2));
@@ -376,7 +376,8 @@ class Batch final : public IBatch {
         return cuda_fail("descriptor upload");
       if ((s = alloc((void**)&d_partial_[hi], (size_t)3 * tl.size() * sizeof(double))) != FG_OK) return s;
     }
-    if (kPlaquetteForce<R> && (s = init_force_rows(row_chain)) != FG_OK) return s;
+    unitary_.assign(n, 1);
+    if (kPlaquetteForce<R> && (s = init_force_rows()) != FG_OK) return s;
     if (b_->prm.tile == 16) hsel_ = 0;
     else if (b_->prm.tile == 32) hsel_ = 1;
     else if (b_->prm.tile == 64) hsel_ = 2;
@@ -406,7 +407,7 @@ class Batch final : public IBatch {
     if ((s = lrun([&] { return launch_gauge_to_device<R, NC>(gh, canon_, (char*)buf_[cur_] + cds_[c].goff, st_); })) !=
         FG_OK)
       return s;
-    return sync();
+    return check_links(c);
   }
   fg_status get_gauge(int c, double* host) override {
     const size_t n = (size_t)4 * cds_[c].g.V * 18;
@@ -488,6 +489,19 @@ class Batch final : public IBatch {
     }
     if ((s = sync()) != FG_OK) return s;
     cur_ = final_buf;
+    if (kPlaquetteForce<R>) {
+      // a rejected chain is back at links that were measured before
+      bool changed = false;
+      for (int c = 0; c < b_->prm.nchains; ++c) {
+        const double* o = host_out_ + (size_t)c * kChainOut;
+        const char u = o[kOutOffUnitary] == 0.0;
+        if (o[6] != 0.0 && u != unitary_[c]) {
+          unitary_[c] = u;
+          changed = true;
+        }
+      }
+      if (changed && (s = upload_rows()) != FG_OK) return s;
+    }
     if (out) {
       const int n = b_->prm.nchains;
       const int nforce = count_forces(ops);
@@ -529,7 +543,12 @@ class Batch final : public IBatch {
   void* P_ = nullptr;
   void* F_ = nullptr;
   void* W_ = nullptr;     // plaquette field of the force evaluation in progress
-  ForceRows rows_{};
+  // Rows of all chains: first those of the chains whose links are unitary to
+  // R, which take the plaquette form of the force, then the others', which
+  // take the staple sums (as Backend::unitary_, chain by chain).
+  int2* d_rows_ = nullptr;
+  int nrows_ = 0, nplaq_ = 0;
+  std::vector<char> unitary_;
   double* h0_ = nullptr;
   ChainDesc* d_chains_h_[3] = {nullptr, nullptr, nullptr};
   Tile* d_tiles_[3] = {nullptr, nullptr, nullptr};
@@ -545,16 +564,47 @@ class Batch final : public IBatch {
   int sms_ = 152;
   std::vector<GraphEntry> graphs_;
 
-  // The rows of all chains for the plaquette-form force launches.
-  fg_status init_force_rows(const std::vector<int>& row_chain) {
-    int* rc;
-    fg_status s;
-    const size_t bytes = row_chain.size() * sizeof(int);
-    if ((s = alloc((void**)&rc, bytes)) != FG_OK) return s;
-    if (cudaMemcpyAsync(rc, row_chain.data(), bytes, cudaMemcpyHostToDevice, st_) != cudaSuccess)
+  fg_status init_force_rows() {
+    nrows_ = 0;
+    for (const ChainDesc& cd : cds_) nrows_ += (cd.g.Vh + 31) / 32;
+    const fg_status s = alloc((void**)&d_rows_, (size_t)nrows_ * sizeof(int2));
+    return s != FG_OK ? s : upload_rows();
+  }
+  // The row list by unitary_.  The captured trajectories hold the counts.
+  fg_status upload_rows() {
+    std::vector<int2> rows;
+    for (int pass = 1; pass >= 0; --pass) {
+      for (int c = 0; c < (int)cds_.size(); ++c)
+        if (unitary_[c] == pass)
+          for (int i = 0; i < cds_[c].g.Vh; i += 32) rows.push_back(make_int2(c, i));
+      if (pass) nplaq_ = (int)rows.size();
+    }
+    for (auto& g : graphs_) cudaGraphExecDestroy(g.exec);
+    graphs_.clear();
+    if (cudaMemcpyAsync(d_rows_, rows.data(), rows.size() * sizeof(int2), cudaMemcpyHostToDevice, st_) != cudaSuccess)
       return cuda_fail("row list upload");
-    rows_ = ForceRows{d_chains_h_[0], rc, (int)row_chain.size()};
     return sync();  // the host copy goes out of scope
+  }
+  ForceRows rows_of(int first, int n) const { return ForceRows{d_chains_h_[0], d_rows_ + first, n}; }
+  // New links of chain c have entered: measure them and wait.
+  fg_status check_links(int c) {
+    if constexpr (kPlaquetteForce<R>) {
+      double* const flag = d_out_ + (size_t)c * kChainOut + kOutOffUnitary;
+      double off = 0.0;
+      const ForceRows one{d_chains_h_[0] + c, nullptr, (cds_[c].g.Vh + 31) / 32};
+      if (cudaMemsetAsync(flag, 0, sizeof(double), st_) != cudaSuccess) return cuda_fail("memset");
+      fg_status s = lrun([&] { return launch_unitarity<R, NC>(one, buf_[cur_], flag, 0, st_); });
+      if (s != FG_OK) return s;
+      if (cudaMemcpyAsync(&off, flag, sizeof(double), cudaMemcpyDeviceToHost, st_) != cudaSuccess)
+        return cuda_fail("unitarity download");
+      if ((s = sync()) != FG_OK) return s;
+      const char u = off == 0.0;
+      if (u == unitary_[c]) return FG_OK;
+      unitary_[c] = u;
+      return upload_rows();
+    } else {
+      return sync();
+    }
   }
 
   static long long align256(long long x) { return (x + 255) & ~255LL; }
@@ -636,9 +686,17 @@ class Batch final : public IBatch {
     a.ckick = ckick; a.cdrift = cdrift; a.cdisp = cdisp;
     a.reunit = b_->prm.reunitarize;
     if constexpr (kPlaquetteForce<R>) {
-      const fg_status s = lrun([&] { return launch_plaquettes<R, NC>(rows_, U, W_, st_); });
-      if (s != FG_OK) return s;
-      return lrun([&] { return launch_gauge_force<R, NC>(geomh(0), rows_, mode, a, st_); });
+      const ForceRows plaq = rows_of(0, nplaq_), rest = rows_of(nplaq_, nrows_ - nplaq_);
+      fg_status s = FG_OK;
+      if (plaq.nrows > 0) {
+        if ((s = lrun([&] { return launch_plaquettes<R, NC>(plaq, U, W_, st_); })) != FG_OK) return s;
+        if ((s = lrun([&] { return launch_gauge_force<R, NC>(geomh(0), plaq, mode, a, st_); })) != FG_OK) return s;
+      }
+      if (rest.nrows > 0) {
+        a.W = nullptr;
+        s = lrun([&] { return launch_gauge_force<R, NC>(geomh(0), rest, mode, a, st_); });
+      }
+      return s;
     } else {
       switch (hsel_) {
         case 0: return staples_h<16>(0, mode, a);
@@ -795,6 +853,12 @@ class Batch final : public IBatch {
     }
     if ((s = misc(1, buf_[cur], 1)) != FG_OK) return s;
     if ((s = misc(2, nullptr, 0, 0, 0, nullptr, nullptr, 3)) != FG_OK) return s;
+    if constexpr (kPlaquetteForce<R>) {
+      if ((s = lrun([&] {
+             return launch_unitarity<R, NC>(rows_of(0, nrows_), buf_[cur], d_out_ + kOutOffUnitary, kChainOut, st_);
+           })) != FG_OK)
+        return s;
+    }
     if ((s = misc(3, nullptr, 0, 0, accept_mode)) != FG_OK) return s;
     if (cur != start && (s = misc(4, nullptr, 0, 0, 0, buf_[start], buf_[cur])) != FG_OK) return s;
     if ((s = misc(5, nullptr, 0, refresh)) != FG_OK) return s;

@@ -25,7 +25,7 @@ enum ForceMode {
 
 struct ForceArgs {
   const void* U;       // links at which the force is evaluated
-  const void* W;       // their plaquette field (launch_plaquettes; unused in FP32)
+  const void* W;       // their plaquette field (launch_plaquettes), or null for the staple sums (FP32: unused)
   void* P;             // momenta
   void* F;             // force out (FM_STORE)
   const void* FF;      // extra force added to the gauge force (fermions) or nullptr
@@ -37,26 +37,31 @@ struct ForceArgs {
   int reunit;
 };
 
-// Whether the force of links in precision R is formed by plaquettes (two
-// launches) or by staples (one).
+// Whether the force of links in precision R can be formed by plaquettes (two
+// launches), or always by staples (one).
 template <typename R>
 constexpr bool kPlaquetteForce = !std::is_same<R, float>::value;
 
-// The lattices of a plaquette-form launch, cut into rows of 32 half-sites.
+// The lattices of an FP64 or double-float force launch, cut into rows of 32
+// half-sites.
 struct ForceRows {
   const void* chains;     // device array of lattice descriptions (fill_chain)
-  const int* row_chain;   // lattice of each row, or null for one lattice
+  const int2* rows;       // lattice and first half-site of each row, or null for all rows of one lattice
   int nrows;
 };
 void fill_chain(void* dst, const GeomH& g, double beta, long long goff, long long moff, long long woff,
-                long long soff, int row0);
+                long long soff);
 size_t chain_bytes();
 
 // The plaquette field of links U into W (6 x 8 reals a site), which the force
 // launch that follows reads.
 template <typename R, int NC>
 cudaError_t launch_plaquettes(const ForceRows& rows, const void* U, void* W, cudaStream_t st);
-// `rows` is used in the plaquette form, `g` otherwise.
+// flag[stride * lattice] = 1.0 for every lattice of `rows` with links too far
+// from unitary for the plaquette form (untouched otherwise).
+template <typename R, int NC>
+cudaError_t launch_unitarity(const ForceRows& rows, const void* U, double* flag, int stride, cudaStream_t st);
+// `rows` is used in FP64 and double-float, `g` in FP32.
 template <typename R, int NC>
 cudaError_t launch_gauge_force(const GeomH& g, const ForceRows& rows, int mode, const ForceArgs& a, cudaStream_t st);
 

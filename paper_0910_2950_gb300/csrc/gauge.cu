@@ -1,7 +1,8 @@
 // Pure-gauge kernels of the force-gradient HMC step (sm_103a).
 //
 //  * staple_force_kernel (FP32), plaquette_kernel and link_force_kernel
-//    (double-float and FP64): Wilson force F^a = (beta/6) Im Tr(lambda^a U A), A the sum of the
+//    (double-float and FP64; staple_rows_kernel where unitarity_kernel finds
+//    the links off unitarity): Wilson force F^a = (beta/6) Im Tr(lambda^a U A), A the sum of the
 //    link's staples (the S-hat vector field of section 3), fused with what
 //    the integrator does next on the same link: store it, kick the momentum,
 //    kick then drift the link, or displace the link along the force for the
@@ -64,12 +65,12 @@ __global__ void __launch_bounds__(4 * kStapleSites, kStapleMinBlocks<NC>)
     if (!ok) return;
     int c[4], par;
     cb_coords(g, s, c, par);
-    force_link_staples<NC, MODE>(U, P, F, FF, Ubase, Uout, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
+    force_link_staples<float, NC, MODE>(U, P, F, FF, Ubase, Uout, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
                                  reunit, ffw);
   }
 }
 
-// The plaquette form walks the lattices of a launch by warps (rows of 32
+// The double-float and FP64 launches walk their lattices by warps (rows of 32
 // consecutive half-sites of one parity): warp w takes part w % parts (a plane
 // or a direction) of row w / parts; all parts and both parities of the same
 // half-sites are in consecutive warps and share the links in L1.
@@ -81,14 +82,16 @@ __device__ __forceinline__ bool row_site(const ForceRows& r, int parts, RowSite&
   const unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const unsigned q = w / (unsigned)parts;
   o.part = (int)(w - q * (unsigned)parts);
-  int row = (int)(q >> 1);
+  const int row = (int)(q >> 1);
   if (row >= r.nrows) return false;
   const ChainDesc* cd = (const ChainDesc*)r.chains;
-  if (r.row_chain != nullptr) {
-    cd += r.row_chain[row];
-    row -= cd->row0;
+  int i = row * 32;
+  if (r.rows != nullptr) {
+    const int2 at = r.rows[row];
+    cd += at.x;
+    i = at.y;
   }
-  const int i = row * 32 + (int)(threadIdx.x & 31);
+  i += (int)(threadIdx.x & 31);
   if (i >= cd->g.Vh) return false;
   o.cd = cd;
   o.s = (int)(q & 1) * cd->g.Vh + i;
@@ -131,6 +134,47 @@ __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
   ff.p = FF == nullptr ? nullptr : FF + cd.moff; ff.V = g.V;
   force_link_plaquettes<R, NC, MODE>(u, w, p, f, ff, ub, uo, g, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, cdisp,
                                      reunit, ffw);
+}
+
+// The same from the staple sums (links that are not unitary to R).
+template <typename R, int NC, int MODE>
+__global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
+    staple_rows_kernel(const __grid_constant__ ForceRows r, char* U, char* P, char* F, char* FF, char* Ubase,
+                       char* Uout, R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+  RowSite o;
+  if (!row_site(r, 4, o)) return;
+  const ChainDesc& cd = *o.cd;
+  const Geom g = cd.g;
+  Gauge<R, NC> u, ub, uo;
+  u.p = U + cd.goff; u.V = g.V;
+  ub.p = Ubase + cd.goff; ub.V = g.V;
+  uo.p = Uout + cd.goff; uo.V = g.V;
+  Mom<R> p, f, ff;
+  p.p = P + cd.moff; p.V = g.V;
+  f.p = F + cd.moff; f.V = g.V;
+  ff.p = FF == nullptr ? nullptr : FF + cd.moff; ff.V = g.V;
+  int c[4], par;
+  cb_coords(g, o.s, c, par);
+  force_link_staples<R, NC, MODE>(u, p, f, ff, ub, uo, g, c, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, cdisp, reunit,
+                                  ffw);
+}
+
+// flag[stride * lattice] = 1 where a link of the lattice is off unitarity by
+// more than `most`.
+template <typename R, int NC>
+__global__ void __launch_bounds__(kForceThreads)
+    unitarity_kernel(const __grid_constant__ ForceRows r, char* U, R most, double* __restrict__ flag, int stride) {
+  RowSite o;
+  const bool in = row_site(r, 4, o);
+  bool off = false;
+  if (in) {
+    Gauge<R, NC> u;
+    u.p = U + o.cd->goff; u.V = o.cd->g.V;
+    off = off_unitary(u.load(o.part, o.s), most);
+  }
+  // lane 0 of a row is always one of its sites; one writer a warp
+  if (__any_sync(0xffffffffu, off) && (threadIdx.x & 31) == 0)
+    atomicExch((unsigned long long*)(flag + stride * (o.cd - (const ChainDesc*)r.chains)), 0x3ff0000000000000ull);  // 1.0
 }
 
 // One thread a link: warp w takes direction w mod 4 of 32 consecutive sites.
@@ -417,7 +461,7 @@ static cudaError_t launch_staple_force(const GeomH& gh, int mode, const ForceArg
 }
 
 void fill_chain(void* dst, const GeomH& gh, double beta, long long goff, long long moff, long long woff,
-                long long soff, int row0) {
+                long long soff) {
   ChainDesc* cd = (ChainDesc*)dst;
   cd->g = to_dev(gh);
   cd->goff = goff; cd->moff = moff; cd->woff = woff; cd->soff = soff;
@@ -425,7 +469,6 @@ void fill_chain(void* dst, const GeomH& gh, double beta, long long goff, long lo
   cd->beta6 = beta / 6.0;
   cd->beta6_hi = (float)cd->beta6;
   cd->beta6_lo = (float)(cd->beta6 - (double)cd->beta6_hi);
-  cd->row0 = row0;
   cd->tile0 = cd->ntiles = 0;
 }
 size_t chain_bytes() { return sizeof(ChainDesc); }
@@ -439,15 +482,31 @@ cudaError_t launch_plaquettes(const ForceRows& r, const void* U, void* W, cudaSt
 }
 
 template <typename R, int NC>
+cudaError_t launch_unitarity(const ForceRows& r, const void* U, double* flag, int stride, cudaStream_t st) {
+  const long long warps = 8LL * r.nrows;
+  const int w = warps_per_block(warps, kForceThreads / 32);
+  unitarity_kernel<R, NC><<<(unsigned)((warps + w - 1) / w), 32 * w, 0, st>>>(r, (char*)U, R(kUnitaryWithin<R>), flag,
+                                                                             stride);
+  return cudaGetLastError();
+}
+
+template <typename R, int NC>
 static cudaError_t launch_link_force(const ForceRows& r, int mode, const ForceArgs& a, cudaStream_t st) {
   const R ffw = R(a.ffw == 0.0 ? 1.0 : a.ffw);
   const long long warps = 8LL * r.nrows;
   const int w = warps_per_block(warps, kForceThreads / 32);
   const unsigned nb = (unsigned)((warps + w - 1) / w);
-#define FG_FORCE(M)                                                                                                 \
-  link_force_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.W, (char*)a.P, (char*)a.F, (char*)a.FF, \
-                                                     (char*)a.Ubase, (char*)a.Uout, R(a.ckick), R(a.cdrift),         \
-                                                     R(a.cdisp), a.reunit, ffw)
+#define FG_FORCE(M)                                                                                                   \
+  do {                                                                                                                \
+    if (a.W != nullptr)                                                                                               \
+      link_force_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.W, (char*)a.P, (char*)a.F, (char*)a.FF, \
+                                                         (char*)a.Ubase, (char*)a.Uout, R(a.ckick), R(a.cdrift),      \
+                                                         R(a.cdisp), a.reunit, ffw);                                  \
+    else                                                                                                              \
+      staple_rows_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.P, (char*)a.F, (char*)a.FF,         \
+                                                          (char*)a.Ubase, (char*)a.Uout, R(a.ckick), R(a.cdrift),     \
+                                                          R(a.cdisp), a.reunit, ffw);                                 \
+  } while (0)
   switch (mode) {
     case FM_STORE: FG_FORCE(FM_STORE); break;
     case FM_KICK: FG_FORCE(FM_KICK); break;
@@ -575,6 +634,10 @@ template cudaError_t launch_kick_ff<double>(const GeomH&, void*, const void*, do
 template cudaError_t launch_kick_ff<float>(const GeomH&, void*, const void*, double, cudaStream_t);
 template cudaError_t launch_kick_ff<DF>(const GeomH&, void*, const void*, double, cudaStream_t);
 
+template cudaError_t launch_unitarity<double, 9>(const ForceRows&, const void*, double*, int, cudaStream_t);
+template cudaError_t launch_unitarity<double, 6>(const ForceRows&, const void*, double*, int, cudaStream_t);
+template cudaError_t launch_unitarity<DF, 9>(const ForceRows&, const void*, double*, int, cudaStream_t);
+template cudaError_t launch_unitarity<DF, 6>(const ForceRows&, const void*, double*, int, cudaStream_t);
 template cudaError_t launch_plaquettes<double, 9>(const ForceRows&, const void*, void*, cudaStream_t);
 template cudaError_t launch_plaquettes<double, 6>(const ForceRows&, const void*, void*, cudaStream_t);
 template cudaError_t launch_plaquettes<DF, 9>(const ForceRows&, const void*, void*, cudaStream_t);

@@ -105,8 +105,10 @@ __device__ __forceinline__ void force_apply(const Gauge<R, NC>& U, const Mom<R>&
 }
 
 // ---------------------------------------------------------------------------
-// The Wilson force by staples (FP32 links): one thread sums the six staples
-// of its link.
+// The Wilson force by staples: one thread sums the six staples of its link.
+// FP32 lattices take this form, and FP64 and double-float ones whose links are
+// not unitary to their precision (kUnitaryWithin below): the staple sum is the
+// derivative of the action for any link matrices.
 
 // Sum of the six staples that close a plaquette with U_mu(x).  Neighbour
 // indices are formed with selects, so mu and nu may be run-time values
@@ -133,31 +135,73 @@ __device__ __forceinline__ M3<R> staple_sum(const Gauge<R, NC>& U, const Geom& g
     const int nu = (mu + k) & 3;
     int dp, dm;
     cb_half_steps(g, c, nu, dp, dm);
-    {
-      // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-      const M3<R> t = mul_nd(U.load(nu, s_pmu), U.load(mu, other + dp));
-      mac_nd(a, t, U.load(nu, s));
-    }
-    {
-      // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) = (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)
-      const int s_mnu = other + dm;
-      const M3<R> t = mul(U.load(mu, s_mnu), U.load(nu, s + dm + dmu));
-      mac_dn(a, t, U.load(nu, s_mnu));
+    const int s_mnu = other + dm;
+    if constexpr (std::is_same<R, DF>::value) {
+      // Double-float: both staples of the plane as X Y^dag Z with run-time
+      // daggers,
+      //   upper  U_nu(x+mu)          U_mu(x+nu)^dag U_nu(x)^dag,
+      //   lower  U_nu(x+mu-nu)^dag   U_mu(x-nu)^dag U_nu(x-nu),
+      // their two products through one loop body (instruction cache), by the
+      // anchored products of df64.cuh: links off unitarity by 1e-7, as
+      // single precision leaves them, stay within the anchor's grid.
+#pragma unroll 1
+      for (int up = 1; up >= 0; --up) {
+        M3<DF> l = dagger_if(U.load(nu, up ? s_pmu : s + dm + dmu), !up);
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+          const int sr = q ? (up ? s : s_mnu) : (up ? other + dp : s_mnu);
+          l = su3_mul(l, dagger_if(U.load(q ? nu : mu, sr), q ? up != 0 : true));
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) a.e[i][j] = a.e[i][j] + l.e[i][j];
+      }
+    } else {
+      {
+        // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
+        const M3<R> t = mul_nd(U.load(nu, s_pmu), U.load(mu, other + dp));
+        mac_nd(a, t, U.load(nu, s));
+      }
+      {
+        // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) = (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)
+        const M3<R> t = mul(U.load(mu, s_mnu), U.load(nu, s + dm + dmu));
+        mac_dn(a, t, U.load(nu, s_mnu));
+      }
     }
   }
   return a;
 }
 
-template <int NC, int MODE>
-__device__ __forceinline__ void force_link_staples(const Gauge<float, NC>& U, const Mom<float>& P, const Mom<float>& F,
-                                                   const Mom<float>& FF, const Gauge<float, NC>& Ubase,
-                                                   const Gauge<float, NC>& Uout, const Geom& g, const int c[4], int s,
-                                                   int mu, float beta6, float ckick, float cdrift, float cdisp,
-                                                   int reunit, float ffw) {
-  const M3<float> a = staple_sum(U, g, c, s, mu);
-  float f[8];
-  im_tr_gellmann(mul(U.load(mu, s), a), f);
-  force_apply<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
+// f^a = Im Tr(lambda^a U A) for the staple sum a.
+template <typename R> __device__ __forceinline__ void staple_force(const M3<R>& u, const M3<R>& a, R f[8]) {
+  if constexpr (std::is_same<R, DF>::value) {
+    // a / 8 (exact) has columns of norm 3/4 at most: within the anchored
+    // products' bounds
+    M3<DF> a8;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        a8.e[i][j] = cx<DF>(DF(a.e[i][j].re.hi * 0.125f, a.e[i][j].re.lo * 0.125f),
+                            DF(a.e[i][j].im.hi * 0.125f, a.e[i][j].im.lo * 0.125f));
+    im_tr_gellmann(su3_mul(u, a8), f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] = f[k] * 8.0f;
+  } else {
+    im_tr_gellmann(mul(u, a), f);
+  }
+}
+
+template <typename R, int NC, int MODE>
+__device__ __forceinline__ void force_link_staples(const Gauge<R, NC>& U, const Mom<R>& P, const Mom<R>& F,
+                                                   const Mom<R>& FF, const Gauge<R, NC>& Ubase,
+                                                   const Gauge<R, NC>& Uout, const Geom& g, const int c[4], int s,
+                                                   int mu, R beta6, R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+  const M3<R> a = staple_sum(U, g, c, s, mu);
+  R f[8];
+  staple_force(U.load(mu, s), a, f);
+  force_apply<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
 }
 
 // Whether the FP32 12-real force kernels share the upper-staple products of
@@ -167,7 +211,7 @@ __device__ __forceinline__ void force_link_staples(const Gauge<float, NC>& U, co
 // 32^4.  With 18-real links the same change executed 8% fewer instructions
 // but ran 2% slower (426 vs 416 us; the slots take L1 capacity from the
 // neighbour loads and the barrier stalls), and the FP64 kernels would need
-// 55 KB of slots per block; those compute every staple in full.
+// 55 KB of slots per block.
 #ifndef FG_FORCE_SHARED_T
 #define FG_FORCE_SHARED_T 1
 #endif
@@ -271,7 +315,7 @@ __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok,
       }
   }
   float f[8];
-  im_tr_gellmann(mul(U.load(mu, s), a), f);
+  staple_force(U.load(mu, s), a, f);
   force_apply<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
 }
 
@@ -285,7 +329,8 @@ __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok,
 //     are W and W^dag);
 //   * U_mu(x+nu) takes -U_nu(x)^dag Q U_nu(x) and U_nu(x+mu) takes
 //     +U_mu(x)^dag Q U_mu(x) (the same closed path read from another corner;
-//     this step uses U^dag U = 1).
+//     this step uses U^dag U = 1: lattices whose links are not unitary to
+//     their precision take the staple sums, see kUnitaryWithin).
 // plaquette_kernel forms Q once for every site and plane (two products and
 // half of a third), link_force_kernel sums six of them for every link, three
 // of them rotated by one neighbour link (90 + 48 multiply-adds, H being
@@ -327,13 +372,63 @@ struct ChainDesc {
   long long soff;  // offset of its sites in per-site arrays
   double beta, beta6;          // beta, beta / 6
   float beta6_hi, beta6_lo;    // beta / 6 as a double-float: no FP64 arithmetic (1/64 of the FP32 rate) there
-  int row0;                    // first of its rows of 32 half-sites
   int tile0, ntiles;           // its tiles (batch.cu)
 };
 template <typename R> __device__ __forceinline__ R beta6_of(const ChainDesc& cd);
 template <> __device__ __forceinline__ double beta6_of<double>(const ChainDesc& cd) { return cd.beta6; }
 template <> __device__ __forceinline__ float beta6_of<float>(const ChainDesc& cd) { return cd.beta6_hi; }
 template <> __device__ __forceinline__ DF beta6_of<DF>(const ChainDesc& cd) { return DF(cd.beta6_hi, cd.beta6_lo); }
+
+// Largest entry of U U^dag - 1 with which a lattice takes the plaquette form.
+// A force by plaquettes is off by about the defect of its links (the staple
+// sums by none of it), and one FG trajectory's dH by some 20 times the
+// defect's mean size on 6^4, growing with the root of the volume: below the
+// lines, less than the rounding of the forces and sums puts into dH (FP64
+// 1e-12, double-float 1e-10 there).  Links held in single precision lie at
+// 1e-7, links made unitary in 64 bits at 1e-15, and a chain that is never
+// re-projected moves away from there with the root of its length: FP64 18-real
+// chains reach 7e-14 and double-float ones 1.8e-11 in 800 trajectories of 16
+// drifts.  12-real links, whose third row is rebuilt from rows that are not
+// quite orthonormal, leave unitarity far faster (1e-11 after 200), so the
+// defect is taken anew after every trajectory.
+template <typename R>
+constexpr double kUnitaryWithin = std::is_same<R, double>::value ? 0x1p-42 : 0x1p-35;
+
+// Whether an entry of U U^dag - 1 is larger than `most` (or not a number).
+// In double-float by anchored sums (df64.cuh; those of the diagonal start at
+// -1): general double-float FMAs took 38 us over a 16^4 lattice.
+template <typename R> __device__ __forceinline__ bool off_unitary(const M3<R>& u, R most) {
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j) {
+      R re = R(i == j ? -1 : 0), im = R(0);
+      if constexpr (std::is_same<R, DF>::value) {
+        Anchored x, y;
+        if (i == j) x.t = 2.0f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          x.add(u.e[i][k].re, u.e[j][k].re);
+          x.add(u.e[i][k].im, u.e[j][k].im);
+          if (i != j) {
+            y.add(u.e[i][k].im, u.e[j][k].re);
+            y.sub(u.e[i][k].re, u.e[j][k].im);
+          }
+        }
+        re = x.value();
+        im = y.value();
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          re = fma(u.e[i][k].re, u.e[j][k].re, fma(u.e[i][k].im, u.e[j][k].im, re));
+          if (i != j) im = fma(u.e[i][k].im, u.e[j][k].re, fma(-u.e[i][k].re, u.e[j][k].im, im));
+        }
+      }
+      ok = ok && fabs(re) < most && fabs(im) < most;
+    }
+  return !ok;
+}
 
 // Plane pl = 0..5 as directions mu < nu, and back.
 __device__ __forceinline__ void plane_dirs(int pl, int& mu, int& nu) {
