@@ -508,17 +508,16 @@ class Backend final : public IBackend {
   // rs_ and p_ always name the current ones
   void *rs2_ = nullptr, *p2_ = nullptr;
   // Folded CG iterations (four launches, vector updates inside the Dslash
-  // launches) or five (four Dslash, one vector update) for FP32 and FP64
-  // inner vectors.  The folded form forms p' at each of a site's eight
-  // neighbours, reading r, Ap and p per hop, to save a streaming vector pass
-  // and a launch.  While the solver's links and vectors fit in L2 the extra
-  // hop reads hit L2 and the saved launch counts (served 8^3 x 16 and
-  // 12^3 x 24 chains); beyond L2 they cost DRAM bandwidth (against six
-  // launches, axpy and xpay apart: FP32 25.7 against 17.9 ms at 20^3 x 40,
-  // 38.8 against 34.2 at 24^3 x 48; FP64 at 16^3 x 32 61.7 against 56.6; the
-  // fifth launch takes another 2% off the FP32 ones).
+  // launches) or six (four Dslash, the residual, x and the direction) for
+  // FP32 and FP64 inner vectors.  The folded form forms p' at each of a site's
+  // eight neighbours, reading r, Ap and p per hop, to save the streaming
+  // vector passes and two launches.  While the solver's links and vectors fit
+  // in L2 the extra hop reads hit L2 and the saved launches count (served
+  // 8^3 x 16 and 12^3 x 24 chains); beyond L2 they cost DRAM bandwidth (FP32
+  // 25.7 against 17.9 ms at 20^3 x 40, 38.8 against 34.2 at 24^3 x 48; FP64 at
+  // 16^3 x 32 61.7 against 56.6).
   // Default: folded when the fields fit in L2; FG_CG_FOLD=1 or 0 in the
-  // environment forces either form.  The 16-bit solvers always take five
+  // environment forces either form.  The 16-bit solvers always take six
   // launches.
   const bool fold_ = [this] {
     const char* e = std::getenv("FG_CG_FOLD");
@@ -1167,27 +1166,31 @@ class Backend final : public IBackend {
     return launch_dslash<R, NC, R>(g_, out, in, x, U, out_par, dag, mode, b, cgd, st_);
   }
 
-  // Launch D of an iteration, and the last one: the vector update of the
-  // five-launch form or A of the folded one, which swaps the current and
+  // Launch D of an iteration, and the last ones: the vector updates of the
+  // six-launch form or A of the folded one, which swaps the current and
   // other buffers of r and p.
   cudaError_t cg_apdot(const void* U) {
     if constexpr (kMixed || std::is_same<R, double>::value) {
       const double k2 = h_->prm.kappa * h_->prm.kappa;
       if constexpr (kMixed) {
         if (half_links_)
-          return launch_cg_apdot_h16<NC>(s16_, g_, ap_, to_, te_, p_, rs_, U, k2, part_pap_, cgd_, st_);
+          return launch_cg_apdot_h16<NC>(s16_, g_, ap_, to_, te_, p_, U, k2, part_pap_, cgd_, st_);
       }
       return launch_cg_apdot<R, NC>(g_, ap_, to_, te_, p_, rs_, U, k2, part_pap_, cgd_, st_, fold_);
     } else {
       return cudaErrorNotSupported;
     }
   }
-  cudaError_t cg_update() {
+  cudaError_t cg_residual() {
     double* const hist = mapped_->hist;
     int* const it = &mapped_->dev_iter;
     const int n = nvec(), most = h_->prm.cg_maxiter;
-    if (half_links_) return launch_cg_update_h16(s16_, xs_, rs_, p_, ap_, cgd_, part_rr_, hist, it, most, n, st_);
-    return launch_cg_update<R>(xs_, rs_, p_, ap_, cgd_, part_rr_, hist, it, most, n, st_);
+    if (half_links_) return launch_cg_residual_h16(s16_, rs_, ap_, cgd_, part_rr_, hist, it, most, n, st_);
+    return launch_cg_residual<R>(rs_, ap_, cgd_, part_rr_, hist, it, most, n, st_);
+  }
+  cudaError_t cg_direction() {
+    if (half_links_) return launch_cg_direction_h16(s16_, xs_, p_, rs_, cgd_, nvec(), st_);
+    return launch_cg_direction<R>(xs_, p_, rs_, cgd_, nvec(), st_);
   }
   cudaError_t fold_update(const void* U) {
     if constexpr (kMixed || std::is_same<R, double>::value) {
@@ -1221,12 +1224,11 @@ class Backend final : public IBackend {
     return run(KC_DSLASH, [&] { return inner_dslash(to_, p_, nullptr, U, 1, 0, 0, 1.0); });
   }
 
-  // One CG iteration in the inner precision R: 4 Dslash launches and a vector
-  // one, which all return at once after convergence (cgd_->done).  Raw launches,
+  // One CG iteration in the inner precision R: 4 Dslash launches and the vector
+  // ones, which all return at once after convergence (cgd_->done).  Raw launches,
   // usable inside stream capture.
   cudaError_t cg_iteration_raw(const void* U) {
     const double k2 = h_->prm.kappa * h_->prm.kappa;
-    const int n = nvec();
     cudaError_t e;
     if (fold_) {
       if ((e = fold_hop(U)) != cudaSuccess) return e;
@@ -1238,14 +1240,14 @@ class Backend final : public IBackend {
     if ((e = inner_dslash(te_, to_, p_, U, 0, 0, 1, -k2)) != cudaSuccess) return e;
     if ((e = inner_dslash(to_, te_, nullptr, U, 1, 1, 0, 1.0)) != cudaSuccess) return e;
     if ((e = cg_apdot(U)) != cudaSuccess) return e;
-    return cg_update();
+    if ((e = cg_residual()) != cudaSuccess) return e;
+    return cg_direction();
   }
 
   // The same through run(), so that per-kernel timing and launch counting see
   // each kernel (used when timing is on or a graph is not available).
   fg_status cg_iteration(const void* U) {
     const double k2 = h_->prm.kappa * h_->prm.kappa;
-    const int n = nvec();
     fg_status s;
     if (fold_) {
       if ((s = run(KC_DSLASH, [&] { return fold_hop(U); })) != FG_OK) return s;
@@ -1264,7 +1266,8 @@ class Backend final : public IBackend {
         FG_OK)
       return s;
     if ((s = run(KC_DSLASH, [&] { return cg_apdot(U); })) != FG_OK) return s;
-    return run(KC_CG_BLAS, [&] { return cg_update(); });
+    if ((s = run(KC_CG_BLAS, [&] { return cg_residual(); })) != FG_OK) return s;
+    return run(KC_CG_BLAS, [&] { return cg_direction(); });
   }
 
   // A CUDA graph of n iterations (n = 2, 4 or 8) on links U, captured on first
@@ -1325,7 +1328,7 @@ class Backend final : public IBackend {
       if (g != nullptr) {
         if (cudaGraphLaunch(g, st_) != cudaSuccess) return cuda_fail("cg graph launch");
         // an even number of folded iterations leaves rs_ and p_ where they were
-        h_->launches += (fold_ ? 4 : 5) * n + (fold_deferred() ? 1 : 0);
+        h_->launches += (fold_ ? 4 : 6) * n + (fold_deferred() ? 1 : 0);
         return FG_OK;
       }
     }

@@ -190,12 +190,19 @@ __device__ __forceinline__ void alpha_beta(double rr, const double tot[3], doubl
   const double rrn = rr - 2.0 * alpha * tot[1] + alpha * alpha * tot[2];
   beta = (rr > 0.0 && rrn > 0.0) ? rrn / rr : 0.0;
 }
-__device__ __forceinline__ void set_alpha_beta(CgDev* cgd, const double tot[3]) {
-  double alpha, beta;
-  alpha_beta(cgd->rr[cgd->iter & 1], tot, alpha, beta);
+// What D's totals settle: alpha and beta from the three sums (folded
+// iteration), alpha alone from <p, Ap>.
+template <int NV> __device__ __forceinline__ void set_scalars(CgDev* cgd, const double tot[NV]) {
+  const double rr = cgd->rr[cgd->iter & 1];
   cgd->pap = tot[0];
-  cgd->alpha = alpha;
-  cgd->beta = beta;
+  if constexpr (NV == 3) {
+    double alpha, beta;
+    alpha_beta(rr, tot, alpha, beta);
+    cgd->alpha = alpha;
+    cgd->beta = beta;
+  } else {
+    cgd->alpha = tot[0] > 0.0 ? rr / tot[0] : 0.0;
+  }
 }
 // |r|^2 of the iteration just done: rr, the history, the count (also to the
 // host), done.
@@ -215,8 +222,9 @@ __device__ __forceinline__ void set_done(CgDev* cgd, bool d) {
   cgd->done = cgd->stop = d ? 1 : 0;
 }
 
-// D: Ap = te + b D^dagger_eo to at the even sites, with the three dot products.
-template <typename RL, int NC, typename R, typename ST = R>
+// D: Ap = te + b D^dagger_eo to at the even sites, with the dot products
+// <p, Ap> and, for NV = 3, Re <r, Ap> and |Ap|^2.
+template <int NV, typename RL, int NC, typename R, typename ST = R>
 __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_apdot_kernel(
     typename Vec2<ST>::T* __restrict__ ap, const typename Vec2<ST>::T* __restrict__ to,
     const typename Vec2<ST>::T* __restrict__ te, const typename Vec2<ST>::T* __restrict__ p,
@@ -224,7 +232,9 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     CgDev* __restrict__ cgd) {
   if (cgd->done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  R pa = R(0), ra = R(0), aa = R(0);  // one site's 24 terms each, in R
+  R v[NV];  // one site's 24 terms each, in R
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = R(0);
   Spinor<R> o;
   if (i < g.Vh) {
     int c[4], par;
@@ -237,20 +247,22 @@ __global__ void __launch_bounds__(kDslashThreads, DslashMinBlocks<R>::value) cg_
     hops_src<1, RL, NC, R>(acc, FieldSrc<R, ST>{to}, U, g, c, i, g.Vh);
     const Spinor<R> tv = load_spinor<R, ST>(te, i, g.Vh);
     const Spinor<R> pv = load_spinor<R, ST>(p, i, g.Vh);
-    const Spinor<R> rv = load_spinor<R, ST>(r, i, g.Vh);
+    Spinor<R> rv;
+    if constexpr (NV == 3) rv = load_spinor<R, ST>(r, i, g.Vh);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
       for (int cc = 0; cc < 3; ++cc) {
         o.s[k][cc] = tv.s[k][cc] + b * acc.s[k][cc];
-        pa += pv.s[k][cc].re * o.s[k][cc].re + pv.s[k][cc].im * o.s[k][cc].im;
-        ra += rv.s[k][cc].re * o.s[k][cc].re + rv.s[k][cc].im * o.s[k][cc].im;
-        aa += o.s[k][cc].re * o.s[k][cc].re + o.s[k][cc].im * o.s[k][cc].im;
+        v[0] += pv.s[k][cc].re * o.s[k][cc].re + pv.s[k][cc].im * o.s[k][cc].im;
+        if constexpr (NV == 3) {
+          v[1] += rv.s[k][cc].re * o.s[k][cc].re + rv.s[k][cc].im * o.s[k][cc].im;
+          v[2] += o.s[k][cc].re * o.s[k][cc].re + o.s[k][cc].im * o.s[k][cc].im;
+        }
       }
   }
-  const R v[3] = {pa, ra, aa};
-  double tot[3];
-  if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_alpha_beta(cgd, tot);
+  double tot[NV];
+  if (block_total<NV>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_scalars<NV>(cgd, tot);
   if (i < g.Vh) store_spinor<R, ST>(ap, i, g.Vh, o);
 }
 
@@ -429,8 +441,9 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_hop_sp
   }
 }
 
-// D: Ap = te + b D^dagger_eo to, block sums of <p, Ap>, Re <r, Ap>, |Ap|^2.
-template <bool DEFER, typename RL, int NC, typename R, typename ST = R>
+// D: Ap = te + b D^dagger_eo to, block sums of <p, Ap> and, for NV = 3,
+// Re <r, Ap> and |Ap|^2.
+template <int NV, bool DEFER, typename RL, int NC, typename R, typename ST = R>
 __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_split_kernel(
     typename Vec2<ST>::T* __restrict__ ap, const typename Vec2<ST>::T* __restrict__ to,
     const typename Vec2<ST>::T* __restrict__ te, const typename Vec2<ST>::T* __restrict__ p,
@@ -441,27 +454,32 @@ __global__ void __launch_bounds__(kDslashThreads, FG_SPLIT_MIN_BLOCKS) cg_apdot_
   const int i = blockIdx.x * 32 + (int)(threadIdx.x & 31), k = (int)(threadIdx.x >> 5);
   Cx<R> row[3];
   hops_split<1, RL, NC, R>(row, sh, FieldSrc<R, ST>{to}, U, g, i, 0, g.Vh);
-  R v[3] = {R(0), R(0), R(0)};  // a thread's 6 terms each
+  R v[NV];  // a thread's 6 terms each
+#pragma unroll
+  for (int q = 0; q < NV; ++q) v[q] = R(0);
   if (i < g.Vh) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const size_t j = entry_index(k, c, i, g.Vh);
       row[c] = Entry<R, ST>::load(te, j) + b * row[c];
       if (DEFER) Entry<R, ST>::store(ap, j, row[c]);
-      const Cx<R> pv = Entry<R, ST>::load(p, j), rv = Entry<R, ST>::load(r, j);
+      const Cx<R> pv = Entry<R, ST>::load(p, j);
       v[0] = fma(pv.re, row[c].re, v[0]);
       v[0] = fma(pv.im, row[c].im, v[0]);
-      v[1] = fma(rv.re, row[c].re, v[1]);
-      v[1] = fma(rv.im, row[c].im, v[1]);
-      v[2] = fma(row[c].re, row[c].re, v[2]);
-      v[2] = fma(row[c].im, row[c].im, v[2]);
+      if constexpr (NV == 3) {
+        const Cx<R> rv = Entry<R, ST>::load(r, j);
+        v[1] = fma(rv.re, row[c].re, v[1]);
+        v[1] = fma(rv.im, row[c].im, v[1]);
+        v[2] = fma(row[c].re, row[c].re, v[2]);
+        v[2] = fma(row[c].im, row[c].im, v[2]);
+      }
     }
   }
   if constexpr (DEFER) {
-    block_sums<3>(v, partial, gridDim.x);
+    block_sums<NV>(v, partial, gridDim.x);
   } else {
-    double tot[3];
-    if (block_total<3>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_alpha_beta(cgd, tot);
+    double tot[NV];
+    if (block_total<NV>(v, partial, &cgd->ticket[0], tot) && threadIdx.x == 0) set_scalars<NV>(cgd, tot);
     if (i < g.Vh) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) Entry<R, ST>::store(ap, entry_index(k, c, i, g.Vh), row[c]);
@@ -638,17 +656,21 @@ __device__ __forceinline__ double block_sum_partials(const double* __restrict__ 
   return r;
 }
 
-// The vector part of a five-launch iteration (Dslash launches to, te, to, D,
-// then this one): x += alpha p, r -= alpha Ap, p = r + beta p with D's alpha
-// and beta; the last block publishes |r|^2.  One pass where an axpy, whose
-// total |r|^2 beta waited for, and an xpay took two (half precision
-// 24^3 x 48: 23.3 + 11.2 us; each thread also divided in FP64).  The search
-// direction is formed on the converging iteration too, so that a reliable
-// update that finds the true residual still too large can simply continue.
-// x has pairs X (FP32 in the 16-bit solvers, whose r, p and Ap are stored as
-// ST and in units of sigma; `scaled` then publishes |r|^2 sigma^2).  The
-// kernels take no iteration argument, so a batch of iterations can be
-// captured once in a CUDA graph and replayed.
+// The vector part of a six-launch iteration (Dslash launches to, te, to, D,
+// then these two).  The first: r -= alpha Ap and |r|^2, which the last block
+// publishes, with beta = |r'|^2 / |r|^2 of the residuals as they are stored.
+// The second: x += alpha p, p = r + beta p.  beta by D's expansion (as the
+// folded iteration takes it) would save a launch, some 2 us, and no memory
+// traffic, as D would read r for it; but the expansion's terms cancel, which
+// leaves beta wrong by some 1e-7 |r|^2 / |r'|^2 in FP32 and by the rounding of
+// the stored r in 16 bits, where the ratio of the sums is good to 1e-8.
+// The search direction is formed on the converging iteration too (`fresh`,
+// not `done`, tells the second launch to go on), so that a reliable update
+// that finds the true residual still too large can simply continue.  x has
+// pairs X (FP32 in the 16-bit solvers, whose r, p and Ap are stored as ST and
+// in units of sigma; `scaled` then publishes |r|^2 sigma^2).  The kernels take
+// no iteration argument, so a batch of iterations can be captured once in a
+// CUDA graph and replayed.
 // A value as its storage holds it.
 template <typename ST, typename R> __device__ __forceinline__ Cx<R> stored(const Cx<R>& v) {
   if constexpr (std::is_same<ST, R>::value) {
@@ -659,35 +681,56 @@ template <typename ST, typename R> __device__ __forceinline__ Cx<R> stored(const
   }
 }
 template <typename R, typename ST>
-__global__ void __launch_bounds__(kVecThreads) cg_update_kernel(
-    typename Vec2<R>::T* __restrict__ x, typename Vec2<ST>::T* __restrict__ r, typename Vec2<ST>::T* __restrict__ p,
-    const typename Vec2<ST>::T* __restrict__ ap, CgDev* __restrict__ cgd, double* __restrict__ rr_part,
-    double* __restrict__ hist, int* __restrict__ iter_out, int maxiter, int scaled, int n) {
-  if (cgd->done) return;
-  const R a = R(cgd->alpha), b = R(cgd->beta);
+__global__ void __launch_bounds__(kVecThreads) cg_residual_kernel(
+    typename Vec2<ST>::T* __restrict__ r, const typename Vec2<ST>::T* __restrict__ ap, CgDev* __restrict__ cgd,
+    double* __restrict__ rr_part, double* __restrict__ hist, int* __restrict__ iter_out, int maxiter, int scaled,
+    int n) {
+  if (cgd->done) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) cgd->fresh = 0;
+    return;
+  }
+  const R a = R(cgd->alpha);
   R acc = R(0);  // a thread's few entries in R; blocks and the total in FP64
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += gridDim.x * blockDim.x) {
-    Cx<R> xv[2], rv[2], pv[2], av[2];
-    Quad<R>::load_cg(x, i, xv[0], xv[1]);
+    Cx<R> rv[2], av[2];
     Quad<ST>::load_cg(r, i, rv[0], rv[1]);
-    Quad<ST>::load_cg(p, i, pv[0], pv[1]);
     Quad<ST>::load_cg(ap, i, av[0], av[1]);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      xv[k] = cx<R>(fma(a, pv[k].re, xv[k].re), fma(a, pv[k].im, xv[k].im));
       rv[k] = stored<ST>(cx<R>(fma(-a, av[k].re, rv[k].re), fma(-a, av[k].im, rv[k].im)));
-      pv[k] = cx<R>(fma(b, pv[k].re, rv[k].re), fma(b, pv[k].im, rv[k].im));
       acc = fma(rv[k].re, rv[k].re, acc);
       acc = fma(rv[k].im, rv[k].im, acc);
     }
-    Quad<R>::store(x, i, xv[0], xv[1]);
     Quad<ST>::store(r, i, rv[0], rv[1]);
-    Quad<ST>::store(p, i, pv[0], pv[1]);
   }
   const R v[1] = {acc};
   double tot[1];
-  if (block_total<1, kVecThreads>(v, rr_part, &cgd->ticket[1], tot) && threadIdx.x == 0)
+  if (block_total<1, kVecThreads>(v, rr_part, &cgd->ticket[1], tot) && threadIdx.x == 0) {
+    const double rr = cgd->rr[cgd->iter & 1];
+    cgd->beta = rr > 0.0 ? tot[0] / rr : 0.0;
+    cgd->fresh = 1;
     publish(cgd, tot[0], hist, iter_out, maxiter, scaled ? cgd->sigma2 : 1.0);
+  }
+}
+template <typename R, typename ST>
+__global__ void __launch_bounds__(kVecThreads) cg_direction_kernel(
+    typename Vec2<R>::T* __restrict__ x, typename Vec2<ST>::T* __restrict__ p,
+    const typename Vec2<ST>::T* __restrict__ r, const CgDev* __restrict__ cgd, int n) {
+  if (!cgd->fresh) return;
+  const R a = R(cgd->alpha), b = R(cgd->beta);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += gridDim.x * blockDim.x) {
+    Cx<R> xv[2], rv[2], pv[2];
+    Quad<R>::load_cg(x, i, xv[0], xv[1]);
+    Quad<ST>::load_cg(p, i, pv[0], pv[1]);
+    Quad<ST>::load_cg(r, i, rv[0], rv[1]);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      xv[k] = cx<R>(fma(a, pv[k].re, xv[k].re), fma(a, pv[k].im, xv[k].im));
+      pv[k] = cx<R>(fma(b, pv[k].re, rv[k].re), fma(b, pv[k].im, rv[k].im));
+    }
+    Quad<R>::store(x, i, xv[0], xv[1]);
+    Quad<ST>::store(p, i, pv[0], pv[1]);
+  }
 }
 
 // Reliable update, first half: x64 += x_s; x_s = 0.
@@ -1118,10 +1161,15 @@ cudaError_t launch_fermion_force(const GeomH& gh, const void* U, const void* Xe,
 }
 
 template <typename R>
-cudaError_t launch_cg_update(void* x, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part, double* hist,
-                             int* iter_out, int maxiter, int n, cudaStream_t st) {
-  cg_update_kernel<R, R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(x), v2<R>(r), v2<R>(p), cv2<R>(ap), cgd, rr_part,
-                                                               hist, iter_out, maxiter, 0, n);
+cudaError_t launch_cg_residual(void* r, const void* ap, CgDev* cgd, double* rr_part, double* hist, int* iter_out,
+                               int maxiter, int n, cudaStream_t st) {
+  cg_residual_kernel<R, R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(r), cv2<R>(ap), cgd, rr_part, hist, iter_out,
+                                                                 maxiter, 0, n);
+  return cudaGetLastError();
+}
+template <typename R>
+cudaError_t launch_cg_direction(void* x, void* p, const void* r, const CgDev* cgd, int n, cudaStream_t st) {
+  cg_direction_kernel<R, R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(x), v2<R>(p), cv2<R>(r), cgd, n);
   return cudaGetLastError();
 }
 template <typename R> static bool cg_defer(int Vh) { return hop_split<R>(Vh) && Vh <= FG_DEFER_MAX; }
@@ -1146,14 +1194,15 @@ cudaError_t launch_cg_publish(const GeomH& gh, const double* partial, CgDev* cgd
 }
 template <typename R, int NC>
 cudaError_t launch_cg_apdot(const GeomH& gh, void* ap, const void* to, const void* te, const void* p, const void* r,
-                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st, bool deferred) {
+                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st, bool folded) {
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  // totals are deferred only with a folded iteration's A behind
-  auto* const k = deferred && cg_defer<R>(gh.Vh)
-                      ? cg_apdot_split_kernel<true, R, NC, R>
-                      : (hop_split<R>(gh.Vh) ? cg_apdot_split_kernel<false, R, NC, R> : cg_apdot_kernel<R, NC, R>);
+  const bool split = hop_split<R>(gh.Vh);
+  auto* const k = folded ? (cg_defer<R>(gh.Vh) ? cg_apdot_split_kernel<3, true, R, NC, R>
+                                               : (split ? cg_apdot_split_kernel<3, false, R, NC, R>
+                                                        : cg_apdot_kernel<3, R, NC, R>))
+                         : (split ? cg_apdot_split_kernel<1, false, R, NC, R> : cg_apdot_kernel<1, R, NC, R>);
   k<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0, st>>>(
       v2<R>(ap), cv2<R>(to), cv2<R>(te), cv2<R>(p), cv2<R>(r), u, to_devg(gh), R(-k2), partial, cgd);
   return cudaGetLastError();
@@ -1257,28 +1306,28 @@ template cudaError_t launch_dslash_h16<9>(int, const GeomH&, void*, const void*,
 template cudaError_t launch_dslash_h16<6>(int, const GeomH&, void*, const void*, const void*, const void*, int, int,
                                           int, double, const CgDev*, cudaStream_t);
 template <typename S, int NC>
-static cudaError_t apdot16(const GeomH& gh, void* ap, const void* to, const void* te, const void* p, const void* r,
-                           const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st) {
+static cudaError_t apdot16(const GeomH& gh, void* ap, const void* to, const void* te, const void* p, const void* U,
+                           double k2, double* partial, CgDev* cgd, cudaStream_t st) {
   typedef typename Conv16<S>::T2 T2;
   Gauge<S, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  auto* const k = hop_split<float>(gh.Vh) ? cg_apdot_split_kernel<false, S, NC, float, S> : cg_apdot_kernel<S, NC, float, S>;
-  k<<<hop_blocks<float>(gh.Vh), kDslashThreads, 0, st>>>((T2*)ap, (const T2*)to, (const T2*)te, (const T2*)p,
-                                                        (const T2*)r, u, to_devg(gh), float(-k2), partial, cgd);
+  auto* const k =
+      hop_split<float>(gh.Vh) ? cg_apdot_split_kernel<1, false, S, NC, float, S> : cg_apdot_kernel<1, S, NC, float, S>;
+  k<<<hop_blocks<float>(gh.Vh), kDslashThreads, 0, st>>>((T2*)ap, (const T2*)to, (const T2*)te, (const T2*)p, nullptr,
+                                                        u, to_devg(gh), float(-k2), partial, cgd);
   return cudaGetLastError();
 }
 template <int NC>
 cudaError_t launch_cg_apdot_h16(int s16, const GeomH& gh, void* ap, const void* to, const void* te, const void* p,
-                                const void* r, const void* U, double k2, double* partial, CgDev* cgd,
-                                cudaStream_t st) {
-  return s16 == S16_BF16 ? apdot16<BF16, NC>(gh, ap, to, te, p, r, U, k2, partial, cgd, st)
-                         : apdot16<Half16, NC>(gh, ap, to, te, p, r, U, k2, partial, cgd, st);
+                                const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st) {
+  return s16 == S16_BF16 ? apdot16<BF16, NC>(gh, ap, to, te, p, U, k2, partial, cgd, st)
+                         : apdot16<Half16, NC>(gh, ap, to, te, p, U, k2, partial, cgd, st);
 }
 template cudaError_t launch_cg_apdot_h16<9>(int, const GeomH&, void*, const void*, const void*, const void*,
-                                            const void*, const void*, double, double*, CgDev*, cudaStream_t);
+                                            const void*, double, double*, CgDev*, cudaStream_t);
 template cudaError_t launch_cg_apdot_h16<6>(int, const GeomH&, void*, const void*, const void*, const void*,
-                                            const void*, const void*, double, double*, CgDev*, cudaStream_t);
+                                            const void*, double, double*, CgDev*, cudaStream_t);
 // Runs KERNEL<S> with the arguments that follow for the 16-bit format s16.
 #define FG_S16(KERNEL, GRID, ...)                                                                              \
   do {                                                                                                         \
@@ -1290,13 +1339,23 @@ template cudaError_t launch_cg_apdot_h16<6>(int, const GeomH&, void*, const void
       KERNEL<Half16><<<GRID, kVecThreads, 0, st>>>(__VA_ARGS__);                                               \
     }                                                                                                          \
   } while (0)
-cudaError_t launch_cg_update_h16(int s16, void* xs, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part,
-                                 double* hist, int* iter_out, int maxiter, int n, cudaStream_t st) {
+cudaError_t launch_cg_residual_h16(int s16, void* r, const void* ap, CgDev* cgd, double* rr_part, double* hist,
+                                   int* iter_out, int maxiter, int n, cudaStream_t st) {
   auto run = [&](auto s) {
     typedef decltype(s) S;
     typedef typename Conv16<S>::T2 T2;
-    cg_update_kernel<float, S><<<vec_blocks(n), kVecThreads, 0, st>>>((float2*)xs, (T2*)r, (T2*)p, (const T2*)ap, cgd,
-                                                                     rr_part, hist, iter_out, maxiter, 1, n);
+    cg_residual_kernel<float, S><<<vec_blocks(n), kVecThreads, 0, st>>>((T2*)r, (const T2*)ap, cgd, rr_part, hist,
+                                                                       iter_out, maxiter, 1, n);
+    return cudaGetLastError();
+  };
+  return s16 == S16_BF16 ? run(BF16{}) : run(Half16{});
+}
+cudaError_t launch_cg_direction_h16(int s16, void* xs, void* p, const void* r, const CgDev* cgd, int n,
+                                    cudaStream_t st) {
+  auto run = [&](auto s) {
+    typedef decltype(s) S;
+    typedef typename Conv16<S>::T2 T2;
+    cg_direction_kernel<float, S><<<vec_blocks(n), kVecThreads, 0, st>>>((float2*)xs, (T2*)p, (const T2*)r, cgd, n);
     return cudaGetLastError();
   };
   return s16 == S16_BF16 ? run(BF16{}) : run(Half16{});
@@ -1426,10 +1485,12 @@ template cudaError_t launch_dslash<float, 9, DF>(const GeomH&, void*, const void
 template cudaError_t launch_dslash<float, 6, DF>(const GeomH&, void*, const void*, const void*, const void*, int, int, int,
                                                      double, const CgDev*, cudaStream_t);
 
-template cudaError_t launch_cg_update<double>(void*, void*, void*, const void*, CgDev*, double*, double*, int*, int, int,
-                                              cudaStream_t);
-template cudaError_t launch_cg_update<float>(void*, void*, void*, const void*, CgDev*, double*, double*, int*, int, int,
-                                             cudaStream_t);
+template cudaError_t launch_cg_residual<double>(void*, const void*, CgDev*, double*, double*, int*, int, int,
+                                                cudaStream_t);
+template cudaError_t launch_cg_residual<float>(void*, const void*, CgDev*, double*, double*, int*, int, int,
+                                               cudaStream_t);
+template cudaError_t launch_cg_direction<double>(void*, void*, const void*, const CgDev*, int, cudaStream_t);
+template cudaError_t launch_cg_direction<float>(void*, void*, const void*, const CgDev*, int, cudaStream_t);
 #define FG_INST_FOLD(R, NC)                                                                                    \
   template cudaError_t launch_cg_hop<R, NC>(const GeomH&, void*, const void*, const void*, const void*, double, \
                                             double*, CgDev*, double*, int*, int, cudaStream_t);                \

@@ -27,6 +27,7 @@ struct CgDev {
   int restart;  // set by a reliable update whose true residual left the recursion far behind
   double pap;       // <p, Ap> of the iteration in progress
   double beta;      // beta of the update in progress
+  int fresh;        // six-launch iteration: r is new, x and p are still to move
   unsigned ticket[2];  // blocks finished, for the two grand totals; the last block resets it to 0
   // half-precision inner vectors hold r / sigma and p / sigma; sigma^2 is
   // reset at every reliable update to |r|^2 / n, and rho rescales p then
@@ -67,12 +68,14 @@ template <typename RL, int NC, typename RS>
 cudaError_t launch_fermion_force(const GeomH& g, const void* U, const void* Xe, const void* Xo, const void* Ye,
                                  const void* Yo, void* FF, double kappa2, int accumulate, cudaStream_t st);
 
-// x += alpha p, r -= alpha Ap, p = r + beta p with cgd's alpha and beta;
-// |r|^2 is published as the residual of iteration iter + 1 (rr[], hist,
-// *iter_out, done).
+// r -= alpha Ap; |r|^2 is published as the residual of iteration iter + 1
+// (rr[], hist, *iter_out, done) and beta = |r'|^2 / |r|^2 is set.
 template <typename R>
-cudaError_t launch_cg_update(void* x, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part, double* hist,
-                             int* iter_out, int maxiter, int n, cudaStream_t st);
+cudaError_t launch_cg_residual(void* r, const void* ap, CgDev* cgd, double* rr_part, double* hist, int* iter_out,
+                               int maxiter, int n, cudaStream_t st);
+// x += alpha p, p = r + beta p if the residual launch before did its work.
+template <typename R>
+cudaError_t launch_cg_direction(void* x, void* p, const void* r, const CgDev* cgd, int n, cudaStream_t st);
 template <typename RI>
 cudaError_t launch_ru_accumulate(void* x64, void* xs, int n, cudaStream_t st);
 template <typename RI>
@@ -93,14 +96,15 @@ cudaError_t launch_df_to_double(void* dst, const void* src, int n, cudaStream_t 
 template <int NC>
 cudaError_t launch_dslash_h16(int s16, const GeomH& g, void* out, const void* in, const void* x, const void* U,
                               int out_par, int dag, int mode, double b, const CgDev* cgd, cudaStream_t st);
-// launch_cg_apdot and launch_cg_update on 16-bit vectors (hist and done in
-// units of |b|).
+// launch_cg_apdot, launch_cg_residual and launch_cg_direction on 16-bit
+// vectors (hist and done in units of |b|).
 template <int NC>
 cudaError_t launch_cg_apdot_h16(int s16, const GeomH& g, void* ap, const void* to, const void* te, const void* p,
-                                const void* r, const void* U, double k2, double* partial, CgDev* cgd,
-                                cudaStream_t st);
-cudaError_t launch_cg_update_h16(int s16, void* xs, void* r, void* p, const void* ap, CgDev* cgd, double* rr_part,
-                                 double* hist, int* iter_out, int maxiter, int n, cudaStream_t st);
+                                const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st);
+cudaError_t launch_cg_residual_h16(int s16, void* r, const void* ap, CgDev* cgd, double* rr_part, double* hist,
+                                   int* iter_out, int maxiter, int n, cudaStream_t st);
+cudaError_t launch_cg_direction_h16(int s16, void* xs, void* p, const void* r, const CgDev* cgd, int n,
+                                    cudaStream_t st);
 // Start of a solve: bb from the partials of |b|^2, sigma^2 = bb / n, rr = n, tol2bb, done.
 cudaError_t launch_cg_init_h16(const double* part, int nparts, CgDev* cgd, double tol2, double* bb_out, int n,
                                cudaStream_t st);
@@ -150,14 +154,14 @@ cudaError_t launch_cg_hop(const GeomH& g, void* te, const void* to, const void* 
                           double* partial, CgDev* cgd, double* hist, int* iter_out, int maxiter, cudaStream_t st);
 cudaError_t launch_cg_publish(const GeomH& g, const double* partial, CgDev* cgd, double* hist, int* iter_out,
                               int maxiter, cudaStream_t st);
-// D: Ap = te - k2 D_eo^dagger to on the even sites, and the sums of <p, Ap>,
-// Re <r, Ap>, |Ap|^2 from which alpha = rr / <p, Ap> and
-// beta = (rr - 2 alpha Re <r, Ap> + alpha^2 |Ap|^2) / rr follow, rr =
-// cgd->rr[iter & 1]: set in cgd, or with `deferred` (a folded iteration) left
-// as block sums to A where cg_deferred().
+// D: Ap = te - k2 D_eo^dagger to on the even sites, and the sum <p, Ap>, with
+// which alpha = rr / <p, Ap> is set, rr = cgd->rr[iter & 1].  `folded`: also
+// Re <r, Ap> and |Ap|^2, with which
+// beta = (rr - 2 alpha Re <r, Ap> + alpha^2 |Ap|^2) / rr is set, or all three
+// are left as block sums to A where cg_deferred().
 template <typename R, int NC>
 cudaError_t launch_cg_apdot(const GeomH& g, void* ap, const void* to, const void* te, const void* p, const void* r,
-                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st, bool deferred);
+                            const void* U, double k2, double* partial, CgDev* cgd, cudaStream_t st, bool folded);
 // A: x += alpha p; r2 = r - alpha Ap; p2 = r2 + beta p (even sites) and
 // to = D_oe p2 (odd sites); |r2|^2 is the residual of iteration iter + 1
 // (rr[], hist, *iter_out, done).  r, p and r2, p2 are different buffers.
