@@ -1388,9 +1388,9 @@ class Backend final : public IBackend {
       return s;
     if (!final) {
       if ((s = apply_mdagm_df(ax64_, xdf_, U)) != FG_OK) return s;
-      if ((s = run(KC_CG_BLAS, [&] { return launch_ru_residual_df_keep(bdf_, ax64_, part_rr_, n, st_); })) != FG_OK)
+      if ((s = run(KC_CG_BLAS, [&] { return launch_ru_residual_df_keep(bdf_, ax64_, cgd_, part_rr_, n, st_); })) != FG_OK)
         return s;
-      if ((s = run(KC_REDUCE, [&] { return launch_ru_publish_h16(part_rr_, nbv, cgd_, tr, n, st_); })) != FG_OK)
+      if ((s = run(KC_REDUCE, [&] { return launch_ru_publish_h16(part_rr_, nbv, cgd_, tr, 1, n, st_); })) != FG_OK)
         return s;
       return run(KC_CG_BLAS, [&] { return launch_ru_rescale_df_h16(s16_, ax64_, rs_, p_, cgd_, n, st_); });
     }
@@ -1398,7 +1398,7 @@ class Backend final : public IBackend {
     if ((s = apply_mdagm64(ax64_, x64_, U)) != FG_OK) return s;
     if ((s = run(KC_CG_BLAS, [&] { return launch_ru_residual64_keep(b64, ax64_, r64_, part_rr_, n, st_); })) != FG_OK)
       return s;
-    if ((s = run(KC_REDUCE, [&] { return launch_ru_publish_h16(part_rr_, nbv, cgd_, tr, n, st_); })) != FG_OK)
+    if ((s = run(KC_REDUCE, [&] { return launch_ru_publish_h16(part_rr_, nbv, cgd_, tr, 0, n, st_); })) != FG_OK)
       return s;
     return run(KC_CG_BLAS, [&] { return launch_ru_rescale64_h16(s16_, r64_, rs_, p_, cgd_, n, st_); });
   }

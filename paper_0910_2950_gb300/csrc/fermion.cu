@@ -827,6 +827,19 @@ __global__ void __launch_bounds__(kVecThreads) df_to_double_kernel(double2* __re
 // |r / sigma|^2 = n after every reliable update keeps the entries O(1), far
 // from the ends of the half range.  Scalars (rr, pAp, alpha, beta) are in the scaled units;
 // the history and the convergence test use rr sigma^2.
+__device__ __forceinline__ void set_sigma(CgDev* cgd, double s2) {
+  cgd->sigma2 = s2;
+  cgd->inv = 1.0 / sqrt(s2);
+  int e;
+  const DF m(frexp(cgd->inv, &e));
+  // a double-float residual has no entries beyond FP32's range
+  e = e < -250 ? -250 : (e > 250 ? 250 : e);
+  cgd->inv_e = e;
+  cgd->inv_hi = m.hi;
+  cgd->inv_lo = m.lo;
+  cgd->inv_s1 = (float)ldexp(1.0, e / 2);
+  cgd->inv_s2 = (float)ldexp(1.0, e - e / 2);
+}
 __global__ void cg_init_h16_kernel(const double* __restrict__ part, int nparts, CgDev* __restrict__ cgd, double tol2,
                                    double* __restrict__ bb_out, int n) {
   const double bb = block_sum_partials(part, nparts);
@@ -834,7 +847,7 @@ __global__ void cg_init_h16_kernel(const double* __restrict__ part, int nparts, 
     const double s2 = bb > 0.0 ? bb / n : 1.0;
     cgd->bb = bb;
     cgd->tol2bb = tol2 * bb;
-    cgd->sigma2 = s2;
+    set_sigma(cgd, s2);
     cgd->rho = 1.0;
     cgd->rr[0] = cgd->rr[1] = bb / s2;
     set_done(cgd, bb == 0.0);
@@ -882,16 +895,21 @@ __global__ void __launch_bounds__(kVecThreads) ru_accumulate_df_scaled_kernel(fl
   }
 }
 
+// r = b - Ax in the place of ax; block sums of |r 2^inv_e|^2 (the squares of
+// the entries themselves leave FP32's range before sigma does).
 __global__ void __launch_bounds__(kVecThreads) ru_residual_df_keep_kernel(const float4* __restrict__ b,
                                                                           float4* __restrict__ ax,
+                                                                          const CgDev* __restrict__ cgd,
                                                                           double* __restrict__ part, int n) {
+  const float s1 = cgd->inv_s1, s2 = cgd->inv_s2;
   float acc = 0.0f;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float4 bv = b[i], av = ax[i];
     const DF re = DF(bv.x, bv.y) - DF(av.x, av.y), im = DF(bv.z, bv.w) - DF(av.z, av.w);
     ax[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
-    acc = fmaf(re.hi, re.hi, acc);
-    acc = fmaf(im.hi, im.hi, acc);
+    const float x = re.hi * s1 * s2, y = im.hi * s1 * s2;
+    acc = fmaf(x, x, acc);
+    acc = fmaf(y, y, acc);
   }
   double v[1] = {double(acc)};
   block_reduce_store<1>(v, part, gridDim.x);
@@ -913,17 +931,15 @@ __global__ void __launch_bounds__(kVecThreads) ru_residual64_keep_kernel(const d
 }
 
 __global__ void ru_publish_h16_kernel(const double* __restrict__ part, int nparts, CgDev* __restrict__ cgd,
-                                      double* __restrict__ true_rr, int n) {
-  const double rr = block_sum_partials(part, nparts);
+                                      double* __restrict__ true_rr, int scaled, int n) {
+  const double sum = block_sum_partials(part, nparts);
   if (threadIdx.x == 0) {
+    const double rr = scaled ? ldexp(sum, -2 * cgd->inv_e) : sum;
     const double rr_iter = cgd->rr[cgd->iter & 1] * cgd->sigma2;
     const double s2 = rr > 0.0 ? rr / n : cgd->sigma2;
     cgd->restart = (rr > 2.0 * rr_iter) ? 1 : 0;
     cgd->rho = sqrt(cgd->sigma2 / s2);
-    cgd->sigma2 = s2;
-    const DF inv(1.0 / sqrt(s2));
-    cgd->inv_hi = inv.hi;
-    cgd->inv_lo = inv.lo;
+    set_sigma(cgd, s2);
     cgd->rr[cgd->iter & 1] = rr / s2;
     set_done(cgd, rr <= cgd->tol2bb);
     *true_rr = rr;
@@ -935,19 +951,20 @@ __global__ void __launch_bounds__(kVecThreads) ru_rescale_h16_kernel(const RV* _
                                                                      typename Conv16<S>::T2* __restrict__ rs,
                                                                      typename Conv16<S>::T2* __restrict__ p,
                                                                      const CgDev* __restrict__ cgd, int n) {
-  // 1 / sigma as ru_publish_h16 left it: a root and a division in FP64 in every
+  // 1 / sigma as set_sigma left it: a root and a division in FP64 in every
   // thread, and FP64 products, made this pass 87 us at 24^3 x 48
   const DF inv(cgd->inv_hi, cgd->inv_lo);
+  const float s1 = cgd->inv_s1, s2 = cgd->inv_s2;
+  const double d = cgd->inv;
   const float rho = float(cgd->rho);
   const bool restart = cgd->restart != 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     float2 f;
     if constexpr (std::is_same<RV, float4>::value) {   // double-float residual
       const float4 v = ((const float4*)r)[i];
-      f = make_float2((DF(v.x, v.y) * inv).hi, (DF(v.z, v.w) * inv).hi);
+      f = make_float2((DF(v.x, v.y) * inv).hi * s1 * s2, (DF(v.z, v.w) * inv).hi * s1 * s2);
     } else {
       const double2 v = ((const double2*)r)[i];
-      const double d = double(inv);
       f = make_float2(float(v.x * d), float(v.y * d));
     }
     const typename Conv16<S>::T2 h = Conv16<S>::of(f);
@@ -1378,8 +1395,9 @@ cudaError_t launch_ru_accumulate_df_scaled(void* xdf, void* xs, const CgDev* cgd
   ru_accumulate_df_scaled_kernel<<<vec_blocks(n), kVecThreads, 0, st>>>((float4*)xdf, (float2*)xs, cgd, n);
   return cudaGetLastError();
 }
-cudaError_t launch_ru_residual_df_keep(const void* bdf, void* axdf, double* part, int n, cudaStream_t st) {
-  ru_residual_df_keep_kernel<<<vec_blocks(n), kVecThreads, 0, st>>>((const float4*)bdf, (float4*)axdf, part, n);
+cudaError_t launch_ru_residual_df_keep(const void* bdf, void* axdf, const CgDev* cgd, double* part, int n,
+                                       cudaStream_t st) {
+  ru_residual_df_keep_kernel<<<vec_blocks(n), kVecThreads, 0, st>>>((const float4*)bdf, (float4*)axdf, cgd, part, n);
   return cudaGetLastError();
 }
 cudaError_t launch_ru_residual64_keep(const void* b64, const void* ax64, void* r64, double* part, int n,
@@ -1388,9 +1406,9 @@ cudaError_t launch_ru_residual64_keep(const void* b64, const void* ax64, void* r
                                                                    (double2*)r64, part, n);
   return cudaGetLastError();
 }
-cudaError_t launch_ru_publish_h16(const double* part, int nparts, CgDev* cgd, double* true_rr, int n,
+cudaError_t launch_ru_publish_h16(const double* part, int nparts, CgDev* cgd, double* true_rr, int scaled, int n,
                                   cudaStream_t st) {
-  ru_publish_h16_kernel<<<1, 256, 0, st>>>(part, nparts, cgd, true_rr, n);
+  ru_publish_h16_kernel<<<1, 256, 0, st>>>(part, nparts, cgd, true_rr, scaled, n);
   return cudaGetLastError();
 }
 cudaError_t launch_ru_rescale_df_h16(int s16, const void* rdf, void* rs, void* p, const CgDev* cgd, int n,

@@ -33,7 +33,11 @@ struct CgDev {
   // reset at every reliable update to |r|^2 / n, and rho rescales p then
   double sigma2;
   double rho;
-  float inv_hi, inv_lo;  // 1 / sigma as a double-float
+  // 1 / sigma, and as the double-float inv_hi + inv_lo in [1/2, 1) times
+  // inv_s1 inv_s2 = 2^inv_e: sigma follows |r| below FP32's range
+  double inv;
+  float inv_hi, inv_lo, inv_s1, inv_s2;
+  int inv_e;
   // folded iteration with one direction a warp: block sums of |r'|^2 are left
   // and not yet published
   int pending;
@@ -116,13 +120,15 @@ cudaError_t launch_h16_to_double_scaled(int s16, void* dst64, const void* src16,
 // x (double-float) += sigma x_s; x_s = 0.
 cudaError_t launch_ru_accumulate_df_scaled(void* xdf, void* xs, const CgDev* cgd, int n, cudaStream_t st);
 // r = b - Ax written over Ax (double-float), partials of |r|^2.
-cudaError_t launch_ru_residual_df_keep(const void* bdf, void* axdf, double* part, int n, cudaStream_t st);
+cudaError_t launch_ru_residual_df_keep(const void* bdf, void* axdf, const CgDev* cgd, double* part, int n,
+                                       cudaStream_t st);
 // r = b - Ax written to r64 (FP64), partials of |r|^2.
 cudaError_t launch_ru_residual64_keep(const void* b64, const void* ax64, void* r64, double* part, int n,
                                       cudaStream_t st);
 // Publish a true residual for the 16-bit solver: rr, restart, new
-// sigma^2 and rho, rr[iter&1] in the new scaling, done.
-cudaError_t launch_ru_publish_h16(const double* part, int nparts, CgDev* cgd, double* true_rr, int n,
+// sigma^2 and rho, rr[iter&1] in the new scaling, done.  `scaled`: the partials
+// are launch_ru_residual_df_keep's.
+cudaError_t launch_ru_publish_h16(const double* part, int nparts, CgDev* cgd, double* true_rr, int scaled, int n,
                                   cudaStream_t st);
 // rs = r / sigma (r double-float or FP64); p = restart ? rs : rho p.
 cudaError_t launch_ru_rescale_df_h16(int s16, const void* rdf, void* rs, void* p, const CgDev* cgd, int n,
