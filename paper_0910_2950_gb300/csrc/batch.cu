@@ -63,7 +63,8 @@ template <> struct TileBounds<64> { static constexpr int min_blocks = 1; };
 template <int NC, int MODE, int H>
 __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
     batch_force_kernel(const Tile* __restrict__ tiles, int ntiles, const ChainDesc* __restrict__ chains, char* U,
-                       char* P, char* F, char* Ubase, char* Uout, float ckick, float cdrift, float cdisp, int reunit) {
+                       char* P, char* F, char* Ubase, char* Uout, Coef<float> ckick0, Coef<float> cdrift, float cdisp,
+                       int reunit) {
   for (int b = blockIdx.x; b < ntiles; b += gridDim.x) {
     const Tile t = tiles[b];
     const ChainDesc& cd = chains[t.chain];
@@ -75,6 +76,10 @@ __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
     u.p = U + cd.goff; u.V = g.V;
     ub.p = Ubase ? Ubase + cd.goff : nullptr; ub.V = g.V;
     uo.p = Uout ? Uout + cd.goff : nullptr; uo.V = g.V;
+    // as make_kick
+    constexpr bool kKick = MODE == FM_KICK || MODE == FM_KICK_DRIFT;
+    const float beta6 = kKick ? 1.0f : cd.beta6_hi;
+    const Coef<float> ckick = product(ckick0, Coef<float>{cd.beta6_hi, cd.beta6_lo}), ffw{1.0f, 0.0f};
     Mom<float> p, f, ff;
     p.p = P ? P + cd.moff : nullptr; p.V = g.V;
     f.p = F ? F + cd.moff : nullptr; f.V = g.V;
@@ -84,13 +89,13 @@ __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
       // block takes the barriers (uniform tile loop)
       extern __shared__ float2 batch_tsh[];
       force_link_shared<NC, MODE, 2 * H>(reinterpret_cast<float2(*)[9][2 * H]>(batch_tsh), ok, s, u, p, f, ff, ub,
-                                         uo, g, cd.beta6_hi, ckick, cdrift, cdisp, reunit, 1.0f);
+                                         uo, g, beta6, ckick, cdrift, cdisp, reunit, ffw);
       __syncthreads();   // the next tile rewrites the slots
     } else {
       int c[4], par;
       cb_coords(g, s, c, par);
-      force_link_staples<float, NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, cd.beta6_hi, ckick, cdrift, cdisp,
-                                   reunit, 1.0f);
+      force_link_staples<float, NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
+                                   reunit, ffw);
     }
   }
 }
@@ -104,7 +109,7 @@ constexpr size_t batch_force_smem() {
 template <typename R, int NC, int H>
 __global__ void __launch_bounds__(8 * H) batch_drift_kernel(const Tile* __restrict__ tiles, int ntiles,
                                                             const ChainDesc* __restrict__ chains, char* Uin,
-                                                            char* P, char* Uout, double c, int reunit) {
+                                                            char* P, char* Uout, Coef<R> c, int reunit) {
   for (int b = blockIdx.x; b < ntiles; b += gridDim.x) {
     const Tile t = tiles[b];
     const ChainDesc& cd = chains[t.chain];
@@ -115,7 +120,7 @@ __global__ void __launch_bounds__(8 * H) batch_drift_kernel(const Tile* __restri
     uo.p = Uout + cd.goff; uo.V = cd.g.V;
     Mom<R> p;
     p.p = P + cd.moff; p.V = cd.g.V;
-    drift_link(ui, p, uo, s, (int)threadIdx.y, R(c), reunit);
+    drift_link(ui, p, uo, s, (int)threadIdx.y, c, reunit);
   }
 }
 
@@ -662,12 +667,12 @@ class Batch final : public IBatch {
     const int gr = grid(nt, TileBounds<H>::min_blocks);
     return lrun([&] {
       const size_t sm = batch_force_smem<NC, H>();
+      const Coef<float> ckick = make_coef<float>(a.ckick), cdrift = make_coef<float>(a.cdrift);
       const Tile* tl = d_tiles_[hi];
       const ChainDesc* cds = d_chains_h_[hi];
 #define FG_FORCE(M)                                                                                                \
   batch_force_kernel<NC, M, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)a.U, (char*)a.P, (char*)a.F, (char*)a.Ubase, \
-                                                     (char*)a.Uout, (float)a.ckick, (float)a.cdrift,              \
-                                                     (float)a.cdisp, a.reunit)
+                                                     (char*)a.Uout, ckick, cdrift, (float)a.cdisp, a.reunit)
       switch (mode) {
         case FM_STORE: FG_FORCE(FM_STORE); break;
         case FM_KICK: FG_FORCE(FM_KICK); break;
@@ -734,8 +739,8 @@ class Batch final : public IBatch {
     const int nt = ntiles_[hi];
     return lrun([&] {
       batch_drift_kernel<R, NC, H><<<grid(nt, 2), dim3(2 * H, 4), 0, st_>>>(d_tiles_[hi], nt, d_chains_h_[hi],
-                                                                            (char*)Uin, (char*)G, (char*)Uout, c,
-                                                                            reunit);
+                                                                            (char*)Uin, (char*)G, (char*)Uout,
+                                                                            make_coef<R>(c), reunit);
       return cudaGetLastError();
     });
   }

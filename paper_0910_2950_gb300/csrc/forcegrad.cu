@@ -153,7 +153,8 @@ __global__ void __launch_bounds__(256) force_tangent_kernel(Gauge<R, NC> U, Gaug
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) kick_fg_kernel(Mom<R> P, Mom<R> F, Mom<R> G, int V, R c, R shift) {
+__global__ void __launch_bounds__(256) kick_fg_kernel(Mom<R> P, Mom<R> F, Mom<R> G, int V, Coef<R> c,
+                                                      R shift) {
   const int s = blockIdx.x * kSites + threadIdx.x;
   const int mu = threadIdx.y;
   if (s >= V) return;
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(256) kick_fg_kernel(Mom<R> P, Mom<R> F, Mom<R>
   F.load(mu, s, f);
   G.load(mu, s, gg);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) p[k] = fma(-c, fma(-shift, gg[k], f[k]), p[k]);
+  for (int k = 0; k < 8; ++k) p[k] = kicked(p[k], fma(-shift, gg[k], f[k]), c);
   P.store(mu, s, p);
 }
 
@@ -204,7 +205,7 @@ template <typename R>
 cudaError_t launch_kick_fg(const GeomH& g, void* P, const void* F, const void* G, double c, double shift,
                            cudaStream_t st) {
   kick_fg_kernel<R><<<grid_of(g.V), block_of(), 0, st>>>(mom_at<R>(P, g.V), mom_at<R>(F, g.V), mom_at<R>(G, g.V),
-                                                         g.V, R(c), R(shift));
+                                                         g.V, make_coef<R>(c), R(shift));
   return cudaGetLastError();
 }
 template <typename RO, typename RX, typename RY>

@@ -53,8 +53,8 @@ constexpr int kStapleSites = 32;
 template <int NC, int MODE>
 __global__ void __launch_bounds__(4 * kStapleSites, kStapleMinBlocks<NC>)
     staple_force_kernel(Gauge<float, NC> U, Mom<float> P, Mom<float> F, Mom<float> FF, Gauge<float, NC> Ubase,
-                        Gauge<float, NC> Uout, Geom g, float beta6, float ckick, float cdrift, float cdisp, int reunit,
-                        float ffw) {
+                        Gauge<float, NC> Uout, Geom g, float beta6, Coef<float> ckick, Coef<float> cdrift, float cdisp,
+                        int reunit, Coef<float> ffw) {
   const int i = (int)(blockIdx.x >> 1) * kStapleSites + (int)threadIdx.x, s = (int)(blockIdx.x & 1) * g.Vh + i;
   const bool ok = i < g.Vh;
   if constexpr (kForceSharedT<float, NC>) {
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kForceThreads, FG_PLAQ_MIN_BLOCKS)
 template <typename R, int NC, int MODE>
 __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
     link_force_kernel(const __grid_constant__ ForceRows r, char* U, char* W, char* P, char* F, char* FF, char* Ubase,
-                      char* Uout, R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+                      char* Uout, Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit, Coef<R> ffw) {
   RowSite o;
   if (!row_site(r, 4, o)) return;
   const ChainDesc& cd = *o.cd;
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
 template <typename R, int NC, int MODE>
 __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
     staple_rows_kernel(const __grid_constant__ ForceRows r, char* U, char* P, char* F, char* FF, char* Ubase,
-                       char* Uout, R ckick, R cdrift, R cdisp, int reunit, R ffw) {
+                       char* Uout, Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit, Coef<R> ffw) {
   RowSite o;
   if (!row_site(r, 4, o)) return;
   const ChainDesc& cd = *o.cd;
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kForceThreads)
 // One thread a link: warp w takes direction w mod 4 of 32 consecutive sites.
 template <typename R, int NC>
 __global__ void __launch_bounds__(256) drift_kernel(Gauge<R, NC> Uin, Mom<R> P, Gauge<R, NC> Uout,
-                                                    int V, R c, int reunit) {
+                                                    int V, Coef<R> c, int reunit) {
   const unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int s = (int)(w >> 2) * 32 + (int)(threadIdx.x & 31);
   if (s >= V) return;
@@ -443,12 +443,16 @@ static cudaError_t launch_staple_force(const GeomH& gh, int mode, const ForceArg
   auto FF = mom_of<float>(a.FF, V);
   auto Ub = gauge_of<float, NC>(a.Ubase, V);
   auto Uo = gauge_of<float, NC>(a.Uout, V);
-  const float b6 = float(a.beta / 6.0);
-  const float ffw = float(a.ffw == 0.0 ? 1.0 : a.ffw);
+  KickCoef<float> k = make_kick(a.beta, a.ckick, a.ffw == 0.0 ? 1.0 : a.ffw);
+  if (mode == FM_STORE || mode == FM_DISPLACE) {  // the force itself
+    k.beta6 = float(a.beta / 6.0);
+    k.ffw = make_coef<float>(a.ffw == 0.0 ? 1.0 : a.ffw);
+  }
+  const Coef<float> cdrift = make_coef<float>(a.cdrift);
   const int nb = 2 * ((g.Vh + kStapleSites - 1) / kStapleSites);
 #define FG_FORCE(M)                                                                                          \
-  staple_force_kernel<NC, M><<<nb, dim3(kStapleSites, 4), 0, st>>>(U, P, F, FF, Ub, Uo, g, b6, float(a.ckick), \
-                                                                  float(a.cdrift), float(a.cdisp), a.reunit, ffw)
+  staple_force_kernel<NC, M><<<nb, dim3(kStapleSites, 4), 0, st>>>(U, P, F, FF, Ub, Uo, g, k.beta6, k.kick, cdrift, \
+                                                                  float(a.cdisp), a.reunit, k.ffw)
   switch (mode) {
     case FM_STORE: FG_FORCE(FM_STORE); break;
     case FM_KICK: FG_FORCE(FM_KICK); break;
@@ -492,7 +496,8 @@ cudaError_t launch_unitarity(const ForceRows& r, const void* U, double* flag, in
 
 template <typename R, int NC>
 static cudaError_t launch_link_force(const ForceRows& r, int mode, const ForceArgs& a, cudaStream_t st) {
-  const R ffw = R(a.ffw == 0.0 ? 1.0 : a.ffw);
+  const Coef<R> ckick = make_coef<R>(a.ckick), ffw = make_coef<R>(a.ffw == 0.0 ? 1.0 : a.ffw);
+  const Coef<R> cdrift = make_coef<R>(a.cdrift);
   const long long warps = 8LL * r.nrows;
   const int w = warps_per_block(warps, kForceThreads / 32);
   const unsigned nb = (unsigned)((warps + w - 1) / w);
@@ -500,12 +505,12 @@ static cudaError_t launch_link_force(const ForceRows& r, int mode, const ForceAr
   do {                                                                                                                \
     if (a.W != nullptr)                                                                                               \
       link_force_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.W, (char*)a.P, (char*)a.F, (char*)a.FF, \
-                                                         (char*)a.Ubase, (char*)a.Uout, R(a.ckick), R(a.cdrift),      \
-                                                         R(a.cdisp), a.reunit, ffw);                                  \
+                                                         (char*)a.Ubase, (char*)a.Uout, ckick, cdrift, R(a.cdisp),    \
+                                                         a.reunit, ffw);                                              \
     else                                                                                                              \
       staple_rows_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.P, (char*)a.F, (char*)a.FF,         \
-                                                          (char*)a.Ubase, (char*)a.Uout, R(a.ckick), R(a.cdrift),     \
-                                                          R(a.cdisp), a.reunit, ffw);                                 \
+                                                          (char*)a.Ubase, (char*)a.Uout, ckick, cdrift, R(a.cdisp),   \
+                                                          a.reunit, ffw);                                             \
   } while (0)
   switch (mode) {
     case FM_STORE: FG_FORCE(FM_STORE); break;
@@ -531,7 +536,8 @@ cudaError_t launch_drift(const GeomH& gh, const void* Uin, const void* P, void* 
   const long long warps = 4LL * ((gh.V + 31) / 32);
   const int w = warps_per_block(warps, 8);
   drift_kernel<R, NC><<<(unsigned)((warps + w - 1) / w), 32 * w, 0, st>>>(
-      gauge_of<R, NC>(Uin, gh.V), mom_of<R>(P, gh.V), gauge_of<R, NC>(Uout, gh.V), gh.V, R(c), reunit);
+      gauge_of<R, NC>(Uin, gh.V), mom_of<R>(P, gh.V), gauge_of<R, NC>(Uout, gh.V), gh.V, make_coef<R>(c),
+      reunit);
   return cudaGetLastError();
 }
 
@@ -613,7 +619,7 @@ cudaError_t launch_mom_to_canon(const GeomH& gh, const void* P, double* canon, c
 // P -= c FF (kick with a force computed elsewhere: the pseudofermion force of
 // a two-level integrator's outer kicks).
 template <typename R>
-__global__ void __launch_bounds__(256) kick_ff_kernel(Mom<R> P, Mom<R> FF, int V, R c) {
+__global__ void __launch_bounds__(256) kick_ff_kernel(Mom<R> P, Mom<R> FF, int V, Coef<R> c) {
   const int s = blockIdx.x * kSitesPerBlock + threadIdx.x;
   const int mu = threadIdx.y;
   if (s >= V) return;
@@ -621,13 +627,13 @@ __global__ void __launch_bounds__(256) kick_ff_kernel(Mom<R> P, Mom<R> FF, int V
   P.load(mu, s, p);
   FF.load(mu, s, f);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) p[k] = fma(-c, f[k], p[k]);
+  for (int k = 0; k < 8; ++k) p[k] = kicked(p[k], f[k], c);
   P.store(mu, s, p);
 }
 template <typename R>
 cudaError_t launch_kick_ff(const GeomH& gh, void* P, const void* FF, double c, cudaStream_t st) {
   kick_ff_kernel<R><<<link_grid(gh.V), link_block(), 0, st>>>(mom_of<R>(P, gh.V), mom_of<R>(FF, gh.V), gh.V,
-                                                              R(c));
+                                                              make_coef<R>(c));
   return cudaGetLastError();
 }
 template cudaError_t launch_kick_ff<double>(const GeomH&, void*, const void*, double, cudaStream_t);
