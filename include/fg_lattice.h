@@ -343,6 +343,15 @@ long long fg_launch_count(const fg_lattice *h);
 /* Block until all work queued on the handle's stream has finished. */
 fg_status fg_sync(fg_lattice *h);
 
+/* Whether the handle runs alone on its GPU (0, the default) or shares it with
+ * others that run at the same time (non-zero), as the chains of a server with
+ * several slots do.  Alone, the FP32 solvers of small lattices (up to 24576
+ * even sites) spend instructions to shorten each launch; shared, they spend
+ * the fewest.  Results of FP32 solves differ in rounding between the two; FP64
+ * handles and pure gauge do not depend on it.  May be set between any two
+ * calls. */
+fg_status fg_set_shared(fg_lattice *h, int shared);
+
 /* Upper limit, in seconds, on every wait of the host for this handle's GPU
  * work (0, the default: no limit).  A call whose wait would last longer
  * returns FG_ETIMEOUT and leaves its work queued on the GPU; the handle's

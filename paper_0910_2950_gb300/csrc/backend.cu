@@ -315,6 +315,15 @@ class Backend final : public IBackend {
     sgc_valid_ = false;
     return check_links();
   }
+  fg_status set_shared(bool shared) override {
+    if (shared == g_.shared) return FG_OK;
+    fg_status s = sync();   // a captured batch may still run
+    if (s != FG_OK) return s;
+    for (const CgGraph& c : cg_graphs_) cudaGraphExecDestroy(c.exec);
+    cg_graphs_.clear();
+    g_.shared = shared;
+    return FG_OK;
+  }
   fg_status set_rng_position(unsigned long long pos) override {
     draw_ = (uint32_t)pos;
     pf_draw_ = (uint32_t)pos;
@@ -1214,7 +1223,7 @@ class Backend final : public IBackend {
   }
   // Whether a batch of folded iterations ends with a launch that publishes
   // the last one, and that launch.
-  bool fold_deferred() const { return fold_ && cg_deferred(g_.Vh, !kMixed); }
+  bool fold_deferred() const { return fold_ && cg_deferred(g_, !kMixed); }
   cudaError_t fold_publish() {
     return launch_cg_publish(g_, part_pap_, cgd_, mapped_->hist, &mapped_->dev_iter, h_->prm.cg_maxiter, st_);
   }

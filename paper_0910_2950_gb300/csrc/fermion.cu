@@ -49,29 +49,31 @@ template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_
 // thread need the fewest instructions and fill the GPU at 16^3 x 32 (65536
 // sites); below some 30 thousand sites they leave it waiting for a few warps'
 // serial loads.  Whole solves, split against whole: FP32 8^3 x 16 (4096
-// sites) 3.43 against 4.95 ms, 12^3 x 24 (20736) 5.22 against 6.50, 16^4
-// (32768) 7.00 against 6.14, 16^3 x 32 12.5 against 9.1.  The double-float
+// sites) 2.64 against 4.59 ms, 12^3 x 24 (20736) 4.61 against 5.96, 14^3 x 16
+// (21952) 4.63 against 5.83, 16^4 (32768) 7.00 against 6.14; half precision
+// 3.95 against 4.56, 5.19 against 5.63, 5.17 against 5.62.  The double-float
 // update gains up to 12^3 x 24 and loses 2% at 24^3 x 48.  FP64 arithmetic
 // waits for its unit, and four times the warps spread over the SMs evenly:
 // 8^3 x 16 7.7 against 21.6 ms, 12^3 x 24 28.3 against 40.7, 16^3 x 32 73.0
 // against 76.6.
-// The line of FP32 and double-float lies lower than those solves put it: with
-// many chains served at once the GPU is full, the extra instructions of the
-// split form count, and eight concurrent slots of the Poisson mix (8^3 x 16
-// and 12^3 x 24 chains) ran 61 trajectories/s with the line at 24576, 74 at
-// 8192, 78 before and 81 with no split.
+// Where the lattice shares the GPU with others that run at the same time
+// (GeomH::shared) the GPU is full without the split and its extra
+// instructions only cost: FP32 and double-float then never split.  Eight
+// concurrent slots of a Poisson mix of pure-gauge, 8^3 x 16 and 12^3 x 24
+// chains run 80.6 trajectories/s so, 61.3 with the split.
 #ifndef FG_SPLIT_MAX32
-#define FG_SPLIT_MAX32 8192
-#endif
-// Most sites with deferred totals (cg_fold_split_kernel).
-#ifndef FG_DEFER_MAX
-#define FG_DEFER_MAX 24576
+#define FG_SPLIT_MAX32 24576
 #endif
 #ifndef FG_SPLIT_MAXDF
-#define FG_SPLIT_MAXDF 8192
+#define FG_SPLIT_MAXDF 24576
 #endif
 #ifndef FG_SPLIT_MAX64
 #define FG_SPLIT_MAX64 131072
+#endif
+// Most sites with deferred totals in FP64 (cg_fold_split_kernel); split FP32
+// iterations always defer them.
+#ifndef FG_DEFER_MAX64
+#define FG_DEFER_MAX64 24576
 #endif
 
 // The grand total of NV values, one a thread in R (blocks of T threads):
@@ -1131,14 +1133,14 @@ int vec_blocks(int n) {
   int b = (n + kVecThreads - 1) / kVecThreads;
   return b > 152 * 8 ? 152 * 8 : b;
 }
-// Whether a Dslash launch over Vh sites gives one direction to a warp
+// Whether a Dslash launch over a parity's sites gives one direction to a warp
 // (blocks of 32 sites) or all eight hops to a thread (blocks of 128).
-template <typename RS> static bool hop_split(int Vh) {
-  return Vh <= (std::is_same<RS, float>::value ? FG_SPLIT_MAX32
-                                               : (std::is_same<RS, DF>::value ? FG_SPLIT_MAXDF : FG_SPLIT_MAX64));
+template <typename RS> static bool hop_split(const GeomH& g) {
+  if (std::is_same<RS, double>::value) return g.Vh <= FG_SPLIT_MAX64;
+  return !g.shared && g.Vh <= (std::is_same<RS, float>::value ? FG_SPLIT_MAX32 : FG_SPLIT_MAXDF);
 }
-template <typename RS> static int hop_blocks(int Vh) {
-  return hop_split<RS>(Vh) ? (Vh + 31) / 32 : (Vh + kDslashThreads - 1) / kDslashThreads;
+template <typename RS> static int hop_blocks(const GeomH& g) {
+  return hop_split<RS>(g) ? (g.Vh + 31) / 32 : (g.Vh + kDslashThreads - 1) / kDslashThreads;
 }
 int dslash_blocks(int Vh) { return (Vh + 31) / 32; }
 
@@ -1149,8 +1151,8 @@ cudaError_t launch_dslash(const GeomH& gh, void* out, const void* in, const void
   u.p = const_cast<void*>(U);
   u.V = gh.V;
   const Geom g = to_devg(gh);
-  const int nb = hop_blocks<RS>(gh.Vh);
-  const bool split = hop_split<RS>(gh.Vh);
+  const int nb = hop_blocks<RS>(gh);
+  const bool split = hop_split<RS>(gh);
 #define FG_DS(D, M)                                                                                       \
   (split ? dslash_split_kernel<RL, NC, RS, D, M> : dslash_kernel<RL, NC, RS, D, M>)<<<nb, kDslashThreads, 0, st>>>( \
       v2<RS>(out), cv2<RS>(in), cv2<RS>(x), u, g, out_par, RS(b), cgd)
@@ -1189,17 +1191,19 @@ cudaError_t launch_cg_direction(void* x, void* p, const void* r, const CgDev* cg
   cg_direction_kernel<R, R><<<vec_blocks(n), kVecThreads, 0, st>>>(v2<R>(x), v2<R>(p), cv2<R>(r), cgd, n);
   return cudaGetLastError();
 }
-template <typename R> static bool cg_defer(int Vh) { return hop_split<R>(Vh) && Vh <= FG_DEFER_MAX; }
-bool cg_deferred(int Vh, bool fp64) { return fp64 ? cg_defer<double>(Vh) : cg_defer<float>(Vh); }
+template <typename R> static bool cg_defer(const GeomH& g) {
+  return hop_split<R>(g) && (std::is_same<R, float>::value || g.Vh <= FG_DEFER_MAX64);
+}
+bool cg_deferred(const GeomH& g, bool fp64) { return fp64 ? cg_defer<double>(g) : cg_defer<float>(g); }
 template <typename R, int NC>
 cudaError_t launch_cg_hop(const GeomH& gh, void* te, const void* to, const void* p, const void* U, double k2,
                           double* partial, CgDev* cgd, double* hist, int* iter_out, int maxiter, cudaStream_t st) {
-  if (!cg_defer<R>(gh.Vh))
+  if (!cg_defer<R>(gh))
     return launch_dslash<R, NC, R>(gh, te, to, p, U, 0, 0, 1, -k2, cgd, st);
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  cg_hop_split_kernel<R, NC><<<hop_blocks<R>(gh.Vh) + 1, kDslashThreads, 0, st>>>(
+  cg_hop_split_kernel<R, NC><<<hop_blocks<R>(gh) + 1, kDslashThreads, 0, st>>>(
       v2<R>(te), cv2<R>(to), cv2<R>(p), u, to_devg(gh), R(-k2), partial, cgd, hist, iter_out, maxiter);
   return cudaGetLastError();
 }
@@ -1215,12 +1219,14 @@ cudaError_t launch_cg_apdot(const GeomH& gh, void* ap, const void* to, const voi
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  const bool split = hop_split<R>(gh.Vh);
-  auto* const k = folded ? (cg_defer<R>(gh.Vh) ? cg_apdot_split_kernel<3, true, R, NC, R>
-                                               : (split ? cg_apdot_split_kernel<3, false, R, NC, R>
-                                                        : cg_apdot_kernel<3, R, NC, R>))
-                         : (split ? cg_apdot_split_kernel<1, false, R, NC, R> : cg_apdot_kernel<1, R, NC, R>);
-  k<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0, st>>>(
+  const bool split = hop_split<R>(gh);
+  auto* k = folded ? cg_apdot_kernel<3, R, NC, R> : cg_apdot_kernel<1, R, NC, R>;
+  if (folded && cg_defer<R>(gh)) k = cg_apdot_split_kernel<3, true, R, NC, R>;
+  else if (split && !folded) k = cg_apdot_split_kernel<1, false, R, NC, R>;
+  else if constexpr (std::is_same<R, double>::value) {  // in FP32 split and folded is deferred
+    if (split) k = cg_apdot_split_kernel<3, false, R, NC, R>;
+  }
+  k<<<hop_blocks<R>(gh), kDslashThreads, 0, st>>>(
       v2<R>(ap), cv2<R>(to), cv2<R>(te), cv2<R>(p), cv2<R>(r), u, to_devg(gh), R(-k2), partial, cgd);
   return cudaGetLastError();
 }
@@ -1231,9 +1237,11 @@ cudaError_t launch_cg_fold(const GeomH& gh, void* to, void* x, const void* r, co
   Gauge<R, NC> u;
   u.p = const_cast<void*>(U);
   u.V = gh.V;
-  auto* const k = cg_defer<R>(gh.Vh) ? cg_fold_split_kernel<R, NC, true>
-                                     : (hop_split<R>(gh.Vh) ? cg_fold_split_kernel<R, NC, false> : cg_fold_kernel<R, NC>);
-  k<<<hop_blocks<R>(gh.Vh), kDslashThreads, 0, st>>>(v2<R>(to), v2<R>(x), cv2<R>(r), cv2<R>(ap), cv2<R>(p), v2<R>(r2),
+  auto* k = cg_defer<R>(gh) ? cg_fold_split_kernel<R, NC, true> : cg_fold_kernel<R, NC>;
+  if constexpr (std::is_same<R, double>::value) {
+    if (!cg_defer<R>(gh) && hop_split<R>(gh)) k = cg_fold_split_kernel<R, NC, false>;
+  }
+  k<<<hop_blocks<R>(gh), kDslashThreads, 0, st>>>(v2<R>(to), v2<R>(x), cv2<R>(r), cv2<R>(ap), cv2<R>(p), v2<R>(r2),
                                                      v2<R>(p2), u, to_devg(gh), partial, cgd, hist, iter_out, maxiter);
   return cudaGetLastError();
 }
@@ -1298,8 +1306,8 @@ static cudaError_t dslash16(const GeomH& gh, void* out, const void* in, const vo
   u.p = const_cast<void*>(U);
   u.V = gh.V;
   const Geom g = to_devg(gh);
-  const int nb = hop_blocks<float>(gh.Vh);
-  const bool split = hop_split<float>(gh.Vh);
+  const int nb = hop_blocks<float>(gh);
+  const bool split = hop_split<float>(gh);
 #define FG_DH(D, M)                                                                                            \
   (split ? dslash_split_kernel<S, NC, float, D, M, S>                                                          \
          : dslash_kernel<S, NC, float, D, M, S>)<<<nb, kDslashThreads, 0, st>>>(                               \
@@ -1330,8 +1338,8 @@ static cudaError_t apdot16(const GeomH& gh, void* ap, const void* to, const void
   u.p = const_cast<void*>(U);
   u.V = gh.V;
   auto* const k =
-      hop_split<float>(gh.Vh) ? cg_apdot_split_kernel<1, false, S, NC, float, S> : cg_apdot_kernel<1, S, NC, float, S>;
-  k<<<hop_blocks<float>(gh.Vh), kDslashThreads, 0, st>>>((T2*)ap, (const T2*)to, (const T2*)te, (const T2*)p, nullptr,
+      hop_split<float>(gh) ? cg_apdot_split_kernel<1, false, S, NC, float, S> : cg_apdot_kernel<1, S, NC, float, S>;
+  k<<<hop_blocks<float>(gh), kDslashThreads, 0, st>>>((T2*)ap, (const T2*)to, (const T2*)te, (const T2*)p, nullptr,
                                                         u, to_devg(gh), float(-k2), partial, cgd);
   return cudaGetLastError();
 }

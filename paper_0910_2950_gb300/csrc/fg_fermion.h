@@ -151,9 +151,9 @@ cudaError_t launch_cg_init_guess(const double* part_b, const double* part_r, int
 // ---- folded CG iteration (FP32 / FP64 inner vectors, links R with NC
 // entries): B, C (launch_dslash), D and A (see fermion.cu); `partial` has
 // 4 x dslash_blocks(Vh) entries.
-// Whether the launches of such an iteration on Vh sites publish it in the
+// Whether the launches of such an iteration on the lattice publish it in the
 // next one's B (launch_cg_publish then ends a batch of them) or in A.
-bool cg_deferred(int Vh, bool fp64);
+bool cg_deferred(const GeomH& g, bool fp64);
 // B: te = p - k2 D_eo to (and publishes the iteration before).
 template <typename R, int NC>
 cudaError_t launch_cg_hop(const GeomH& g, void* te, const void* to, const void* p, const void* U, double k2,

@@ -13,6 +13,7 @@ namespace fg {
 struct GeomH {
   int L[4];
   int Lxh, Vh, V;
+  bool shared = false;   // the lattice shares the GPU with others (fg_set_shared)
 };
 
 // Fused gauge-force kernel modes.

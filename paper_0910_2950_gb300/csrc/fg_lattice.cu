@@ -528,6 +528,10 @@ fg_status fg_sync(fg_lattice* h) {
   if (s != FG_OK) return h->fail(s, why);
   return FG_OK;
 }
+fg_status fg_set_shared(fg_lattice* h, int shared) {
+  FG_CHECK_HANDLE(h);
+  return h->be->set_shared(shared != 0);
+}
 fg_status fg_set_wait_limit(fg_lattice* h, double seconds) {
   FG_CHECK_HANDLE(h);
   if (!(seconds >= 0.0)) return h->fail(FG_EINVAL, "wait limit must be >= 0");

@@ -93,6 +93,7 @@ struct IBackend {
   virtual fg_status reunitarize_all() = 0;
   virtual fg_status random_gauge() = 0;
   virtual fg_status set_rng_position(unsigned long long pos) = 0;
+  virtual fg_status set_shared(bool shared) = 0;
 };
 
 }  // namespace fg

@@ -94,6 +94,7 @@ SIGNATURES = {
                                          C.POINTER(FgTrajResult)]),
     "fg_launch_count": (C.c_longlong, [_vp]),
     "fg_sync": (_i, [_vp]),
+    "fg_set_shared": (_i, [_vp, _i]),
     "fg_set_wait_limit": (_i, [_vp, _d]),
     "fg_device_bytes": (C.c_ulonglong, [_vp]),
     "fg_action_sums_noalloc": (_i, [_vp, _vp, C.POINTER(C.c_int), _d, _vp, _vp]),
@@ -356,6 +357,9 @@ class Lattice:
 
     def launch_count(self):
         return int(self._lib.fg_launch_count(self._h))
+
+    def set_shared(self, shared=True):
+        self._call("fg_set_shared", int(shared))
 
     def set_wait_limit(self, seconds):
         self._call("fg_set_wait_limit", float(seconds))

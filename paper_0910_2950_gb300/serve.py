@@ -153,15 +153,19 @@ class TrajectoryServer:
         self.cg_tol = cg_tol
         self.cg_tol_action = cg_tol_action
         self.clock = clock
-        self.lattice_factory = lattice_factory or (
-            lambda spec: _fg.Lattice(spec.dims, spec.beta, kappa=spec.kappa, precision=self.precision,
-                                     cg_tol=self.cg_tol, cg_tol_action=self.cg_tol_action, seed=spec.seed))
+        self.lattice_factory = lattice_factory or self._lattice
         self.chains = {}
         self.resident_bytes = 0
         self.evictions = 0
         self.peak_resident_bytes = 0
         self._lock = threading.Lock()
         self._pool = cf.ThreadPoolExecutor(max_workers=slots)
+
+    def _lattice(self, spec):
+        lat = _fg.Lattice(spec.dims, spec.beta, kappa=spec.kappa, precision=self.precision, cg_tol=self.cg_tol,
+                          cg_tol_action=self.cg_tol_action, seed=spec.seed)
+        lat.set_shared(self.slots > 1)   # several slots run at the same time
+        return lat
 
     # -- chain residency ------------------------------------------------
     def _make_resident(self, ch: _Chain):
