@@ -50,6 +50,7 @@ class Backend final : public IBackend {
 
   ~Backend() override {
     for (void* p : allocs_) cudaFree(p);
+    if (W_) cudaFree(W_);
     if (host_out_) cudaFreeHost(host_out_);
     if (mapped_) cudaFreeHost(mapped_);
     for (int i = 0; i < 2; ++i) {
@@ -70,10 +71,7 @@ class Backend final : public IBackend {
     U_ = buf_[0];
     if ((s = alloc(&P_, mom_bytes)) != FG_OK) return s;
     if ((s = alloc(&F_, mom_bytes)) != FG_OK) return s;
-    if (kPlaquetteForce<R>) {
-      if ((s = alloc(&W_, (size_t)6 * 4 * V * sizeof(C2))) != FG_OK) return s;
-      if ((s = init_force_rows()) != FG_OK) return s;
-    }
+    if (kPlaquetteForce<R> && (s = init_force_rows()) != FG_OK) return s;
     if ((s = alloc((void**)&h0_, V * sizeof(double))) != FG_OK) return s;
     for (int k = 0; k < 2; ++k)
       if ((s = alloc((void**)&sgc_[k], V * sizeof(double))) != FG_OK) return s;
@@ -122,6 +120,7 @@ class Backend final : public IBackend {
       return cuda_fail("momenta upload");
     s = run(KC_CONVERT, [&] { return launch_mom_to_device<R>(g_, canon_, P_, st_); });
     if (s != FG_OK) return s;
+    if (unitary_) plaquettes();   // forces will follow
     return sync();
   }
   fg_status get_momenta(double* host) override { return download_mom(P_, host); }
@@ -442,7 +441,35 @@ class Backend final : public IBackend {
   void* P_ = nullptr;
   void* F_ = nullptr;
   ForceRows rows_{};
-  void* W_ = nullptr;   // plaquette field of the force evaluation in progress
+  // Plaquette field of the force evaluation in progress (384 bytes a site):
+  // allocated when the first force or momenta ask for it, and given up for the
+  // staple sums where memory does not suffice for it or for anything else of
+  // the handle, so that a lattice that fits without it runs.  FG_PLAQUETTES=0
+  // in the environment does without it from the start.
+  void* W_ = nullptr;
+  bool no_plaquettes_ = plaquettes_off();
+  void* plaquettes() {
+    if (!kPlaquetteForce<R> || no_plaquettes_) return nullptr;
+    const size_t bytes = (size_t)6 * 4 * g_.V * sizeof(C2);
+    if (W_ == nullptr) {
+      if (cudaMalloc(&W_, bytes) == cudaSuccess) {
+        h_->dev_bytes += bytes;
+      } else {
+        cudaGetLastError();
+        W_ = nullptr;
+        no_plaquettes_ = true;
+      }
+    }
+    return W_;
+  }
+  bool drop_plaquettes() {
+    if (W_ == nullptr) return false;
+    cudaFree(W_);   // waits for the launches that use it
+    h_->dev_bytes -= (size_t)6 * 4 * g_.V * sizeof(C2);
+    W_ = nullptr;
+    no_plaquettes_ = true;
+    return true;
+  }
   // Whether the current links are unitary to R, which the plaquette form of
   // the force needs (kUnitaryWithin): measured whenever links enter and after
   // every trajectory and step, so that the form depends on the links alone
@@ -608,7 +635,12 @@ class Backend final : public IBackend {
 
   fg_status alloc(void** p, size_t bytes) {
     *p = nullptr;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();   // or the next launch reports it
+      if (drop_plaquettes()) e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) {
       cudaGetLastError();
       *p = nullptr;
       return h_->fail(FG_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed");
@@ -686,7 +718,7 @@ class Backend final : public IBackend {
     ForceArgs a;
     std::memset(&a, 0, sizeof(a));
     a.U = Uf;
-    a.W = unitary_ ? W_ : nullptr;
+    a.W = unitary_ ? plaquettes() : nullptr;
     a.P = P_;
     a.Ubase = Uf;
     a.beta = h_->prm.beta;

@@ -311,6 +311,7 @@ class Batch final : public IBatch {
   ~Batch() override {
     for (auto& g : graphs_) cudaGraphExecDestroy(g.exec);
     for (void* p : allocs_) cudaFree(p);
+    if (W_) cudaFree(W_);
     if (host_out_) cudaFreeHost(host_out_);
   }
 
@@ -348,7 +349,6 @@ class Batch final : public IBatch {
     cur_ = 0;
     if ((s = alloc(&P_, mom_bytes_)) != FG_OK) return s;
     if ((s = alloc(&F_, mom_bytes_)) != FG_OK) return s;
-    if (kPlaquetteForce<R> && (s = alloc(&W_, woff)) != FG_OK) return s;
     if ((s = alloc((void**)&h0_, sites_ * sizeof(double))) != FG_OK) return s;
     if ((s = alloc((void**)&d_out_, (size_t)n * kChainOut * sizeof(double))) != FG_OK) return s;
     if ((s = alloc((void**)&d_acc_, (size_t)n * sizeof(int))) != FG_OK) return s;
@@ -382,7 +382,13 @@ class Batch final : public IBatch {
       if ((s = alloc((void**)&d_partial_[hi], (size_t)3 * tl.size() * sizeof(double))) != FG_OK) return s;
     }
     unitary_.assign(n, 1);
-    if (kPlaquetteForce<R> && (s = init_force_rows()) != FG_OK) return s;
+    if constexpr (kPlaquetteForce<R>) {
+      if (!plaquettes_off() && cudaMalloc(&W_, woff) != cudaSuccess) {
+        cudaGetLastError();
+        W_ = nullptr;
+      }
+      if ((s = init_force_rows()) != FG_OK) return s;
+    }
     if (b_->prm.tile == 16) hsel_ = 0;
     else if (b_->prm.tile == 32) hsel_ = 1;
     else if (b_->prm.tile == 64) hsel_ = 2;
@@ -547,7 +553,10 @@ class Batch final : public IBatch {
   int cur_ = 0;
   void* P_ = nullptr;
   void* F_ = nullptr;
-  void* W_ = nullptr;     // plaquette field of the force evaluation in progress
+  // Plaquette field of the force evaluation in progress; null, and every chain
+  // with the staple sums, where memory does not suffice for it or for anything
+  // else of the batch.
+  void* W_ = nullptr;
   // Rows of all chains: first those of the chains whose links are unitary to
   // R, which take the plaquette form of the force, then the others', which
   // take the staple sums (as Backend::unitary_, chain by chain).
@@ -580,7 +589,7 @@ class Batch final : public IBatch {
     std::vector<int2> rows;
     for (int pass = 1; pass >= 0; --pass) {
       for (int c = 0; c < (int)cds_.size(); ++c)
-        if (unitary_[c] == pass)
+        if ((unitary_[c] && W_ != nullptr) == (pass != 0))
           for (int i = 0; i < cds_[c].g.Vh; i += 32) rows.push_back(make_int2(c, i));
       if (pass) nplaq_ = (int)rows.size();
     }
@@ -623,13 +632,24 @@ class Batch final : public IBatch {
   }
   fg_status alloc(void** p, size_t bytes) {
     *p = nullptr;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();   // or the next launch reports it
+      if (drop_plaquettes()) e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) {
       cudaGetLastError();
       *p = nullptr;
       return b_->fail(FG_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed");
     }
     allocs_.push_back(*p);
     return FG_OK;
+  }
+  bool drop_plaquettes() {
+    if (W_ == nullptr) return false;
+    cudaFree(W_);   // waits for the launches that use it
+    W_ = nullptr;
+    return d_rows_ == nullptr || upload_rows() == FG_OK;   // init uploads them otherwise
   }
   fg_status ensure_canon(size_t n) {
     if (canon_n_ >= n) return FG_OK;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstdlib>
 #include <type_traits>
 
 namespace fg {
@@ -42,6 +43,11 @@ struct ForceArgs {
 // launches), or always by staples (one).
 template <typename R>
 constexpr bool kPlaquetteForce = !std::is_same<R, float>::value;
+
+inline bool plaquettes_off() {
+  const char* e = std::getenv("FG_PLAQUETTES");
+  return e && e[0] == '0';
+}
 
 // The lattices of an FP64 or double-float force launch, cut into rows of 32
 // half-sites.
