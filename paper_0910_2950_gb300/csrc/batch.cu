@@ -9,9 +9,10 @@
 // assigns blocks of H half-sites (both parities, four directions) to chains,
 // and the kernels walk it with a grid-stride loop over a grid sized to fill
 // the GPU once (a persistent launch).  The double-float and FP64 force takes
-// the single-lattice launches instead, over the rows of all chains.  Per-link arithmetic is the same code
-// as for one lattice (gauge_device.cuh), so a chain gives the same links alone
-// and in a batch.  The dH of every chain is summed in FP64 per chain and the
+// the single-lattice launches instead, over the rows of the chains that take
+// its plaquette form and over those of the others.  Per-link arithmetic is the
+// same code as for one lattice (gauge_device.cuh), so a chain gives the same
+// links alone and in a batch.  The dH of every chain is summed in FP64 per chain and the
 // Metropolis step runs on the device, so a whole trajectory of all chains is
 // one CUDA graph: refresh, start energies, the fused force launches, end
 // energies, accept/reject, restore of rejected chains.  The tile size H is
@@ -304,8 +305,9 @@ class Batch final : public IBatch {
  public:
   typedef typename Vec2<R>::T C2;
   // Tile sizes compiled for this precision: 16, 32 and 64 half-sites, or 16
-  // and 32 for double-float links (their force kernel is several times the
-  // size of the FP32 one; fg_batch_create rejects tile 64 for them).
+  // and 32 for double-float links (a tile of 64 is a drift block of 512
+  // threads, with the 128 registers of a double-float exponential a whole
+  // SM's; fg_batch_create rejects tile 64 for them).
   static constexpr int kTileSizes = std::is_same<R, DF>::value ? 2 : 3;
   explicit Batch(fg_batch* b) : b_(b), st_(b->st) {}
   ~Batch() override {

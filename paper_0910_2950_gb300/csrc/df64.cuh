@@ -102,9 +102,8 @@ __device__ __forceinline__ DF operator*(DF a, float f) {
 // with the remainder r1 = a - q1 b, q3 = r2.hi / b.hi with r2 = r1 - q2 b.
 // One step is accurate to ~2^-47 but not unbiased: dividing r1 (which
 // contains -q1 b.lo) by b.hi instead of b leaves -q (b.lo / b.hi)^2, never
-// positive, so 1/x came out low by 6.5e-16 on average and every exp(iA)
-// (its coefficients divide by 9u^2 - w^2) shrank the links.  The second
-// step's own error is ~2^-72.
+// positive, so 1/x came out low by 6.5e-16 on average, and whatever was
+// scaled by such a quotient shrank.  The second step's own error is ~2^-72.
 __device__ __forceinline__ DF operator/(DF a, DF b) {
   const float q1 = __fdiv_rn(a.hi, b.hi);
   const DF r1 = a - b * q1;
@@ -250,7 +249,7 @@ __device__ __forceinline__ M3<DF> dagger_if(const M3<DF>& m, bool d) {
   return r;
 }
 
-// a b, a b^dagger and a^dagger b for unitary double-float matrices.
+// a b for unitary double-float matrices.
 __device__ __forceinline__ M3<DF> su3_mul(const M3<DF>& a, const M3<DF>& b) {
   M3<DF> c;
 #pragma unroll
@@ -269,42 +268,5 @@ __device__ __forceinline__ M3<DF> su3_mul(const M3<DF>& a, const M3<DF>& b) {
     }
   return c;
 }
-__device__ __forceinline__ M3<DF> su3_mul_nd(const M3<DF>& a, const M3<DF>& b) {
-  M3<DF> c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      Anchored re, im;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        re.add(a.e[i][k].re, b.e[j][k].re);
-        re.add(a.e[i][k].im, b.e[j][k].im);
-        im.add(a.e[i][k].im, b.e[j][k].re);
-        im.sub(a.e[i][k].re, b.e[j][k].im);
-      }
-      c.e[i][j] = cx<DF>(re.value(), im.value());
-    }
-  return c;
-}
-__device__ __forceinline__ M3<DF> su3_mul_dn(const M3<DF>& a, const M3<DF>& b) {
-  M3<DF> c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      Anchored re, im;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        re.add(a.e[k][i].re, b.e[k][j].re);
-        re.add(a.e[k][i].im, b.e[k][j].im);
-        im.add(a.e[k][i].re, b.e[k][j].im);
-        im.sub(a.e[k][i].im, b.e[k][j].re);
-      }
-      c.e[i][j] = cx<DF>(re.value(), im.value());
-    }
-  return c;
-}
-
 
 }  // namespace fg

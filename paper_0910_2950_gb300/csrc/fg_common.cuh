@@ -54,12 +54,6 @@ template <typename R> __device__ __forceinline__ void cmac_jc(Cx<R>& acc, Cx<R> 
   acc.re = fma(a.re, b.re, acc.re); acc.re = fma(a.im, b.im, acc.re);
   acc.im = fma(a.im, b.re, acc.im); acc.im = fma(-a.re, b.im, acc.im);
 }
-// acc += conj(a) * conj(b)
-template <typename R> __device__ __forceinline__ void cmac_cc(Cx<R>& acc, Cx<R> a, Cx<R> b) {
-  acc.re = fma(a.re, b.re, acc.re); acc.re = fma(-a.im, b.im, acc.re);
-  acc.im = fma(-a.re, b.im, acc.im); acc.im = fma(-a.im, b.re, acc.im);
-}
-
 template <typename R> struct M3 {
   Cx<R> e[3][3];
 };
@@ -115,20 +109,6 @@ template <typename R> __device__ __forceinline__ M3<R> mul_nd(const M3<R>& a, co
       Cx<R> s = cx<R>(0, 0);
 #pragma unroll
       for (int k = 0; k < 3; ++k) cmac_jc(s, a.e[i][k], b.e[j][k]);
-      c.e[i][j] = s;
-    }
-  return c;
-}
-// c = a^dagger * b
-template <typename R> __device__ __forceinline__ M3<R> mul_dn(const M3<R>& a, const M3<R>& b) {
-  M3<R> c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      Cx<R> s = cx<R>(0, 0);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) cmac_cj(s, a.e[k][i], b.e[k][j]);
       c.e[i][j] = s;
     }
   return c;

@@ -13,8 +13,9 @@
 //    (summed as site-by-site differences).
 //  * refresh_momenta_kernel: unit-Gaussian momenta from a counter-based RNG.
 //
-// One thread per link; a block is 64 consecutive checkerboard sites x 4
-// directions, so the four links of a site and their staples share L1/L2 lines.
+// One thread per link (or plaquette); blocks take 32 consecutive half-sites of
+// a parity in all directions, or some of their warps, so the links of a site
+// and their staples share L1/L2 lines.
 #include <type_traits>
 
 #include "fg_common.cuh"
