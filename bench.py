@@ -1129,7 +1129,8 @@ def run_ours(args):
     roof = {"bound": "alu", "achieved": achieved, "peak": peak,
             "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic,
-            "traffic_note": "bytes per launch: 203 B/link measured by ncu at 28^4, scaled by links" if traffic
+            "traffic_note": f"bytes per launch: {FORCE_TRAFFIC_BYTES_PER_LINK} B/link measured by ncu at 28^4, scaled by "
+                            "links" if traffic
             else None,
             "peak_derivation": f"{sm_count} SMs x 128 FP32 lanes x 2 flop x {sm_max_mhz:g} MHz (maximum SM clock "
                                "sampled by nvidia-smi during the timed region); FP64 at 1/64 of it",

@@ -141,7 +141,8 @@ typedef struct {
   int precision;           /* fg_precision (default FG_FP64); FG_DF64 needs kappa == 0 */
   int link_reals;          /* 18 (full) or 12 (two rows + reconstruction); default 18 */
   int reunitarize;         /* 1: re-project links onto SU(3) after every drift;
-                              default 0 for FG_FP64 and FG_DF64, 1 for FG_FP32 */
+                              default 0 for FG_FP64 and FG_DF64, 1 for FG_FP32.
+                              12-real links are re-projected in any case */
   double cg_tol;           /* relative residual |phi - M x| / |phi| for force solves (1e-10) */
   double cg_tol_action;    /* the same for the action solve at trajectory end (1e-12) */
   int cg_maxiter;          /* CG iteration cap (default 20000) */

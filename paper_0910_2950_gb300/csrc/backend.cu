@@ -387,11 +387,11 @@ class Backend final : public IBackend {
     sf0_valid_ = false;
     if ((s = execute(ops, dt, start)) != FG_OK) return s;
     if ((s = energy(1, P_, 3, nullptr, sgc_[1 - sgc_cur_])) != FG_OK) return s;
-    if ((s = queue_unitarity()) != FG_OK) return s;
+    if (!drifts_project() && (s = queue_unitarity()) != FG_OK) return s;
     if ((s = fetch(7)) != FG_OK) return s;
     double o[6];
     std::memcpy(o, host_out_, sizeof(o));
-    const bool unitary1 = read_unitarity();
+    const bool unitary1 = drifts_project() || read_unitarity();
     double sf1 = 0.0;
     if (ferm_ && (s = fermion_action(U_, &sf1)) != FG_OK) return s;
     r->S_gauge0 = o[0];
@@ -472,9 +472,11 @@ class Backend final : public IBackend {
   }
   // Whether the current links are unitary to R, which the plaquette form of
   // the force needs (kUnitaryWithin): measured whenever links enter and after
-  // every trajectory and step, so that the form depends on the links alone
-  // and a chain goes on from a stored configuration with the same bits.
+  // every trajectory and step whose drifts do not project them, so that the
+  // form depends on the links alone and a chain goes on from a stored
+  // configuration with the same bits.
   bool unitary_ = true;
+  bool drifts_project() const { return NC == 6 || h_->prm.reunitarize; }
   bool flag_set_ = false;   // the device's flag (dout_ + 6) is up
   double* h0_ = nullptr;
   // per-site gauge action of the current links (sgc_[sgc_cur_]) and of the

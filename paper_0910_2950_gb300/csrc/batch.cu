@@ -507,7 +507,7 @@ class Batch final : public IBatch {
       bool changed = false;
       for (int c = 0; c < b_->prm.nchains; ++c) {
         const double* o = host_out_ + (size_t)c * kChainOut;
-        const char u = o[kOutOffUnitary] == 0.0;
+        const char u = drifts_project() || o[kOutOffUnitary] == 0.0;
         if (o[6] != 0.0 && u != unitary_[c]) {
           unitary_[c] = u;
           changed = true;
@@ -565,6 +565,7 @@ class Batch final : public IBatch {
   int2* d_rows_ = nullptr;
   int nrows_ = 0, nplaq_ = 0;
   std::vector<char> unitary_;
+  bool drifts_project() const { return NC == 6 || b_->prm.reunitarize; }
   double* h0_ = nullptr;
   ChainDesc* d_chains_h_[3] = {nullptr, nullptr, nullptr};
   Tile* d_tiles_[3] = {nullptr, nullptr, nullptr};
@@ -881,7 +882,7 @@ class Batch final : public IBatch {
     if ((s = misc(1, buf_[cur], 1)) != FG_OK) return s;
     if ((s = misc(2, nullptr, 0, 0, 0, nullptr, nullptr, 3)) != FG_OK) return s;
     if constexpr (kPlaquetteForce<R>) {
-      if ((s = lrun([&] {
+      if (!drifts_project() && (s = lrun([&] {
              return launch_unitarity<R, NC>(rows_of(0, nrows_), buf_[cur], d_out_ + kOutOffUnitary, kChainOut, st_);
            })) != FG_OK)
         return s;

@@ -48,8 +48,77 @@ __device__ __forceinline__ M3<R> link_mul(const M3<R>& a, const M3<R>& b) {
   else return mul(a, b);
 }
 
+// reunitarize of a product of two unitary matrices, rows 0 and 1.  The
+// corrections are a few roundings: they are formed to first order, the three
+// side by side, and in double-float added in FP32 (the general form took 6% of
+// a double-float 12-real trajectory, this one 2%); where their squares would
+// show, the general form takes over.  The norms are summed with all terms of a
+// square: anchored double-float sums leave errors of one sign in them, 6e-15
+// of |U|^2 after every drift.
+template <typename R> __device__ __forceinline__ void project_product(M3<R>& u) {
+  constexpr bool kDF = std::is_same<R, DF>::value;
+  typedef typename std::conditional<kDF, float, R>::type C;   // a correction
+  constexpr C most = kDF ? C(0x1p-25f) : (std::is_same<R, double>::value ? C(0x1p-27) : C(0x1p-13f));
+  R n0 = R(-1), n1 = R(-1);   // |row0|^2 - 1, |row1|^2 - 1
+  C c0, c1, pr, pi;           // and <row0, row1>, with the signs of the corrections
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    n0 = fma(u.e[0][k].im, u.e[0][k].im, fma(u.e[0][k].re, u.e[0][k].re, n0));
+    n1 = fma(u.e[1][k].im, u.e[1][k].im, fma(u.e[1][k].re, u.e[1][k].re, n1));
+  }
+  if constexpr (kDF) {
+    Anchored re, im;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const Cx<DF> a = u.e[0][k], b = u.e[1][k];
+      re.add(a.re, b.re);
+      re.add(a.im, b.im);
+      im.add(a.re, b.im);
+      im.sub(a.im, b.re);
+    }
+    c0 = -0.5f * n0.hi;
+    c1 = -0.5f * n1.hi;
+    pr = -re.value().hi;
+    pi = -im.value().hi;
+  } else {
+    Cx<R> p = cx<R>(R(0), R(0));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) cmac_cj(p, u.e[0][k], u.e[1][k]);
+    c0 = R(-0.5) * n0;
+    c1 = R(-0.5) * n1;
+    pr = -p.re;
+    pi = -p.im;
+  }
+  if (fabs(c0) + fabs(c1) + fabs(pr) + fabs(pi) < most) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      Cx<R>& a = u.e[0][k];
+      Cx<R>& b = u.e[1][k];
+      if constexpr (kDF) {
+        const float x = a.re.hi, y = a.im.hi;
+        b.re = df_add_f(b.re, fmaf(c1, b.re.hi, fmaf(pr, x, -pi * y)));
+        b.im = df_add_f(b.im, fmaf(c1, b.im.hi, fmaf(pr, y, pi * x)));
+        a.re = df_add_f(a.re, c0 * x);
+        a.im = df_add_f(a.im, c0 * y);
+      } else {
+        const Cx<R> t = a;
+        b.re = fma(pr, t.re, fma(-pi, t.im, fma(c1, b.re, b.re)));
+        b.im = fma(pr, t.im, fma(pi, t.re, fma(c1, b.im, b.im)));
+        a = cx<R>(fma(c0, t.re, t.re), fma(c0, t.im, t.im));
+      }
+    }
+  } else {
+    reunitarize(u);
+  }
+}
+
 // Stores exp(i P) u, re-projected onto SU(3) if reunit is set (then rows 0
-// and 1 of the product suffice).
+// and 1 of the product suffice) and always with 12-real links: their third row
+// is rebuilt as (row0 x row1)^*, whose norm is off by the sum of the other
+// two's, and the next product mixes that back into them, so that the defect of
+// links that are only multiplied doubles every 20 trajectories (FP64 and
+// double-float links were off by 1e-11 and 2e-9 after 200, by 3e-3 and 1
+// after 800).
 template <typename R, int NC>
 __device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const Gauge<R, NC>& Uout, int mu, int s,
                                             int reunit) {
@@ -59,7 +128,9 @@ __device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const 
     reunitarize(un);
     Uout.store(mu, s, un);
   } else {
-    Uout.store(mu, s, link_mul(e, u));
+    M3<R> un = link_mul(e, u);
+    if constexpr (NC == 6) project_product(un);
+    Uout.store(mu, s, un);
   }
 }
 
@@ -414,9 +485,7 @@ template <> __device__ __forceinline__ DF beta6_of<DF>(const ChainDesc& cd) { re
 // 1e-7, links made unitary in 64 bits at 1e-15, and a chain that is never
 // re-projected moves away from there with the root of its length: FP64 18-real
 // chains reach 7e-14 and double-float ones 1.8e-11 in 800 trajectories of 16
-// drifts.  12-real links, whose third row is rebuilt from rows that are not
-// quite orthonormal, leave unitarity far faster (1e-11 after 200), so the
-// defect is taken anew after every trajectory.
+// drifts.  The defect is therefore taken anew after every trajectory.
 template <typename R>
 constexpr double kUnitaryWithin = std::is_same<R, double>::value ? 0x1p-42 : 0x1p-35;
 
