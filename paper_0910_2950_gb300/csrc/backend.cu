@@ -750,7 +750,26 @@ class Backend final : public IBackend {
     const char* e = std::getenv("FG_SPLIT_EXP");
     return e ? e[0] == '1' : std::is_same<R, DF>::value;
   }();
-  fg_status gauge_launch(int mode, const ForceArgs& a) {
+  // kick_pair for the coefficients in use (a trajectory has a handful)
+  struct PairOf {
+    double k, c;
+    KickPair pair;
+  };
+  std::vector<PairOf> pairs_;
+  KickPair pair_of(double k, double c) {
+    for (const PairOf& p : pairs_)
+      if (p.k == k && p.c == c) return p.pair;
+    if (pairs_.size() >= 32) pairs_.clear();
+    pairs_.push_back(PairOf{k, c, kick_pair(k, c)});
+    return pairs_.back().pair;
+  }
+  fg_status gauge_launch(int mode, ForceArgs a) {
+    if (std::is_same<R, float>::value && mode == FM_KICK_DRIFT) {
+      const KickPair d = pair_of(0.5 * a.cdrift, 0.0);
+      a.drift = DriftPair{d.a, d.b};
+    }
+    if (std::is_same<R, float>::value && (mode == FM_KICK || mode == FM_KICK_DRIFT))
+      a.pair = pair_of(a.ckick * (a.beta / 6.0), a.FF == nullptr ? 0.0 : a.ckick * (a.ffw == 0.0 ? 1.0 : a.ffw));
     if constexpr (kPlaquetteForce<R>) {
       if (a.W != nullptr) {
         const fg_status w = run(KC_PLAQUETTE, [&] { return launch_plaquettes<R, NC>(rows_, a.U, W_, st_); });

@@ -64,8 +64,8 @@ template <> struct TileBounds<64> { static constexpr int min_blocks = 1; };
 template <int NC, int MODE, int H>
 __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
     batch_force_kernel(const Tile* __restrict__ tiles, int ntiles, const ChainDesc* __restrict__ chains, char* U,
-                       char* P, char* F, char* Ubase, char* Uout, Coef<float> ckick0, Coef<float> cdrift, float cdisp,
-                       int reunit) {
+                       char* P, char* F, char* Ubase, char* Uout, const float2* __restrict__ kicks, float cdrift,
+                       float half, float cdisp, int reunit) {
   for (int b = blockIdx.x; b < ntiles; b += gridDim.x) {
     const Tile t = tiles[b];
     const ChainDesc& cd = chains[t.chain];
@@ -77,10 +77,8 @@ __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
     u.p = U + cd.goff; u.V = g.V;
     ub.p = Ubase ? Ubase + cd.goff : nullptr; ub.V = g.V;
     uo.p = Uout ? Uout + cd.goff : nullptr; uo.V = g.V;
-    // as make_kick
     constexpr bool kKick = MODE == FM_KICK || MODE == FM_KICK_DRIFT;
-    const float beta6 = kKick ? 1.0f : cd.beta6_hi;
-    const Coef<float> ckick = product(ckick0, Coef<float>{cd.beta6_hi, cd.beta6_lo}), ffw{1.0f, 0.0f};
+    const float2 kick = kKick ? kicks[t.chain] : make_float2(cd.beta6_hi, 0.0f);   // kick_pair's a and b
     Mom<float> p, f, ff;
     p.p = P ? P + cd.moff : nullptr; p.V = g.V;
     f.p = F ? F + cd.moff : nullptr; f.V = g.V;
@@ -90,13 +88,13 @@ __global__ void __launch_bounds__(8 * H, TileBounds<H>::min_blocks)
       // block takes the barriers (uniform tile loop)
       extern __shared__ float2 batch_tsh[];
       force_link_shared<NC, MODE, 2 * H>(reinterpret_cast<float2(*)[9][2 * H]>(batch_tsh), ok, s, u, p, f, ff, ub,
-                                         uo, g, beta6, ckick, cdrift, cdisp, reunit, ffw);
+                                         uo, g, kick.x, kick.y, cdrift, half, cdisp, reunit, 0.0f);
       __syncthreads();   // the next tile rewrites the slots
     } else {
       int c[4], par;
       cb_coords(g, s, c, par);
-      force_link_staples<float, NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
-                                   reunit, ffw);
+      force_link_staples<float, NC, MODE>(u, p, f, ff, ub, uo, g, c, s, (int)threadIdx.y, kick.x, kick.y, cdrift, half, cdisp,
+                                   reunit, 0.0f);
     }
   }
 }
@@ -110,7 +108,7 @@ constexpr size_t batch_force_smem() {
 template <typename R, int NC, int H>
 __global__ void __launch_bounds__(8 * H) batch_drift_kernel(const Tile* __restrict__ tiles, int ntiles,
                                                             const ChainDesc* __restrict__ chains, char* Uin,
-                                                            char* P, char* Uout, Coef<R> c, int reunit) {
+                                                            char* P, char* Uout, R c, R half, int reunit) {
   for (int b = blockIdx.x; b < ntiles; b += gridDim.x) {
     const Tile t = tiles[b];
     const ChainDesc& cd = chains[t.chain];
@@ -121,7 +119,7 @@ __global__ void __launch_bounds__(8 * H) batch_drift_kernel(const Tile* __restri
     uo.p = Uout + cd.goff; uo.V = cd.g.V;
     Mom<R> p;
     p.p = P + cd.moff; p.V = cd.g.V;
-    drift_link(ui, p, uo, s, (int)threadIdx.y, c, reunit);
+    drift_link(ui, p, uo, s, (int)threadIdx.y, c, half, reunit);
   }
 }
 
@@ -383,6 +381,8 @@ class Batch final : public IBatch {
         return cuda_fail("descriptor upload");
       if ((s = alloc((void**)&d_partial_[hi], (size_t)3 * tl.size() * sizeof(double))) != FG_OK) return s;
     }
+    if (!kPlaquetteForce<R> && (s = alloc((void**)&d_kicks_, (size_t)kMostKicks * n * sizeof(float2))) != FG_OK)
+      return s;
     unitary_.assign(n, 1);
     if constexpr (kPlaquetteForce<R>) {
       if (!plaquettes_off() && cudaMalloc(&W_, woff) != cudaSuccess) {
@@ -464,6 +464,7 @@ class Batch final : public IBatch {
     const int start = cur_;
     std::vector<Op> ops = trajectory_ops(integ, b_->prm.alpha, nsteps, true);
     int final_buf = start;
+    if (std::is_same<R, float>::value && (s = prepare_kicks(ops, dt)) != FG_OK) return s;
     if (b_->prm.use_graphs) {
       cudaGraphExec_t g = nullptr;
       for (auto& e : graphs_)
@@ -580,6 +581,46 @@ class Batch final : public IBatch {
   int hsel_ = 1;
   int sms_ = 152;
   std::vector<GraphEntry> graphs_;
+  // FP32 kicks: kick_pair's a and b of every chain for the coefficients in use
+  // (kick_c_, a row of d_kicks_ each).  Captured trajectories point into it.
+  static constexpr int kMostKicks = 32;
+  float2* d_kicks_ = nullptr;
+  std::vector<double> kick_c_;
+  const float2* kicks_of(double c) const {
+    for (size_t i = 0; i < kick_c_.size(); ++i)
+      if (kick_c_[i] == c) return d_kicks_ + i * cds_.size();
+    return nullptr;
+  }
+  // The rows of a trajectory's kicks, before it is queued or captured.
+  fg_status prepare_kicks(const std::vector<Op>& ops, double dt) {
+    fg_status s;
+    std::vector<double> fresh;
+    for (const Op& o : ops) {
+      const double c = o.c * dt;
+      if (o.kind != 'Q' && kicks_of(c) == nullptr && std::find(fresh.begin(), fresh.end(), c) == fresh.end())
+        fresh.push_back(c);
+    }
+    if (fresh.empty()) return FG_OK;
+    if (fresh.size() > kMostKicks) return b_->fail(FG_EINVAL, "too many different kicks in one step");
+    if (kick_c_.size() + fresh.size() > kMostKicks) {   // a trajectory has a handful
+      if ((s = sync()) != FG_OK) return s;
+      for (auto& g : graphs_) cudaGraphExecDestroy(g.exec);
+      graphs_.clear();
+      kick_c_.clear();
+      return prepare_kicks(ops, dt);
+    }
+    std::vector<float2> rows;
+    for (double c : fresh)
+      for (const ChainDesc& cd : cds_) {
+        const KickPair k = kick_pair(c * (cd.beta / 6.0));
+        rows.push_back(make_float2(k.a, k.b));
+      }
+    if (cudaMemcpyAsync(d_kicks_ + kick_c_.size() * cds_.size(), rows.data(), rows.size() * sizeof(float2),
+                        cudaMemcpyHostToDevice, st_) != cudaSuccess)
+      return cuda_fail("kick coefficient upload");
+    kick_c_.insert(kick_c_.end(), fresh.begin(), fresh.end());
+    return sync();  // the host copy goes out of scope
+  }
 
   fg_status init_force_rows() {
     nrows_ = 0;
@@ -690,12 +731,14 @@ class Batch final : public IBatch {
     const int gr = grid(nt, TileBounds<H>::min_blocks);
     return lrun([&] {
       const size_t sm = batch_force_smem<NC, H>();
-      const Coef<float> ckick = make_coef<float>(a.ckick), cdrift = make_coef<float>(a.cdrift);
+      const DriftPair drift = drift_pair(a.cdrift);
+      const float2* const kicks = mode == FM_KICK || mode == FM_KICK_DRIFT ? kicks_of(a.ckick) : nullptr;
       const Tile* tl = d_tiles_[hi];
       const ChainDesc* cds = d_chains_h_[hi];
 #define FG_FORCE(M)                                                                                                \
   batch_force_kernel<NC, M, H><<<gr, blk, sm, st_>>>(tl, nt, cds, (char*)a.U, (char*)a.P, (char*)a.F, (char*)a.Ubase, \
-                                                     (char*)a.Uout, ckick, cdrift, (float)a.cdisp, a.reunit)
+                                                     (char*)a.Uout, kicks, drift.x, drift.y, (float)a.cdisp,  \
+                                                     a.reunit)
       switch (mode) {
         case FM_STORE: FG_FORCE(FM_STORE); break;
         case FM_KICK: FG_FORCE(FM_KICK); break;
@@ -760,10 +803,16 @@ class Batch final : public IBatch {
   template <int H>
   fg_status drift_h(int hi, void* Uin, void* Uout, double c, void* G, int reunit) {
     const int nt = ntiles_[hi];
+    R x = R(c), y = R(0);
+    if constexpr (std::is_same<R, float>::value) {
+      const DriftPair d = drift_pair(c);
+      x = d.x;
+      y = d.y;
+    }
     return lrun([&] {
       batch_drift_kernel<R, NC, H><<<grid(nt, 2), dim3(2 * H, 4), 0, st_>>>(d_tiles_[hi], nt, d_chains_h_[hi],
-                                                                            (char*)Uin, (char*)G, (char*)Uout,
-                                                                            make_coef<R>(c), reunit);
+                                                                            (char*)Uin, (char*)G, (char*)Uout, x,
+                                                                            y, reunit);
       return cudaGetLastError();
     });
   }

@@ -172,45 +172,20 @@ template <typename R> __device__ __forceinline__ M3<R> alg_to_mat(const R p[8]) 
   return q;
 }
 
-// Step coefficients.  FP32 ones carry the part that FP32 leaves off: a kick of
-// c = 1/48 rounded to FP32 is too strong by 3e-8 of itself on every link, and
-// because the products of 1/48's periodic digits with a force often lie just
-// at the middle between two momenta, more than that.  Such errors have one
-// sign: the trajectory conserves T + (1 + e) S, and dH is off by e times what
-// S has gained, in proportion to the volume.  FG, dt = 1/8, from links still
-// relaxing: dH off by 0.112 at 32^4 and 6.3e-3 at 16^4 with rounded
-// coefficients, 4.2e-3 and 1.0e-3 with their low parts, which cost 56
-// operations of some 2300 a link and no time that could be measured.
-template <typename R> struct Coef {
-  R c;
-};
-template <> struct Coef<float> {
-  float c, lo;
-};
-template <typename R> inline Coef<R> make_coef(double x) { return Coef<R>{R(x)}; }
-template <> inline Coef<float> make_coef<float>(double x) { return Coef<float>{(float)x, (float)(x - (double)(float)x)}; }
-
-__host__ __device__ __forceinline__ Coef<float> product(Coef<float> a, Coef<float> b) {
-  const float c = a.c * b.c;
-  return Coef<float>{c, fmaf(a.c, b.lo, fmaf(a.lo, b.c, fmaf(a.c, b.c, -c)))};
-}
-
-// c x
-template <typename R> __device__ __forceinline__ R scaled(R x, Coef<R> c) { return x * c.c; }
-template <> __device__ __forceinline__ float scaled<float>(float x, Coef<float> c) {
-  const float d = __fmul_rn(c.c, x);
-  return __fadd_rn(d, __fmaf_rn(c.lo, x, __fmaf_rn(c.c, x, -d)));
-}
-// p - c f - low, rounded once: what the first rounding lost is
-// (p - s) - c f (p - s is exact unless the momentum changes by a factor of 2).
-template <typename R> __device__ __forceinline__ R kicked(R p, R f, R c, R low) { return fma(-c, f, p); }
-template <> __device__ __forceinline__ float kicked<float>(float p, float f, float c, float low) {
-  const float s = __fmaf_rn(-c, f, p);
-  return __fadd_rn(s, __fsub_rn(__fmaf_rn(-c, f, __fsub_rn(p, s)), low));
-}
-template <typename R> __device__ __forceinline__ R kicked(R p, R f, Coef<R> c) { return kicked(p, f, c.c, R(0)); }
-template <> __device__ __forceinline__ float kicked<float>(float p, float f, Coef<float> c) {
-  return kicked(p, f, c.c, c.lo * f);
+// h sum_a p^a lambda^a: the exponent of an FP32 drift (drift_pair).
+__device__ __forceinline__ M3<float> alg_to_mat(const float p[8], float h) {
+  const float t = 0.57735026918962576451f * p[7];
+  M3<float> q;
+  q.e[0][0] = cx<float>(h * (p[2] + t), 0.0f);
+  q.e[1][1] = cx<float>(h * (t - p[2]), 0.0f);
+  q.e[2][2] = cx<float>(-2.0f * h * t, 0.0f);
+  q.e[0][1] = cx<float>(h * p[0], -(h * p[1]));
+  q.e[1][0] = conj(q.e[0][1]);
+  q.e[0][2] = cx<float>(h * p[3], -(h * p[4]));
+  q.e[2][0] = conj(q.e[0][2]);
+  q.e[1][2] = cx<float>(h * p[5], -(h * p[6]));
+  q.e[2][1] = conj(q.e[1][2]);
+  return q;
 }
 
 // exp(i A) for Hermitian traceless A = f0 + f1 A + f2 A^2 (Cayley-Hamilton,

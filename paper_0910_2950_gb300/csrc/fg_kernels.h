@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <cstdlib>
 #include <type_traits>
 
@@ -25,6 +26,52 @@ enum ForceMode {
   FM_DISPLACE = 3     // U_out = exp(-i cdisp F(U)) U
 };
 
+// FP32 kicks P -= k F + c FF are formed as f = a F + w FF, P -= b f.  A
+// coefficient rounded to FP32 is an error of one sign: k = 1/48 comes out too
+// strong by 3e-8 on every link, and by more because products with its periodic
+// digits often lie just at the middle between two momenta, so the trajectory
+// conserves T + (1 + e) S and dH is off by e times what S has gained, in
+// proportion to the volume.  a and b are two FP32 numbers whose product is k to
+// some 1e-10 (and b w is c to 1e-9), with digits of no pattern: a is taken
+// near the golden ratio.  FG, dt = 1/8, from links still relaxing: dH off by
+// 5.0e-3 (32^4) and 5e-4 (16^4), with rounded coefficients 0.112 and 6.3e-3.
+// The device executes the same operations (coefficients with low parts, added
+// by compensated arithmetic, did as well and took 1.5% of a 32^4 trajectory).
+struct KickPair {
+  float a, b, w;
+};
+inline KickPair kick_pair(double k, double c = 0.0) {
+  KickPair best{0.0f, 0.0f, 0.0f};
+  double least = 1e300;
+  const int n = c != 0.0 ? 1024 : 128;
+  for (int i = 0; i < n; ++i) {
+    const double x = (double)(float)(1.6180339887498949 * (1.0 + i * 0x1p-18));
+    const float b = (float)((k != 0.0 ? k : c) / x);
+    double e = std::fabs(x * b - k);
+    float w = 0.0f;
+    if (c != 0.0) {
+      w = (float)(c / b);
+      e = std::fabs((double)w * b / c - 1.0);
+      if (k != 0.0) e = std::fmax(e, std::fabs(x * b / k - 1.0));
+    }
+    if (e < least) {
+      least = e;
+      best = KickPair{k != 0.0 ? (float)x : 0.0f, b, w};
+    }
+  }
+  return best;
+}
+
+// FP32 drifts by exp(i c P) likewise: the exponent is y sum_a (x p^a) lambda^a
+// with x y = c / 2.
+struct DriftPair {
+  float x, y;
+};
+inline DriftPair drift_pair(double c) {
+  const KickPair k = kick_pair(0.5 * c);
+  return DriftPair{k.a, k.b};
+}
+
 struct ForceArgs {
   const void* U;       // links at which the force is evaluated
   const void* W;       // their plaquette field (launch_plaquettes), or null for the staple sums (FP32: unused)
@@ -35,6 +82,8 @@ struct ForceArgs {
   void* Uout;          // output links (FM_KICK_DRIFT, FM_DISPLACE)
   double beta;
   double ckick, cdrift, cdisp;
+  KickPair pair;       // FP32 kicks, in place of ckick, beta and ffw
+  DriftPair drift;     // FP32 drifts, in place of cdrift
   double ffw;          // weight of FF relative to the gauge force (0 is treated as 1)
   int reunit;
 };

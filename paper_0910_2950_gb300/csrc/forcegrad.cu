@@ -15,6 +15,8 @@
 //    backend.cu).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "fg_common.cuh"
 #include "fg_fermion.h"
 #include "fg_kernels.h"
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(256) force_tangent_kernel(Gauge<R, NC> U, Gaug
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) kick_fg_kernel(Mom<R> P, Mom<R> F, Mom<R> G, int V, Coef<R> c,
+__global__ void __launch_bounds__(256) kick_fg_kernel(Mom<R> P, Mom<R> F, Mom<R> G, int V, R a, R b,
                                                       R shift) {
   const int s = blockIdx.x * kSites + threadIdx.x;
   const int mu = threadIdx.y;
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(256) kick_fg_kernel(Mom<R> P, Mom<R> F, Mom<R>
   F.load(mu, s, f);
   G.load(mu, s, gg);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) p[k] = kicked(p[k], fma(-shift, gg[k], f[k]), c);
+  for (int k = 0; k < 8; ++k) p[k] = fma(-b, a * fma(-shift, gg[k], f[k]), p[k]);
   P.store(mu, s, p);
 }
 
@@ -204,8 +206,14 @@ cudaError_t launch_force_tangent(const GeomH& g, const void* U, const void* dU, 
 template <typename R>
 cudaError_t launch_kick_fg(const GeomH& g, void* P, const void* F, const void* G, double c, double shift,
                            cudaStream_t st) {
-  kick_fg_kernel<R><<<grid_of(g.V), block_of(), 0, st>>>(mom_at<R>(P, g.V), mom_at<R>(F, g.V), mom_at<R>(G, g.V),
-                                                         g.V, make_coef<R>(c), R(shift));
+  R a = R(1.0f), b = R(c);
+  if constexpr (std::is_same<R, float>::value) {
+    const KickPair k = kick_pair(c);
+    a = k.a;
+    b = k.b;
+  }
+  kick_fg_kernel<R><<<grid_of(g.V), block_of(), 0, st>>>(mom_at<R>(P, g.V), mom_at<R>(F, g.V), mom_at<R>(G, g.V), g.V,
+                                                         a, b, R(shift));
   return cudaGetLastError();
 }
 template <typename RO, typename RX, typename RY>

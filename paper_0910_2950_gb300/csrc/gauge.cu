@@ -54,19 +54,19 @@ constexpr int kStapleSites = 32;
 template <int NC, int MODE>
 __global__ void __launch_bounds__(4 * kStapleSites, kStapleMinBlocks<NC>)
     staple_force_kernel(Gauge<float, NC> U, Mom<float> P, Mom<float> F, Mom<float> FF, Gauge<float, NC> Ubase,
-                        Gauge<float, NC> Uout, Geom g, float beta6, Coef<float> ckick, Coef<float> cdrift, float cdisp,
-                        int reunit, Coef<float> ffw) {
+                        Gauge<float, NC> Uout, Geom g, float beta6, float ckick, float cdrift, float half, float cdisp,
+                        int reunit, float ffw) {
   const int i = (int)(blockIdx.x >> 1) * kStapleSites + (int)threadIdx.x, s = (int)(blockIdx.x & 1) * g.Vh + i;
   const bool ok = i < g.Vh;
   if constexpr (kForceSharedT<float, NC>) {
     __shared__ float2 tsh[6][9][kStapleSites];
-    force_link_shared<NC, MODE, kStapleSites>(tsh, ok, s, U, P, F, FF, Ubase, Uout, g, beta6, ckick, cdrift, cdisp, reunit,
+    force_link_shared<NC, MODE, kStapleSites>(tsh, ok, s, U, P, F, FF, Ubase, Uout, g, beta6, ckick, cdrift, half, cdisp, reunit,
                                     ffw);
   } else {
     if (!ok) return;
     int c[4], par;
     cb_coords(g, s, c, par);
-    force_link_staples<float, NC, MODE>(U, P, F, FF, Ubase, Uout, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, cdisp,
+    force_link_staples<float, NC, MODE>(U, P, F, FF, Ubase, Uout, g, c, s, (int)threadIdx.y, beta6, ckick, cdrift, half, cdisp,
                                  reunit, ffw);
   }
 }
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kForceThreads, FG_PLAQ_MIN_BLOCKS)
 template <typename R, int NC, int MODE>
 __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
     link_force_kernel(const __grid_constant__ ForceRows r, char* U, char* W, char* P, char* F, char* FF, char* Ubase,
-                      char* Uout, Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit, Coef<R> ffw) {
+                      char* Uout, R ckick, R cdrift, R half, R cdisp, int reunit, R ffw) {
   RowSite o;
   if (!row_site(r, 4, o)) return;
   const ChainDesc& cd = *o.cd;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
   p.p = P + cd.moff; p.V = g.V;
   f.p = F + cd.moff; f.V = g.V;
   ff.p = FF == nullptr ? nullptr : FF + cd.moff; ff.V = g.V;
-  force_link_plaquettes<R, NC, MODE>(u, w, p, f, ff, ub, uo, g, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, cdisp,
+  force_link_plaquettes<R, NC, MODE>(u, w, p, f, ff, ub, uo, g, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, half, cdisp,
                                      reunit, ffw);
 }
 
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
 template <typename R, int NC, int MODE>
 __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
     staple_rows_kernel(const __grid_constant__ ForceRows r, char* U, char* P, char* F, char* FF, char* Ubase,
-                       char* Uout, Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit, Coef<R> ffw) {
+                       char* Uout, R ckick, R cdrift, R half, R cdisp, int reunit, R ffw) {
   RowSite o;
   if (!row_site(r, 4, o)) return;
   const ChainDesc& cd = *o.cd;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kForceThreads, FG_LINK_MIN_BLOCKS)
   ff.p = FF == nullptr ? nullptr : FF + cd.moff; ff.V = g.V;
   int c[4], par;
   cb_coords(g, o.s, c, par);
-  force_link_staples<R, NC, MODE>(u, p, f, ff, ub, uo, g, c, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, cdisp, reunit,
+  force_link_staples<R, NC, MODE>(u, p, f, ff, ub, uo, g, c, o.s, o.part, beta6_of<R>(cd), ckick, cdrift, half, cdisp, reunit,
                                   ffw);
 }
 
@@ -181,11 +181,11 @@ __global__ void __launch_bounds__(kForceThreads)
 // One thread a link: warp w takes direction w mod 4 of 32 consecutive sites.
 template <typename R, int NC>
 __global__ void __launch_bounds__(256) drift_kernel(Gauge<R, NC> Uin, Mom<R> P, Gauge<R, NC> Uout,
-                                                    int V, Coef<R> c, int reunit) {
+                                                    int V, R c, R half, int reunit) {
   const unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int s = (int)(w >> 2) * 32 + (int)(threadIdx.x & 31);
   if (s >= V) return;
-  drift_link(Uin, P, Uout, s, (int)(w & 3), c, reunit);
+  drift_link(Uin, P, Uout, s, (int)(w & 3), c, half, reunit);
 }
 
 template <typename R, int NC>
@@ -444,16 +444,12 @@ static cudaError_t launch_staple_force(const GeomH& gh, int mode, const ForceArg
   auto FF = mom_of<float>(a.FF, V);
   auto Ub = gauge_of<float, NC>(a.Ubase, V);
   auto Uo = gauge_of<float, NC>(a.Uout, V);
-  KickCoef<float> k = make_kick(a.beta, a.ckick, a.ffw == 0.0 ? 1.0 : a.ffw);
-  if (mode == FM_STORE || mode == FM_DISPLACE) {  // the force itself
-    k.beta6 = float(a.beta / 6.0);
-    k.ffw = make_coef<float>(a.ffw == 0.0 ? 1.0 : a.ffw);
-  }
-  const Coef<float> cdrift = make_coef<float>(a.cdrift);
+  const bool kick = mode == FM_KICK || mode == FM_KICK_DRIFT;
+  const KickPair k = kick ? a.pair : KickPair{float(a.beta / 6.0), 0.0f, float(a.ffw == 0.0 ? 1.0 : a.ffw)};
   const int nb = 2 * ((g.Vh + kStapleSites - 1) / kStapleSites);
 #define FG_FORCE(M)                                                                                          \
-  staple_force_kernel<NC, M><<<nb, dim3(kStapleSites, 4), 0, st>>>(U, P, F, FF, Ub, Uo, g, k.beta6, k.kick, cdrift, \
-                                                                  float(a.cdisp), a.reunit, k.ffw)
+  staple_force_kernel<NC, M><<<nb, dim3(kStapleSites, 4), 0, st>>>(U, P, F, FF, Ub, Uo, g, k.a, k.b,        \
+                                                                  a.drift.x, a.drift.y, float(a.cdisp), a.reunit, k.w)
   switch (mode) {
     case FM_STORE: FG_FORCE(FM_STORE); break;
     case FM_KICK: FG_FORCE(FM_KICK); break;
@@ -497,8 +493,7 @@ cudaError_t launch_unitarity(const ForceRows& r, const void* U, double* flag, in
 
 template <typename R, int NC>
 static cudaError_t launch_link_force(const ForceRows& r, int mode, const ForceArgs& a, cudaStream_t st) {
-  const Coef<R> ckick = make_coef<R>(a.ckick), ffw = make_coef<R>(a.ffw == 0.0 ? 1.0 : a.ffw);
-  const Coef<R> cdrift = make_coef<R>(a.cdrift);
+  const R ckick = R(a.ckick), ffw = R(a.ffw == 0.0 ? 1.0 : a.ffw), cdrift = R(a.cdrift);
   const long long warps = 8LL * r.nrows;
   const int w = warps_per_block(warps, kForceThreads / 32);
   const unsigned nb = (unsigned)((warps + w - 1) / w);
@@ -506,11 +501,11 @@ static cudaError_t launch_link_force(const ForceRows& r, int mode, const ForceAr
   do {                                                                                                                \
     if (a.W != nullptr)                                                                                               \
       link_force_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.W, (char*)a.P, (char*)a.F, (char*)a.FF, \
-                                                         (char*)a.Ubase, (char*)a.Uout, ckick, cdrift, R(a.cdisp),    \
+                                                         (char*)a.Ubase, (char*)a.Uout, ckick, cdrift, R(0), R(a.cdisp), \
                                                          a.reunit, ffw);                                              \
     else                                                                                                              \
       staple_rows_kernel<R, NC, M><<<nb, 32 * w, 0, st>>>(r, (char*)a.U, (char*)a.P, (char*)a.F, (char*)a.FF,         \
-                                                          (char*)a.Ubase, (char*)a.Uout, ckick, cdrift, R(a.cdisp),   \
+                                                          (char*)a.Ubase, (char*)a.Uout, ckick, cdrift, R(0), R(a.cdisp), \
                                                           a.reunit, ffw);                                             \
   } while (0)
   switch (mode) {
@@ -536,9 +531,14 @@ cudaError_t launch_drift(const GeomH& gh, const void* Uin, const void* P, void* 
                          int reunit, cudaStream_t st) {
   const long long warps = 4LL * ((gh.V + 31) / 32);
   const int w = warps_per_block(warps, 8);
+  R x = R(c), y = R(0);
+  if constexpr (std::is_same<R, float>::value) {
+    const DriftPair d = drift_pair(c);
+    x = d.x;
+    y = d.y;
+  }
   drift_kernel<R, NC><<<(unsigned)((warps + w - 1) / w), 32 * w, 0, st>>>(
-      gauge_of<R, NC>(Uin, gh.V), mom_of<R>(P, gh.V), gauge_of<R, NC>(Uout, gh.V), gh.V, make_coef<R>(c),
-      reunit);
+      gauge_of<R, NC>(Uin, gh.V), mom_of<R>(P, gh.V), gauge_of<R, NC>(Uout, gh.V), gh.V, x, y, reunit);
   return cudaGetLastError();
 }
 
@@ -620,7 +620,7 @@ cudaError_t launch_mom_to_canon(const GeomH& gh, const void* P, double* canon, c
 // P -= c FF (kick with a force computed elsewhere: the pseudofermion force of
 // a two-level integrator's outer kicks).
 template <typename R>
-__global__ void __launch_bounds__(256) kick_ff_kernel(Mom<R> P, Mom<R> FF, int V, Coef<R> c) {
+__global__ void __launch_bounds__(256) kick_ff_kernel(Mom<R> P, Mom<R> FF, int V, R a, R b) {
   const int s = blockIdx.x * kSitesPerBlock + threadIdx.x;
   const int mu = threadIdx.y;
   if (s >= V) return;
@@ -628,13 +628,18 @@ __global__ void __launch_bounds__(256) kick_ff_kernel(Mom<R> P, Mom<R> FF, int V
   P.load(mu, s, p);
   FF.load(mu, s, f);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) p[k] = kicked(p[k], f[k], c);
+  for (int k = 0; k < 8; ++k) p[k] = fma(-b, a * f[k], p[k]);
   P.store(mu, s, p);
 }
 template <typename R>
 cudaError_t launch_kick_ff(const GeomH& gh, void* P, const void* FF, double c, cudaStream_t st) {
-  kick_ff_kernel<R><<<link_grid(gh.V), link_block(), 0, st>>>(mom_of<R>(P, gh.V), mom_of<R>(FF, gh.V), gh.V,
-                                                              make_coef<R>(c));
+  R a = R(1.0f), b = R(c);
+  if constexpr (std::is_same<R, float>::value) {
+    const KickPair k = kick_pair(c);
+    a = k.a;
+    b = k.b;
+  }
+  kick_ff_kernel<R><<<link_grid(gh.V), link_block(), 0, st>>>(mom_of<R>(P, gh.V), mom_of<R>(FF, gh.V), gh.V, a, b);
   return cudaGetLastError();
 }
 template cudaError_t launch_kick_ff<double>(const GeomH&, void*, const void*, double, cudaStream_t);

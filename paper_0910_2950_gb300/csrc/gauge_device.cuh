@@ -112,7 +112,8 @@ template <typename R> __device__ __forceinline__ void project_product(M3<R>& u) 
   }
 }
 
-// Stores exp(i P) u, re-projected onto SU(3) if reunit is set (then rows 0
+// Stores exp(i c P) u (FP32: drift_pair's x and y in place of c and `half`),
+// re-projected onto SU(3) if reunit is set (then rows 0
 // and 1 of the product suffice) and always with 12-real links: their third row
 // is rebuilt as (row0 x row1)^*, whose norm is off by the sum of the other
 // two's, and the next product mixes that back into them, so that the defect of
@@ -120,9 +121,13 @@ template <typename R> __device__ __forceinline__ void project_product(M3<R>& u) 
 // double-float links were off by 1e-11 and 2e-9 after 200, by 3e-3 and 1
 // after 800).
 template <typename R, int NC>
-__device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const Gauge<R, NC>& Uout, int mu, int s,
-                                            int reunit) {
-  const M3<R> e = expi_herm(alg_to_mat(p));
+__device__ __forceinline__ void drift_store(R p[8], R c, R half, const M3<R>& u, const Gauge<R, NC>& Uout, int mu,
+                                            int s, int reunit) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) p[k] *= c;
+  M3<R> e;
+  if constexpr (std::is_same<R, float>::value) e = expi_herm(alg_to_mat(p, half));
+  else e = expi_herm(alg_to_mat(p));
   if (reunit) {
     M3<R> un = mul_rows01(e, u);
     reunitarize(un);
@@ -134,46 +139,20 @@ __device__ __forceinline__ void drift_store(const R p[8], const M3<R>& u, const 
   }
 }
 
-// The coefficients of a kick P -= kick (beta6 f + ffw FF), FF the extra force
-// that joins the gauge force.  In FP32 beta / 6 goes into `kick` (beta6 = 1),
-// so that nothing is rounded in between, and ffw.lo is what kick.c ffw.c lacks.
-template <typename R> struct KickCoef {
-  R beta6;
-  Coef<R> kick, ffw;
-};
-inline KickCoef<float> make_kick(double beta, double c, double ffw) {
-  KickCoef<float> k;
-  const double b6 = beta / 6.0, w = b6 > 0.0 ? ffw / b6 : ffw;
-  k.beta6 = b6 > 0.0 ? 1.0f : 0.0f;
-  k.kick = b6 > 0.0 ? product(make_coef<float>(c), make_coef<float>(b6)) : make_coef<float>(c);
-  k.ffw.c = (float)w;
-  k.ffw.lo = (float)(c * ffw - (double)k.kick.c * (double)k.ffw.c);
-  return k;
-}
-
-// What MODE does with link (s, mu), f^a = Im Tr(lambda^a U A) given.
+// What MODE does with link (s, mu), f^a = Im Tr(lambda^a U A) given: the force
+// is beta6 f + ffw FF (FP32 kicks: kick_pair's a, w and b in place of beta6, ffw
+// and ckick).
 template <typename R, int NC, int MODE>
 __device__ __forceinline__ void force_apply(const Gauge<R, NC>& U, const Mom<R>& P, const Mom<R>& F, const Mom<R>& FF,
                                             const Gauge<R, NC>& Ubase, const Gauge<R, NC>& Uout, int s, int mu,
-                                            R f[8], R beta6, Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit,
-                                            Coef<R> ffw) {
-  // FP32: what c F lacks of the kick (KickCoef)
-  constexpr bool kLow = std::is_same<R, float>::value && (MODE == FM_KICK || MODE == FM_KICK_DRIFT);
-  R low[8];
+                                            R f[8], R beta6, R ckick, R cdrift, R half, R cdisp, int reunit, R ffw) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    f[k] = f[k] * beta6;
-    if constexpr (kLow) low[k] = ckick.lo * f[k];
-    else low[k] = R(0);
-  }
+  for (int k = 0; k < 8; ++k) f[k] = f[k] * beta6;
   if (FF.p != nullptr) {
     R ff[8];
     FF.load(mu, s, ff);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      f[k] = fma(ffw.c, ff[k], f[k]);
-      if constexpr (kLow) low[k] = fma(ffw.lo, ff[k], low[k]);
-    }
+    for (int k = 0; k < 8; ++k) f[k] = fma(ffw, ff[k], f[k]);
   }
   if (MODE == FM_STORE) {
     F.store(mu, s, f);
@@ -181,12 +160,10 @@ __device__ __forceinline__ void force_apply(const Gauge<R, NC>& U, const Mom<R>&
     R p[8];
     P.load(mu, s, p);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) p[k] = kicked(p[k], f[k], ckick.c, low[k]);
+    for (int k = 0; k < 8; ++k) p[k] = fma(-ckick, f[k], p[k]);
     P.store(mu, s, p);
     if (MODE == FM_KICK_DRIFT) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) p[k] = scaled(p[k], cdrift);
-      drift_store(p, Ubase.load(mu, s), Uout, mu, s, reunit);
+      drift_store(p, cdrift, half, Ubase.load(mu, s), Uout, mu, s, reunit);
     }
   } else {  // FM_DISPLACE
     // The displaced links only serve one force evaluation and are then
@@ -293,12 +270,12 @@ template <typename R, int NC, int MODE>
 __device__ __forceinline__ void force_link_staples(const Gauge<R, NC>& U, const Mom<R>& P, const Mom<R>& F,
                                                    const Mom<R>& FF, const Gauge<R, NC>& Ubase,
                                                    const Gauge<R, NC>& Uout, const Geom& g, const int c[4], int s,
-                                                   int mu, R beta6, Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit,
-                                                   Coef<R> ffw) {
+                                                   int mu, R beta6, R ckick, R cdrift, R half, R cdisp, int reunit,
+                                                   R ffw) {
   const M3<R> a = staple_sum(U, g, c, s, mu);
   R f[8];
   staple_force(U.load(mu, s), a, f);
-  force_apply<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
+  force_apply<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, half, cdisp, reunit, ffw);
 }
 
 // Whether the FP32 12-real force kernels share the upper-staple products of
@@ -345,8 +322,8 @@ template <int NC, int MODE, int NS>
 __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok, int s, const Gauge<float, NC>& U,
                                                   const Mom<float>& P, const Mom<float>& F, const Mom<float>& FF,
                                                   const Gauge<float, NC>& Ubase, const Gauge<float, NC>& Uout,
-                                                  const Geom& g, float beta6, Coef<float> ckick, Coef<float> cdrift,
-                                                  float cdisp, int reunit, Coef<float> ffw) {
+                                                  const Geom& g, float beta6, float ckick, float cdrift,
+                                                  float half, float cdisp, int reunit, float ffw) {
   const int x = threadIdx.x;
   const int mu = threadIdx.y;
   M3<float> a;
@@ -413,7 +390,7 @@ __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok,
   }
   float f[8];
   staple_force(U.load(mu, s), a, f);
-  force_apply<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
+  force_apply<float, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, half, cdisp, reunit, ffw);
 }
 
 // ---------------------------------------------------------------------------
@@ -777,22 +754,20 @@ template <typename R, int NC, int MODE>
 __device__ __forceinline__ void force_link_plaquettes(const Gauge<R, NC>& U, const Mom<R>& W, const Mom<R>& P,
                                                       const Mom<R>& F, const Mom<R>& FF, const Gauge<R, NC>& Ubase,
                                                       const Gauge<R, NC>& Uout, const Geom& g, int s, int mu, R beta6,
-                                                      Coef<R> ckick, Coef<R> cdrift, R cdisp, int reunit,
-                                                      Coef<R> ffw) {
+                                                      R ckick, R cdrift, R half, R cdisp, int reunit,
+                                                      R ffw) {
   R f[8];
   link_force(U, W, g, s, mu, f);
-  force_apply<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, cdisp, reunit, ffw);
+  force_apply<R, NC, MODE>(U, P, F, FF, Ubase, Uout, s, mu, f, beta6, ckick, cdrift, half, cdisp, reunit, ffw);
 }
 
 // U_out(s, mu) = exp(i c P) U_in(s, mu), the exact T-hat flow of section 2.
 template <typename R, int NC>
 __device__ __forceinline__ void drift_link(const Gauge<R, NC>& Uin, const Mom<R>& P, const Gauge<R, NC>& Uout,
-                                           int s, int mu, Coef<R> c, int reunit) {
+                                           int s, int mu, R c, R half, int reunit) {
   R p[8];
   P.load(mu, s, p);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) p[k] = scaled(p[k], c);
-  drift_store(p, Uin.load(mu, s), Uout, mu, s, reunit);
+  drift_store(p, c, half, Uin.load(mu, s), Uout, mu, s, reunit);
 }
 
 // Per-site energy h(x) = T(x) + S_G(x) (T = 0 if P is null), with
