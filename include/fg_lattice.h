@@ -198,7 +198,8 @@ const char *fg_last_error(const fg_lattice *h);
  * rebuilds a row from the other two).  FP64 and FG_DF64 forces of links that
  * are unitary to that precision use U^dagger U = 1; of links that are not
  * (a configuration held in single precision, say), and until fg_reunitarize,
- * they are formed by the staple sums, at 1.3 to 2.3 times the time. */
+ * they are formed by the staple sums (trajectories of 1.1 to 1.4 times the
+ * time). */
 fg_status fg_set_gauge(fg_lattice *h, const double *host_links);
 fg_status fg_get_gauge(fg_lattice *h, double *host_links);
 

@@ -411,12 +411,11 @@ __device__ __forceinline__ void force_link_shared(float2 (*tsh)[9][NS], bool ok,
 // Hermitian).  A site then takes 6 x 306 + 12 x 138 = 3492 multiply-adds
 // instead of the 4 x 13 x 108 = 5616 of a staple sum for every link.
 // Double-float and FP64 forces are bound by that arithmetic (FP32 and FP64
-// issue), so they take this form: a trajectory against the staple sums takes
-// 1.94 instead of 2.51 ms (double-float 16^4), 12.1 instead of 16.0 ms
-// (64-chain double-float batch), 3.03 instead of 4.6 ms (FP64 12^4), and on
-// small lattices, where a thread's serial chain counts, 0.45 instead of
-// 0.55 ms (double-float 8^4) and 1.32 instead of 3.00 ms (FP64 4^4, with its
-// warps spread over the SMs).  The FP32 force executes 18% fewer instructions
+// issue), so they take this form: an FG trajectory against the staple sums over
+// the same rows takes 1.65 instead of 2.25 ms (double-float 16^4), 7.56 instead
+// of 10.3 (24^4), 7.92 instead of 10.1 (FP64 16^4), and on small lattices 0.37
+// instead of 0.39 ms (double-float 8^4) and 0.67 instead of 0.85 (FP64 4^4).
+// The FP32 force executes 18% fewer instructions
 // this way but waits for the memory traffic of Q (193 + 233 us a launch pair
 // against 405 us at 32^4; 12% slower at 8^4): it stays with the staples.  One
 // launch of both kinds of work, link blocks waiting for the plaquettes they
