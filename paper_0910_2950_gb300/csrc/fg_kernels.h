@@ -32,8 +32,9 @@ enum ForceMode {
 // digits often lie just at the middle between two momenta, so the trajectory
 // conserves T + (1 + e) S and dH is off by e times what S has gained, in
 // proportion to the volume.  a and b are two FP32 numbers whose product is k to
-// some 1e-10 (and b w is c to 1e-9), with digits of no pattern: a is taken
-// near the golden ratio.  FG, dt = 1/8, from links still relaxing: dH off by
+// some 1e-10 (7e-9 at worst of 20000 coefficients; with b w = c beside it some
+// 1e-9, 1.4e-8 at worst), with digits of no pattern: a is taken near the golden
+// ratio.  FG, dt = 1/8, from links still relaxing: dH off by
 // 5.0e-3 (32^4) and 5e-4 (16^4), with rounded coefficients 0.112 and 6.3e-3.
 // The device executes the same operations (coefficients with low parts, added
 // by compensated arithmetic, did as well and took 1.5% of a 32^4 trajectory).
@@ -41,7 +42,8 @@ struct KickPair {
   float a, b, w;
 };
 inline KickPair kick_pair(double k, double c = 0.0) {
-  KickPair best{0.0f, 0.0f, 0.0f};
+  // for coefficients out of FP32's range, whose products say so
+  KickPair best = k != 0.0 ? KickPair{1.0f, (float)k, (float)(c / k)} : KickPair{0.0f, (float)c, c != 0.0 ? 1.0f : 0.0f};
   double least = 1e300;
   const int n = c != 0.0 ? 1024 : 128;
   for (int i = 0; i < n; ++i) {
