@@ -1563,6 +1563,7 @@ class Backend final : public IBackend {
     int checked = 0;     // device iterations whose residual the host has read
     int iters = 0;
     int pending = -1;    // event slot of the batch queued before the last one
+    int queued_at[2] = {0, 0};   // iterations queued up to the event of each slot
     mapped_->dev_iter = 0;
     for (;;) {
       bool converged = false;
@@ -1594,6 +1595,7 @@ class Backend final : public IBackend {
         queued += nb;
         const int slot = (pending + 1) & 1;
         if (cudaEventRecord(ev_[slot], st_) != cudaSuccess) return cuda_fail("event");
+        queued_at[slot] = queued;
         if (pending >= 0) {
           // wait for the batch before this one; the GPU keeps working on this one
           std::string why;
@@ -1612,7 +1614,10 @@ class Backend final : public IBackend {
               break;
             }
           }
-          const int upto = *(volatile int*)&mapped_->dev_iter;
+          // only the iterations up to the event: the batch on the GPU goes on
+          // counting, and where a reliable update lands would depend on timing
+          const int now = *(volatile int*)&mapped_->dev_iter;
+          const int upto = std::min(now, queued_at[pending]);
           const int first = checked + 1;
           double first_rr = -1.0, last = -1.0;
           for (int j = first; j <= upto; ++j) {
