@@ -388,7 +388,7 @@ typedef struct {
   const double *beta;      /* nchains couplings; copied */
   int precision;           /* FG_FP32 (default), FG_FP64 or FG_DF64 */
   int link_reals;          /* 18 or 12 */
-  int reunitarize;         /* -1: after every drift for FP32, never for FP64 and FG_DF64 */
+  int reunitarize;         /* -1: after every drift for FP32 and for 12-real links, otherwise not */
   double alpha;            /* PQPQP parameter for FG_OMELYAN (0.1932) */
   int tile;                /* half-sites per block: 16, 32 or 64; 0 = time all three on the
                               first trajectory and keep the fastest (autotuning) */

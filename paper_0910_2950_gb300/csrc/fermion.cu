@@ -60,7 +60,7 @@ template <> struct DslashMinBlocks<DF> { static constexpr int value = FG_DSLASH_
 // (GeomH::shared) the GPU is full without the split and its extra
 // instructions only cost: FP32 and double-float then never split.  Eight
 // concurrent slots of a Poisson mix of pure-gauge, 8^3 x 16 and 12^3 x 24
-// chains run 80.6 trajectories/s so, 61.3 with the split.
+// chains run 79 to 81 trajectories/s so, 61 with the split.
 #ifndef FG_SPLIT_MAX32
 #define FG_SPLIT_MAX32 24576
 #endif
